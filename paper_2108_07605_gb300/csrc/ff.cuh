@@ -177,6 +177,173 @@ __device__ __forceinline__ ff ff_log(ff x) {
   return y0 + t;
 }
 
+// Sums kept as hi + lo without renormalising after every term: the head by
+// an exact two-sum, the errors and low parts in one FP32 word (8 operations
+// against 20 for operator+; each term's rounding stays below 2^-47 of the
+// largest partial sum).  ff_norm closes a sum.
+__device__ __forceinline__ void ff_acc(ff& s, ff b) {
+  const ff t = two_sum(s.hi, b.hi);
+  s.hi = t.hi;
+  s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, b.lo));
+}
+// s += a b, the product's head exact (12 operations against 27)
+__device__ __forceinline__ void ff_fma_acc(ff& s, ff a, ff b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p);
+  e = __fmaf_rn(a.hi, b.lo, e);
+  e = __fmaf_rn(a.lo, b.hi, e);
+  const ff t = two_sum(s.hi, p);
+  s.hi = t.hi;
+  s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, e));
+}
+__device__ __forceinline__ ff ff_norm(ff s) { return fast_two_sum(s.hi, s.lo); }
+
+// Conversions through the bit patterns.  GB300's FP32 <-> FP64 conversion
+// instructions run at the rate of its FP64 pipes (measured: 17 cycles per
+// warp and SM, as a DFMA, against 0.26 for an FP32 or integer instruction),
+// so the moves between the two formats are integer work here.
+//
+// |d| < 2^-126 becomes 0, |d| >= 2^128 (and infinities, NaN) NaN; hi is the
+// nearest float, lo the 24 leading of the 28 bits that remain (dropped, 0, for
+// |d| < 2^-74).
+__device__ __forceinline__ ff ff_of_double(double d) {
+  const int h = __double2hiint(d), l = __double2loint(d);
+  const int mag = h & 0x7fffffff, sgn = h & 0x80000000;
+  const int tr = (int)(__funnelshift_l(l, mag, 3) - (896u << 23));   // truncated
+  const int up = (l >> 28) & 1;                       // the first bit below it
+  const int rest = (l & 0x1fffffff) - (up << 29);
+  int hb = tr + up;
+  if (mag < 0x38100000) hb = 0;                       // below 2^-126
+  if (mag >= 0x47f00000) hb = 0x7fffffff;             // 2^128 and above
+  const int sc = max((tr & 0x7f800000) - (52 << 23), 0);
+  const float lo = __fmul_rn(__int2float_rn(rest), __int_as_float(sc | sgn));
+  return ff(__int_as_float(hb | sgn), mag < 0x38100000 ? 0.f : lo);
+}
+// exact for 0 and normal numbers; denormals become 0
+__device__ __forceinline__ double double_of_float(float f) {
+  const int b = __float_as_int(f);
+  const int m = b & 0x7fffffff;
+  int h = (m >> 3) + (896 << 20);
+  if (m < 0x00800000) h = 0;
+  if (m >= 0x7f800000) h = m > 0x7f800000 ? 0x7ff80000 : 0x7ff00000;
+  return __hiloint2double(h | (b & 0x80000000), m < 0x00800000 ? 0 : b << 29);
+}
+__device__ __forceinline__ double double_of_ff(ff a) {
+  return double_of_float(a.hi) + double_of_float(a.lo);
+}
+// The same for a normalised pair (|lo| <= ulp(hi) / 2), the low part joined to
+// the head's mantissa by an integer addition; through the FP64 pipe below
+// 2^-75, where lo's weight leaves FP32's range.
+__device__ __forceinline__ double double_join(ff a) {
+  const int b = __float_as_int(a.hi), m = b & 0x7fffffff;
+  if (m < (52 << 23) || m >= 0x7f800000) return double_of_ff(a);
+  const float w = __int_as_float((int)((306u << 23) - (m & 0x7f800000u)));   // 2^(52 - exponent)
+  int l = __float2int_rn(__fmul_rn(a.lo, w));
+  if (b < 0) l = -l;
+  const unsigned long long d =
+      ((unsigned long long)((m >> 3) + (896 << 20)) << 32 | ((unsigned)b << 29)) + (long long)l;
+  return __longlong_as_double((long long)(d | (unsigned long long)(b & 0x80000000u) << 32));
+}
+// 1 / a
+__device__ __forceinline__ ff ff_rcp(ff a) {
+  const float q = __fdiv_rn(1.f, a.hi);
+  float e = __fmaf_rn(-q, a.hi, 1.f);
+  e = __fmaf_rn(-q, a.lo, e);
+  return fast_two_sum(q, __fmul_rn(q, e));
+}
+// a pair in a double's place
+__device__ __forceinline__ double ff_pack(ff a) {
+  return __hiloint2double(__float_as_int(a.hi), __float_as_int(a.lo));
+}
+__device__ __forceinline__ ff ff_unpack(double d) {
+  return ff(__int_as_float(__double2hiint(d)), __int_as_float(__double2loint(d)));
+}
+
+// Exponentials of the reaction rates.  The argument comes in units of ln2/64
+// (the mechanism's coefficients are scaled by 64/ln2 on the host), as the
+// nearest integer n and the rest r = rh + rl, |r| <= 1/2; e^x = y 2^e with
+// e = floor(n / 64) and y = 2^(j/64) e^z, z = r ln2/64 (Tang's reduction,
+// as ff_exp).  e is applied after the concentrations (ff_scale), so that a
+// rate constant beyond FP32's range is no overflow by itself.
+struct ExpArg {
+  int n;
+  float rh, rl;
+};
+// arguments beyond +-16000 (e^+-173) are held at that bound; NaN stays NaN
+constexpr float kExpArgMax = 16000.f;
+
+// x = xh + xl in units of ln2/64
+__device__ __forceinline__ ExpArg exp_arg(ff x) {
+  ExpArg a;
+  const float xh = fminf(fmaxf(x.hi, -kExpArgMax), kExpArgMax);   // NaN: -kExpArgMax
+  const float t = __fadd_rn(xh, 12582912.f);                       // 1.5 2^23: rounds
+  a.n = __float_as_int(t) - 0x4b400000;
+  const ff r = two_sum(__fsub_rn(xh, __fsub_rn(t, 12582912.f)),
+                       fabsf(x.hi) <= kExpArgMax ? x.lo : (x.hi != x.hi ? x.hi : 0.f));
+  a.rh = r.hi;
+  a.rl = r.lo;
+  return a;
+}
+// x in FP64: integer part and rest from its fixed-point form with 46 fraction
+// bits, in integer arithmetic (the FP64 pipe would take three additions)
+__device__ __forceinline__ ExpArg exp_arg(double x) {
+  const int h = __double2hiint(x), l = __double2loint(x);
+  const int mag = h & 0x7fffffff;
+  if (mag >= 0x40cf4000) {                 // 16000 and above
+    ExpArg b{h < 0 ? -16000 : 16000, 0.f, 0.f};
+    if (x != x) b.rh = __int_as_float(0x7fffffff);
+    return b;
+  }
+  const unsigned long long m =
+      ((unsigned long long)(unsigned)((mag & 0xfffff) | 0x100000) << 42) |
+      ((unsigned long long)(unsigned)l << 10);            // mantissa, 62 fraction bits
+  const int sh = min(1039 - (mag >> 20), 63);             // 16 - exponent
+  long long v = (long long)(m >> sh);
+  if (h < 0) v = -v;
+  const int vh = (int)(v >> 32);
+  ExpArg a;
+  a.n = (vh + (1 << 13)) >> 14;
+  const int fh = vh - (a.n << 14);
+  const unsigned fl = (unsigned)v;
+  const int f1 = (int)__funnelshift_l(fl, (unsigned)fh, 18);      // rest, 32 fraction bits
+  a.rh = __fmul_rn(__int2float_rn(f1 & ~0xff), 0x1p-32f);
+  a.rl = __fmul_rn(__int2float_rn(((f1 & 0xff) << 14) | (int)(fl & 0x3fffu)), 0x1p-46f);
+  return a;
+}
+
+__device__ __forceinline__ ff exp_frac(const ExpArg& a) {
+  // z = r ln2/64 as p + e
+  const float C1 = 0x1.62e43p-7f, C2 = -0x1.05c61p-35f;   // ln2/64 = C1 + C2
+  const float p = __fmul_rn(a.rh, C1);
+  float e = __fmaf_rn(a.rh, C1, -p);
+  e = __fmaf_rn(a.rh, C2, e);
+  e = __fmaf_rn(a.rl, C1, e);
+  // e^z - 1 = z + z^2/2 + z^3 (1/6 + z/24 + z^2/120 + z^3/720), the last
+  // group (below 3e-8) in FP32
+  const float q = __fmul_rn(p, p);
+  const float qe = __fmaf_rn(p, p, -q);
+  float c = __fmaf_rn(p, 1.3888889225e-3f, 8.3333337680e-3f);
+  c = __fmaf_rn(p, c, 4.1666667908e-2f);
+  c = __fmaf_rn(p, c, 1.6666667163e-1f);
+  const ff s = fast_two_sum(p, __fmul_rn(0.5f, q));
+  float lo = __fmaf_rn(0.5f, qe, __fmaf_rn(p, e, e));
+  lo = __fmaf_rn(__fmul_rn(p, q), c, lo);
+  lo = __fadd_rn(s.lo, lo);
+  // 2^(j/64) (1 + em1)
+  const float2 t = __ldg(&kExp2Tab64[a.n & 63]);
+  const ff w = two_prod(t.x, s.hi);
+  const ff y = fast_two_sum(t.x, w.hi);
+  lo = __fmaf_rn(t.x, lo, __fmaf_rn(t.y, s.hi, __fadd_rn(w.lo, t.y)));
+  return fast_two_sum(y.hi, __fadd_rn(y.lo, lo));
+}
+// a 2^e, |e| <= 256, in two exact factors
+__device__ __forceinline__ ff ff_scale(ff a, int e) {
+  const int e1 = e >> 1;
+  const float s1 = __int_as_float((e1 + 127) << 23);
+  const float s2 = __int_as_float((e - e1 + 127) << 23);
+  return ff(__fmul_rn(__fmul_rn(a.hi, s1), s2), __fmul_rn(__fmul_rn(a.lo, s1), s2));
+}
+
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ ff ff_from_double(double d) {
   const float h = __double2float_rn(d);

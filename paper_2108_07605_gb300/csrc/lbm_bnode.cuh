@@ -635,6 +635,7 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
   for (int a = 0; a < M; ++a) {
     rec[(RC::Y + a) * N + n] = s.Y[a * kBnd];
 #pragma unroll
-    for (int d = 0; d < D; ++d) rec[(RC::US + a * D + d) * N + n] = s.us[(a * D + d) * kBnd];
+    for (int d = 0; d < D; ++d)
+      rec[(RC::US + a * D + d) * N + n] = s.us[(a * D + d) * kBnd] - s.u[d];
   }
 }

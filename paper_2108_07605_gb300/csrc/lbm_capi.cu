@@ -83,9 +83,7 @@ Launch resolve_launch(const lbm_launch& opt, long long nodes, lbm_precision prec
   lc.persistent = opt.persistent >= 0
                       ? opt.persistent
                       : (plan && prec == LBM_FP64 && nodes < kPlanSingleLaunch ? 2 : 0);
-  lc.coll_split = opt.collide_split >= 0
-                      ? opt.collide_split
-                      : (prec == LBM_FP64 && !small && lc.persistent != 2 ? 0 : 1);
+  lc.coll_split = opt.collide_split >= 0 ? opt.collide_split : 1;
   lc.npt = opt.nodes_per_thread > 0 ? opt.nodes_per_thread : 1;
   return lc;
 }
@@ -249,6 +247,9 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
   d.M = m.n_species;
   d.R = m.n_reactions;
   const double T0 = T_REF;
+  // Gibbs functions g_a/(R_U T) = gi/T + g0 + g1 T + g2 T^2 - a0 ln T
+  double gi[LBM_MAX_SPECIES], g0[LBM_MAX_SPECIES], g1[LBM_MAX_SPECIES], g2[LBM_MAX_SPECIES],
+      ga[LBM_MAX_SPECIES];
   for (int a = 0; a < m.n_species; ++a) {
     const double mm = m.molar_mass[a];
     const double a0 = m.cp[a][0], a1 = m.cp[a][1], a2 = m.cp[a][2];
@@ -260,37 +261,59 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
     d.u1[a] = d.Ra[a] * (a0 - 1.0);
     d.u2[a] = d.Ra[a] * 0.5 * a1;
     d.u3[a] = d.Ra[a] * a2 / 3.0;
-    d.g_inv[a] = m.h_formation[a] / R_U - poly0;
-    d.g0[a] = a0 - m.s_standard[a] / R_U + a0 * std::log(T0) + a1 * T0 + 0.5 * a2 * T0 * T0;
-    d.g1[a] = -0.5 * a1;
-    d.g2[a] = -a2 / 6.0;
-    d.a0[a] = a0;
+    gi[a] = m.h_formation[a] / R_U - poly0;
+    g0[a] = a0 - m.s_standard[a] / R_U + a0 * std::log(T0) + a1 * T0 + 0.5 * a2 * T0 * T0;
+    g1[a] = -0.5 * a1;
+    g2[a] = -a2 / 6.0;
+    ga[a] = a0;
     for (int b = 0; b < m.n_species; ++b) {
       d.K[a][b] = a == b ? 0.0 : 1.0 / (mm * m.molar_mass[b] * m.D0[a][b]);
       d.Kf[a][b] = (float)d.K[a][b];
+      d.K_f[a][b] = ff_host(d.K[a][b]);
     }
   }
-  d.ln_p0_over_ru = std::log(P_REF / R_U);
+  // the reactions without a third body, then those of each distinct row of
+  // efficiencies
+  int rows = 0, set[LBM_MAX_REACTIONS];
+  double eff[LBM_MAX_REACTIONS][LBM_MAX_SPECIES];
   for (int r = 0; r < m.n_reactions; ++r) {
-    DevReaction& x = d.rx[r];
-    x.nr = x.np = 0;
-    x.dn = 0;
-    for (int a = 0; a < m.n_species; ++a) {
-      for (int k = 0; k < m.nu_f[r][a]; ++k) x.reac[x.nr++] = a;
-      for (int k = 0; k < m.nu_r[r][a]; ++k) x.prod[x.np++] = a;
-      x.dn += m.nu_r[r][a] - m.nu_f[r][a];
-      d.eff[r][a] = m.efficiency[r][a];
-    }
-    x.reversible = m.reversible[r] ? 1 : 0;
-    x.third_body = m.third_body[r] ? 1 : 0;
-    x.lnA = std::log(m.arrhenius[r][0]);
-    x.b = m.arrhenius[r][1];
-    x.EaR = m.arrhenius[r][2] / R_U;
-    x.lnA_f = ff_host(x.lnA);
-    x.b_f = ff_host(x.b);
-    x.EaR_f = ff_host(x.EaR);
-    for (int a = 0; a < m.n_species; ++a) d.eff_f[r][a] = ff_host(m.efficiency[r][a]);
+    set[r] = -1;
+    if (!m.third_body[r]) continue;
+    for (int k = 0; k < rows && set[r] < 0; ++k)
+      if (std::equal(m.efficiency[r], m.efficiency[r] + m.n_species, eff[k])) set[r] = k;
+    if (set[r] >= 0) continue;
+    std::copy(m.efficiency[r], m.efficiency[r] + m.n_species, eff[rows]);
+    for (int a = 0; a < m.n_species; ++a) d.eff_f[rows][a] = ff_host(m.efficiency[r][a]);
+    set[r] = rows++;
   }
+  const long double ln_p0 = std::log(P_REF / R_U), S = 64.0L / std::log(2.0L);
+  int n = 0;
+  for (int k = -1; k < rows; ++k)
+    for (int r = 0; r < m.n_reactions; ++r) {
+      if (set[r] != k) continue;
+      DevReaction& x = d.rx[n++];
+      x.third_body = k;
+      x.reversible = m.reversible[r] ? 1 : 0;
+      const long double lnA = std::log((long double)m.arrhenius[r][0]), b = m.arrhenius[r][1],
+                        EaR = m.arrhenius[r][2] / R_U;
+      // k_r = k_f / K_c, ln K_c = -sum_a nu_a g_a/(R_U T) + dn ln(P0 / (R_U T))
+      long double c[5] = {lnA, b, -EaR, 0.0L, 0.0L};
+      auto molecule = [&](int a, long double sgn) {
+        c[0] += sgn * (g0[a] - ln_p0);
+        c[1] += sgn * (1.0L - ga[a]);
+        c[2] += sgn * gi[a];
+        c[3] += sgn * g1[a];
+        c[4] += sgn * g2[a];
+      };
+      x.nr = x.np = 0;
+      for (int a = 0; a < m.n_species; ++a) {
+        for (int j = 0; j < m.nu_f[r][a]; ++j) { x.reac[x.nr++] = a; molecule(a, -1.0L); }
+        for (int j = 0; j < m.nu_r[r][a]; ++j) { x.prod[x.np++] = a; molecule(a, 1.0L); }
+      }
+      const long double f[3] = {lnA, b, -EaR};
+      for (int j = 0; j < 3; ++j) x.f_f[j] = ff_host(x.f[j] = (double)(S * f[j]));
+      for (int j = 0; j < 5; ++j) x.r_f[j] = ff_host(x.r[j] = (double)(S * c[j]));
+    }
   d.D_T_exp = m.D_T_exponent;
   d.mu0 = m.mu0;
   d.mu_T_exp = m.mu_T_exponent;
@@ -302,15 +325,9 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
     d.u1_f[a] = ff_host(d.u1[a]);
     d.u2_f[a] = ff_host(d.u2[a]);
     d.u3_f[a] = ff_host(d.u3[a]);
-    d.g_inv_f[a] = ff_host(d.g_inv[a]);
-    d.g0_f[a] = ff_host(d.g0[a]);
-    d.g1_f[a] = ff_host(d.g1[a]);
-    d.g2_f[a] = ff_host(d.g2[a]);
-    d.a0_f[a] = ff_host(d.a0[a]);
     d.inv_mm_s[a] = (float)d.inv_mm[a];
     d.Ra_s[a] = (float)d.Ra[a];
   }
-  d.ln_p0_over_ru_f = ff_host(d.ln_p0_over_ru);
   d.D_T_exp_s = (float)d.D_T_exp;
   d.mu0_s = (float)d.mu0;
   d.mu_T_exp_s = (float)d.mu_T_exp;
@@ -659,6 +676,7 @@ lbm_status init_common(lbm_ctx* h, const double* rho_or_P, int is_pressure, cons
 
 namespace lbm {
 void fill_mixed_units(Units& un) {
+  un.dt_sub = un.dt / un.substeps;
   un.c2_f = ff_host(un.c * un.c);
   un.inv_c2_f = ff_host(un.inv_c2);
   un.dt_sub_f = ff_host(un.dt / un.substeps);
@@ -666,6 +684,12 @@ void fill_mixed_units(Units& un) {
   un.inv_c2_s = (float)un.inv_c2;
   un.s_pref_s = (float)un.s_pref;
   un.nu_pref_s = (float)un.nu_pref;
+}
+void fill_enthalpies(const DevMech& m, Units& un) {
+  for (int a = 0; a < m.M; ++a) {
+    const double h[4] = {m.u0[a], m.u1[a] + m.Ra[a], m.u2[a], m.u3[a]};
+    for (int k = 0; k < 4; ++k) un.hl_f[k][a] = ff_host(un.hl[k][a] = h[k] * un.inv_c2);
+  }
 }
 // Host helpers shared with the allocation-free entry point (lbm_noalloc.cu).
 std::string validate_config(const lbm_config* c) { return validate(c); }
@@ -793,6 +817,7 @@ lbm_status lbm_create(const lbm_config* cfg, lbm_t* out) {
   h->un.newton_rtol = cfg->newton_rtol;
   fill_mixed_units(h->un);
   build_mech(cfg->mech, h->mech);
+  fill_enthalpies(h->mech, h->un);
   h->elem = elem_size(cfg->precision);
   h->stream = static_cast<cudaStream_t>(cfg->stream);
   const HostBC hb = classify(*cfg, c);

@@ -58,7 +58,7 @@ template <int D, int M> struct Rec {
   static constexpr int QF = P + Lat<D>::NP;
   static constexpr int E = QF + D;
   static constexpr int Y = E + 1;
-  static constexpr int US = Y + M;
+  static constexpr int US = Y + M;              // u_a - u
   static constexpr int PHI = US + M * D;
   static constexpr int DRHO = PHI + D;          // reaction increments, species a < M
   static constexpr int NF = DRHO + M - 1;
@@ -104,53 +104,9 @@ __device__ __forceinline__ double species_U(const DevMech& m, int a, double T) {
 }
 
 // ------------------------------------------------------------------------
-// chemistry: mass production rates rho_dot_a (kg/(m^3 s)) at (T, rho_a).
-template <int M>
-__device__ void production_rates(const DevMech& m, double T, const double* r,
-                                 double* rdot) {
-  const double lnT = log(T);
-  const double invT = 1.0 / T;
-  double C[M], G[M], w[M];
-#pragma unroll
-  for (int a = 0; a < M; ++a) {
-    C[a] = r[a] * m.inv_mm[a];
-    G[a] = m.g_inv[a] * invT + m.g0[a] + T * (m.g1[a] + T * m.g2[a]) - m.a0[a] * lnT;
-    w[a] = 0.0;
-  }
-  const double ln_p0_rut = m.ln_p0_over_ru - lnT;   // ln(P0 / (R_U T))
-  for (int k = 0; k < m.R; ++k) {
-    const DevReaction& rx = m.rx[k];
-    const double lnkf = rx.lnA + rx.b * lnT - rx.EaR * invT;
-    double fwd = exp_tang(lnkf);
-    for (int j = 0; j < rx.nr; ++j) fwd *= C[rx.reac[j]];
-    double rev = 0.0;
-    if (rx.reversible) {
-      double dG = 0.0;                               // sum_a nu_a G_a
-      for (int j = 0; j < rx.np; ++j) dG += G[rx.prod[j]];
-      for (int j = 0; j < rx.nr; ++j) dG -= G[rx.reac[j]];
-      // k_r = k_f / K_c, ln K_c = -dG + dn ln(P0/(R_U T))
-      rev = exp_tang(lnkf + dG - rx.dn * ln_p0_rut);
-      for (int j = 0; j < rx.np; ++j) rev *= C[rx.prod[j]];
-    }
-    double q = fwd - rev;
-    if (rx.third_body) {
-      double cm = 0.0;
-#pragma unroll
-      for (int a = 0; a < M; ++a) cm += m.eff[k][a] * C[a];
-      q *= cm;
-    }
-    for (int j = 0; j < rx.nr; ++j) w[rx.reac[j]] -= q;
-    for (int j = 0; j < rx.np; ++j) w[rx.prod[j]] += q;
-  }
-#pragma unroll
-  for (int a = 0; a < M; ++a) rdot[a] = w[a] * m.mm[a];
-}
-
-// ------------------------------------------------------------------------
-// The same temperature solve and rates in float-float (mixed path).  The
-// formulas are those of newton_T and production_rates; the stopping rule
-// uses max(rtol, 4e-13), the resolution of float-float sums of the
-// formation-energy-sized terms.
+// The same temperature solve in float-float (mixed path).  The formulas are
+// those of newton_T; the stopping rule uses max(rtol, 4e-13), the resolution
+// of float-float sums of the formation-energy-sized terms.
 __device__ __forceinline__ ff species_U_ff(const DevMech& m, int a, ff T) {
   return m.u0_f[a] + T * (m.u1_f[a] + T * (m.u2_f[a] + T * m.u3_f[a]));
 }
@@ -178,60 +134,117 @@ __device__ ff newton_T_ff(const DevMech& m, const ff* Y, ff U, ff T, int max_ite
   return T;
 }
 
-// The arrays the reaction loop indexes by species (concentrations, Gibbs
-// functions, rates) live in a per-thread slice of shared memory: a runtime
-// index into a register array would put it in local memory.  Every kernel
-// that runs the float-float rates has kChemThreads threads per block.
-constexpr int kChemThreads = 128;
+// ------------------------------------------------------------------------
+// Chemistry: rates of progress and mass production rates (Sec. 2.4, Sec.
+// 3.6), the temperature in CT: FP64 (the FP64 path, and FP32 storage with
+// chem_fp64) or float-float.
+//
+// What bounds it is the arithmetic of two exponentials per reaction.  In
+// FP64 the whole took ~42 FP64 instructions per reaction of 64 cycles each
+// per SM quarter, in float-float ~410 FP32 instructions.  So (1) the
+// logarithm of each rate constant is one sum over the basis (1, ln T, 1/T, T,
+// T^2) with coefficients folded on the host, which replaces the species' Gibbs
+// functions; (2) only these sums run in FP64 (six instructions per
+// reaction), where the argument's size (up to ~100) would cost a
+// float-float its accuracy; the exponentials, products and sums that follow
+// keep ~48 bits in pairs of FP32, below the ~1e-14 that the rounding of T
+// leaves in a rate constant; (3) sums stay unnormalised (ff_acc); (4) the
+// third-body sums are formed once per distinct row of efficiencies.
+template <typename CT> struct TBasis { CT lnT, invT, T, T2; };
 
-// bytes of one block's slices (kChemThreads threads, C, G and W per species)
-template <int M, typename CT> constexpr size_t chem_slice_bytes() {
-  return (size_t)3 * M * kChemThreads * sizeof(CT);
+__device__ __forceinline__ TBasis<double> tbasis(double T) {
+  return TBasis<double>{log(T), 1.0 / T, T, T * T};
+}
+__device__ __forceinline__ TBasis<ff> tbasis(ff T) {
+  return TBasis<ff>{ff_log(T), ff(1.f) / T, T, T * T};
+}
+__device__ __forceinline__ ExpArg forward_arg(const DevReaction& x, const TBasis<double>& b) {
+  return exp_arg(fma(x.f[2], b.invT, fma(x.f[1], b.lnT, x.f[0])));
+}
+__device__ __forceinline__ ExpArg reverse_arg(const DevReaction& x, const TBasis<double>& b) {
+  return exp_arg(fma(x.r[2], b.invT,
+                     fma(x.r[1], b.lnT, fma(x.r[4], b.T2, fma(x.r[3], b.T, x.r[0])))));
+}
+__device__ __forceinline__ ExpArg forward_arg(const DevReaction& x, const TBasis<ff>& b) {
+  ff s = x.f_f[0];
+  ff_fma_acc(s, x.f_f[1], b.lnT);
+  ff_fma_acc(s, x.f_f[2], b.invT);
+  return exp_arg(ff_norm(s));
+}
+__device__ __forceinline__ ExpArg reverse_arg(const DevReaction& x, const TBasis<ff>& b) {
+  ff s = x.r_f[0];
+  ff_fma_acc(s, x.r_f[3], b.T);
+  ff_fma_acc(s, x.r_f[4], b.T2);
+  ff_fma_acc(s, x.r_f[1], b.lnT);
+  ff_fma_acc(s, x.r_f[2], b.invT);
+  return exp_arg(ff_norm(s));
 }
 
-// Cs: this thread's slice (entry a of C at Cs[a kChemThreads], then G and W)
-template <int M>
-__device__ void production_rates_ff(const DevMech& m, ff T, const ff* r, ff* rdot,
-                                    ff* const Cs) {
-  ff* const Gs = Cs + M * kChemThreads;
-  ff* const Ws = Gs + M * kChemThreads;
-  const ff lnT = ff_log(T);
-  const ff invT = ff(1.f) / T;
-  ff C[M];
-#pragma unroll
-  for (int a = 0; a < M; ++a) {
-    C[a] = r[a] * m.inv_mm_f[a];
-    Cs[a * kChemThreads] = C[a];
-    Gs[a * kChemThreads] =
-        m.g_inv_f[a] * invT + m.g0_f[a] + T * (m.g1_f[a] + T * m.g2_f[a]) - m.a0_f[a] * lnT;
-    Ws[a * kChemThreads] = ff();
+// The arrays the reaction loop indexes by species (concentrations C, molar
+// rates W) live in a per-thread slice of shared memory: a runtime index into
+// a register array would put it in local memory.  Every kernel that runs the
+// rates has kChemThreads threads per block (or fewer).
+constexpr int kChemThreads = 128;
+
+// bytes of one block's slices (kChemThreads threads, C and W per species)
+template <int M> constexpr size_t chem_slice_bytes() {
+  return (size_t)2 * M * kChemThreads * sizeof(ff);
+}
+
+// Rate of progress of a reaction without its third body; C: this thread's
+// concentrations (entry a at C[a kChemThreads]).
+template <typename CT>
+__device__ __forceinline__ ff reaction_rate(const DevReaction& x, const TBasis<CT>& b,
+                                            const ff* C) {
+  const ExpArg af = forward_arg(x, b);
+  ff q = exp_frac(af);
+  for (int j = 0; j < x.nr; ++j) q *= C[x.reac[j] * kChemThreads];
+  q = ff_scale(q, af.n >> 6);
+  if (x.reversible) {
+    const ExpArg ar = reverse_arg(x, b);
+    ff rev = exp_frac(ar);
+    for (int j = 0; j < x.np; ++j) rev *= C[x.prod[j] * kChemThreads];
+    ff_acc(q, -ff_scale(rev, ar.n >> 6));
+    q = ff_norm(q);
   }
-  const ff ln_p0_rut = m.ln_p0_over_ru_f - lnT;
-  for (int k = 0; k < m.R; ++k) {
-    const DevReaction& rx = m.rx[k];
-    const ff lnkf = rx.lnA_f + rx.b_f * lnT - rx.EaR_f * invT;
-    ff fwd = ff_exp(lnkf);
-    for (int j = 0; j < rx.nr; ++j) fwd *= Cs[rx.reac[j] * kChemThreads];
-    ff rev;
-    if (rx.reversible) {
-      ff dG;
-      for (int j = 0; j < rx.np; ++j) dG += Gs[rx.prod[j] * kChemThreads];
-      for (int j = 0; j < rx.nr; ++j) dG -= Gs[rx.reac[j] * kChemThreads];
-      rev = ff_exp(lnkf + dG - ff((float)rx.dn) * ln_p0_rut);
-      for (int j = 0; j < rx.np; ++j) rev *= Cs[rx.prod[j] * kChemThreads];
-    }
-    ff q = fwd - rev;
-    if (rx.third_body) {
-      ff cm;
+  return q;
+}
+
+// The reactions first, first + step, ... added to this thread's molar rates W
+// (entry a at W[a kChemThreads], unnormalised).
+template <int M, typename CT>
+__device__ __forceinline__ void add_reactions(const DevMech& m, const TBasis<CT>& b,
+                                              const ff* C, ff* W, int first, int step) {
+  int row = -1;
+  ff cm;
+  for (int k = first; k < m.R; k += step) {
+    const DevReaction& x = m.rx[k];
+    ff q = reaction_rate(x, b, C);
+    if (x.third_body >= 0) {
+      if (x.third_body != row) {
+        row = x.third_body;
+        cm = ff();
 #pragma unroll
-      for (int a = 0; a < M; ++a) cm += m.eff_f[k][a] * C[a];
+        for (int a = 0; a < M; ++a) ff_fma_acc(cm, m.eff_f[row][a], C[a * kChemThreads]);
+        cm = ff_norm(cm);
+      }
       q *= cm;
     }
-    for (int j = 0; j < rx.nr; ++j) Ws[rx.reac[j] * kChemThreads] -= q;
-    for (int j = 0; j < rx.np; ++j) Ws[rx.prod[j] * kChemThreads] += q;
+    for (int j = 0; j < x.nr; ++j) ff_acc(W[x.reac[j] * kChemThreads], -q);
+    for (int j = 0; j < x.np; ++j) ff_acc(W[x.prod[j] * kChemThreads], q);
   }
+}
+
+// Molar rates w_a (mol/(m^3 s)) at T of the concentrations already in this
+// thread's slice Cs; the slice's rates are overwritten.
+template <int M, typename CT>
+__device__ __forceinline__ void molar_rates(const DevMech& m, CT T, ff (&w)[M], ff* const Cs) {
+  ff* const Ws = Cs + M * kChemThreads;
 #pragma unroll
-  for (int a = 0; a < M; ++a) rdot[a] = Ws[a * kChemThreads] * m.mm_f[a];
+  for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
+  add_reactions<M>(m, tbasis(T), Cs, Ws, 0, 1);
+#pragma unroll
+  for (int a = 0; a < M; ++a) w[a] = ff_norm(Ws[a * kChemThreads]);
 }
 
 // ------------------------------------------------------------------------
@@ -262,6 +275,44 @@ __device__ __forceinline__ void solve_dd_strided(R* A, int st, R (&B)[M][D]) {
 #pragma unroll
       for (int c = k + 1; c < M; ++c) s -= A[(k * M + c) * st] * B[c][d];
       B[k][d] = s * inv;
+    }
+  }
+}
+
+// The same in float-float (the FP64 path's diffusion velocities, which enter
+// the collision only through corrections a thousand times below what they
+// correct: 48 bits of a correction are beyond FP64's rounding of the sum.  In
+// FP64 the elimination took ~800 instructions of 64 cycles).
+template <int M, int D>
+__device__ __forceinline__ void solve_dd_strided(ff* A, int st, ff (&B)[M][D]) {
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    const ff inv = ff_rcp(A[(k * M + k) * st]);
+    A[(k * M + k) * st] = inv;
+#pragma unroll
+    for (int r = k + 1; r < M; ++r) {
+      const ff f = -(A[(r * M + k) * st] * inv);
+#pragma unroll
+      for (int c = k + 1; c < M; ++c) {
+        ff v = A[(r * M + c) * st];
+        ff_fma_acc(v, f, A[(k * M + c) * st]);
+        A[(r * M + c) * st] = ff_norm(v);
+      }
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        ff_fma_acc(B[r][d], f, B[k][d]);
+        B[r][d] = ff_norm(B[r][d]);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = M - 1; k >= 0; --k) {
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      ff s = B[k][d];
+#pragma unroll
+      for (int c = k + 1; c < M; ++c) ff_fma_acc(s, -A[(k * M + c) * st], B[c][d]);
+      B[k][d] = ff_norm(s) * A[(k * M + k) * st];
     }
   }
 }

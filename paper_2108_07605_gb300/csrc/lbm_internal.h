@@ -25,13 +25,18 @@ constexpr int ST_NONFINITE = 2;
 constexpr int ST_RANGE = 4;
 constexpr int ST_TIMEOUT = 8;   // a bounded device wait gave up
 
+// Logarithms of a reaction's rate constants, in units of ln2/64 (ExpArg), as
+// sums over T alone:
+//   forward  f[0] + f[1] ln T + f[2] / T
+//   reverse  r[0] + r[1] ln T + r[2] / T + r[3] T + r[4] T^2,
+// the reverse one with the reaction's equilibrium constant folded in.
 struct DevReaction {
   int nr, np;            // number of reactant / product molecules (<= 3)
   int reac[3], prod[3];  // species index per molecule (repeated for nu = 2)
-  int dn;                // sum of product minus reactant coefficients
-  int reversible, third_body;
-  double lnA, b, EaR;    // ln A, temperature exponent, Ea / R_U
-  ff lnA_f, b_f, EaR_f;  // the same as float-float (mixed path)
+  int reversible;
+  int third_body;        // row of DevMech::eff_f, -1: none
+  double f[3], r[5];
+  ff f_f[3], r_f[5];     // the same as float-float (mixed path)
 };
 
 // Mechanism in the forms the kernels evaluate (built on the host).
@@ -41,15 +46,13 @@ struct DevMech {
   // U_a(T) = u0 + u1 T + u2 T^2 + u3 T^3  (J/kg, incl. formation)
   double u0[LBM_MAX_SPECIES], u1[LBM_MAX_SPECIES], u2[LBM_MAX_SPECIES],
       u3[LBM_MAX_SPECIES];
-  // g_a/(R_U T) = g_inv/T + g0 + g1 T + g2 T^2 - a0 ln T
-  double g_inv[LBM_MAX_SPECIES], g0[LBM_MAX_SPECIES], g1[LBM_MAX_SPECIES],
-      g2[LBM_MAX_SPECIES], a0[LBM_MAX_SPECIES];
-  double ln_p0_over_ru;
+  // reactions, those of equal third-body efficiencies in a row (the sum over
+  // the species is formed once per row)
   DevReaction rx[LBM_MAX_REACTIONS];
-  double eff[LBM_MAX_REACTIONS][LBM_MAX_SPECIES];
   // 1/tau_ab = s(node) * K[a][b], K = 1/(m_a m_b D0_ab)
   double K[LBM_MAX_SPECIES][LBM_MAX_SPECIES];
   float Kf[LBM_MAX_SPECIES][LBM_MAX_SPECIES];   // K rounded to FP32 (mixed path)
+  ff K_f[LBM_MAX_SPECIES][LBM_MAX_SPECIES];     // and as float-float (FP64 path)
   double D_T_exp, mu0, mu_T_exp, inv_prandtl;
   // Wilke's mixing rule (wilke = 1): species viscosities at T0 and the
   // T-independent Phi_ab (the species share the T exponent)
@@ -61,10 +64,7 @@ struct DevMech {
   // float-float copies for the mixed path's temperature solve and chemistry
   ff mm_f[LBM_MAX_SPECIES], inv_mm_f[LBM_MAX_SPECIES];
   ff u0_f[LBM_MAX_SPECIES], u1_f[LBM_MAX_SPECIES], u2_f[LBM_MAX_SPECIES], u3_f[LBM_MAX_SPECIES];
-  ff g_inv_f[LBM_MAX_SPECIES], g0_f[LBM_MAX_SPECIES], g1_f[LBM_MAX_SPECIES],
-      g2_f[LBM_MAX_SPECIES], a0_f[LBM_MAX_SPECIES];
-  ff ln_p0_over_ru_f;
-  ff eff_f[LBM_MAX_REACTIONS][LBM_MAX_SPECIES];
+  ff eff_f[LBM_MAX_REACTIONS][LBM_MAX_SPECIES];   // distinct rows of third-body efficiencies
   // FP32 copies for the mixed path's transport and energy-flux terms
   float inv_mm_s[LBM_MAX_SPECIES], Ra_s[LBM_MAX_SPECIES];
   float D_T_exp_s, mu0_s, mu_T_exp_s, inv_prandtl_s;
@@ -77,6 +77,10 @@ struct Units {
   int substeps;
   int newton_max_iter;
   double newton_rtol;
+  double dt_sub;         // dt / substeps
+  // species enthalpies H_a/c^2 = sum_k hl[k][a] T^k (with formation)
+  double hl[4][LBM_MAX_SPECIES];
+  ff hl_f[4][LBM_MAX_SPECIES];
   // mixed path: float-float and FP32 copies
   ff c2_f, inv_c2_f, dt_sub_f;   // c^2, 1/c^2, dt / substeps
   float newton_rtol_f;           // max(newton_rtol, 4e-13): float-float resolution
@@ -316,5 +320,6 @@ std::string validate_config(const lbm_config* c);   // "" when valid
 void build_device_mechanism(const lbm_mechanism& m, DevMech& d);
 void fill_units(const lbm_config& cfg, Units& un);
 void fill_mixed_units(Units& un);
+void fill_enthalpies(const DevMech& m, Units& un);
 
 }  // namespace lbm

@@ -145,13 +145,13 @@ __device__ __forceinline__ constexpr int pidx(int a, int b) {
 // (Sec. 2.4 Eq. R3): rs the post-stream species densities (the slaved one
 // included), rho, ER = E / rho and usqR = |u|^2 of the moments, T_0 = T
 // their temperature; dr receives the increments drho_a (a < M - 1).  The
-// mixed path runs it in float-float, whose rate arrays live in the thread's
-// shared-memory slice (kDynChem: chem_slice, the block's slices of
-// chem_slice_bytes in dynamic shared memory; else a static array of the
-// calling kernel); FP64 chemistry otherwise.  Blocks of kChemThreads threads.
+// temperature solve in float-float (mixed path) or FP64; the rate arrays live
+// in the thread's shared-memory slice (kDynChem: chem_slice, the block's
+// slices of chem_slice_bytes in dynamic shared memory; else a static array of
+// the calling kernel).  Blocks of kChemThreads threads.
 template <int M>
 __device__ __forceinline__ ff* chem_static_slice() {
-  __shared__ __align__(8) unsigned char chem_raw[chem_slice_bytes<M, ff>()];
+  __shared__ __align__(8) unsigned char chem_raw[chem_slice_bytes<M>()];
   return reinterpret_cast<ff*>(chem_raw);
 }
 
@@ -160,12 +160,13 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
                                               double T, const Units& un, const DevMech& mech,
                                               int* __restrict__ status, void* chem_slice,
                                               RT (&dr)[M - 1]) {
+  ff* Cs;
+  if constexpr (kDynChem) Cs = static_cast<ff*>(chem_slice) + threadIdx.x;
+  else Cs = chem_static_slice<M>() + threadIdx.x;
+  ff w[M];
   if constexpr (kFF<RT>) {
-    ff* Cs;
-    if constexpr (kDynChem) Cs = static_cast<ff*>(chem_slice) + threadIdx.x;
-    else Cs = chem_static_slice<M>() + threadIdx.x;
     const ff Uphys = (ff(ER) + ff(-0.5f * usqR)) * un.c2_f;
-    ff r[M], rdot[M];
+    ff r[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) r[a] = ff(rs[a]);
     ff Ts = ff_from_double(T);
@@ -179,33 +180,35 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
         Ts = newton_T_ff<M>(mech, Ys, Uphys, Ts, un.newton_max_iter, un.newton_rtol_f, oks);
         if (!oks) atomicOr(status, ST_NEWTON);
       }
-      production_rates_ff<M>(mech, Ts, r, rdot, Cs);
 #pragma unroll
-      for (int a = 0; a < M; ++a) r[a] += un.dt_sub_f * rdot[a];
+      for (int a = 0; a < M; ++a) Cs[a * kChemThreads] = r[a] * mech.inv_mm_f[a];
+      molar_rates<M>(mech, Ts, w, Cs);
+#pragma unroll
+      for (int a = 0; a < M; ++a) r[a] += un.dt_sub_f * (w[a] * mech.mm_f[a]);
     }
 #pragma unroll
     for (int a = 0; a < M - 1; ++a) dr[a] = (r[a] - ff(rs[a])).hi;
   } else {
     const double Uphys = (double(ER) - 0.5 * double(usqR)) * un.c * un.c;
-    const double dtr = un.dt / un.substeps;
-    const double rho_d = double(rho);
-    double r[M], rdot[M];
+    const double dtr = un.dt_sub, ir = 1.0 / double(rho);
+    double r[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) r[a] = double(rs[a]);
     double Ts = T;
     for (int s = 0; s < un.substeps; ++s) {
       if (s > 0) {
         double Ys[M];
-        const double ir = 1.0 / rho_d;
 #pragma unroll
         for (int a = 0; a < M; ++a) Ys[a] = r[a] * ir;
         bool oks;
         Ts = newton_T<M>(mech, Ys, Uphys, Ts, un.newton_max_iter, un.newton_rtol, oks);
         if (!oks) atomicOr(status, ST_NEWTON);
       }
-      production_rates<M>(mech, Ts, r, rdot);
 #pragma unroll
-      for (int a = 0; a < M; ++a) r[a] += dtr * rdot[a];
+      for (int a = 0; a < M; ++a) Cs[a * kChemThreads] = ff_of_double(r[a] * mech.inv_mm[a]);
+      molar_rates<M>(mech, Ts, w, Cs);
+#pragma unroll
+      for (int a = 0; a < M; ++a) r[a] = fma(double_of_ff(w[a]), dtr * mech.mm[a], r[a]);
     }
 #pragma unroll
     for (int a = 0; a < M - 1; ++a) dr[a] = RT(r[a] - double(rs[a]));
@@ -311,14 +314,14 @@ __device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __r
     // components
     const bool tiny = species_velocity_undefined<D, RT>(rs[a], js[a]);
     if constexpr (sizeof(RT) == 8) {
-      const RT ira = tiny ? RT(0) : RT(1) / rs[a];
+      const RT ira = RT(1) / rs[a];
 #pragma unroll
       for (int d = 0; d < D; ++d)
-        rec[(RC::US + a * D + d) * N + n] = tiny ? uR[d] : js[a][d] * ira;
+        rec[(RC::US + a * D + d) * N + n] = tiny ? RT(0) : fma(js[a][d], ira, -uR[d]);
     } else {
 #pragma unroll
       for (int d = 0; d < D; ++d)
-        rec[(RC::US + a * D + d) * N + n] = tiny ? uR[d] : js[a][d] / rs[a];
+        rec[(RC::US + a * D + d) * N + n] = tiny ? RT(0) : js[a][d] / rs[a] - uR[d];
     }
   }
 }
@@ -433,25 +436,15 @@ __device__ __forceinline__ ff shfl_xor_ct(unsigned mask, ff v, int o) {
 
 template <typename CT> struct Chem;
 template <> struct Chem<double> {
-  __device__ static double ex(double x) { return exp_tang(x); }
-  __device__ static double ln(double x) { return log(x); }
   __device__ static double inv(double x) { return 1.0 / x; }
-  __device__ static double inv_mm(const DevMech& m, int a) { return m.inv_mm[a]; }
-  __device__ static double mm(const DevMech& m, int a) { return m.mm[a]; }
-  __device__ static double gibbs(const DevMech& m, int a, double T, double invT, double lnT) {
-    return m.g_inv[a] * invT + m.g0[a] + T * (m.g1[a] + T * m.g2[a]) - m.a0[a] * lnT;
-  }
-  __device__ static double lnkf(const DevReaction& rx, double lnT, double invT) {
-    return rx.lnA + rx.b * lnT - rx.EaR * invT;
-  }
-  __device__ static double rev_arg(const DevReaction& rx, double lk, double dG, double lp) {
-    return lk + dG - rx.dn * lp;
-  }
-  __device__ static double ln_p0(const DevMech& m) { return m.ln_p0_over_ru; }
-  __device__ static double eff(const DevMech& m, int k, int a) { return m.eff[k][a]; }
-  __device__ static double dt_sub(const Units& u) { return u.dt / u.substeps; }
   __device__ static double of(double v) { return v; }
   __device__ static double of_T(double T) { return T; }
+  __device__ static ff concentration(const DevMech& m, int a, double r) {
+    return ff_of_double(r * m.inv_mm[a]);
+  }
+  __device__ static double increment(const DevMech& m, const Units& u, int a, ff w) {
+    return double_of_ff(w) * (u.dt_sub * m.mm[a]);
+  }
   __device__ static double ucoef(const DevMech& m, int k, int a) {
     return k == 0 ? m.u0[a] : (k == 1 ? m.u1[a] : (k == 2 ? m.u2[a] : m.u3[a]));
   }
@@ -459,25 +452,13 @@ template <> struct Chem<double> {
   __device__ static double rtol(const Units& u) { return u.newton_rtol; }
 };
 template <> struct Chem<ff> {
-  __device__ static ff ex(ff x) { return ff_exp(x); }
-  __device__ static ff ln(ff x) { return ff_log(x); }
   __device__ static ff inv(ff x) { return ff(1.f) / x; }
-  __device__ static ff inv_mm(const DevMech& m, int a) { return m.inv_mm_f[a]; }
-  __device__ static ff mm(const DevMech& m, int a) { return m.mm_f[a]; }
-  __device__ static ff gibbs(const DevMech& m, int a, ff T, ff invT, ff lnT) {
-    return m.g_inv_f[a] * invT + m.g0_f[a] + T * (m.g1_f[a] + T * m.g2_f[a]) - m.a0_f[a] * lnT;
-  }
-  __device__ static ff lnkf(const DevReaction& rx, ff lnT, ff invT) {
-    return rx.lnA_f + rx.b_f * lnT - rx.EaR_f * invT;
-  }
-  __device__ static ff rev_arg(const DevReaction& rx, ff lk, ff dG, ff lp) {
-    return lk + dG - ff((float)rx.dn) * lp;
-  }
-  __device__ static ff ln_p0(const DevMech& m) { return m.ln_p0_over_ru_f; }
-  __device__ static ff eff(const DevMech& m, int k, int a) { return m.eff_f[k][a]; }
-  __device__ static ff dt_sub(const Units& u) { return u.dt_sub_f; }
   __device__ static ff of(float v) { return ff(v); }
   __device__ static ff of_T(double T) { return ff_from_double(T); }
+  __device__ static ff concentration(const DevMech& m, int a, ff r) { return r * m.inv_mm_f[a]; }
+  __device__ static ff increment(const DevMech& m, const Units& u, int a, ff w) {
+    return u.dt_sub_f * (w * m.mm_f[a]);
+  }
   __device__ static ff ucoef(const DevMech& m, int k, int a) {
     return k == 0 ? m.u0_f[a] : (k == 1 ? m.u1_f[a] : (k == 2 ? m.u2_f[a] : m.u3_f[a]));
   }
@@ -487,13 +468,6 @@ template <> struct Chem<ff> {
 
 template <typename RT> struct ChemType { using type = double; };
 template <> struct ChemType<float> { using type = std::conditional_t<LBM_CHEM64 != 0, double, ff>; };
-
-__device__ __forceinline__ double shfl_ct(unsigned mask, double v, int src) {
-  return __shfl_sync(mask, v, src);
-}
-__device__ __forceinline__ ff shfl_ct(unsigned mask, ff v, int src) {
-  return ff(__shfl_sync(mask, v.hi, src), __shfl_sync(mask, v.lo, src));
-}
 
 // Register r[a] for a lane-dependent species index a (a select per species:
 // a runtime index into a register array would put it in local memory).
@@ -552,73 +526,32 @@ __device__ __forceinline__ void chem_group_substeps(CT (&r)[M], const CT irho, c
                                                     int sub, unsigned gmask,
                                                     int* __restrict__ status) {
   using X = Chem<CT>;
-  const int base = (int)(threadIdx.x & 31) - sub;      // the group's first lane
-  // the arrays the reaction loop indexes by species: a per-thread slice of
-  // shared memory (as in production_rates_ff; 128-thread blocks)
-  __shared__ __align__(8) unsigned char chem_raw[3 * M * kChemThreads * sizeof(CT)];
-  CT* const Cs = reinterpret_cast<CT*>(chem_raw) + threadIdx.x;
-  CT* const Gs = Cs + M * kChemThreads;
-  CT* const Ws = Gs + M * kChemThreads;
+  // concentrations and rates: a per-thread slice of shared memory
+  // (128-thread blocks)
+  ff* const Cs = chem_static_slice<M>() + threadIdx.x;
+  ff* const Ws = Cs + M * kChemThreads;
   for (int s = 0; s < un.substeps; ++s) {
     if (s > 0) {
       bool ok;
       Ts = group_newton<M, L, CT>(m, r, irho, U, Ts, un, sub, gmask, ok);
       if (!ok && sub == 0) atomicOr(status, ST_NEWTON);
     }
-    const CT lnT = X::ln(Ts);
-    const CT invT = X::inv(Ts);
-    // Gibbs functions: lane `sub` evaluates species sub, sub + L, ...; the
-    // group exchanges them with shuffles
-    CT Gown[(M + L - 1) / L];
-#pragma unroll
-    for (int j = 0; j < (M + L - 1) / L; ++j) {
-      const int a = sub + j * L;
-      Gown[j] = a < M ? X::gibbs(m, a, Ts, invT, lnT) : CT();
-    }
-    // species-indexed arrays in the thread's shared-memory slice (the
-    // register copy of C serves the unrolled third-body sums)
-    CT C[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-      C[a] = r[a] * X::inv_mm(m, a);
-      Cs[a * kChemThreads] = C[a];
-      Gs[a * kChemThreads] = shfl_ct(gmask, Gown[a / L], base + a % L);
-      Ws[a * kChemThreads] = CT();
+      Cs[a * kChemThreads] = X::concentration(m, a, r[a]);
+      Ws[a * kChemThreads] = ff();
     }
-    const CT lp = X::ln_p0(m) - lnT;   // ln(P0 / (R_U T))
-    for (int k = sub; k < m.R; k += L) {
-      const DevReaction& rx = m.rx[k];
-      const CT lk = X::lnkf(rx, lnT, invT);
-      CT fwd = X::ex(lk);
-      for (int j = 0; j < rx.nr; ++j) fwd *= Cs[rx.reac[j] * kChemThreads];
-      CT rev = CT();
-      if (rx.reversible) {
-        CT dG = CT();
-        for (int j = 0; j < rx.np; ++j) dG += Gs[rx.prod[j] * kChemThreads];
-        for (int j = 0; j < rx.nr; ++j) dG -= Gs[rx.reac[j] * kChemThreads];
-        rev = X::ex(X::rev_arg(rx, lk, dG, lp));
-        for (int j = 0; j < rx.np; ++j) rev *= Cs[rx.prod[j] * kChemThreads];
-      }
-      CT q = fwd - rev;
-      if (rx.third_body) {
-        CT cm = CT();
-#pragma unroll
-        for (int a = 0; a < M; ++a) cm += X::eff(m, k, a) * C[a];
-        q *= cm;
-      }
-      for (int j = 0; j < rx.nr; ++j) Ws[rx.reac[j] * kChemThreads] -= q;
-      for (int j = 0; j < rx.np; ++j) Ws[rx.prod[j] * kChemThreads] += q;
-    }
-    CT w[M];
+    add_reactions<M>(m, tbasis(Ts), Cs, Ws, sub, L);
+    ff w[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) w[a] = Ws[a * kChemThreads];
     // butterfly sums over the group: every lane ends with the same total
 #pragma unroll
     for (int o = 1; o < L; o <<= 1)
 #pragma unroll
-      for (int a = 0; a < M; ++a) w[a] += shfl_xor_ct(gmask, w[a], o);
+      for (int a = 0; a < M; ++a) ff_acc(w[a], shfl_xor_ct(gmask, w[a], o));
 #pragma unroll
-    for (int a = 0; a < M; ++a) r[a] += X::dt_sub(un) * (w[a] * X::mm(m, a));
+    for (int a = 0; a < M; ++a) r[a] += X::increment(m, un, a, ff_norm(w[a]));
   }
 }
 
@@ -815,7 +748,7 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
     put(RC::Y + a, YR[a]);
     const bool tiny = species_velocity_undefined<D, RT>(rs[a], js[a]);
 #pragma unroll
-    for (int d = 0; d < D; ++d) put(RC::US + a * D + d, tiny ? uR[d] : js[a][d] / rs[a]);
+    for (int d = 0; d < D; ++d) put(RC::US + a * D + d, tiny ? RT(0) : js[a][d] / rs[a] - uR[d]);
   }
   // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3), T_0 the T just solved
   CT r0[M - 1];
@@ -863,18 +796,27 @@ template <> struct MixParams<float> {
   }
 };
 
+__device__ __forceinline__ float exp_of(float x) { return exp(x); }
+__device__ __forceinline__ double exp_of(double x) { return exp_tang(x); }
+
 // ---------------------------------------------------------------------------
 // Per-node collision parameters: everything the direction loop needs
 // (Sec. 2.3 Eqs. betaa, taua, transform1; Sec. 3.3 Eq. Pex; Sec. 3.4 Eqs.
 // gstar, qdiff, corrFourier; Sec. 2.4 Eq. R3).
+// The diffusion velocities and what only they need: float-float in the FP64
+// path (solve_dd_strided), FP32 in the mixed path.
+template <typename RT> struct DiffType { using type = RT; };
+template <> struct DiffType<double> { using type = ff; };
 template <int D, int M, typename RT> struct NodePar {
   RT rho, om, U, theta;          // density, omega, internal energy, R T (lattice)
   RT u[D], Pex[D], W[D];         // velocity, extended diagonal pressure, energy-flux term
-  RT th[M], V[M][D], rs[M];      // theta_b, diffusion velocities, rho_b
-  RT cF[M - 1], om1[M - 1], hh[M - 1];  // (beta_a - 1) Y_a s, 1 - 2 beta_a, 2 beta_a rho_a + drho_a
+  RT th[M], rs[M];               // theta_b, rho_b
+  typename DiffType<RT>::type V[M][D], cF[M - 1];  // diffusion velocities, (beta_a - 1) Y_a s
+  RT om1[M - 1], hh[M - 1];      // 1 - 2 beta_a, 2 beta_a rho_a + drho_a
 };
 
-// Field offsets of NodePar stored field-major [field][N] (split collision).
+// Field offsets of NodePar stored field-major [field][N] (split collision);
+// float-float fields as packed pairs (ff_pack).
 template <int D, int M> struct CPar {
   static constexpr int TH = 0;
   static constexpr int V = TH + M;
@@ -909,41 +851,53 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
   const int y = (int)((n / g.nx) % g.ny);
   const int z = (int)(n / ((long long)g.nx * g.ny));
 
-  // node scalars in the parameter type PT (FP64 in the FP64 path, FP32 in
-  // the mixed path, whose temperature and chemistry run in float-float);
-  // lattice-type values (RT) for gradients, the solve and the collision
-  using PT = RT;
-  using MP = MixParams<PT>;
-  const PT rho = PT(rec[RC::RHO * N + n]);
+  // node scalars in the lattice type; the diffusion velocities in VT
+  using MP = MixParams<RT>;
+  using VT = typename DiffType<RT>::type;
+  const RT rho = rec[RC::RHO * N + n];
   const double T_d = __ldcg(Tf + n);
-  const PT T = PT(T_d);
-  const PT E = PT(rec[RC::E * N + n]);
-  PT u[D], Y[M];
-  RT q[D], P[NP], V[M][D];
-  PT usq = PT(0);
+  const RT T = RT(T_d);
+  const RT E = rec[RC::E * N + n];
+  RT u[D], Y[M], q[D], P[NP], usq = RT(0);
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    u[d] = PT(rec[(RC::U + d) * N + n]);
+    u[d] = rec[(RC::U + d) * N + n];
     q[d] = rec[(RC::QF + d) * N + n];
     usq += u[d] * u[d];
   }
 #pragma unroll
   for (int k = 0; k < NP; ++k) P[k] = rec[(RC::P + k) * N + n];
 #pragma unroll
-  for (int a = 0; a < M; ++a) {
-    Y[a] = PT(rec[(RC::Y + a) * N + n]);
+  for (int a = 0; a < M; ++a) Y[a] = rec[(RC::Y + a) * N + n];
+
+  // species enthalpies H_a/c^2 (Horner in FP64; in the mixed path summed in
+  // float-float, rounded)
+  RT Ha[M];
+  if constexpr (sizeof(RT) == 8) {
 #pragma unroll
-    for (int d = 0; d < D; ++d) V[a][d] = rec[(RC::US + a * D + d) * N + n] - RT(u[d]);
+    for (int a = 0; a < M; ++a)
+      Ha[a] = fma(T, fma(T, fma(T, un.hl[3][a], un.hl[2][a]), un.hl[1][a]), un.hl[0][a]);
+  } else {
+    const ff T1 = ff_of_double(T_d), T2 = T1 * T1, T3 = T2 * T1;
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+      ff h = un.hl_f[0][a];
+      ff_fma_acc(h, un.hl_f[1][a], T1);
+      ff_fma_acc(h, un.hl_f[2][a], T2);
+      ff_fma_acc(h, un.hl_f[3][a], T3);
+      Ha[a] = ff_norm(h).hi;
+    }
   }
 
-  // isotropic gradients d_a Phi_a and grad Y_a: 3 sum_i w_i c_ia phi(x + c_i)
-  RT dPhi[D], gY[M][D];
+  // isotropic gradients: d_a Phi_a, and sum_a H_a grad Y_a with this node's
+  // H_a, whose sum over the species is taken at each neighbour first (M + 3
+  // multiply-adds per neighbour instead of 3 M, and three sums in registers
+  // instead of 3 M): 3 sum_i w_i c_i phi(x + c_i)
+  RT dPhi[D], corr[D], HYself = RT(0);
 #pragma unroll
-  for (int d = 0; d < D; ++d) {
-    dPhi[d] = RT(0);
+  for (int d = 0; d < D; ++d) dPhi[d] = corr[d] = RT(0);
 #pragma unroll
-    for (int a = 0; a < M; ++a) gY[a][d] = RT(0);
-  }
+  for (int a = 0; a < M; ++a) HYself += Ha[a] * Y[a];
   // ghost values beyond non-periodic faces and on solid nodes: walls Phi = 0,
   // inlet the inlet state's Phi, outlet the node's own Phi; Y the node's own
   RT phi_self[D], phi_in[D];
@@ -995,6 +949,12 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
       const RT wy = cyi == 0 ? RT(2.0 / 3.0) : RT(1.0 / 6.0);
       const RT wz = D == 3 ? (czi == 0 ? RT(2.0 / 3.0) : RT(1.0 / 6.0)) : RT(1);
       const RT w3 = RT(3) * ((ix == 1 ? RT(2.0 / 3.0) : RT(1.0 / 6.0)) * wy * wz);
+      RT hy = HYself;
+      if (gk == BK_NONE) {
+        hy = RT(0);
+#pragma unroll
+        for (int a = 0; a < M; ++a) hy += Ha[a] * __ldg(rec + (RC::Y + a) * N + nb);
+      }
 #pragma unroll
       for (int d = 0; d < D; ++d) {
         if (cvi[d] == 0) continue;
@@ -1002,144 +962,189 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
         const RT pv = gk == BK_NONE ? __ldg(rec + (RC::PHI + d) * N + nb)
                       : (gk == BK_INLET ? phi_in[d] : (gk == BK_OUTLET ? phi_self[d] : RT(0)));
         dPhi[d] += wc * pv;
-#pragma unroll
-        for (int a = 0; a < M; ++a)
-          gY[a][d] += wc * (gk == BK_NONE ? __ldg(rec + (RC::Y + a) * N + nb) : RT(Y[a]));
+        corr[d] += wc * hy;
       }
     }
   }
 
-  // relaxation parameters (Sec. 2.3 Eqs. betaa, taua; Sec. 3.5 Eqs. mu, lambda)
-  PT Rmix = PT(0);
+  // relaxation parameters (Sec. 2.3 Eqs. betaa, taua; Sec. 3.5 Eqs. mu,
+  // lambda): 1/tau_ab = s K_ab; with xr = nu/theta, omega = 1/(xr + 1/2),
+  // omega1 = 1/(xr/Pr + 1/2) and (2 - omega)/(2 omega) = xr
+  RT Rmix = RT(0);
 #pragma unroll
   for (int a = 0; a < M; ++a) Rmix += Y[a] * MP::inv_mm(mech, a);
-  Rmix *= PT(R_U);
-  const PT theta = Rmix * T * MP::inv_c2(un);
-  const PT lnTr = log(T * PT(1.0 / T_REF));
-  const PT s_tau = MP::s_pref(un) * rho * T * T * exp(-MP::D_T_exp(mech) * lnTr);
-  PT mu = MP::mu0(mech);
+  Rmix *= RT(R_U);
+  const RT theta = Rmix * T * MP::inv_c2(un);
+  const RT lnTr = log(T * RT(1.0 / T_REF));
+  const RT s_tau = MP::s_pref(un) * rho * T * T * exp_of(-MP::D_T_exp(mech) * lnTr);
+  RT mu = MP::mu0(mech);
   if (mech.wilke) {
     // Wilke's mixing rule over the species viscosities (the mole fractions'
     // normalisation cancels between numerator and denominator)
-    PT X[M];
+    RT X[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) X[a] = Y[a] * MP::inv_mm(mech, a);
-    mu = PT(0);
+    mu = RT(0);
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-      PT den = PT(0);
+      RT den = RT(0);
 #pragma unroll
       for (int b = 0; b < M; ++b) den += X[b] * MP::wilke_phi(mech, a, b);
       mu += X[a] * MP::mu0_sp(mech, a) / den;
     }
   }
-  mu *= exp(MP::mu_T_exp(mech) * lnTr);
-  const PT nu = mu / rho * MP::nu_pref(un);
-  const PT omega = PT(1) / (nu / theta + PT(0.5));
-  const PT omega1 = PT(1) / (nu * MP::inv_prandtl(mech) / theta + PT(0.5));
-  PT inv_tau_a[M];
-#pragma unroll
-  for (int a = 0; a < M; ++a) {
-    PT acc = PT(0);
-#pragma unroll
-    for (int b = 0; b < M; ++b)
-      if (b != a) acc += Y[b] * (s_tau * kcoef<PT>(mech, a, b));
-    inv_tau_a[a] = acc;
-  }
+  mu *= exp_of(MP::mu_T_exp(mech) * lnTr);
+  const RT Pres = rho * theta;
+  const RT iP = RT(1) / Pres;
+  const RT xr = mu * MP::nu_pref(un) * iP;
+  const RT h0 = xr + RT(0.5), h1 = xr * MP::inv_prandtl(mech) + RT(0.5);
+  const RT ih = RT(1) / (h0 * h1);
+  const RT omega = h1 * ih, omega1 = h0 * ih;
 
-  // diffusion velocities, Eq. transform1: A V = u_a - u  (V holds the rhs).
-  // Each thread's matrix lives in shared memory, entry-major with the block's
-  // threads contiguous (no bank conflicts): in registers it would not fit
-  // beside the node's other state and spills to local memory.
+  // diffusion velocities, Eq. transform1: A V = u_a - u  (V holds the rhs),
+  // A_aa = 1 + 1/(2 tau_a), A_ab = -Y_b/(2 tau_ab).  Each thread's matrix lives
+  // in shared memory, entry-major with the block's threads contiguous (no
+  // bank conflicts): in registers it would not fit beside the node's other
+  // state and spills to local memory.
+  VT V[M][D], inv_tau_a[M], sv;
   {
     extern __shared__ unsigned char smem_raw[];
-    RT* As = reinterpret_cast<RT*>(smem_raw) + threadIdx.x;
+    VT* As = reinterpret_cast<VT*>(smem_raw) + threadIdx.x;
     const int st = kBS;
+    if constexpr (sizeof(RT) == 8) {
+      sv = ff_of_double(s_tau);
+      const ff sh(-0.5f * sv.hi, -0.5f * sv.lo);
+      ff Yv[M];
 #pragma unroll
-    for (int a = 0; a < M; ++a)
+      for (int a = 0; a < M; ++a) Yv[a] = ff_of_double(Y[a]);
 #pragma unroll
-      for (int b = 0; b < M; ++b)
-        As[(a * M + b) * st] = RT(a == b ? PT(1) + PT(0.5) * inv_tau_a[a]
-                                         : PT(-0.5) * Y[b] * (s_tau * kcoef<PT>(mech, a, b)));
-    solve_dd_strided<M, D, RT>(As, st, V);
+      for (int a = 0; a < M; ++a) {
+        ff acc;
+#pragma unroll
+        for (int b = 0; b < M; ++b)
+          if (b != a) ff_fma_acc(acc, mech.K_f[a][b], Yv[b]);
+        inv_tau_a[a] = sv * ff_norm(acc);
+        ff dg(1.f);
+        ff_acc(dg, ff(0.5f * inv_tau_a[a].hi, 0.5f * inv_tau_a[a].lo));
+        As[(a * M + a) * st] = ff_norm(dg);
+#pragma unroll
+        for (int d = 0; d < D; ++d) V[a][d] = ff_of_double(rec[(RC::US + a * D + d) * N + n]);
+      }
+#pragma unroll
+      for (int b = 0; b < M; ++b) {
+        const ff y = sh * Yv[b];
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+          if (b != a) As[(a * M + b) * st] = y * mech.K_f[a][b];
+      }
+    } else {
+      sv = s_tau;
+#pragma unroll
+      for (int a = 0; a < M; ++a) {
+        RT acc = RT(0);
+#pragma unroll
+        for (int b = 0; b < M; ++b)
+          if (b != a) acc += Y[b] * kcoef<RT>(mech, a, b);
+        inv_tau_a[a] = s_tau * acc;
+        As[(a * M + a) * st] = RT(1) + RT(0.5) * inv_tau_a[a];
+#pragma unroll
+        for (int d = 0; d < D; ++d) V[a][d] = rec[(RC::US + a * D + d) * N + n];
+      }
+#pragma unroll
+      for (int b = 0; b < M; ++b) {
+        const RT y = RT(-0.5) * s_tau * Y[b];
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+          if (b != a) As[(a * M + b) * st] = y * kcoef<RT>(mech, a, b);
+      }
+    }
+    solve_dd_strided<M, D>(As, st, V);
   }
 
   // species densities; the reaction increments come from the moments kernel
-  PT rs[M];
+  RT rs[M];
 #pragma unroll
   for (int a = 0; a < M; ++a) rs[a] = rho * Y[a];
 
   // energy-flux correction W = (omega - omega1)(q* - q^eq), folded form
-  const PT U_lat = E - PT(0.5) * usq;
+  const RT U_lat = E - RT(0.5) * usq;
   RT W[D];
   {
-    RT diff[D], corr[D];
+    VT diff[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) { diff[d] = RT(0); corr[d] = RT(0); }
+    for (int d = 0; d < D; ++d) diff[d] = VT();
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-      RT Ha;
-      if constexpr (kFF<RT>) {
-        const ff Tf_(T);
-        Ha = ((species_U_ff(mech, a, Tf_) + ff(mech.Ra_s[a]) * Tf_) * un.inv_c2_f).hi;
-      } else {
-        Ha = RT((species_U(mech, a, T_d) + mech.Ra[a] * T_d) * un.inv_c2);
-      }
-      const RT HY = Ha * RT(Y[a]);
+      if constexpr (sizeof(RT) == 8) {
+        const ff HY = ff_of_double(Ha[a] * Y[a]);
 #pragma unroll
-      for (int d = 0; d < D; ++d) {
-        diff[d] += HY * V[a][d];
-        corr[d] += Ha * gY[a][d];
+        for (int d = 0; d < D; ++d) ff_fma_acc(diff[d], HY, V[a][d]);
+      } else {
+        const RT HY = Ha[a] * Y[a];
+#pragma unroll
+        for (int d = 0; d < D; ++d) diff[d] += HY * V[a][d];
       }
     }
-    const RT rhoR = RT(rho), thR = RT(theta), ER = RT(E);
-    const RT Pres = rhoR * thR;
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      const RT ud = RT(u[d]);
-      const RT q_eq = rhoR * ud * (ER + thR);
+      const RT ud = u[d];
+      const RT q_eq = rho * ud * (E + theta);
       RT uP = RT(0);
 #pragma unroll
       for (int b = 0; b < D; ++b) {
-        const RT ub = RT(u[b]);
-        const RT Peq = rhoR * ub * ud + (b == d ? Pres : RT(0));
-        uP += ub * (P[pidx<D>(b, d)] - Peq);
+        const RT Peq = rho * u[b] * ud + (b == d ? Pres : RT(0));
+        uP += u[b] * (P[pidx<D>(b, d)] - Peq);
       }
       const RT q_ex = RT(-0.5) * ud * dPhi[d];
-      W[d] = RT(omega - omega1) * (q[d] - q_eq - uP + q_ex) + RT(omega1) * rhoR * diff[d] +
-             RT(PT(0.5) * (PT(2) - omega1)) * Pres * corr[d];
+      RT df;
+      if constexpr (sizeof(RT) == 8) df = double_of_ff(diff[d]);
+      else df = diff[d];
+      W[d] = (omega - omega1) * (q[d] - q_eq - uP + q_ex) + omega1 * rho * df +
+             (RT(0.5) * (RT(2) - omega1)) * Pres * corr[d];
     }
   }
 
-  // per-lattice parameters in the collision type
+  // per-lattice parameters
 #pragma unroll
   for (int a = 0; a < M; ++a) {
-    p.th[a] = RT(MP::Ra(mech, a) * T * MP::inv_c2(un));
-    p.rs[a] = RT(rs[a]);
+    p.th[a] = MP::Ra(mech, a) * T * MP::inv_c2(un);
+    p.rs[a] = rs[a];
 #pragma unroll
     for (int d = 0; d < D; ++d) p.V[a][d] = V[a][d];
   }
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    p.u[d] = RT(u[d]);
-    p.Pex[d] = RT(theta + u[d] * u[d] + (PT(2) - omega) / (PT(2) * rho * omega) * PT(dPhi[d]));
+    p.u[d] = u[d];
+    p.Pex[d] = theta + u[d] * u[d] + xr * (iP * theta) * dPhi[d];
     p.W[d] = W[d];
   }
-  p.rho = RT(rho);
-  p.om = RT(omega);
-  p.U = RT(U_lat);
-  p.theta = RT(theta);
+  p.rho = rho;
+  p.om = omega;
+  p.U = U_lat;
+  p.theta = theta;
   // species coefficients of the update
   //   f_a + 2 beta_a (rho_a psi_a - f_a) + cF_a sum_b K_ab d_b + drho_a psi_a
   //     = f_a om1_a + psi_a hh_a + cF_a sum_b K_ab d_b,
   // cF_a = (beta_a - 1) Y_a s (1/tau_ab = s K_ab), om1_a = 1 - 2 beta_a,
-  // hh_a = 2 beta_a rho_a + drho_a
+  // hh_a = 2 beta_a rho_a + drho_a; beta = 1 / (2 tau + 1) to the precision of
+  // the diffusion velocities (om1 and hh share its rounding, so that mass is
+  // conserved)
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
-    const PT beta = inv_tau_a[a] / (PT(2) + inv_tau_a[a]);
-    p.cF[a] = RT((beta - PT(1)) * Y[a] * s_tau);
-    p.om1[a] = RT(PT(1) - PT(2) * beta);
-    p.hh[a] = RT(PT(2) * beta * rs[a] + PT(rec[(RC::DRHO + a) * N + n]));
+    RT beta;
+    if constexpr (sizeof(RT) == 8) {
+      ff den(2.f);
+      ff_acc(den, inv_tau_a[a]);
+      const ff r = ff_rcp(ff_norm(den));
+      beta = double_of_ff(inv_tau_a[a] * r);
+      // beta - 1 = -2 / (2 + 1/tau)
+      p.cF[a] = ff(-2.f * r.hi, -2.f * r.lo) * (ff_of_double(Y[a]) * sv);
+    } else {
+      beta = inv_tau_a[a] / (RT(2) + inv_tau_a[a]);
+      p.cF[a] = (beta - RT(1)) * Y[a] * s_tau;
+    }
+    p.om1[a] = RT(1) - RT(2) * beta;
+    p.hh[a] = RT(2) * beta * rs[a] + rec[(RC::DRHO + a) * N + n];
   }
 }
 
@@ -1270,6 +1275,11 @@ __device__ __forceinline__ void collide_direction(const PS& ps, const XYPart<D, 
   }
 }
 
+__device__ __forceinline__ float value_of(float v) { return v; }
+__device__ __forceinline__ double value_of(ff v) { return double_of_ff(v); }
+__device__ __forceinline__ float stored(float v) { return v; }
+__device__ __forceinline__ double stored(ff v) { return ff_pack(v); }
+
 // Parameters held in registers (fused placement).  The species axis factors
 // come from a table in this thread's shared-memory column (FP32, entry stride
 // kBS) or are formed directly, except, in FP64 3D, those of the y and z axes,
@@ -1277,12 +1287,16 @@ __device__ __forceinline__ void collide_direction(const PS& ps, const XYPart<D, 
 // kBS, d = 1, 2).
 template <int D, int M, typename RT> struct RegPar {
   const NodePar<D, M, RT>& p;
-  RT Afv[D][3], Bfv[D][3];
+  RT Afv[D][3], Bfv[D][3], cFv[M - 1], Vx[M];
   const RT* tab;
   const RT* yztab;
   __device__ RegPar(const NodePar<D, M, RT>& p_, const RT* tab_, const RT* yztab_ = nullptr)
       : p(p_), tab(tab_), yztab(yztab_) {
     energy_factors<D, RT>(p.u, p.theta, Afv, Bfv);
+#pragma unroll
+    for (int a = 0; a < M - 1; ++a) cFv[a] = value_of(p.cF[a]);
+#pragma unroll
+    for (int b = 0; b < M; ++b) Vx[b] = value_of(p.V[b][0]);
   }
   __device__ RT rho() const { return p.rho; }
   __device__ RT om() const { return p.om; }
@@ -1291,7 +1305,7 @@ template <int D, int M, typename RT> struct RegPar {
   __device__ RT Pex(int d) const { return p.Pex[d]; }
   __device__ RT W(int d) const { return p.W[d]; }
   __device__ RT rs(int a) const { return p.rs[a]; }
-  __device__ RT cF(int a) const { return p.cF[a]; }
+  __device__ RT cF(int a) const { return cFv[a]; }
   __device__ RT om1(int a) const { return p.om1[a]; }
   __device__ RT hh(int a) const { return p.hh[a]; }
   __device__ RT Af(int d, int c) const { return c == 0 ? Afv[d][1] : (c > 0 ? Afv[d][2] : Afv[d][0]); }
@@ -1300,7 +1314,7 @@ template <int D, int M, typename RT> struct RegPar {
   __device__ RT sp(int set, int b, int d, int c) const {
     if (tab) return tab[(((set * M + b) * D + d) * 3 + c + 1) * kBS];
     if (D == 3 && d > 0 && yztab) return yztab[(((set * M + b) * 2 + d - 1) * 3 + c + 1) * kBS];
-    const RT xs = set ? p.u[d] + p.V[b][d] : p.u[d];
+    const RT xs = set ? p.u[d] + (d == 0 ? Vx[b] : RT(value_of(p.V[b][d]))) : p.u[d];
     return psi1<RT>(c, xs, p.th[b] + xs * xs);
   }
 };
@@ -1345,7 +1359,7 @@ __device__ __forceinline__ void collide_body(const S* __restrict__ src, S* __res
       for (int b = 0; b < M; ++b)
 #pragma unroll
         for (int d = 1; d < 3; ++d) {
-          const RT xs = set ? p.u[d] + p.V[b][d] : p.u[d];
+          const RT xs = set ? p.u[d] + RT(value_of(p.V[b][d])) : p.u[d];
           const RT Ps = p.th[b] + xs * xs;
 #pragma unroll
           for (int c = -1; c <= 1; ++c)
@@ -1392,11 +1406,11 @@ __device__ __forceinline__ void prep_body(const RT* __restrict__ rec,
     cp[(CP::TH + b) * N + n] = p.th[b];
     cp[(CP::RS + b) * N + n] = p.rs[b];
 #pragma unroll
-    for (int d = 0; d < D; ++d) cp[(CP::V + b * D + d) * N + n] = p.V[b][d];
+    for (int d = 0; d < D; ++d) cp[(CP::V + b * D + d) * N + n] = stored(p.V[b][d]);
   }
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
-    cp[(CP::CF + a) * N + n] = p.cF[a];
+    cp[(CP::CF + a) * N + n] = stored(p.cF[a]);
     cp[(CP::OM1 + a) * N + n] = p.om1[a];
     cp[(CP::HH + a) * N + n] = p.hh[a];
   }
@@ -1417,9 +1431,7 @@ constexpr int kCollTPN = 9;      // threads per node (warps per block)
 
 // shared-memory entries per node of k_coll: parameters, energy factors,
 // species axis-factor tables
-template <int D, int M> constexpr int coll_smem_entries() {
-  return CPar<D, M>::NF + 6 * D + 2 * M * D * 3;
-}
+template <int D, int M, typename RT> constexpr int coll_smem_entries();
 
 // Parameters of node j of the block, field f at s[f * kCollNodes + j].
 template <int D, int M, typename RT> struct SmemPar {
@@ -1445,6 +1457,177 @@ template <int D, int M, typename RT> struct SmemPar {
   }
 };
 
+// Layout of k_coll's shared memory in FP64 (8-byte entries per node): the
+// parameters, the energy factors, the FP64 axis factors E of every species'
+// equilibrium, and float-float tables (packed pairs) of the Stefan-Maxwell
+// term's factors:
+//   e_d(c), the axis factor of psi(u, theta_b), and t_d(c) = s_d(c) - e_d(c),
+//   s_d(c) that of psi(u + V_b, theta_b), formed without cancellation from
+//   V_b (t(0) = -V (2u + V), t(+-1) = (V (2u + V) +- V)/2); for x, s and t
+//   times -rho_b.
+template <int D, int M> struct Coll64 {
+  static constexpr int AF = CPar<D, M>::NF, BF = AF + 3 * D, E = BF + 3 * D;
+  static constexpr int F = E + M * D * 3;       // ff pairs of (b, d): 6 entries
+  static constexpr int N = F + M * D * 6;
+  static constexpr int e(int b, int d, int c) { return E + (b * D + d) * 3 + c + 1; }
+  // first of a pair: x: -rho s(c), then -rho t(c); y, z: e(c), then t(c)
+  static constexpr int f(int b, int d, int c) { return F + (b * D + d) * 6 + c + 1; }
+};
+template <int D, int M, typename RT> constexpr int coll_smem_entries() {
+  return sizeof(RT) == 8 ? Coll64<D, M>::N : CPar<D, M>::NF + 6 * D + 2 * M * D * 3;
+}
+
+// The FP64 collision of one block of TPN warps, 32 nodes (lane = node), the
+// directions dealt to the warps as in coll_block.
+//
+// What bounds it is the FP64 pipe: an FP64 instruction occupies an SM quarter
+// for 64 cycles, an FP32 one for 1.  So only what must carry 53 bits runs
+// there: per population the equilibrium and the relaxation (two fused
+// multiply-adds for a species, f om1 + cF F + psi hh with hh folded into the
+// (c_x, c_y) part), f^ex, g^eq and the axis factors.  The Stefan-Maxwell term
+//   F_a = sum_b K_ab d_b,  d_b = rho_b (psi(u) - psi(u + V_b)),
+// half of the FP64 work before, is a correction of the relative size of V:
+// float-float (48 bits) differences and sums of it stay below FP64's
+// rounding of the population.  d_b is formed from the differences t of the
+// axis factors, without the cancellation of psi(u) - psi(u + V_b):
+//   -d_b / rho_b = (t_x e_y + s_x t_y) e_z + s_x s_y t_z.
+template <int D, int M, typename S, int TPN>
+__device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __restrict__ dst,
+                                             const double* __restrict__ cp, const Geom& g,
+                                             const BCDev& bc, const DevMech& mech,
+                                             long long n0, double* __restrict__ sm) {
+  using CP = CPar<D, M>;
+  using T = Coll64<D, M>;
+  constexpr int Q = Lat<D>::Q;
+  const long long N = g.N;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long n = n0 + lane;
+  const int tag = n < N ? (bc.tag ? bc.tag[n] : TAG_BULK) : TAG_SOLID;
+  const bool valid = tag != TAG_SOLID;
+  double* const s = sm + lane;
+  for (int f = w; f < CP::NF; f += TPN)
+    s[f * kCollNodes] = valid ? __ldcg(cp + f * N + n) : 0.0;
+  __syncthreads();
+  if (valid) {
+    if (w == TPN - 1) {
+      double u[D], Af[D][3], Bf[D][3];
+#pragma unroll
+      for (int d = 0; d < D; ++d) u[d] = s[(CP::U + d) * kCollNodes];
+      energy_factors<D, double>(u, s[CP::THETA * kCollNodes], Af, Bf);
+#pragma unroll
+      for (int d = 0; d < D; ++d)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          s[(T::AF + d * 3 + k) * kCollNodes] = Af[d][k];
+          s[(T::BF + d * 3 + k) * kCollNodes] = Bf[d][k];
+        }
+    }
+    for (int e = w; e < M * D; e += TPN) {
+      const int b = e / D, d = e % D;
+      const double u = s[(CP::U + d) * kCollNodes];
+      const double P = fma(u, u, s[(CP::TH + b) * kCollNodes]), hu = 0.5 * u;
+      const double E[3] = {fma(0.5, P, -hu), 1.0 - P, fma(0.5, P, hu)};
+      const ff V = ff_unpack(s[(CP::V + b * D + d) * kCollNodes]);
+      ff uf = ff_of_double(u);
+      uf = ff(2.f * uf.hi, 2.f * uf.lo) + V;
+      const ff dP = V * uf;                     // V (2u + V)
+      const ff t0 = -dP, tp = dP + V, tm = dP - V;
+      const ff t[3] = {ff(0.5f * tm.hi, 0.5f * tm.lo), t0, ff(0.5f * tp.hi, 0.5f * tp.lo)};
+      const ff mr = -ff_of_double(s[(CP::RS + b) * kCollNodes]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        s[(T::E + e * 3 + c) * kCollNodes] = E[c];
+        const ff ef = ff_of_double(E[c]);
+        const ff first = d == 0 ? mr * (ef + t[c]) : ef;
+        const ff second = d == 0 ? mr * t[c] : t[c];
+        s[(T::F + e * 6 + c) * kCollNodes] = ff_pack(first);
+        s[(T::F + e * 6 + 3 + c) * kCollNodes] = ff_pack(second);
+      }
+    }
+  }
+  __syncthreads();
+  if (!valid) return;
+  auto P = [&](int f) { return s[f * kCollNodes]; };
+  auto PF = [&](int f) { return ff_unpack(s[f * kCollNodes]); };
+  const int x = (int)(n % g.nx);
+  const int y = (int)((n / g.nx) % g.ny);
+  const int z = (int)(n / ((long long)g.nx * g.ny));
+  constexpr int NZ = D == 3 ? 3 : 1;
+  constexpr int CH = (Q + TPN - 1) / TPN;
+  const int k0 = w * CH, k1 = min(k0 + CH, Q);
+  if (k0 >= k1) return;
+  ff A[M], SS[M];              // t_x e_y + s_x t_y and s_x s_y, times -rho_b
+  double eh[M - 1];            // hh_a e_x e_y
+  double fxy = 0.0, gP = 0.0, gQ = 0.0;
+  const double rho = P(CP::RHO), om = P(CP::OM);
+  int jcur = -1;
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) {
+    const int j = k / NZ, i = j + 9 * (k % NZ);
+    const int cx = cvel(j, 0), cy = cvel(j, 1), cz = D == 3 ? k % NZ - 1 : 0;
+    double fin[M + 1];
+    load_direction<D, M, S, double>(src, bc, tag, N, node_shift<D>(x, y, z, i, -1, g), i,
+                                    g.codec, fin);
+    if (j != jcur) {
+      jcur = j;
+#pragma unroll
+      for (int b = 0; b < M; ++b) {
+        const ff sx = PF(T::f(b, 0, cx)), tx = PF(T::f(b, 0, cx) + 3);
+        const ff ey = PF(T::f(b, 1, cy)), ty = PF(T::f(b, 1, cy) + 3);
+        ff v = tx * ey;
+        ff_fma_acc(v, sx, ty);
+        A[b] = ff_norm(v);
+        if constexpr (D == 3) {
+          ff sy = ey;
+          ff_acc(sy, ty);
+          SS[b] = sx * ff_norm(sy);
+        }
+        if (b < M - 1) eh[b] = P(T::e(b, 0, cx)) * P(T::e(b, 1, cy)) * P(CP::HH + b);
+      }
+      fxy = rho * psi1<double>(cx, P(CP::U), P(CP::PEX)) *
+            psi1<double>(cy, P(CP::U + 1), P(CP::PEX + 1));
+      const double ax = P(T::AF + cx + 1), ay = P(T::AF + 3 + cy + 1);
+      gP = ax * ay;
+      gQ = fma(P(CP::UL), gP, fma(P(T::BF + cx + 1), ay, ax * P(T::BF + 3 + cy + 1)));
+    }
+    ff dd[M];
+#pragma unroll
+    for (int b = 0; b < M; ++b) {
+      if constexpr (D == 3) {
+        ff v = A[b] * PF(T::f(b, 2, cz));
+        ff_fma_acc(v, SS[b], PF(T::f(b, 2, cz) + 3));
+        dd[b] = ff_norm(v);
+      } else {
+        dd[b] = A[b];
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < M - 1; ++a) {
+      ff F;
+#pragma unroll
+      for (int b = 0; b < M; ++b)
+        if (b != a) ff_fma_acc(F, mech.K_f[a][b], dd[b]);
+      F = PF(CP::CF + a) * ff_norm(F);
+      const double ez = D == 3 ? P(T::e(a, D - 1, cz)) : 1.0;
+      const double base = fma(fin[a], P(CP::OM1 + a), double_join(F));
+      dst[(long long)(a * Q + i) * N + n] = D == 3 ? fma(eh[a], ez, base) : eh[a] + base;
+    }
+    double fex = fxy, geq = gQ;
+    if constexpr (D == 3) {
+      fex *= psi1<double>(cz, P(CP::U + 2), P(CP::PEX + 2));
+      geq = fma(P(T::AF + 6 + cz + 1), gQ, gP * P(T::BF + 6 + cz + 1));
+    }
+    dst[(long long)((M - 1) * Q + i) * N + n] = fma(om, fex - fin[M - 1], fin[M - 1]);
+    double gn = fma(om, fma(rho, geq, -fin[M]), fin[M]);
+    if (csq(i, D) == 1) {
+#pragma unroll
+      for (int d = 0; d < D; ++d)
+        if (cvel(i, d) != 0) gn += (cvel(i, d) > 0 ? 0.5 : -0.5) * P(CP::W + d);
+    }
+    dst[(long long)(M * Q + i) * N + n] = gn;
+  }
+}
+
 // One block of TPN warps: nodes n0 .. n0 + 31.  sm holds coll_smem_entries *
 // kCollNodes.  The Q directions, taken in the order k = 0 .. Q - 1 with
 // direction (k / NZ) + 9 (k % NZ) (NZ = 3 in 3D: the directions of one
@@ -1454,6 +1637,9 @@ __device__ __forceinline__ void coll_block(const S* __restrict__ src, S* __restr
                                            const RT* __restrict__ cp, const Geom& g,
                                            const BCDev& bc, const DevMech& mech, long long n0,
                                            RT* __restrict__ sm) {
+  if constexpr (sizeof(RT) == 8) {
+    coll_block64<D, M, S, TPN>(src, dst, cp, g, bc, mech, n0, sm);
+  } else {
   using CP = CPar<D, M>;
   using SP = SmemPar<D, M, RT>;
   constexpr int Q = Lat<D>::Q;
@@ -1499,15 +1685,12 @@ __device__ __forceinline__ void coll_block(const S* __restrict__ src, S* __restr
   const int y = (int)((n / g.nx) % g.ny);
   const int z = (int)(n / ((long long)g.nx * g.ny));
   // software pipeline: the next direction's populations are in flight while
-  // this one collides.  FP64 forms the (c_x, c_y) part once per pair and
-  // keeps it in registers; FP32 forms it per direction, which keeps k_coll
-  // within its 56-register budget.
+  // this one collides.  The (c_x, c_y) part is formed per direction, which
+  // keeps k_coll within its 56-register budget.
   constexpr int NZ = D == 3 ? 3 : 1;
   constexpr int CH = (Q + TPN - 1) / TPN;
   const int k0 = w * CH, k1 = min(k0 + CH, Q);
   if (k0 >= k1) return;
-  XYPart<D, M, RT> h;
-  int jcur = -1;
   RT fa[M + 1], fb[M + 1];
   int i = k0 / NZ + 9 * (k0 % NZ);
   load_direction<D, M, S, RT>(src, bc, tag, N, node_shift<D>(x, y, z, i, -1, g), i, g.codec, fa);
@@ -1518,14 +1701,13 @@ __device__ __forceinline__ void coll_block(const S* __restrict__ src, S* __restr
       load_direction<D, M, S, RT>(src, bc, tag, N, node_shift<D>(x, y, z, inext, -1, g), inext,
                                   g.codec, fb);
     const int j = k / NZ;
-    if (sizeof(RT) == 4 || j != jcur) {
-      xy_part<D, M, RT>(ps, cvel(j, 0), cvel(j, 1), h);
-      jcur = j;
-    }
+    XYPart<D, M, RT> h;
+    xy_part<D, M, RT>(ps, cvel(j, 0), cvel(j, 1), h);
     collide_direction<D, M, S, RT>(ps, h, i, fa, dst, N, n, mech, g.codec);
 #pragma unroll
     for (int l = 0; l <= M; ++l) fa[l] = fb[l];
     i = inext;
+  }
   }
 }
 
@@ -1624,7 +1806,7 @@ k_prep(const RT* __restrict__ rec, const double* __restrict__ Tf, RT* __restrict
 }
 
 // FP32: four 288-thread blocks per SM (at most 56 registers), so a grid of
-// the 16k-node flame fits the GPU in one wave; FP64 would spill
+// the 16k-node flame fits the GPU in one wave
 template <int D, int M, typename S, typename RT>
 __global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? 4 : 1)
 k_coll(const S* __restrict__ src, S* __restrict__ dst, const RT* __restrict__ cp,
@@ -1995,9 +2177,9 @@ template <int D, int M, typename S, typename RT> constexpr size_t persist_smem(b
   using R = typename ComputeType<S>::type;
   const size_t bnd = bnode_smem<D, M, R>() * (kPersistThreads / kBnd);
   const size_t prep = (size_t)M * M * kBS * sizeof(RT);
-  const size_t coll = (size_t)coll_smem_entries<D, M>() * kCollNodes * sizeof(RT);
+  const size_t coll = (size_t)coll_smem_entries<D, M, RT>() * kCollNodes * sizeof(RT);
   const size_t fused = (size_t)collide_smem_entries<D, M, RT>() * kBS * sizeof(RT);
-  const size_t chem = kFF<RT> ? chem_slice_bytes<M, ff>() : 0;
+  const size_t chem = chem_slice_bytes<M>();
   size_t m = bnd > chem ? bnd : chem;
   if (split) {
     m = m > prep ? m : prep;
@@ -2110,9 +2292,12 @@ k_diag(const S* __restrict__ pops, const double* __restrict__ Tf, const int* __r
     const double T = newton_T<M>(mech, Y, (rhoE / rho - 0.5 * usq) * un.c * un.c, Tf[n],
                                  un.newton_max_iter, un.newton_rtol, ok);
     if (!ok) atomicOr(status, ST_NEWTON);
-    double rdot[M];
-    production_rates<M>(mech, T, rs, rdot);
-    for (int a = 0; a < M; ++a) q -= (species_U(mech, a, T) + mech.Ra[a] * T) * rdot[a];
+    ff w[M];
+    ff* const Cs = chem_static_slice<M>() + threadIdx.x;
+    for (int a = 0; a < M; ++a) Cs[a * kChemThreads] = ff_of_double(rs[a] * mech.inv_mm[a]);
+    molar_rates<M>(mech, T, w, Cs);
+    for (int a = 0; a < M; ++a)
+      q -= (species_U(mech, a, T) + mech.Ra[a] * T) * (double_of_ff(w[a]) * mech.mm[a]);
     qmax = q;
     nmax = n;
     Tmax = T;
@@ -2195,7 +2380,7 @@ template <int D, int M, typename RT> constexpr size_t prep_smem() {
   return (size_t)M * M * kBS * sizeof(RT);
 }
 template <int D, int M, typename RT> constexpr size_t coll_smem() {
-  return (size_t)coll_smem_entries<D, M>() * kCollNodes * sizeof(RT);
+  return (size_t)coll_smem_entries<D, M, RT>() * kCollNodes * sizeof(RT);
 }
 
 // Kernel attributes (shared memory above the 48 KB default) of every kernel a
@@ -2226,7 +2411,7 @@ static void launch_chem(const Launch& lc, cudaStream_t s, RT* rec, const double*
                         int* status, long long N, const BCDev& bc, const Units& un,
                         const DevMech* mech, int node_set) {
   if (node_set == NODES_INTERFACE && bc.n_if >= kIfChemThreadNodes) {
-    const size_t sm = kFF<RT> ? chem_slice_bytes<M, ff>() : 0;
+    const size_t sm = chem_slice_bytes<M>();
     k_iface_chem<D, M, RT><<<blocks_for(bc.n_if, kChemThreads), kChemThreads, sm, s>>>(
         rec, Tf, status, N, bc.if_node, bc.n_if, un, mech);
     return;
@@ -2414,7 +2599,7 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
     if (node_set == NODES_INTERFACE && gr.n_if_total >= kIfChemThreadNodes) {
       // enough interface nodes to fill the GPU with one thread each
       auto k = k_iface_chem_batch<D, M, RT>;
-      const size_t sm = kFF<RT> ? chem_slice_bytes<M, ff>() : 0;
+      const size_t sm = chem_slice_bytes<M>();
       k<<<batch_grid(k, gr.ntblocks, kBnd, sm, ps), kBnd, sm, st>>>(doms, ndom, gr.ntblocks);
       return;
     }
