@@ -282,37 +282,43 @@ __device__ __forceinline__ void solve_dd_strided(R* A, int st, R (&B)[M][D]) {
 // The same in float-float (the FP64 path's diffusion velocities, which enter
 // the collision only through corrections a thousand times below what they
 // correct: 48 bits of a correction are beyond FP64's rounding of the sum.  In
-// FP64 the elimination took ~800 instructions of 64 cycles).
+// FP64 the elimination took ~800 instructions of 64 cycles), the right-hand
+// sides in the matrix's columns M .. M + D - 1 (rows of M + D entries); they
+// become the solution.  The loop over the rows below the pivot is rolled:
+// unrolled, the code (a dozen instructions per update) outgrows the
+// instruction cache, and fetching it took half of the time.
 template <int M, int D>
-__device__ __forceinline__ void solve_dd_strided(ff* A, int st, ff (&B)[M][D]) {
+__device__ __forceinline__ void solve_dd_ff(ff* A, int st) {
+  constexpr int W = M + D;
 #pragma unroll
   for (int k = 0; k < M; ++k) {
-    const ff inv = ff_rcp(A[(k * M + k) * st]);
-    A[(k * M + k) * st] = inv;
+    const ff inv = ff_rcp(A[(k * W + k) * st]);
+    A[(k * W + k) * st] = inv;
+    ff piv[W];
 #pragma unroll
+    for (int c = k + 1; c < W; ++c) piv[c] = A[(k * W + c) * st];
+#pragma unroll 1
     for (int r = k + 1; r < M; ++r) {
-      const ff f = -(A[(r * M + k) * st] * inv);
+      ff* const row = A + r * W * st;
+      const ff f = -(row[k * st] * inv);
 #pragma unroll
-      for (int c = k + 1; c < M; ++c) {
-        ff v = A[(r * M + c) * st];
-        ff_fma_acc(v, f, A[(k * M + c) * st]);
-        A[(r * M + c) * st] = ff_norm(v);
-      }
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        ff_fma_acc(B[r][d], f, B[k][d]);
-        B[r][d] = ff_norm(B[r][d]);
+      for (int c = k + 1; c < W; ++c) {
+        ff v = row[c * st];
+        ff_fma_acc(v, f, piv[c]);
+        row[c * st] = ff_norm(v);
       }
     }
   }
+#pragma unroll 1
+  for (int d = 0; d < D; ++d) {
+    ff x[M];
 #pragma unroll
-  for (int k = M - 1; k >= 0; --k) {
+    for (int k = M - 1; k >= 0; --k) {
+      ff s = A[(k * W + M + d) * st];
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      ff s = B[k][d];
-#pragma unroll
-      for (int c = k + 1; c < M; ++c) ff_fma_acc(s, -A[(k * M + c) * st], B[c][d]);
-      B[k][d] = ff_norm(s) * A[(k * M + k) * st];
+      for (int c = k + 1; c < M; ++c) ff_fma_acc(s, -A[(k * W + c) * st], x[c]);
+      x[k] = ff_norm(s) * A[(k * W + k) * st];
+      A[(k * W + M + d) * st] = x[k];
     }
   }
 }

@@ -127,12 +127,19 @@ template <> __device__ __forceinline__ float kcoef<float>(const DevMech& m, int 
 constexpr int kBS = 128;
 static_assert(kBS == kChemThreads, "the chemistry's shared-memory slices assume kBS threads");
 
+// shared-memory entries per thread of the diffusion-velocity solve: the
+// matrix, in FP64 (float-float pairs) with the right-hand sides
+template <int D, int M, typename RT> constexpr int solve_smem_entries() {
+  return sizeof(RT) == 8 ? M * (M + D) : M * M;
+}
+
 // shared memory of the collision kernel per thread: the diffusion-velocity
 // matrix, then the axis-factor tables (FP32: every axis; FP64 in 3D: the y
 // and z axes, the whole table would halve the occupancy)
 template <int D, int M, typename RT> constexpr int collide_smem_entries() {
   constexpr int tab = sizeof(RT) == 4 ? 2 * M * D * 3 : (D == 3 ? 2 * M * 2 * 3 : 0);
-  return tab > M * M ? tab : M * M;
+  constexpr int solve = solve_smem_entries<D, M, RT>();
+  return tab > solve ? tab : solve;
 }
 
 template <int D>
@@ -1013,10 +1020,21 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
     const int st = kBS;
     if constexpr (sizeof(RT) == 8) {
       sv = ff_of_double(s_tau);
-      const ff sh(-0.5f * sv.hi, -0.5f * sv.lo);
-      ff Yv[M];
+      constexpr int W = M + D;
+      ff Yv[M], yh[M];
 #pragma unroll
-      for (int a = 0; a < M; ++a) Yv[a] = ff_of_double(Y[a]);
+      for (int a = 0; a < M; ++a) {
+        Yv[a] = ff_of_double(Y[a]);
+        yh[a] = ff(-0.5f * sv.hi, -0.5f * sv.lo) * Yv[a];
+      }
+#pragma unroll 1
+      for (int a = 0; a < M; ++a) {
+#pragma unroll
+        for (int b = 0; b < M; ++b) As[(a * W + b) * st] = yh[b] * mech.K_f[a][b];
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+          As[(a * W + M + d) * st] = ff_of_double(rec[(RC::US + a * D + d) * N + n]);
+      }
 #pragma unroll
       for (int a = 0; a < M; ++a) {
         ff acc;
@@ -1026,17 +1044,13 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
         inv_tau_a[a] = sv * ff_norm(acc);
         ff dg(1.f);
         ff_acc(dg, ff(0.5f * inv_tau_a[a].hi, 0.5f * inv_tau_a[a].lo));
-        As[(a * M + a) * st] = ff_norm(dg);
-#pragma unroll
-        for (int d = 0; d < D; ++d) V[a][d] = ff_of_double(rec[(RC::US + a * D + d) * N + n]);
+        As[(a * W + a) * st] = ff_norm(dg);
       }
+      solve_dd_ff<M, D>(As, st);
 #pragma unroll
-      for (int b = 0; b < M; ++b) {
-        const ff y = sh * Yv[b];
+      for (int a = 0; a < M; ++a)
 #pragma unroll
-        for (int a = 0; a < M; ++a)
-          if (b != a) As[(a * M + b) * st] = y * mech.K_f[a][b];
-      }
+        for (int d = 0; d < D; ++d) V[a][d] = As[(a * W + M + d) * st];
     } else {
       sv = s_tau;
 #pragma unroll
@@ -1057,8 +1071,8 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
         for (int a = 0; a < M; ++a)
           if (b != a) As[(a * M + b) * st] = y * kcoef<RT>(mech, a, b);
       }
+      solve_dd_strided<M, D, RT>(As, st, V);
     }
-    solve_dd_strided<M, D>(As, st, V);
   }
 
   // species densities; the reaction increments come from the moments kernel
@@ -1808,7 +1822,7 @@ k_prep(const RT* __restrict__ rec, const double* __restrict__ Tf, RT* __restrict
 // FP32: four 288-thread blocks per SM (at most 56 registers), so a grid of
 // the 16k-node flame fits the GPU in one wave
 template <int D, int M, typename S, typename RT>
-__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? 4 : 1)
+__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? 4 : 2)
 k_coll(const S* __restrict__ src, S* __restrict__ dst, const RT* __restrict__ cp,
        const __grid_constant__ Geom g, const __grid_constant__ BCDev bc,
        const __grid_constant__ DevMech mech) {
@@ -1970,7 +1984,7 @@ k_prep_batch(const DomainDev* __restrict__ doms, int ndom, int nblk) {
 }
 
 template <int D, int M, typename S, typename RT>
-__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? 4 : 1)
+__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? 4 : 2)
 k_coll_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   extern __shared__ __align__(16) unsigned char coll_raw[];
@@ -2176,7 +2190,7 @@ k_step_persist(const DomainDev* __restrict__ doms, int ndom, int parity,
 template <int D, int M, typename S, typename RT> constexpr size_t persist_smem(bool split) {
   using R = typename ComputeType<S>::type;
   const size_t bnd = bnode_smem<D, M, R>() * (kPersistThreads / kBnd);
-  const size_t prep = (size_t)M * M * kBS * sizeof(RT);
+  const size_t prep = (size_t)solve_smem_entries<D, M, RT>() * kBS * sizeof(RT);
   const size_t coll = (size_t)coll_smem_entries<D, M, RT>() * kCollNodes * sizeof(RT);
   const size_t fused = (size_t)collide_smem_entries<D, M, RT>() * kBS * sizeof(RT);
   const size_t chem = chem_slice_bytes<M>();
@@ -2377,7 +2391,7 @@ template <int D, int M, typename RT> constexpr size_t fused_smem() {
   return (size_t)collide_smem_entries<D, M, RT>() * kBS * sizeof(RT);
 }
 template <int D, int M, typename RT> constexpr size_t prep_smem() {
-  return (size_t)M * M * kBS * sizeof(RT);
+  return (size_t)solve_smem_entries<D, M, RT>() * kBS * sizeof(RT);
 }
 template <int D, int M, typename RT> constexpr size_t coll_smem() {
   return (size_t)coll_smem_entries<D, M, RT>() * kCollNodes * sizeof(RT);
