@@ -251,6 +251,15 @@ __device__ __forceinline__ ff ff_rcp(ff a) {
   e = __fmaf_rn(-q, a.lo, e);
   return fast_two_sum(q, __fmul_rn(q, e));
 }
+// a / b to ~46 bits (a Newton update's quotient)
+__device__ __forceinline__ ff ff_quotient(ff a, ff b) {
+  const float r = __fdiv_rn(1.f, b.hi);
+  const float q = __fmul_rn(a.hi, r);
+  const ff p = two_prod(q, b.hi);
+  float e = __fsub_rn(__fsub_rn(a.hi, p.hi), p.lo);
+  e = __fadd_rn(e, __fmaf_rn(-q, b.lo, a.lo));
+  return fast_two_sum(q, __fmul_rn(e, r));
+}
 // a pair in a double's place
 __device__ __forceinline__ double ff_pack(ff a) {
   return __hiloint2double(__float_as_int(a.hi), __float_as_int(a.lo));

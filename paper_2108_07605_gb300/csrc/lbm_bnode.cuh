@@ -160,6 +160,12 @@ template <typename R> __device__ __forceinline__ R sel3(int c, const R (&t)[3]) 
   return c < 0 ? t[0] : (c == 0 ? t[1] : t[2]);
 }
 
+// FP32 products rounded on their own, and below sums fused explicitly: left
+// to the compiler, a thread's and a warp's procedure (bnode_body, bnode_warp)
+// would not be fused alike
+__device__ __forceinline__ float mul1(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul1(double a, double b) { return a * b; }
+
 template <int D, int M, int l, typename R>
 __device__ __forceinline__ void ptab(const BState<D, M, R>& s, PTab<D, R>& e, const DevMech& m,
                                      const Units& un) {
@@ -189,14 +195,15 @@ __device__ __forceinline__ void gtab(const BState<D, M, R>& s, GTab<D, R>& g) {
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const R ua = s.u[d];
-    const R O1 = s.th * ua + R(0.5) * ua * ua * ua;
-    const R O2 = s.th * s.th + R(2.5) * s.th * ua * ua + R(0.5) * ua * ua * ua * ua;
-    const R P = s.th + ua * ua;
+    const R q = mul1(ua, ua), hq = R(0.5) * q;
+    const R O1 = mul1(ua, s.th + hq);                                  // theta u + u^3/2
+    const R O2 = fma(s.th, s.th, mul1(q, fma(R(2.5), s.th, hq)));
+    const R P = s.th + q;
     g.A[d][0] = R(0.5) * (P - ua);
     g.A[d][1] = R(1) - P;
     g.A[d][2] = R(0.5) * (P + ua);
     g.B[d][0] = R(0.5) * (O2 - O1);
-    g.B[d][1] = R(0.5) * ua * ua - O2;
+    g.B[d][1] = hq - O2;
     g.B[d][2] = R(0.5) * (O2 + O1);
   }
 }
@@ -221,11 +228,11 @@ template <int D, int M, typename R> struct ETab {
       const R ay = sel3(cy, g.A[1]), by = sel3(cy, g.B[1]);
       if constexpr (D == 3) {
         const R az = sel3(cz, g.A[2]), bz = sel3(cz, g.B[2]);
-        rP = ay * az;
-        rQ = g.U * rP + by * az + ay * bz;
+        rP = mul1(ay, az);
+        rQ = fma(g.U, rP, fma(by, az, mul1(ay, bz)));
       } else {
         rP = ay;
-        rQ = g.U * ay + by;
+        rQ = fma(g.U, ay, by);
       }
     } else {
       rp = p.pref * sel3(cy, p.t[1]);
@@ -233,8 +240,9 @@ template <int D, int M, typename R> struct ETab {
     }
   }
   template <int l> __device__ __forceinline__ R evalx(int cx) const {
-    if constexpr (l == M) return g.rho * (sel3(cx, g.A[0]) * rQ + sel3(cx, g.B[0]) * rP);
-    else return rp * sel3(cx, p.t[0]);
+    if constexpr (l == M)
+      return mul1(g.rho, fma(sel3(cx, g.A[0]), rQ, mul1(sel3(cx, g.B[0]), rP)));
+    else return mul1(rp, sel3(cx, p.t[0]));
   }
 };
 
@@ -637,5 +645,504 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
 #pragma unroll
     for (int d = 0; d < D; ++d)
       rec[(RC::US + a * D + d) * N + n] = s.us[(a * D + d) * kBnd] - s.u[d];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The same procedure with one warp per interface node, for grids with few of
+// them (bnode_warp_limit): a thread per node is then a single chain of some
+// thousand dependent loads and sums, whatever the node count (444 us in FP64,
+// 355 us in FP32 for the 32 interface nodes of the 1024x4x4 flame, the
+// critical path of its step; with a warp each, sub-steps included, 70 and 56).  Lane 3 l + p holds lattice l's directions of
+// c_z = p - 1 (D3Q27: 9 populations; D2Q9: 3, of c_y = p - 1); its loads are
+// in flight together, its sums go through shared memory to every lane, and
+// the sums over the species are butterflies over 16 lanes (lane & 15 = the
+// species).  In FP64 the sums are taken in another order than in bnode_body
+// (the two agree to rounding); FP32 sums keep its order, whose rounding a
+// flame's front would amplify.
+
+template <int D, int M> struct WB {
+  static constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP;
+  static constexpr int NR = D == 3 ? 9 : 3;        // populations per lane
+  static constexpr int ZS = 1 + D;                 // sums per lattice
+  static constexpr int Z = 0, P = Z + (M + 1) * ZS;    // sums, momentum flux of f
+  static constexpr int ST = P + NP;                // states: Y [M], u_a [M D]
+  static constexpr int SS = M + M * D;
+  static constexpr int N = ST + 4 * SS;            // R entries per warp
+};
+
+// A state: scalars in every lane, Y and the species velocities (us; used:
+// nullptr when u serves every species) in the warp's shared memory.
+template <int D, int M, typename R> struct WState {
+  R rho, T, th, U;
+  R u[D];
+  R *Y, *us;
+  bool own_us;
+  double T_full;
+};
+
+__device__ __forceinline__ float shfl_xor_ct(unsigned mask, float v, int o) {
+  return __shfl_xor_sync(mask, v, o);
+}
+template <typename V>
+__device__ __forceinline__ V species_sum(V v) {
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) v += shfl_xor_ct(0xffffffffu, v, o);
+  return v;
+}
+
+// theta, U/c^2 from T and Y (bstate_prepare)
+template <int D, int M, typename R>
+__device__ __forceinline__ void wprepare(WState<D, M, R>& s, const DevMech& m, const Units& un,
+                                         int lane) {
+  using CT = typename ChemType<R>::type;
+  const int a = min(lane & 15, M - 1);
+  const R Ya = (lane & 15) < M ? s.Y[a] : R(0);
+  if constexpr (!kFF<R>) {
+    const double Rm = species_sum(double(Ya) * m.inv_mm[a]);
+    const double U = species_sum(double(Ya) * species_U(m, a, double(s.T)));
+    s.th = R(R_U * Rm * double(s.T) * un.inv_c2);
+    s.U = R(U * un.inv_c2);
+  } else {
+    float Rm = 0.f;
+#pragma unroll
+    for (int b = 0; b < M; ++b) Rm += s.Y[b] * m.inv_mm_s[b];
+    const CT U = species_sum(ff(Ya) * species_U_ff(m, a, ff(s.T)));
+    s.th = float(R_U) * Rm * s.T * un.inv_c2_s;
+    s.U = (U * un.inv_c2_f).hi;
+  }
+}
+
+// This lane's partial sums of its populations v; the lattice's totals (and
+// the f lattice's momentum flux) in z.
+template <int D, int M, typename R>
+__device__ __forceinline__ void wsums(const R (&v)[WB<D, M>::NR], R* z, int lane) {
+  using W = WB<D, M>;
+  const int l = lane / 3, p = lane % 3;
+  const bool on = lane < 3 * (M + 1);
+  R sum = R(0), sj[D], sP[W::NP];
+#pragma unroll
+  for (int d = 0; d < D; ++d) sj[d] = R(0);
+#pragma unroll
+  for (int q = 0; q < W::NP; ++q) sP[q] = R(0);
+  // a row (c_y, c_z) of sum sr, difference dx and sx = f_+ + f_-
+  auto add_row = [&](R sr, R dx, R sx, int cy, int cz) {
+    sum += sr;
+    sj[0] += dx;
+    sP[pidx<D>(0, 0)] += sx;
+    if (cy != 0) {
+      sj[1] += cy > 0 ? sr : -sr;
+      sP[pidx<D>(1, 1)] += sr;
+      sP[pidx<D>(0, 1)] += cy > 0 ? dx : -dx;
+    }
+    if constexpr (D == 3) {
+      if (cz != 0) {
+        sj[2] += cz > 0 ? sr : -sr;
+        sP[pidx<D>(2, 2)] += sr;
+        sP[pidx<D>(0, 2)] += cz > 0 ? dx : -dx;
+        if (cy != 0) sP[pidx<D>(1, 2)] += cy == cz ? sr : -sr;
+      }
+    }
+  };
+  const int l0 = min(3 * l, 27);
+  if constexpr (sizeof(R) == 4) {
+    // bsums' order: row after row, every lane of the lattice the whole sum
+#pragma unroll
+    for (int pp = 0; pp < 3; ++pp)
+#pragma unroll
+      for (int r = 0; r < W::NR / 3; ++r) {
+        R w[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) w[q] = __shfl_sync(0xffffffffu, v[3 * r + q], l0 + pp);
+        const R sx = w[0] + w[2];
+        if constexpr (D == 3) add_row(sx + w[1], w[2] - w[0], sx, r - 1, pp - 1);
+        else add_row(sx + w[1], w[2] - w[0], sx, pp - 1, 0);
+      }
+  } else {
+#pragma unroll
+    for (int r = 0; r < W::NR / 3; ++r) {
+      const R sx = v[3 * r] + v[3 * r + 2], dx = v[3 * r + 2] - v[3 * r];
+      add_row(sx + v[3 * r + 1], dx, sx, D == 3 ? r - 1 : 0, 0);
+    }
+    // the terms with this lane's own velocity component p - 1 (c_z; D2Q9: c_y)
+    const R c = on ? R(p - 1) : R(0);
+    sj[D - 1] = c * sum;
+    if constexpr (D == 3) {
+      sP[pidx<D>(2, 2)] = c * c * sum;
+      sP[pidx<D>(0, 2)] = c * sj[0];
+      sP[pidx<D>(1, 2)] = c * sj[1];
+    } else {
+      sP[pidx<D>(1, 1)] = c * c * sum;
+      sP[pidx<D>(0, 1)] = c * sj[0];
+    }
+    auto total = [&](R x) {
+      const R y0 = __shfl_sync(0xffffffffu, x, l0), y1 = __shfl_sync(0xffffffffu, x, l0 + 1),
+              y2 = __shfl_sync(0xffffffffu, x, l0 + 2);
+      return y0 + y1 + y2;
+    };
+    sum = total(sum);
+#pragma unroll
+    for (int d = 0; d < D; ++d) sj[d] = total(sj[d]);
+#pragma unroll
+    for (int q = 0; q < W::NP; ++q) sP[q] = total(sP[q]);
+  }
+  __syncwarp();                        // the previous sums' readers are done
+  if (on && p == 0) {
+    z[W::Z + l * W::ZS] = sum;
+#pragma unroll
+    for (int d = 0; d < D; ++d) z[W::Z + l * W::ZS + 1 + d] = sj[d];
+    if (l == M - 1)
+#pragma unroll
+      for (int q = 0; q < W::NP; ++q) z[W::P + q] = sP[q];
+  }
+  __syncwarp();
+}
+
+// The macroscopic state of the sums in z (bstate_of).
+template <int D, int M, typename R>
+__device__ __forceinline__ void wstate_of(WState<D, M, R>& s, const R* z, double T_guess,
+                                          const DevMech& m, const Units& un, int* status,
+                                          int lane) {
+  using W = WB<D, M>;
+  using CT = typename ChemType<R>::type;
+  using X = Chem<CT>;
+  const int sp = lane & 15, a = min(sp, M - 1);
+  const R* zf = z + W::Z + (M - 1) * W::ZS;
+  s.rho = zf[0];
+  const R irho = R(1) / s.rho;
+  R usq = R(0);
+#pragma unroll
+  for (int d = 0; d < D; ++d) { s.u[d] = zf[1 + d] * irho; usq += s.u[d] * s.u[d]; }
+  // rho_a, j_a: the slaved species from the mixture
+  R q[W::ZS];
+#pragma unroll
+  for (int e = 0; e < W::ZS; ++e) {
+    const R mine = sp < M - 1 ? z[W::Z + a * W::ZS + e] : R(0);
+    R rest = zf[e];
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+      for (int b = 0; b < M - 1; ++b) rest -= z[W::Z + b * W::ZS + e];
+    } else {
+      rest -= species_sum(mine);
+    }
+    q[e] = sp < M - 1 ? mine : rest;
+  }
+  const R Ya = sp < M ? q[0] * irho : R(0);
+  if (lane < M) {
+    s.Y[a] = Ya;
+    if (s.own_us) {
+      R ja[D];
+#pragma unroll
+      for (int d = 0; d < D; ++d) ja[d] = q[1 + d];
+      const bool tiny = species_velocity_undefined<D, R>(q[0], ja);
+#pragma unroll
+      for (int d = 0; d < D; ++d) s.us[a * D + d] = tiny ? s.u[d] : ja[d] / q[0];
+    }
+  }
+  __syncwarp();
+  CT c[4], U;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c[k] = species_sum(X::of(Ya) * X::ucoef(m, k, a));
+  const R rhoE = z[W::Z + M * W::ZS];
+  if constexpr (!kFF<R>) U = (double(rhoE * irho) - 0.5 * double(usq)) * un.c * un.c;
+  else U = (ff(rhoE * irho) + ff(-0.5f * usq)) * un.c2_f;
+  bool ok;
+  const CT T = newton_poly(c, U, X::of_T(T_guess), un.newton_max_iter, X::rtol(un), ok);
+  if constexpr (!kFF<R>) {
+    s.T = R(T);
+    s.T_full = T;
+  } else {
+    s.T = T.hi;
+    s.T_full = ff_to_double(T);
+  }
+  if (!ok && lane == 0) atomicOr(status, ST_NEWTON);
+  wprepare<D, M, R>(s, m, un, lane);
+}
+
+// Equilibrium populations of a state in this lane's lattice and directions.
+template <int D, int M, typename R>
+__device__ __forceinline__ void wequilibrium(const WState<D, M, R>& s, const DevMech& m,
+                                             const Units& un, int lane, R (&e)[WB<D, M>::NR]) {
+  using W = WB<D, M>;
+  const int l = min(lane / 3, M), p = lane % 3;
+  if (l < M) {
+    R th = s.th, pref = s.rho;
+    if (l < M - 1) {
+      if constexpr (sizeof(R) == 8) th = R(m.Ra[l] * double(s.T) * un.inv_c2);
+      else th = m.Ra_s[l] * s.T * un.inv_c2_s;
+      pref = s.rho * s.Y[l];
+    }
+    R t[D][3];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const R xi = l < M - 1 && s.own_us ? s.us[l * D + d] : s.u[d];
+      const R P = th + xi * xi;
+      t[d][0] = R(0.5) * (P - xi);
+      t[d][1] = R(1) - P;
+      t[d][2] = R(0.5) * (P + xi);
+    }
+    const R tp = sel3(p - 1, t[D - 1]);
+#pragma unroll
+    for (int r = 0; r < W::NR / 3; ++r) {
+      const R w = D == 3 ? pref * t[1][r] * tp : pref * tp;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) e[3 * r + k] = mul1(w, t[0][k]);
+    }
+  } else {
+    BState<D, M, R> b;
+    b.rho = s.rho;
+    b.th = s.th;
+    b.U = s.U;
+#pragma unroll
+    for (int d = 0; d < D; ++d) b.u[d] = s.u[d];
+    GTab<D, R> g;
+    gtab<D, M, R>(b, g);
+    const R az = sel3(p - 1, g.A[D - 1]), bz = sel3(p - 1, g.B[D - 1]);
+#pragma unroll
+    for (int r = 0; r < W::NR / 3; ++r) {
+      const R P = D == 3 ? mul1(g.A[1][r], az) : az;
+      const R Qv = D == 3 ? fma(g.U, P, fma(g.B[1][r], az, mul1(g.A[1][r], bz)))
+                          : fma(g.U, az, bz);
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        e[3 * r + k] = mul1(g.rho, fma(g.A[0][k], Qv, mul1(g.B[0][k], P)));
+    }
+  }
+}
+
+// Interface node k by one warp; sm: the warp's WB::N entries; m: the
+// mechanism's global copy (indexed by lane); Cs: this thread's slice for the
+// sub-steps.
+template <int D, int M, typename S, typename R>
+__device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDev& bc,
+                                           R* __restrict__ rec, double* __restrict__ Tf,
+                                           int* __restrict__ status, const Geom& g,
+                                           const Units& un, const DevMech& m, int k, R* sm,
+                                           int lane, ff* const Cs) {
+  using W = WB<D, M>;
+  using RC = Rec<D, M>;
+  constexpr int Q = W::Q;
+  const long long N = g.N;
+  const long long n = bc.if_node[k];
+  const int info = bc.if_info[k], kind = info & 15;
+  const unsigned inc = bc.if_inc[k];
+  const bool on = lane < 3 * (M + 1);
+  const int l = min(lane / 3, M), p = lane % 3;
+  const int i0 = p * W::NR;                        // the lane's directions i0 .. i0 + NR - 1
+  const int x = (int)(n % g.nx);
+  const int y = (int)((n / g.nx) % g.ny);
+  const int z = (int)(n / ((long long)g.nx * g.ny));
+  auto at = [&](long long node, int i) {
+    return Codec<S>::template dec<R>(__ldg(src + (long long)(l * Q + i) * N + node), g.codec,
+                                     l * Q + i);
+  };
+  auto stored = [&](long long node, R (&v)[W::NR]) {
+#pragma unroll
+    for (int j = 0; j < W::NR; ++j) v[j] = at(node, i0 + j);
+  };
+  R pull[W::NR], v[W::NR];
+#pragma unroll
+  for (int j = 0; j < W::NR; ++j) pull[j] = at(node_shift<D>(x, y, z, i0 + j, -1, g), i0 + j);
+  const double Tg = __ldcg(Tf + n);
+  auto incoming = [&](int j) { return (inc >> (i0 + j) & 1u) != 0; };
+  WState<D, M, R> A, B, L;
+  A.Y = sm + W::ST;
+  B.Y = A.Y + W::SS;
+  L.Y = B.Y + W::SS;
+  R* const Fs = L.Y + W::SS;
+  A.us = A.Y + M;
+  B.us = B.Y + M;
+  L.us = L.Y + M;
+  A.own_us = B.own_us = L.own_us = false;
+
+  if (kind == BK_BB) {
+#pragma unroll
+    for (int j = 0; j < W::NR; ++j) v[j] = incoming(j) ? at(n, Q - 1 - i0 - j) : pull[j];
+  } else {
+    if (kind == BK_TMS) {
+#pragma unroll
+      for (int j = 0; j < W::NR; ++j) v[j] = incoming(j) ? at(n, Q - 1 - i0 - j) : pull[j];
+      wsums<D, M, R>(v, sm, lane);
+      A.rho = sm[W::Z + (M - 1) * W::ZS];
+      const R irho = R(1) / A.rho;
+      const int sp = lane & 15;
+      const R Ya = sp < M - 1 ? sm[W::Z + min(sp, M - 1) * W::ZS] * irho : R(0);
+      R last = R(1);
+      if constexpr (sizeof(R) == 4) {
+        R ysum = R(0);
+#pragma unroll
+        for (int b = 0; b < M - 1; ++b) ysum += mul1(sm[W::Z + b * W::ZS], irho);
+        last -= ysum;
+      } else {
+        last -= species_sum(Ya);
+      }
+      if (lane < M) A.Y[lane] = lane < M - 1 ? Ya : last;
+#pragma unroll
+      for (int d = 0; d < D; ++d) A.u[d] = R(0);
+      A.T = R(bc.if_wallT[k]);
+      __syncwarp();
+      if (bc.if_nbr && bc.if_nbr[k] >= 0) {
+        B.own_us = true;
+        stored(bc.if_nbr[k], v);
+        wsums<D, M, R>(v, sm, lane);
+        wstate_of<D, M, R>(B, sm, Tg, m, un, status, lane);
+        const double h = bc.if_wh[k], dl = bc.if_wd[k];
+        const R w = R(dl / (h + dl));
+#pragma unroll
+        for (int d = 0; d < D; ++d) A.u[d] = w * B.u[d];
+        A.own_us = true;
+        for (int e = lane; e < M * D; e += 32) A.us[e] = w * B.us[e];
+        A.T = R((h * bc.if_wallT[k] + dl * B.T_full) / (h + dl));
+        B.own_us = false;
+        __syncwarp();
+      }
+    } else if (kind == BK_INLET) {
+      A.rho = R(bc.rho_in);
+      if (lane < M) A.Y[lane] = R(bc.Y_in[lane]);
+#pragma unroll
+      for (int d = 0; d < D; ++d) A.u[d] = R(bc.if_uin[(long long)d * bc.n_if + k]);
+      A.T = R(bc.T_in);
+      __syncwarp();
+    } else {
+      const int ax = (info >> 4) & 3;
+      const int sg = (info >> 6) & 1 ? 1 : -1;
+      const long long stride =
+          ax == 0 ? 1 : (ax == 1 ? (long long)g.nx : (long long)g.nx * g.ny);
+      R v1[W::NR];
+      stored(n, v);
+      stored(n - sg * stride, v1);
+      wsums<D, M, R>(v, sm, lane);
+      wstate_of<D, M, R>(L, sm, Tg, m, un, status, lane);
+      wsums<D, M, R>(v1, sm, lane);
+      wstate_of<D, M, R>(B, sm, Tg, m, un, status, lane);
+      auto pick3 = [&](const R (&u)[D]) {
+        R w = u[0];
+#pragma unroll
+        for (int d = 1; d < D; ++d)
+          if (ax == d) w = u[d];
+        return double(w);
+      };
+      const int sp = lane & 15, a = min(sp, M - 1);
+      const double T0 = L.T, T1 = B.T;
+      const double Y0 = sp < M ? double(L.Y[a]) : 0.0, Y1 = sp < M ? double(B.Y[a]) : 0.0;
+      const double R0 = R_U * species_sum(Y0 * m.inv_mm[a]);
+      const double R1 = R_U * species_sum(Y1 * m.inv_mm[a]);
+      const double Cv =
+          species_sum(Y0 * (m.u1[a] + T0 * (2.0 * m.u2[a] + 3.0 * T0 * m.u3[a])));
+      const double r0 = L.rho, r1 = B.rho;
+      const double p0 = r0 * R0 * T0 * un.inv_c2;
+      const double p1 = r1 * R1 * T1 * un.inv_c2;
+      const double un0 = sg * pick3(L.u), un1 = sg * pick3(B.u);
+      const double gamma = (Cv + R0) / Cv;
+      const double cs = sqrt(gamma * R0 * T0 * un.inv_c2);
+      const double Ma = un0 / cs;
+      const double Ln =
+          bc.outlet_L > 0.0 ? bc.outlet_L : (ax == 0 ? g.nx : (ax == 1 ? g.ny : g.nz));
+      const double K = bc.sigma * (1.0 - Ma * Ma) * cs / Ln;
+      const double L1 = K * (p0 - bc.p_out_lat);
+      const double L2 = un0 * (cs * cs * (r0 - r1) - (p0 - p1));
+      const double L5 = (un0 + cs) * ((p0 - p1) + r0 * cs * (un0 - un1));
+      const double rho_o = r0 - (L2 + 0.5 * (L5 + L1)) / (cs * cs);
+      const double p_o = p0 - 0.5 * (L5 + L1);
+      const double un_o = un0 - (L5 - L1) / (2.0 * r0 * cs);
+      A.rho = R(rho_o);
+#pragma unroll
+      for (int d = 0; d < D; ++d)
+        A.u[d] = d == ax ? R(sg * un_o) : R(double(L.u[d]) - un0 * double(L.u[d] - B.u[d]));
+      const double Ya = Y0 - un0 * (Y0 - Y1);
+      const double Ro = species_sum(Ya * m.inv_mm[a]);
+      if (lane < M) A.Y[lane] = R(Ya);
+      A.T = R(p_o * un.c * un.c / (rho_o * R_U * Ro));
+      __syncwarp();
+    }
+    wprepare<D, M, R>(A, m, un, lane);
+    // the local state: incoming links at A, the others pulled
+    R ea[W::NR], el[W::NR];
+    wequilibrium<D, M, R>(A, m, un, lane, ea);
+#pragma unroll
+    for (int j = 0; j < W::NR; ++j) v[j] = incoming(j) ? ea[j] : pull[j];
+    wsums<D, M, R>(v, sm, lane);
+    L.own_us = kind == BK_TMS;
+    wstate_of<D, M, R>(L, sm, Tg, m, un, status, lane);
+    wequilibrium<D, M, R>(L, m, un, lane, el);
+    if (kind == BK_INLET && bc.inlet_simplified != 0) {
+#pragma unroll
+      for (int j = 0; j < W::NR; ++j) v[j] = el[j];
+    } else if (kind == BK_INLET) {
+      R eb[W::NR];
+      B.rho = L.rho;
+      B.Y = L.Y;
+#pragma unroll
+      for (int d = 0; d < D; ++d) B.u[d] = A.u[d];
+      B.T = R(bc.T_in);
+      wprepare<D, M, R>(B, m, un, lane);
+      wequilibrium<D, M, R>(B, m, un, lane, eb);
+#pragma unroll
+      for (int j = 0; j < W::NR; ++j) v[j] = eb[j] + (incoming(j) ? ea[j] : pull[j]) - el[j];
+    } else {
+#pragma unroll
+      for (int j = 0; j < W::NR; ++j) v[j] = ea[j] + (incoming(j) ? ea[j] : pull[j]) - el[j];
+    }
+  }
+  if (on)
+#pragma unroll
+    for (int j = 0; j < W::NR; ++j)
+      bc.pops[(long long)(l * Q + i0 + j) * bc.n_if + k] = double(v[j]);
+
+  // the record
+  wsums<D, M, R>(v, sm, lane);
+  WState<D, M, R> s;
+  s.Y = Fs;
+  s.us = Fs + M;
+  s.own_us = true;
+  wstate_of<D, M, R>(s, sm, Tg, m, un, status, lane);
+  const R rr = s.rho;
+  if (lane == 0) {
+    if (!(rr > R(0)) || !isfinite(double(rr)) || !isfinite(s.T_full))
+      atomicOr(status, ST_NONFINITE);
+    Tf[n] = s.T_full;
+    rec[RC::RHO * N + n] = rr;
+    rec[RC::E * N + n] = sm[W::Z + M * W::ZS] * (R(1) / rr);
+  }
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    if (lane == 1 + d) {
+      rec[(RC::U + d) * N + n] = s.u[d];
+      rec[(RC::QF + d) * N + n] = sm[W::Z + M * W::ZS + 1 + d];
+      rec[(RC::PHI + d) * N + n] =
+          rr * s.u[d] * (R(1) - R(3) * s.th) - rr * s.u[d] * s.u[d] * s.u[d];
+    }
+  }
+  for (int e = lane; e < W::NP; e += 32) rec[(RC::P + e) * N + n] = sm[W::P + e];
+  for (int a = lane; a < M; a += 32) rec[(RC::Y + a) * N + n] = s.Y[a];
+#pragma unroll
+  for (int d = 0; d < D; ++d)
+    for (int a = lane; a < M; a += 32)
+      rec[(RC::US + a * D + d) * N + n] = s.us[a * D + d] - s.u[d];
+
+  // the reaction sub-steps, the reactions over the warp's lanes
+  using CT = typename ChemType<R>::type;
+  using X = Chem<CT>;
+  CT r[M], r0[M - 1], U;
+  R last = rr, usq = R(0);
+#pragma unroll
+  for (int a = 0; a < M - 1; ++a) {
+    const R ra = s.Y[a] * rr;
+    last -= ra;
+    r0[a] = r[a] = X::of(ra);
+  }
+  r[M - 1] = X::of(last);
+#pragma unroll
+  for (int d = 0; d < D; ++d) usq += s.u[d] * s.u[d];
+  const R ER = sm[W::Z + M * W::ZS] * (R(1) / rr);
+  if constexpr (kFF<R>) U = (ff(ER) + ff(-0.5f * usq)) * un.c2_f;
+  else U = (double(ER) - 0.5 * double(usq)) * un.c * un.c;
+  chem_group_substeps<M, CT, 32>(r, X::inv(X::of(rr)), U, X::of_T(s.T_full), un, m, lane,
+                                 0xffffffffu, status, Cs);
+#pragma unroll
+  for (int a = 0; a < M - 1; ++a) {
+    if (a != lane) continue;
+    if constexpr (kFF<R>) rec[(RC::DRHO + a) * N + n] = (r[a] - r0[a]).hi;
+    else rec[(RC::DRHO + a) * N + n] = R(r[a] - r0[a]);
   }
 }

@@ -56,33 +56,22 @@ lbm_status cuda_fail(lbm_ctx* h, cudaError_t e, const char* where) {
   return fail(h, LBM_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
-// Default placement.  The split collision measured faster than the fused
-// one on every grid tried (FP32 and FP64, 16k to 524k nodes).  Below
-// kSmallGrid nodes a thread-per-node grid holds fewer than four 128-thread
-// blocks per SM of a 152-SM GB300, too few warps to hide the latency of the
-// float-float chemistry, which then runs with four lanes per node; in FP64
-// the extra redundant work of the lanes costs more than it hides.
+// Default placement, measured on one GB300.  The split collision is faster
+// than the fused one on every grid tried (FP64 and FP32).  Below kSmallGrid
+// nodes a thread-per-node grid of the FP32 path holds fewer than four
+// 128-thread blocks per SM of a 152-SM GB300, too few warps to hide the latency
+// of the float-float chemistry, which then runs with four lanes per node; in
+// FP64 the extra redundant work of the lanes costs more than it hides.  Batch
+// plans take one launch per kernel (six reactors and flames of 69k nodes in
+// all, FP64: 0.84 ms per step against 1.05 as a single launch over the
+// work-list, whose registers the kernels' largest stage sets).
 constexpr long long kSmallGrid = 152LL * 4 * 128;
-
-// Defaults, measured on one GB300.  plan: a batch plan's placement, whose
-// default for FP64 storage below kPlanSingleLaunch nodes in total is the
-// single launch over the work-list with split collision (14 % faster than
-// one launch per kernel on a mix of eight domains of 92k nodes in all; on
-// batches of about a million nodes one launch per kernel is 2-6 % faster);
-// FP32 and FP16 plans keep one launch per kernel, whose kernels hold fewer
-// registers than the single launch.  FP64, a grid that fills the GPU at one
-// thread per node: the fused collision (3 % faster on the 600x40x40 tube);
-// else the split one.
-constexpr long long kPlanSingleLaunch = 4 * kSmallGrid;
-Launch resolve_launch(const lbm_launch& opt, long long nodes, lbm_precision prec,
-                      bool plan = false) {
+Launch resolve_launch(const lbm_launch& opt, long long nodes, lbm_precision prec) {
   Launch lc;
   const bool small = nodes < kSmallGrid;
   lc.chem_lanes = opt.chem_lanes > 0 ? opt.chem_lanes
                                      : (small && prec == LBM_FP32_STORE ? 4 : 1);
-  lc.persistent = opt.persistent >= 0
-                      ? opt.persistent
-                      : (plan && prec == LBM_FP64 && nodes < kPlanSingleLaunch ? 2 : 0);
+  lc.persistent = opt.persistent >= 0 ? opt.persistent : 0;
   lc.coll_split = opt.collide_split >= 0 ? opt.collide_split : 1;
   lc.npt = opt.nodes_per_thread > 0 ? opt.nodes_per_thread : 1;
   return lc;
@@ -99,6 +88,9 @@ void fill_domains(lbm_ctx* const* hs, int n, const Launch& lc, std::vector<Domai
                   BatchGrids& gr) {
   doms.assign(n, DomainDev());
   gr = BatchGrids();
+  for (int k = 0; k < n; ++k) gr.n_if_total += hs[k]->bc.n_if;
+  gr.bnd_warp = n > 0 && gr.n_if_total <= bnode_warp_limit(hs[0]->cfg.precision);
+  const int per_bnd = gr.bnd_warp ? kBnodeWarps : kBndNodesPerBlock;
   for (int k = 0; k < n; ++k) {
     lbm_ctx* h = hs[k];
     DomainDev& d = doms[k];
@@ -120,8 +112,7 @@ void fill_domains(lbm_ctx* const* hs, int n, const Launch& lc, std::vector<Domai
     d.kblock_begin = gr.nkblocks;
     gr.nblocks += (int)((h->g.N + 127) / 128);
     gr.nbblocks += (h->bc.n_if + kIfChemNodesPerBlock - 1) / kIfChemNodesPerBlock;
-    gr.ntblocks += (h->bc.n_if + kBndNodesPerBlock - 1) / kBndNodesPerBlock;
-    gr.n_if_total += h->bc.n_if;
+    gr.ntblocks += (h->bc.n_if + per_bnd - 1) / per_bnd;
     if (lc.chem_lanes > 1) {
       const int per = 128 / lc.chem_lanes;
       gr.ncblocks += (int)((h->g.N + per - 1) / per);
@@ -1138,10 +1129,9 @@ lbm_status lbm_batch_step(lbm_t* hs, int n, int nsteps) {
   DeviceGuard dg(h0->cfg.device);
   std::vector<DomainDev> doms;
   BatchGrids gr;
-  // the placement a new plan of these handles starts with (for FP64 under
-  // kPlanSingleLaunch nodes: the whole step as one launch over a work-list)
+  // the placement a new plan of these handles starts with
   const Launch lc = resolve_launch(lbm_launch{-1, -1, -1, -1}, total_nodes(hs, n),
-                                   hs[0]->cfg.precision, true);
+                                   hs[0]->cfg.precision);
   fill_domains(hs, n, lc, doms, gr);
   // every handle's earlier work precedes the batch; the batch runs on the
   // first handle's stream and each handle's stream waits for it afterwards
@@ -1326,8 +1316,7 @@ lbm_status lbm_batch_create(lbm_t* hs, int n, lbm_batch_t* out) {
     b->ddev = static_cast<DomainDev*>(dalloc(h0->cfg, n * sizeof(DomainDev)));
     if (!b->ddev) e = cudaErrorMemoryAllocation;
   }
-  b->lc = resolve_launch(lbm_launch{-1, -1, -1, -1}, total_nodes(hs, n), hs[0]->cfg.precision,
-                         true);
+  b->lc = resolve_launch(lbm_launch{-1, -1, -1, -1}, total_nodes(hs, n), hs[0]->cfg.precision);
   if (e == cudaSuccess) e = batch_upload(b);
   if (e == cudaSuccess) e = prepare_batch_step(h0->D, h0->M, kernel_precision(h0->cfg));
   if (e == cudaSuccess) e = batch_capture_all(b);
@@ -1388,8 +1377,7 @@ lbm_status lbm_batch_set_launch(lbm_batch_t b, const lbm_launch* l) {
     return fail(h0, LBM_ERR_INVALID, "placement out of range");
   DeviceGuard dg(h0->cfg.device);
   cudaError_t e = cudaStreamSynchronize(b->stream);
-  b->lc = resolve_launch(*l, total_nodes(b->hs.data(), (int)b->hs.size()), h0->cfg.precision,
-                         true);
+  b->lc = resolve_launch(*l, total_nodes(b->hs.data(), (int)b->hs.size()), h0->cfg.precision);
   if (e == cudaSuccess) e = batch_upload(b);
   if (e == cudaSuccess) e = batch_capture_all(b);
   return e == cudaSuccess ? LBM_OK : cuda_fail(h0, e, "batch placement");

@@ -219,6 +219,7 @@ struct BatchGrids {
   int ncblocks = 0;   // k_chem, 128 / chem_lanes nodes per block (0 without it)
   int nkblocks = 0;   // k_coll, 32 nodes per block (0 without it)
   long long n_if_total = 0;   // interface nodes of every domain
+  int bnd_warp = 0;           // the boundary grid holds kBnodeWarps nodes per block
   // persistent == 2: the device work-list and its sync words (zeroed before
   // every launch), the domains' interface-node presence
   const PItem* items = nullptr;
@@ -229,6 +230,15 @@ struct BatchGrids {
   long long timeout_ns = kPersistTimeoutNs;
 };
 
+// Grids (of a plan: handles together) with up to this many interface nodes take
+// the boundary kernel with a warp per node, which does more work in all but
+// not in one chain: with the 4078 nodes of the 2000x40 channel a step takes
+// 0.69 ms against 0.75 in FP64, 0.36 against 0.33 in FP32 with FP64 chemistry
+// (there the chain hides behind the bulk nodes); with the flame's 32 nodes
+// 0.29 against 0.60 (FP64) and 0.15 against 0.34 (FP32).
+inline int bnode_warp_limit(lbm_precision p) { return p == LBM_FP64 ? 6144 : 1536; }
+// nodes (warps) per block of it
+constexpr int kBnodeWarps = 2;
 // interface nodes per block of the boundary kernel (one thread each)
 constexpr int kBndNodesPerBlock = 64;
 // interface nodes per block of the batched interface chemistry (8 lanes each)

@@ -455,7 +455,6 @@ template <> struct Chem<double> {
   __device__ static double ucoef(const DevMech& m, int k, int a) {
     return k == 0 ? m.u0[a] : (k == 1 ? m.u1[a] : (k == 2 ? m.u2[a] : m.u3[a]));
   }
-  __device__ static double mag(double x) { return fabs(x); }
   __device__ static double rtol(const Units& u) { return u.newton_rtol; }
 };
 template <> struct Chem<ff> {
@@ -469,7 +468,6 @@ template <> struct Chem<ff> {
   __device__ static ff ucoef(const DevMech& m, int k, int a) {
     return k == 0 ? m.u0_f[a] : (k == 1 ? m.u1_f[a] : (k == 2 ? m.u2_f[a] : m.u3_f[a]));
   }
-  __device__ static float mag(ff x) { return fabsf(x.hi); }
   __device__ static float rtol(const Units& u) { return u.newton_rtol_f; }
 };
 
@@ -511,31 +509,19 @@ __device__ __forceinline__ CT group_newton(const DevMech& m, const CT (&r)[M], C
   for (int o = 1; o < L; o <<= 1)
 #pragma unroll
     for (int k = 0; k < 4; ++k) c[k] += shfl_xor_ct(gmask, c[k], o);
-  const CT two = X::of(2.f), three = X::of(3.f);
-  ok = false;
-  for (int it = 0; it < un.newton_max_iter; ++it) {
-    const CT F = c[0] + T * (c[1] + T * (c[2] + T * c[3])) - U;
-    const CT dF = c[1] + T * (two * c[2] + three * T * c[3]);
-    const CT dT = -(F / dF);
-    T += dT;
-    if (X::mag(dT) <= X::rtol(un) * X::mag(T)) { ok = true; break; }
-  }
-  return T;
+  return newton_poly(c, U, T, un.newton_max_iter, X::rtol(un), ok);
 }
 
 // The reaction sub-steps of one node by its lane group (Sec. 2.4 Eq. R3),
 // from the post-stream species densities r (replaced by the densities after
 // the sub-steps), 1/rho, the internal energy U and the temperature T_0 of
-// the moments.
+// the moments.  Cs: this thread's slice for concentrations and rates.
 template <int M, typename CT, int L>
 __device__ __forceinline__ void chem_group_substeps(CT (&r)[M], const CT irho, const CT U,
                                                     CT Ts, const Units& un, const DevMech& m,
                                                     int sub, unsigned gmask,
-                                                    int* __restrict__ status) {
+                                                    int* __restrict__ status, ff* const Cs) {
   using X = Chem<CT>;
-  // concentrations and rates: a per-thread slice of shared memory
-  // (128-thread blocks)
-  ff* const Cs = chem_static_slice<M>() + threadIdx.x;
   ff* const Ws = Cs + M * kChemThreads;
   for (int s = 0; s < un.substeps; ++s) {
     if (s > 0) {
@@ -601,7 +587,7 @@ __device__ __forceinline__ void chem_lanes_body(RT* __restrict__ rec,
   }
   r[M - 1] = X::of(last);
   chem_group_substeps<M, CT, L>(r, X::inv(X::of(rho)), U, X::of_T(Tf[n]), un, m, sub, gmask,
-                                status);
+                                status, chem_static_slice<M>() + threadIdx.x);
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
     if (a % L != sub) continue;
@@ -761,7 +747,8 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
   CT r0[M - 1];
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) r0[a] = r[a];
-  chem_group_substeps<M, CT, L>(r, irho, U, X::of_T(T), un, mg, sub, gmask, status);
+  chem_group_substeps<M, CT, L>(r, irho, U, X::of_T(T), un, mg, sub, gmask, status,
+                                chem_static_slice<M>() + threadIdx.x);
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
     if constexpr (kFF<RT>) put(RC::DRHO + a, (r[a] - r0[a]).hi);
@@ -1850,6 +1837,22 @@ k_bnode(const S* __restrict__ src, const __grid_constant__ BCDev bc, double* __r
                              threadIdx.x);
 }
 
+// The interface nodes with a warp each: reconstruction, record and reaction
+// sub-steps (lbm_bnode.cuh).
+template <int D, int M, typename S>
+__global__ void __launch_bounds__(32 * kBnodeWarps)
+k_bnode_warp(const S* __restrict__ src, const __grid_constant__ BCDev bc,
+             double* __restrict__ Tf, int* __restrict__ status, const __grid_constant__ Geom g,
+             const __grid_constant__ Units un, const DevMech* __restrict__ mech,
+             typename ComputeType<S>::type* __restrict__ rec) {
+  using R = typename ComputeType<S>::type;
+  __shared__ R ws[kBnodeWarps][WB<D, M>::N];
+  const int w = threadIdx.x >> 5, k = blockIdx.x * kBnodeWarps + w;
+  if (k >= bc.n_if) return;
+  bnode_warp<D, M, S, R>(src, bc, rec, Tf, status, g, un, *mech, k, ws[w], threadIdx.x & 31,
+                         chem_static_slice<M>() + threadIdx.x);
+}
+
 // ---------------------------------------------------------------------------
 // Batched kernels: the grid is the concatenation of every domain's tiles; a
 // block finds its domain by binary search over the domains' first blocks.
@@ -2022,6 +2025,23 @@ k_bnode_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nblk
   }
 }
 
+template <int D, int M, typename S>
+__global__ void __launch_bounds__(32 * kBnodeWarps)
+k_bnode_warp_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nblk) {
+  LBM_BLOCK_DOMAIN(bd);
+  using R = typename ComputeType<S>::type;
+  __shared__ R ws[kBnodeWarps][WB<D, M>::N];
+  const int w = threadIdx.x >> 5;
+  for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
+    const DomainDev& d = bd.get(doms, domain_of_block(doms, ndom, b, GRID_BNODE));
+    const int k = (b - d.tblock_begin) * kBnodeWarps + w;
+    if (k >= d.bc.n_if) continue;
+    bnode_warp<D, M, S, R>(static_cast<const S*>(d.pops[d.cur0 ^ parity]), d.bc,
+                           static_cast<R*>(d.rec), d.Tf, d.status, d.g, d.un, *d.mech, k, ws[w],
+                           threadIdx.x & 31, chem_static_slice<M>() + threadIdx.x);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // The whole batched step as one persistent launch over a work-list (PItem,
 // lbm_internal.h).  Dependencies go through sync words: a producer block
@@ -2099,6 +2119,10 @@ k_iface_chem_batch(const DomainDev* __restrict__ doms, int ndom, int nblk) {
 }
 
 template <typename RT> constexpr int kPersistMinBlocks = sizeof(RT) == 8 ? 2 : 3;
+// a boundary item of up to this many interface nodes gives each a warp (the
+// thread-per-node procedure of a 128-node item takes as long as ~15 nodes of a
+// warp each)
+constexpr int kPersistWarpNodes = 32;
 constexpr int kPersistCollWarps = kPersistThreads / 32;
 
 template <int D, int M, typename S, typename RT>
@@ -2136,7 +2160,15 @@ k_step_persist(const DomainDev* __restrict__ doms, int ndom, int parity,
     const int c = d.cur0 ^ parity;
     const S* src = static_cast<const S*>(d.pops[c]);
     RT* rec = static_cast<RT*>(d.rec);
-    if (w.kind == PI_BND) {
+    if (w.kind == PI_BND && d.bc.n_if - w.first <= kPersistWarpNodes) {
+      // few interface nodes: the block's warps take them in turn
+      const int wp = threadIdx.x >> 5;
+      R* ws = reinterpret_cast<R*>(ps_raw + chem_slice_bytes<M>()) + wp * WB<D, M>::N;
+      for (int k = (int)w.first + wp; k < d.bc.n_if; k += kPersistThreads / 32)
+        bnode_warp<D, M, S, R>(src, d.bc, static_cast<R*>(d.rec), d.Tf, d.status, d.g, d.un,
+                               *d.mech, k, ws, threadIdx.x & 31,
+                               reinterpret_cast<ff*>(ps_raw) + threadIdx.x);
+    } else if (w.kind == PI_BND) {
       // two groups of kBnd threads, each with its boundary columns
       const int grp = threadIdx.x / kBnd, t = threadIdx.x % kBnd;
       constexpr int E = bnode_col_entries<D, M>();
@@ -2193,7 +2225,8 @@ template <int D, int M, typename S, typename RT> constexpr size_t persist_smem(b
   const size_t prep = (size_t)solve_smem_entries<D, M, RT>() * kBS * sizeof(RT);
   const size_t coll = (size_t)coll_smem_entries<D, M, RT>() * kCollNodes * sizeof(RT);
   const size_t fused = (size_t)collide_smem_entries<D, M, RT>() * kBS * sizeof(RT);
-  const size_t chem = chem_slice_bytes<M>();
+  const size_t chem =
+      chem_slice_bytes<M>() + sizeof(R) * WB<D, M>::N * (kPersistThreads / 32);
   size_t m = bnd > chem ? bnd : chem;
   if (split) {
     m = m > prep ? m : prep;
@@ -2490,36 +2523,39 @@ static cudaError_t step_impl(const DevMech& mech, const StepArgs& a, cudaStream_
     // allocation-free step accepts no interface nodes).
     if (a.bc.n_if > 0 && !a.mech_dev) return cudaErrorInvalidValue;
     const bool fork = a.bc.n_if > 0 && a.side && a.ev_fork && a.ev_join;
+    // the boundary kernel and the interface nodes' sub-steps
+    auto boundary = [&](cudaStream_t st) {
+      if (a.bc.n_if <= bnode_warp_limit(sizeof(RT) == 8 ? LBM_FP64 : LBM_FP32_STORE)) {
+        k_bnode_warp<D, M, S><<<blocks_for(a.bc.n_if, kBnodeWarps), 32 * kBnodeWarps, 0, st>>>(
+            src, a.bc, a.Tfield, a.status, a.g, a.un, a.mech_dev, rec);
+        return;
+      }
+      k_bnode<D, M, S><<<blocks_for(a.bc.n_if, kBnd), kBnd, bnode_smem<D, M, RT>(), st>>>(
+          src, a.bc, a.Tfield, a.status, a.g, a.un, mech, rec);
+      launch_chem<D, M, RT>(lc, st, rec, a.Tfield, a.status, a.g.N, a.bc, a.un, a.mech_dev,
+                            NODES_INTERFACE);
+    };
+    auto bulk = [&](int node_set) {
+      if (chem_sep)
+        mchem(s, node_set);
+      else
+        k_moments<D, M, S, RT><<<nb, bs, 0, s>>>(src, rec, a.Tfield, a.status, a.g, a.un, a.bc,
+                                                 mech, 1, node_set);
+    };
     if (fork) {
       cudaError_t e = cudaEventRecord(a.ev_fork, s);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(a.side, a.ev_fork, 0);
       if (e != cudaSuccess) return e;
-      k_bnode<D, M, S><<<blocks_for(a.bc.n_if, kBnd), kBnd, bnode_smem<D, M, RT>(), a.side>>>(
-          src, a.bc, a.Tfield, a.status, a.g, a.un, mech, rec);
-      launch_chem<D, M, RT>(lc, a.side, rec, a.Tfield, a.status, a.g.N, a.bc, a.un,
-                            a.mech_dev, NODES_INTERFACE);
+      boundary(a.side);
       e = cudaEventRecord(a.ev_join, a.side);
       if (e != cudaSuccess) return e;
-      if (chem_sep)
-        mchem(s, NODES_BULK);
-      else
-        k_moments<D, M, S, RT><<<nb, bs, 0, s>>>(src, rec, a.Tfield, a.status, a.g, a.un, a.bc,
-                                                 mech, 1, NODES_BULK);
+      bulk(NODES_BULK);
       e = cudaStreamWaitEvent(s, a.ev_join, 0);
       if (e != cudaSuccess) return e;
     } else {
       const bool bnd = a.bc.n_if > 0;
-      if (bnd)
-        k_bnode<D, M, S><<<blocks_for(a.bc.n_if, kBnd), kBnd, bnode_smem<D, M, RT>(), s>>>(
-            src, a.bc, a.Tfield, a.status, a.g, a.un, mech, rec);
-      if (chem_sep)
-        mchem(s, bnd ? NODES_BULK : NODES_ALL);
-      else
-        k_moments<D, M, S, RT><<<nb, bs, 0, s>>>(src, rec, a.Tfield, a.status, a.g, a.un, a.bc,
-                                                 mech, 1, bnd ? NODES_BULK : NODES_ALL);
-      if (bnd)
-        launch_chem<D, M, RT>(lc, s, rec, a.Tfield, a.status, a.g.N, a.bc, a.un, a.mech_dev,
-                              NODES_INTERFACE);
+      if (bnd) boundary(s);
+      bulk(bnd ? NODES_BULK : NODES_ALL);
     }
   }
   if (which != 0) {
@@ -2605,11 +2641,23 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
   const int chem_inline = lc.chem_lanes <= 1;
   const bool ps = lc.persistent != 0;
   auto kmom = k_moments_batch<D, M, S, RT>;
-  auto kbnd = k_bnode_batch<D, M, S>;
-  const size_t sbnd = bnode_smem<D, M, RT>();
+  // the boundary kernel: a warp or a thread per interface node
+  auto bnd = [&](cudaStream_t st) {
+    if (gr.bnd_warp) {
+      auto k = k_bnode_warp_batch<D, M, S>;
+      k<<<batch_grid(k, gr.ntblocks, 32 * kBnodeWarps, 0, ps), 32 * kBnodeWarps, 0, st>>>(
+          doms, ndom, parity, gr.ntblocks);
+    } else {
+      auto k = k_bnode_batch<D, M, S>;
+      const size_t sm = bnode_smem<D, M, RT>();
+      k<<<batch_grid(k, gr.ntblocks, kBnd, sm, ps), kBnd, sm, st>>>(doms, ndom, parity,
+                                                                    gr.ntblocks);
+    }
+  };
   // the reaction sub-steps in k_chem over a node set (the grid of the set)
   static_assert(128 / 8 == kIfChemNodesPerBlock, "interface chemistry: 8 lanes per node");
   auto chem = [&](int node_set, cudaStream_t st) {
+    if (gr.bnd_warp) return;          // done by the boundary kernel
     if (node_set == NODES_INTERFACE && gr.n_if_total >= kIfChemThreadNodes) {
       // enough interface nodes to fill the GPU with one thread each
       auto k = k_iface_chem_batch<D, M, RT>;
@@ -2651,8 +2699,7 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
     if (e != cudaSuccess) return e;
     // (the interface nodes: records by the boundary warps, sub-steps with
     // eight lanes per node, whatever the bulk placement)
-    kbnd<<<batch_grid(kbnd, gr.ntblocks, kBnd, sbnd, ps), kBnd, sbnd, side.stream>>>(
-        doms, ndom, parity, gr.ntblocks);
+    bnd(side.stream);
     chem(NODES_INTERFACE, side.stream);
     e = cudaEventRecord(side.join, side.stream);
     if (e != cudaSuccess) return e;
@@ -2666,8 +2713,7 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
   } else {
     const bool bnd_rec = gr.nbblocks > 0;
     if (gr.nbblocks > 0)
-      kbnd<<<batch_grid(kbnd, gr.ntblocks, kBnd, sbnd, ps), kBnd, sbnd, s>>>(doms, ndom, parity,
-                                                                          gr.ntblocks);
+      bnd(s);
     if (chem_inline)
       kmom<<<batch_grid(kmom, gr.nblocks, bs, 0, ps), bs, 0, s>>>(
           doms, ndom, parity, 1, bnd_rec ? NODES_BULK : NODES_ALL, gr.nblocks);
