@@ -240,6 +240,7 @@ __device__ __forceinline__ double double_join(ff a) {
   const float w = __int_as_float((int)((306u << 23) - (m & 0x7f800000u)));   // 2^(52 - exponent)
   int l = __float2int_rn(__fmul_rn(a.lo, w));
   if (b < 0) l = -l;
+  if (l < 0 && (m & 0x007fffff) == 0) l += l;   // below a power of two the last bit counts half
   const unsigned long long d =
       ((unsigned long long)((m >> 3) + (896 << 20)) << 32 | ((unsigned)b << 29)) + (long long)l;
   return __longlong_as_double((long long)(d | (unsigned long long)(b & 0x80000000u) << 32));

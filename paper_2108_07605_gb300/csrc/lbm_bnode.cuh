@@ -644,7 +644,7 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
     rec[(RC::Y + a) * N + n] = s.Y[a * kBnd];
 #pragma unroll
     for (int d = 0; d < D; ++d)
-      rec[(RC::US + a * D + d) * N + n] = s.us[(a * D + d) * kBnd] - s.u[d];
+      rec[(RC::US + a * D + d) * N + n] = record_us(s.us[(a * D + d) * kBnd] - s.u[d]);
   }
 }
 
@@ -1118,7 +1118,7 @@ __device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDe
 #pragma unroll
   for (int d = 0; d < D; ++d)
     for (int a = lane; a < M; a += 32)
-      rec[(RC::US + a * D + d) * N + n] = s.us[a * D + d] - s.u[d];
+      rec[(RC::US + a * D + d) * N + n] = record_us(s.us[a * D + d] - s.u[d]);
 
   // the reaction sub-steps, the reactions over the warp's lanes
   using CT = typename ChemType<R>::type;

@@ -89,7 +89,8 @@ void fill_domains(lbm_ctx* const* hs, int n, const Launch& lc, std::vector<Domai
   doms.assign(n, DomainDev());
   gr = BatchGrids();
   for (int k = 0; k < n; ++k) gr.n_if_total += hs[k]->bc.n_if;
-  gr.bnd_warp = n > 0 && gr.n_if_total <= bnode_warp_limit(hs[0]->cfg.precision);
+  gr.bnd_warp = n > 0 && gr.n_if_total <= bnode_warp_limit(
+                                        hs[0]->D, hs[0]->cfg.precision == LBM_FP64);
   const int per_bnd = gr.bnd_warp ? kBnodeWarps : kBndNodesPerBlock;
   for (int k = 0; k < n; ++k) {
     lbm_ctx* h = hs[k];
@@ -676,10 +677,11 @@ void fill_mixed_units(Units& un) {
   un.s_pref_s = (float)un.s_pref;
   un.nu_pref_s = (float)un.nu_pref;
 }
-void fill_enthalpies(const DevMech& m, Units& un) {
+void fill_species_units(const DevMech& m, Units& un) {
   for (int a = 0; a < m.M; ++a) {
     const double h[4] = {m.u0[a], m.u1[a] + m.Ra[a], m.u2[a], m.u3[a]};
     for (int k = 0; k < 4; ++k) un.hl_f[k][a] = ff_host(un.hl[k][a] = h[k] * un.inv_c2);
+    un.dtmm_f[a] = ff_host(un.dtmm[a] = un.dt_sub * m.mm[a]);
   }
 }
 // Host helpers shared with the allocation-free entry point (lbm_noalloc.cu).
@@ -808,7 +810,7 @@ lbm_status lbm_create(const lbm_config* cfg, lbm_t* out) {
   h->un.newton_rtol = cfg->newton_rtol;
   fill_mixed_units(h->un);
   build_mech(cfg->mech, h->mech);
-  fill_enthalpies(h->mech, h->un);
+  fill_species_units(h->mech, h->un);
   h->elem = elem_size(cfg->precision);
   h->stream = static_cast<cudaStream_t>(cfg->stream);
   const HostBC hb = classify(*cfg, c);

@@ -58,11 +58,84 @@ template <int D, int M> struct Rec {
   static constexpr int QF = P + Lat<D>::NP;
   static constexpr int E = QF + D;
   static constexpr int Y = E + 1;
-  static constexpr int US = Y + M;              // u_a - u
+  static constexpr int US = Y + M;              // u_a - u (record_us)
   static constexpr int PHI = US + M * D;
   static constexpr int DRHO = PHI + D;          // reaction increments, species a < M
   static constexpr int NF = DRHO + M - 1;
 };
+
+// u_a - u as the record holds it: in FP64 a float-float pair, the type of the
+// diffusion velocities it becomes
+__device__ __forceinline__ float record_us(float v) { return v; }
+__device__ __forceinline__ double record_us(double v) { return ff_pack(ff_of_double(v)); }
+
+// ------------------------------------------------------------------------
+// Sums of FP64 values in fixed point.  An FP64 addition occupies an SM quarter
+// of GB300 for 75 cycles, an integer one for 1: a group of values (one
+// lattice's populations at a node) is shifted to a common exponent, that of
+// the largest, and added in integers.  A value is cut at 2^-63 of the largest
+// one's power of two (a double's own last bit lies at 2^-52 of it), and the
+// sums of up to 32 terms are exact; with the small differences that a momentum
+// is made of, this is what FP64 differences keep, and more.
+//
+// Fix: the value modulo 2^64 in units of 2^(e - 63), and a, the same in units
+// of 2^(e - 25), each term rounded towards 0, which says which multiple of
+// 2^64 was lost.
+struct Fix {
+  unsigned long long lo;
+  int a;
+  __device__ Fix() : lo(0), a(0) {}
+  __device__ Fix(unsigned long long l, int a_) : lo(l), a(a_) {}
+};
+__device__ __forceinline__ Fix operator+(Fix x, Fix y) { return Fix(x.lo + y.lo, x.a + y.a); }
+__device__ __forceinline__ Fix operator-(Fix x, Fix y) { return Fix(x.lo - y.lo, x.a - y.a); }
+
+// biased exponent of v; the common one is the maximum over the group
+__device__ __forceinline__ int fix_exponent(double v) {
+  return (__double2hiint(v) >> 20) & 0x7ff;
+}
+__device__ __forceinline__ Fix fix_of(double v, int e) {
+  const int h = __double2hiint(v), l = __double2loint(v);
+  const int ev = (h >> 20) & 0x7ff;
+  const unsigned hm = (unsigned)((h & 0xfffff) | 0x100000);
+  unsigned long long m = ((unsigned long long)(hm << 11 | (unsigned)l >> 21) << 32) |
+                         (unsigned)(l << 11);
+  m >>= min(e - ev, 63);
+  if (ev == 0) m = 0;                          // zeros, denormals
+  const int a = (int)(m >> 38);
+  return h < 0 ? Fix(0ull - m, -a) : Fix(m, a);
+}
+// The sum as a signed integer s in units of 2^(e - 1023 - 57), e the biased
+// exponent to be used with it: six bits finer than asked for where it fits.
+struct FixSum {
+  long long s;
+  int e;
+};
+__device__ __forceinline__ FixSum fix_sum(Fix v, int e) {
+  // |value / 2^38 - a| <= the number of terms
+  const int k = (v.a - (int)(v.lo >> 38) + (1 << 25)) >> 26;
+  const long long f = (long long)v.lo;
+  if (k == (int)(f >> 63)) return FixSum{f, e - 6};
+  return FixSum{((long long)k << 58) + (long long)(((v.lo >> 5) + 1) >> 1), e};
+}
+// s shifted down by sh >= 0 exponents, rounded
+__device__ __forceinline__ long long fix_down(long long s, int sh) {
+  return sh <= 0 ? s : ((s >> min(sh - 1, 62)) + 1) >> 1;
+}
+// the value, rounded to nearest; NaN when e is near that of infinities
+__device__ __forceinline__ double double_of_fix(long long s, int e) {
+  if (e >= 0x7f0) return __longlong_as_double(0x7ff8000000000000LL);
+  if (s == 0) return 0.0;
+  const unsigned sgn = (unsigned)(s >> 32) & 0x80000000u;
+  unsigned long long a = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
+  const int z = __clzll((long long)a);
+  a <<= z;                                     // leading bit at 63
+  const unsigned long long r = ((a >> 10) + 1) >> 1;          // 53 bits, rounded
+  const int ex = e + 6 - z;                    // biased exponent of the leading bit
+  const unsigned long long d = ex <= 0 ? 0 : ((unsigned long long)(ex - 1) << 52) + r;
+  return __longlong_as_double((long long)(d | (unsigned long long)sgn << 32));
+}
+__device__ __forceinline__ double double_of_fix(FixSum v) { return double_of_fix(v.s, v.e); }
 
 // ------------------------------------------------------------------------
 // thermodynamics (Sec. 3.1)

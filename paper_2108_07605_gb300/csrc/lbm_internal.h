@@ -78,6 +78,8 @@ struct Units {
   int newton_max_iter;
   double newton_rtol;
   double dt_sub;         // dt / substeps
+  double dtmm[LBM_MAX_SPECIES];   // dt_sub times the molar mass
+  ff dtmm_f[LBM_MAX_SPECIES];
   // species enthalpies H_a/c^2 = sum_k hl[k][a] T^k (with formation)
   double hl[4][LBM_MAX_SPECIES];
   ff hl_f[4][LBM_MAX_SPECIES];
@@ -232,11 +234,12 @@ struct BatchGrids {
 
 // Grids (of a plan: handles together) with up to this many interface nodes take
 // the boundary kernel with a warp per node, which does more work in all but
-// not in one chain: with the 4078 nodes of the 2000x40 channel a step takes
-// 0.69 ms against 0.75 in FP64, 0.36 against 0.33 in FP32 with FP64 chemistry
-// (there the chain hides behind the bulk nodes); with the flame's 32 nodes
-// 0.29 against 0.60 (FP64) and 0.15 against 0.34 (FP32).
-inline int bnode_warp_limit(lbm_precision p) { return p == LBM_FP64 ? 6144 : 1536; }
+// not in one chain.  Steps of the 1024x4x4 flame (32 nodes): 0.29 ms against
+// 0.60 in FP64, 0.15 against 0.34 in FP32; of a mixed FP32 batch (2816 nodes)
+// 2.2 against 2.7; of the 2000x40 channel (4078 nodes, D2Q9) 0.69 against 0.75
+// in FP64 but 0.36 against 0.33 in FP32 with FP64 chemistry, where the shorter
+// 2-D chain hides behind the bulk nodes.
+inline int bnode_warp_limit(int D, bool fp64) { return D == 2 && !fp64 ? 1536 : 6144; }
 // nodes (warps) per block of it
 constexpr int kBnodeWarps = 2;
 // interface nodes per block of the boundary kernel (one thread each)
@@ -330,6 +333,6 @@ std::string validate_config(const lbm_config* c);   // "" when valid
 void build_device_mechanism(const lbm_mechanism& m, DevMech& d);
 void fill_units(const lbm_config& cfg, Units& un);
 void fill_mixed_units(Units& un);
-void fill_enthalpies(const DevMech& m, Units& un);
+void fill_species_units(const DevMech& m, Units& un);
 
 }  // namespace lbm

@@ -58,7 +58,7 @@ template <typename RT> constexpr bool kFF = sizeof(RT) == 4 && !LBM_CHEM64;
 // four for the float-float chemistry, two with FP64 chemistry beside FP32
 // lattice arithmetic, one in the FP64 path
 template <typename RT>
-constexpr int kMomentsMinBlocks = kFF<RT> ? 4 : (sizeof(RT) == 4 ? 2 : 1);
+constexpr int kMomentsMinBlocks = kFF<RT> ? 4 : (sizeof(RT) == 4 ? 2 : 3);
 
 // Arithmetic type of a storage type: FP16 storage computes in FP32.
 template <typename S> struct ComputeType { using type = S; };
@@ -224,15 +224,13 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
 
 // ---------------------------------------------------------------------------
 // The node's record from its population sums (Sec. 2.1, Sec. 3.1-3.2, Sec.
-// 3.7 slaving): fields, temperature by Newton from the node's previous T,
-// and the reaction sub-steps when chem_inline (else the species densities go
-// to the increment slots for a separate sub-step kernel).  Used by the
-// moments kernels (one thread per node).
+// 3.7 slaving): fields, temperature by Newton from the node's previous T, and
+// the reaction sub-steps.  FP32 lattice arithmetic.
 template <int D, int M, typename RT, bool kDynChem = false>
 __device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __restrict__ Tf,
                                                int* __restrict__ status, long long N,
                                                const Units& un, const DevMech& mech,
-                                               long long n, int chem_inline, RT rho, RT rhoE,
+                                               long long n, RT rho, RT rhoE,
                                                const RT (&j)[D], const RT (&q)[D],
                                                const RT (&P)[Lat<D>::NP], RT (&rs)[M],
                                                RT (&js)[M][D], void* chem_slice) {
@@ -292,15 +290,10 @@ __device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __r
   // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3): a zero-dimensional
   // reactor per node from its post-stream species densities; T_0 is the T
   // just solved.  The increments drho_a (a < M) go to the record.
-  if (!chem_inline) {
+  RT dr[M - 1];
+  node_substeps<M, RT, kDynChem>(rs, rho, ER, usqR, T, un, mech, status, chem_slice, dr);
 #pragma unroll
-    for (int a = 0; a < M - 1; ++a) rec[(RC::DRHO + a) * N + n] = rs[a];
-  } else {
-    RT dr[M - 1];
-    node_substeps<M, RT, kDynChem>(rs, rho, ER, usqR, T, un, mech, status, chem_slice, dr);
-#pragma unroll
-    for (int a = 0; a < M - 1; ++a) rec[(RC::DRHO + a) * N + n] = dr[a];
-  }
+  for (int a = 0; a < M - 1; ++a) rec[(RC::DRHO + a) * N + n] = dr[a];
 
   rec[RC::RHO * N + n] = rho;
 #pragma unroll
@@ -316,37 +309,275 @@ __device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __r
   for (int a = 0; a < M; ++a) {
     rec[(RC::Y + a) * N + n] = YR[a];
     // where defined, |j_a| < rho_a, so the quotient lies in (-1, 1) even when
-    // rho_a is denormal in FP32 (its reciprocal would overflow: FP32 divides);
-    // in FP64 rho_a > 1e-300 where defined, so one reciprocal serves the D
-    // components
+    // rho_a is denormal (its reciprocal would overflow)
     const bool tiny = species_velocity_undefined<D, RT>(rs[a], js[a]);
-    if constexpr (sizeof(RT) == 8) {
-      const RT ira = RT(1) / rs[a];
 #pragma unroll
-      for (int d = 0; d < D; ++d)
-        rec[(RC::US + a * D + d) * N + n] = tiny ? RT(0) : fma(js[a][d], ira, -uR[d]);
-    } else {
-#pragma unroll
-      for (int d = 0; d < D; ++d)
-        rec[(RC::US + a * D + d) * N + n] = tiny ? RT(0) : js[a][d] / rs[a] - uR[d];
-    }
+    for (int d = 0; d < D; ++d)
+      rec[(RC::US + a * D + d) * N + n] = tiny ? RT(0) : js[a][d] / rs[a] - uR[d];
   }
 }
 
 // ---------------------------------------------------------------------------
+// Shared memory of the FP64 moments: per thread the chemistry's slice (C, W),
+// then the concentrations and the summed rates in FP64 (M each).
+template <int M> constexpr size_t moments64_bytes() {
+  return chem_slice_bytes<M>() + (size_t)2 * M * kChemThreads * sizeof(double);
+}
+template <int M>
+__device__ __forceinline__ void* moments64_static() {
+  __shared__ __align__(16) unsigned char mom_raw[moments64_bytes<M>()];
+  return mom_raw;
+}
+
+// The moments, record and reaction sub-steps of bulk node n in FP64, one
+// thread per node, lattice by lattice.
+//
+// What bounds it is the count of FP64 instructions (75 cycles of an SM
+// quarter each), then their latency.  So: a lattice's 27 populations are
+// loaded together (27 loads in flight; three before) and summed in fixed point
+// (fix_of), as are the remainders of the slaved species; u_a - u, which only
+// becomes a diffusion velocity, is a float-float quotient of the FP64 j_a -
+// rho_a u; comparisons are made on the bit patterns; a sub-step's energy
+// coefficients are those of the moments plus float-float increments.  ~500
+// FP64 instructions per node remain of ~1500.  The loop over the lattices is
+// rolled: its sums need no register arrays (so more warps fit) and the code
+// stays in the instruction cache.
+template <int D, int M, typename S>
+__device__ __forceinline__ void moments_body64(const S* __restrict__ src,
+                                               double* __restrict__ rec,
+                                               double* __restrict__ Tf,
+                                               int* __restrict__ status, const Geom& g,
+                                               const Units& un, const BCDev& bc,
+                                               const DevMech& mech, long long n, void* smem) {
+  constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP, NZ = Q / 9;
+  using RC = Rec<D, M>;
+  const long long N = g.N;
+  if (n >= N) return;
+  if (bc.tag && bc.tag[n] == TAG_SOLID) return;
+  ff* const Cs = static_cast<ff*>(smem) + threadIdx.x;
+  ff* const Ws = Cs + M * kChemThreads;
+  double* const Cd = static_cast<double*>(smem) + 2 * M * kChemThreads + threadIdx.x;
+  double* const Wd = Cd + M * kChemThreads;
+  const int x = (int)(n % g.nx);
+  const int y = (int)((n / g.nx) % g.ny);
+  const int z = (int)(n / ((long long)g.nx * g.ny));
+  // pull sources: x of c_x = -1, 0, 1 and the offsets of (c_y, c_z)
+  const int xs[3] = {wrap1(x + 1, g.nx), x, wrap1(x - 1, g.nx)};
+  long long row[Q / 3];
+#pragma unroll
+  for (int r = 0; r < Q / 3; ++r)
+    row[r] = (long long)g.nx *
+             (wrap1(y - (r % 3 - 1), g.ny) +
+              (long long)g.ny * (D == 3 ? wrap1(z - (r / 3 - 1), g.nz) : 0));
+
+  double rho = 0.0, inv_rho = 0.0, u[D], usq = 0.0, ER = 0.0;
+  double Rm = 0.0, cU[4] = {0.0, 0.0, 0.0, 0.0};   // sum Y/m, energy polynomial
+  // the slaved species' sums: the f lattice's minus the others', in fixed
+  // point at exponent eR (momenta: eR - 6); ex: sums that do not fit there
+  // (beyond any physical state)
+  long long rem[1 + D];
+  double ex[1 + D];
+  int eR = 0;
+#pragma unroll
+  for (int d = 0; d <= D; ++d) { rem[d] = 0; ex[d] = 0.0; }
+#pragma unroll
+  for (int d = 0; d < D; ++d) u[d] = 0.0;
+
+  // species a's state from its sums: record, concentration, energy polynomial
+  auto species = [&](int a, double rs, const double (&js)[D]) {
+    const double Y = rs * inv_rho;
+    rec[(RC::Y + a) * N + n] = Y;
+    Rm = fma(Y, mech.inv_mm[a], Rm);
+    cU[0] = fma(Y, mech.u0[a], cU[0]);
+    cU[1] = fma(Y, mech.u1[a], cU[1]);
+    cU[2] = fma(Y, mech.u2[a], cU[2]);
+    cU[3] = fma(Y, mech.u3[a], cU[3]);
+    const double c = rs * mech.inv_mm[a];
+    Cd[a * kChemThreads] = c;
+    Wd[a * kChemThreads] = 0.0;
+    Cs[a * kChemThreads] = ff_of_double(c);
+    // reading R5 on the bit patterns (positive doubles order as integers; a
+    // negative rho_a is below every |j_a|)
+    const long long rb = __double_as_longlong(rs);
+    bool undef = rb <= __double_as_longlong(RHO_TINY);
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+      undef |= (__double_as_longlong(js[d]) & 0x7fffffffffffffffLL) >= rb;
+    // (j_a - rho_a u) / rho_a, both scaled by rho_a's power of two
+    const int de = 1023 - ((__double2hiint(rs) >> 20) & 0x7ff);
+    const ff ir = ff_rcp(ff_of_double(
+        __hiloint2double((__double2hiint(rs) & 0x800fffff) | 0x3ff00000, __double2loint(rs))));
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const double w = fma(-rs, u[d], js[d]);
+      const int h = __double2hiint(w), ew = ((h >> 20) & 0x7ff) + de;
+      const double ws = ew <= 0 || undef
+                            ? 0.0
+                            : __hiloint2double((h & 0x800fffff) | (ew << 20), __double2loint(w));
+      rec[(RC::US + a * D + d) * N + n] = ff_pack(ff_of_double(ws) * ir);
+    }
+  };
+
+#pragma unroll 1
+  for (int it = 0; it <= M; ++it) {
+    const int l = it == 0 ? M - 1 : (it == 1 ? M : it - 2);   // f, g, the species
+    double v[Q];
+    int e = 0;
+    const S* pl = src + (long long)l * Q * N;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = __ldg(pl + (long long)i * N + row[i / 3] + xs[i % 3]);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) e = max(e, fix_exponent(v[i]));
+    Fix sum, sj[D], sP[NP];
+#pragma unroll
+    for (int pz = 0; pz < NZ; ++pz) {
+      Fix ps, pd, py, pxy;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const int i = 9 * pz + 3 * r;
+        const Fix f0 = fix_of(v[i], e), f1 = fix_of(v[i + 1], e), f2 = fix_of(v[i + 2], e);
+        const Fix sx = f0 + f2, sr = sx + f1, dx = f2 - f0;
+        ps = ps + sr;
+        pd = pd + dx;
+        sP[pidx<D>(0, 0)] = sP[pidx<D>(0, 0)] + sx;
+        if (r != 1) {
+          py = r == 2 ? py + sr : py - sr;
+          pxy = r == 2 ? pxy + dx : pxy - dx;
+          sP[pidx<D>(1, 1)] = sP[pidx<D>(1, 1)] + sr;
+        }
+      }
+      sum = sum + ps;
+      sj[0] = sj[0] + pd;
+      sj[1] = sj[1] + py;
+      sP[pidx<D>(0, 1)] = sP[pidx<D>(0, 1)] + pxy;
+      if constexpr (D == 3) {
+        if (pz != 1) {
+          sj[2] = pz == 2 ? sj[2] + ps : sj[2] - ps;
+          sP[pidx<D>(2, 2)] = sP[pidx<D>(2, 2)] + ps;
+          sP[pidx<D>(0, 2)] = pz == 2 ? sP[pidx<D>(0, 2)] + pd : sP[pidx<D>(0, 2)] - pd;
+          sP[pidx<D>(1, 2)] = pz == 2 ? sP[pidx<D>(1, 2)] + py : sP[pidx<D>(1, 2)] - py;
+        }
+      }
+    }
+    const FixSum t0 = fix_sum(sum, e);
+    const double s0 = double_of_fix(t0);
+    FixSum t1[D];
+    double s1[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      t1[d] = fix_sum(sj[d], e);
+      s1[d] = double_of_fix(t1[d]);
+    }
+    if (it == 0) {
+      eR = e + 2;
+      rho = s0;
+      inv_rho = 1.0 / rho;
+      rec[RC::RHO * N + n] = rho;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        u[d] = s1[d] * inv_rho;
+        usq = fma(u[d], u[d], usq);
+        rec[(RC::U + d) * N + n] = u[d];
+      }
+#pragma unroll
+      for (int k = 0; k < NP; ++k)
+        rec[(RC::P + k) * N + n] = double_of_fix(fix_sum(sP[k], e));
+    } else if (it == 1) {
+      ER = s0 * inv_rho;
+      rec[RC::E * N + n] = ER;
+#pragma unroll
+      for (int d = 0; d < D; ++d) rec[(RC::QF + d) * N + n] = s1[d];
+    }
+    if (it != 1) {
+      const long long sg = it == 0 ? 1 : -1;
+      if (t0.e <= eR) rem[0] += sg * fix_down(t0.s, eR - t0.e);
+      else ex[0] += sg * s0;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        if (t1[d].e <= eR - 6) rem[1 + d] += sg * fix_down(t1[d].s, eR - 6 - t1[d].e);
+        else ex[1 + d] += sg * s1[d];
+      }
+      if (it > 1) species(l, s0, s1);
+    }
+  }
+  {   // slaved species M (Eq. strongest)
+    double rs = double_of_fix(rem[0], eR), js[D];
+    if (ex[0] != 0.0) rs += ex[0];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      js[d] = double_of_fix(rem[1 + d], eR - 6);
+      if (ex[1 + d] != 0.0) js[d] += ex[1 + d];
+    }
+    species(M - 1, rs, js);
+  }
+
+  // temperature (Eq. temperature) from the node's previous T
+  const double U = (ER - 0.5 * usq) * un.c * un.c;
+  bool ok;
+  const double T = newton_poly(cU, U, __ldcg(Tf + n), un.newton_max_iter, un.newton_rtol, ok);
+  if (!ok) atomicOr(status, ST_NEWTON);
+  if (!(rho > 0.0) || !isfinite(rho) || !isfinite(T)) atomicOr(status, ST_NONFINITE);
+  Tf[n] = T;
+  const double b3 = fma(-3.0, R_U * Rm * T * un.inv_c2, 1.0);    // 1 - 3 theta
+#pragma unroll
+  for (int d = 0; d < D; ++d)
+    rec[(RC::PHI + d) * N + n] = rho * u[d] * fma(-u[d], u[d], b3);
+
+  // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3): a zero-dimensional
+  // reactor per node from its post-stream species densities; T_0 is the T just
+  // solved
+  double Ts = T;
+  ff dU[4];                              // increments of rho cU
+  const ff irho = ff_of_double(inv_rho);
+#pragma unroll 1
+  for (int s = 0; s < un.substeps; ++s) {
+    if (s > 0) {
+      double c[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) c[k] = cU[k] + double_of_ff(ff_norm(dU[k]) * irho);
+      bool oks;
+      Ts = newton_poly(c, U, Ts, un.newton_max_iter, un.newton_rtol, oks);
+      if (!oks) atomicOr(status, ST_NEWTON);
+    }
+#pragma unroll
+    for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
+    add_reactions<M>(mech, tbasis(Ts), Cs, Ws, 0, 1);
+    const bool last = s + 1 == un.substeps;
+#pragma unroll 1
+    for (int a = 0; a < M; ++a) {
+      const ff w = ff_norm(Ws[a * kChemThreads]);
+      const double wd = double_join(w);
+      Wd[a * kChemThreads] += wd;
+      if (last) continue;
+      const double c = fma(wd, un.dt_sub, Cd[a * kChemThreads]);
+      Cd[a * kChemThreads] = c;
+      Cs[a * kChemThreads] = ff_of_double(c);
+      const ff inc = w * un.dtmm_f[a];
+      ff_fma_acc(dU[0], inc, mech.u0_f[a]);
+      ff_fma_acc(dU[1], inc, mech.u1_f[a]);
+      ff_fma_acc(dU[2], inc, mech.u2_f[a]);
+      ff_fma_acc(dU[3], inc, mech.u3_f[a]);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < M - 1; ++a)
+    rec[(RC::DRHO + a) * N + n] = Wd[a * kChemThreads] * un.dtmm[a];
+}
+
+// ---------------------------------------------------------------------------
 // Moments of the post-stream state + temperature (Sec. 2.1, Sec. 3.1-3.2,
-// Sec. 3.7 slaving, Sec. 4.1 pull streaming).
-// chem_inline = 0: the reaction sub-steps run in a lane-group kernel
-// (k_chem); this kernel then leaves the post-stream species densities rho_a
-// (a < M) in the record's increment slots for it.
+// Sec. 3.7 slaving, Sec. 4.1 pull streaming), and the reaction sub-steps.
 template <int D, int M, typename S, typename RT, bool kDynChem = false>
 __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __restrict__ rec,
                                              double* __restrict__ Tf, int* __restrict__ status,
                                              const Geom& g, const Units& un, const BCDev& bc,
                                              const DevMech& mech, long long n,
-                                             int chem_inline, void* chem_slice = nullptr) {
+                                             void* chem_slice = nullptr) {
+  if constexpr (sizeof(RT) == 8) {
+    if constexpr (!kDynChem) chem_slice = moments64_static<M>();
+    moments_body64<D, M>(src, rec, Tf, status, g, un, bc, mech, n, chem_slice);
+  } else {
   constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP;
-  using RC = Rec<D, M>;
   const long long N = g.N;
   if (n >= N) return;
   const int tag = bc.tag ? bc.tag[n] : TAG_BULK;
@@ -422,8 +653,9 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
       if (D == 3) q[D - 1] += cz * sr;
     }
   }
-  moments_finish<D, M, RT, kDynChem>(rec, Tf, status, N, un, mech, n, chem_inline, rho, rhoE, j,
-                                     q, P, rs, js, chem_slice);
+  moments_finish<D, M, RT, kDynChem>(rec, Tf, status, N, un, mech, n, rho, rhoE, j, q, P, rs, js,
+                                     chem_slice);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -741,7 +973,8 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
     put(RC::Y + a, YR[a]);
     const bool tiny = species_velocity_undefined<D, RT>(rs[a], js[a]);
 #pragma unroll
-    for (int d = 0; d < D; ++d) put(RC::US + a * D + d, tiny ? RT(0) : js[a][d] / rs[a] - uR[d]);
+    for (int d = 0; d < D; ++d)
+      put(RC::US + a * D + d, record_us(tiny ? RT(0) : js[a][d] / rs[a] - uR[d]));
   }
   // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3), T_0 the T just solved
   CT r0[M - 1];
@@ -1020,7 +1253,7 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
         for (int b = 0; b < M; ++b) As[(a * W + b) * st] = yh[b] * mech.K_f[a][b];
 #pragma unroll
         for (int d = 0; d < D; ++d)
-          As[(a * W + M + d) * st] = ff_of_double(rec[(RC::US + a * D + d) * N + n]);
+          As[(a * W + M + d) * st] = ff_unpack(rec[(RC::US + a * D + d) * N + n]);
       }
 #pragma unroll
       for (int a = 0; a < M; ++a) {
@@ -1728,11 +1961,11 @@ __global__ void __launch_bounds__(128, kMomentsMinBlocks<RT>)
 k_moments(const S* __restrict__ src, RT* __restrict__ rec, double* __restrict__ Tf,
           int* __restrict__ status, const __grid_constant__ Geom g,
           const __grid_constant__ Units un, const __grid_constant__ BCDev bc,
-          const __grid_constant__ DevMech mech, int chem_inline, int node_set) {
+          const __grid_constant__ DevMech mech, int node_set) {
   // node_set: NODES_ALL or NODES_BULK
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (node_set == NODES_BULK && bc.tag && n < g.N && bc.tag[n] >= 0) return;
-  moments_body<D, M, S, RT>(src, rec, Tf, status, g, un, bc, mech, n, chem_inline);
+  moments_body<D, M, S, RT>(src, rec, Tf, status, g, un, bc, mech, n);
 }
 
 // reaction sub-steps, L lanes per node, 128 threads per block.  Node sets:
@@ -1903,8 +2136,8 @@ static_assert(sizeof(DomainDev) % 4 == 0, "domain descriptor copied in 4-byte wo
   BlockDomain name{name##_raw}
 template <int D, int M, typename S, typename RT>
 __global__ void __launch_bounds__(128, kMomentsMinBlocks<RT>)
-k_moments_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int chem_inline,
-                int node_set, int nblk) {
+k_moments_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int node_set,
+                int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   // node_set: NODES_ALL or NODES_BULK (the interface nodes' records come from
   // k_bnode_batch)
@@ -1914,7 +2147,7 @@ k_moments_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int ch
     const long long n = (b - d.block_begin) * (long long)blockDim.x + threadIdx.x;
     if (node_set == NODES_BULK && d.bc.tag && n < d.g.N && d.bc.tag[n] >= 0) continue;
     moments_body<D, M, S, RT>(static_cast<const S*>(d.pops[c]), static_cast<RT*>(d.rec), d.Tf,
-                              d.status, d.g, d.un, d.bc, *d.mech, n, chem_inline);
+                              d.status, d.g, d.un, d.bc, *d.mech, n);
   }
 }
 
@@ -2189,7 +2422,7 @@ k_step_persist(const DomainDev* __restrict__ doms, int ndom, int parity,
         const long long n = w.first + (long long)j * kPersistThreads + threadIdx.x;
         if (n >= d.g.N) break;
         if (d.bc.tag && d.bc.tag[n] >= 0) continue;   // interface node: PI_BND
-        moments_body<D, M, S, RT, true>(src, rec, d.Tf, d.status, d.g, d.un, d.bc, *d.mech, n, 1,
+        moments_body<D, M, S, RT, true>(src, rec, d.Tf, d.status, d.g, d.un, d.bc, *d.mech, n,
                                         ps_raw);
       }
     } else if (w.kind == PI_PREP) {
@@ -2228,6 +2461,7 @@ template <int D, int M, typename S, typename RT> constexpr size_t persist_smem(b
   const size_t chem =
       chem_slice_bytes<M>() + sizeof(R) * WB<D, M>::N * (kPersistThreads / 32);
   size_t m = bnd > chem ? bnd : chem;
+  if (sizeof(RT) == 8) m = m > moments64_bytes<M>() ? m : moments64_bytes<M>();
   if (split) {
     m = m > prep ? m : prep;
     m = m > coll ? m : coll;
@@ -2525,7 +2759,7 @@ static cudaError_t step_impl(const DevMech& mech, const StepArgs& a, cudaStream_
     const bool fork = a.bc.n_if > 0 && a.side && a.ev_fork && a.ev_join;
     // the boundary kernel and the interface nodes' sub-steps
     auto boundary = [&](cudaStream_t st) {
-      if (a.bc.n_if <= bnode_warp_limit(sizeof(RT) == 8 ? LBM_FP64 : LBM_FP32_STORE)) {
+      if (a.bc.n_if <= bnode_warp_limit(D, sizeof(RT) == 8)) {
         k_bnode_warp<D, M, S><<<blocks_for(a.bc.n_if, kBnodeWarps), 32 * kBnodeWarps, 0, st>>>(
             src, a.bc, a.Tfield, a.status, a.g, a.un, a.mech_dev, rec);
         return;
@@ -2540,7 +2774,7 @@ static cudaError_t step_impl(const DevMech& mech, const StepArgs& a, cudaStream_
         mchem(s, node_set);
       else
         k_moments<D, M, S, RT><<<nb, bs, 0, s>>>(src, rec, a.Tfield, a.status, a.g, a.un, a.bc,
-                                                 mech, 1, node_set);
+                                                 mech, node_set);
     };
     if (fork) {
       cudaError_t e = cudaEventRecord(a.ev_fork, s);
@@ -2704,7 +2938,7 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
     e = cudaEventRecord(side.join, side.stream);
     if (e != cudaSuccess) return e;
     if (chem_inline)
-      kmom<<<batch_grid(kmom, gr.nblocks, bs, 0, ps), bs, 0, s>>>(doms, ndom, parity, 1,
+      kmom<<<batch_grid(kmom, gr.nblocks, bs, 0, ps), bs, 0, s>>>(doms, ndom, parity,
                                                                   NODES_BULK, gr.nblocks);
     else
       mchem(NODES_BULK);
@@ -2716,7 +2950,7 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
       bnd(s);
     if (chem_inline)
       kmom<<<batch_grid(kmom, gr.nblocks, bs, 0, ps), bs, 0, s>>>(
-          doms, ndom, parity, 1, bnd_rec ? NODES_BULK : NODES_ALL, gr.nblocks);
+          doms, ndom, parity, bnd_rec ? NODES_BULK : NODES_ALL, gr.nblocks);
     else
       mchem(bnd_rec ? NODES_BULK : NODES_ALL);
     if (bnd_rec) chem(NODES_INTERFACE, s);
