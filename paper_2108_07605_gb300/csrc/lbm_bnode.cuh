@@ -85,11 +85,12 @@ template <int D, int M, typename R> struct BSums {
 // The macroscopic state of population sums (Eqs. density1, momentum1,
 // fdensity, f1momMomentum, g0momTotalEnergy, slaving Eq. strongest): rho,
 // u, Y, u_a (reading R5) and T by Newton on Eq. temperature from T_guess,
-// then theta and U/c^2 as bstate_prepare.
+// then theta and U/c^2 as bstate_prepare; the record's enthalpy polynomial in
+// H if given.
 template <int D, int M, typename R>
 __device__ __forceinline__ void bstate_of(BState<D, M, R>& s, const BSums<D, M, R>& z,
                                           double T_guess, const DevMech& m, const Units& un,
-                                          int* status) {
+                                          int* status, R* H = nullptr) {
   s.rho = z.rho;
   const R irho = R(1) / z.rho;
   R usq = R(0);
@@ -131,18 +132,39 @@ __device__ __forceinline__ void bstate_of(BState<D, M, R>& s, const BSums<D, M, 
 #pragma unroll
     for (int a = 0; a < M; ++a) Y[a] = double(s.Y[a * kBnd]);
     const double U = (double(z.rhoE * irho) - 0.5 * double(usq)) * un.c * un.c;
-    const double T = newton_T<M>(m, Y, U, T_guess, un.newton_max_iter, un.newton_rtol, ok);
+    double c[4];
+    const double T = newton_T<M>(m, Y, U, T_guess, un.newton_max_iter, un.newton_rtol, ok, c);
     s.T = R(T);
     s.T_full = T;
+    if (H) {
+      R Rm = R(0), h[4];
+#pragma unroll
+      for (int a = 0; a < M; ++a) {
+        if constexpr (sizeof(R) == 8) Rm += Y[a] * m.inv_mm[a];
+        else Rm += s.Y[a * kBnd] * m.inv_mm_s[a];
+      }
+      enthalpy_poly(c, Rm, un, h);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) H[k] = h[k];
+    }
   } else {
     ff Yf[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) Yf[a] = ff(s.Y[a * kBnd]);
     const ff U = (ff(z.rhoE * irho) + ff(-0.5f * usq)) * un.c2_f;
+    ff c[4];
     const ff T = newton_T_ff<M>(m, Yf, U, ff_from_double(T_guess), un.newton_max_iter,
-                                un.newton_rtol_f, ok);
+                                un.newton_rtol_f, ok, c);
     s.T = T.hi;
     s.T_full = ff_to_double(T);
+    if (H) {
+      float Rm = 0.f, h[4];
+#pragma unroll
+      for (int a = 0; a < M; ++a) Rm += s.Y[a * kBnd] * m.inv_mm_s[a];
+      enthalpy_poly(c, Rm, un, h);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) H[k] = h[k];
+    }
   }
   if (!ok) atomicOr(status, ST_NEWTON);
   bstate_prepare<D, M, R>(s, m, un);
@@ -609,22 +631,11 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
   BState<D, M, R> s;
   s.Y = A.Y;                                    // the target columns are free now
   s.us = col + 3 * M * kBnd;
-  bstate_of<D, M, R>(s, z, __ldcg(Tf + n), m, un, status);
+  R H[4];
+  bstate_of<D, M, R>(s, z, __ldcg(Tf + n), m, un, status, H);
   if (!(s.rho > R(0)) || !isfinite(double(s.rho)) || !isfinite(s.T_full))
     atomicOr(status, ST_NONFINITE);
   Tf[n] = s.T_full;
-  R thR;
-  if constexpr (sizeof(R) == 4) {
-    float Rm = 0.f;
-#pragma unroll
-    for (int a = 0; a < M; ++a) Rm += s.Y[a * kBnd] * m.inv_mm_s[a];
-    thR = Rm * float(R_U) * s.T * un.inv_c2_s;
-  } else {
-    double Rmix = 0.0;
-#pragma unroll
-    for (int a = 0; a < M; ++a) Rmix += s.Y[a * kBnd] * m.inv_mm[a];
-    thR = R(Rmix * R_U * s.T * un.inv_c2);
-  }
   const R rr = s.rho;
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) rec[(RC::DRHO + a) * N + n] = s.Y[a * kBnd] * rr;
@@ -632,13 +643,15 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     rec[(RC::U + d) * N + n] = s.u[d];
-    rec[(RC::QF + d) * N + n] = z.q[d];
+    rec[(RC::Z + d) * N + n] = flux_less_work<D, R>(d, s.u, z.q, z.P);
     rec[(RC::PHI + d) * N + n] =
-        rr * s.u[d] * (R(1) - R(3) * thR) - rr * s.u[d] * s.u[d] * s.u[d];
+        rr * s.u[d] * (R(1) - R(3) * s.th) - rr * s.u[d] * s.u[d] * s.u[d];
   }
-#pragma unroll
-  for (int p = 0; p < NP; ++p) rec[(RC::P + p) * N + n] = z.P[p];
   rec[RC::E * N + n] = z.rhoE * (R(1) / rr);
+  rec[RC::TH * N + n] = s.th;
+  rec[RC::LNT * N + n] = ln_T0(s.T);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) rec[(RC::H + k) * N + n] = H[k];
 #pragma unroll
   for (int a = 0; a < M; ++a) {
     rec[(RC::Y + a) * N + n] = s.Y[a * kBnd];
@@ -802,7 +815,7 @@ __device__ __forceinline__ void wsums(const R (&v)[WB<D, M>::NR], R* z, int lane
 template <int D, int M, typename R>
 __device__ __forceinline__ void wstate_of(WState<D, M, R>& s, const R* z, double T_guess,
                                           const DevMech& m, const Units& un, int* status,
-                                          int lane) {
+                                          int lane, R* H = nullptr) {
   using W = WB<D, M>;
   using CT = typename ChemType<R>::type;
   using X = Chem<CT>;
@@ -856,6 +869,18 @@ __device__ __forceinline__ void wstate_of(WState<D, M, R>& s, const R* z, double
     s.T_full = ff_to_double(T);
   }
   if (!ok && lane == 0) atomicOr(status, ST_NEWTON);
+  if (H) {
+    R Rm = R(0), h[4];
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+      for (int b = 0; b < M; ++b) Rm += s.Y[b] * m.inv_mm_s[b];
+    } else {
+      Rm = species_sum(Ya * m.inv_mm[a]);
+    }
+    enthalpy_poly(c, Rm, un, h);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) H[k] = h[k];
+  }
   wprepare<D, M, R>(s, m, un, lane);
 }
 
@@ -1095,7 +1120,8 @@ __device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDe
   s.Y = Fs;
   s.us = Fs + M;
   s.own_us = true;
-  wstate_of<D, M, R>(s, sm, Tg, m, un, status, lane);
+  R H[4];
+  wstate_of<D, M, R>(s, sm, Tg, m, un, status, lane, H);
   const R rr = s.rho;
   if (lane == 0) {
     if (!(rr > R(0)) || !isfinite(double(rr)) || !isfinite(s.T_full))
@@ -1103,17 +1129,21 @@ __device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDe
     Tf[n] = s.T_full;
     rec[RC::RHO * N + n] = rr;
     rec[RC::E * N + n] = sm[W::Z + M * W::ZS] * (R(1) / rr);
+    rec[RC::TH * N + n] = s.th;
+    rec[RC::LNT * N + n] = ln_T0(s.T);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) rec[(RC::H + k) * N + n] = H[k];
   }
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     if (lane == 1 + d) {
       rec[(RC::U + d) * N + n] = s.u[d];
-      rec[(RC::QF + d) * N + n] = sm[W::Z + M * W::ZS + 1 + d];
+      rec[(RC::Z + d) * N + n] =
+          flux_less_work<D, R>(d, s.u, sm + W::Z + M * W::ZS + 1, sm + W::P);
       rec[(RC::PHI + d) * N + n] =
           rr * s.u[d] * (R(1) - R(3) * s.th) - rr * s.u[d] * s.u[d] * s.u[d];
     }
   }
-  for (int e = lane; e < W::NP; e += 32) rec[(RC::P + e) * N + n] = sm[W::P + e];
   for (int a = lane; a < M; a += 32) rec[(RC::Y + a) * N + n] = s.Y[a];
 #pragma unroll
   for (int d = 0; d < D; ++d)

@@ -680,7 +680,7 @@ void fill_mixed_units(Units& un) {
 void fill_species_units(const DevMech& m, Units& un) {
   for (int a = 0; a < m.M; ++a) {
     const double h[4] = {m.u0[a], m.u1[a] + m.Ra[a], m.u2[a], m.u3[a]};
-    for (int k = 0; k < 4; ++k) un.hl_f[k][a] = ff_host(un.hl[k][a] = h[k] * un.inv_c2);
+    for (int k = 0; k < 4; ++k) un.hl_f[k][a] = ff_host(h[k] * un.inv_c2);
     un.dtmm_f[a] = ff_host(un.dtmm[a] = un.dt_sub * m.mm[a]);
   }
 }

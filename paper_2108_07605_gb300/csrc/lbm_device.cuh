@@ -50,18 +50,23 @@ __host__ __device__ __forceinline__ bool species_velocity_undefined(R rho_a, con
 }
 
 // Moment-record field offsets ([field][N] scratch in the lattice compute
-// type, written by the moments kernel, read by the collision kernel).
+// type, written by the moments and boundary kernels, read by the collision
+// kernel).  Neighbours read H and PHI only.
 template <int D, int M> struct Rec {
   static constexpr int RHO = 0;
   static constexpr int U = 1;
-  static constexpr int P = U + D;
-  static constexpr int QF = P + Lat<D>::NP;
-  static constexpr int E = QF + D;
+  static constexpr int Z = U + D;               // q - u . P (energy flux less the work of P)
+  static constexpr int E = Z + D;
   static constexpr int Y = E + 1;
-  static constexpr int US = Y + M;              // u_a - u (record_us)
+  // sum_a Y_a H_a(T)/c^2 as a polynomial in T: its gradient at a node's own T
+  // is sum_a H_a grad Y_a, from four fields per neighbour instead of M
+  static constexpr int H = Y + M;
+  static constexpr int US = H + 4;              // u_a - u (record_us)
   static constexpr int PHI = US + M * D;
   static constexpr int DRHO = PHI + D;          // reaction increments, species a < M
-  static constexpr int NF = DRHO + M - 1;
+  static constexpr int TH = DRHO + M - 1;       // theta = R T / c^2
+  static constexpr int LNT = TH + 1;            // ln(T / T0)
+  static constexpr int NF = LNT + 1;
 };
 
 // u_a - u as the record holds it: in FP64 a float-float pair, the type of the
@@ -182,12 +187,19 @@ __device__ __forceinline__ double newton_poly(const double (&c)[4], double U, do
   return T;
 }
 
+// c receives the polynomial's coefficients
+template <int M>
+__device__ __forceinline__ double newton_T(const DevMech& m, const double* Y, double U,
+                                           double T, int max_iter, double rtol, bool& ok,
+                                           double (&c)[4]) {
+  mixture_energy_poly<M>(m, Y, c);
+  return newton_poly(c, U, T, max_iter, rtol, ok);
+}
 template <int M>
 __device__ __forceinline__ double newton_T(const DevMech& m, const double* Y, double U,
                                            double T, int max_iter, double rtol, bool& ok) {
   double c[4];
-  mixture_energy_poly<M>(m, Y, c);
-  return newton_poly(c, U, T, max_iter, rtol, ok);
+  return newton_T<M>(m, Y, U, T, max_iter, rtol, ok, c);
 }
 
 __device__ __forceinline__ double species_U(const DevMech& m, int a, double T) {
@@ -222,8 +234,9 @@ __device__ __forceinline__ ff newton_poly(const ff (&c)[4], ff U, ff T, int max_
 
 template <int M>
 __device__ __forceinline__ ff newton_T_ff(const DevMech& m, const ff* Y, ff U, ff T,
-                                          int max_iter, float rtol, bool& ok) {
-  ff c[4];
+                                          int max_iter, float rtol, bool& ok, ff (&c)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c[k] = ff();
 #pragma unroll
   for (int a = 0; a < M; ++a) {
     ff_fma_acc(c[0], Y[a], m.u0_f[a]);
@@ -234,6 +247,42 @@ __device__ __forceinline__ ff newton_T_ff(const DevMech& m, const ff* Y, ff U, f
 #pragma unroll
   for (int k = 0; k < 4; ++k) c[k] = ff_norm(c[k]);
   return newton_poly(c, U, T, max_iter, rtol, ok);
+}
+
+// The record's enthalpy polynomial from the energy polynomial c (J/kg) and
+// sum Y_a/m_a: H_a = U_a + R_a T.
+__device__ __forceinline__ void enthalpy_poly(const double (&c)[4], double Rm, const Units& un,
+                                              double (&H)[4]) {
+  H[0] = c[0] * un.inv_c2;
+  H[1] = fma(Rm, R_U, c[1]) * un.inv_c2;
+  H[2] = c[2] * un.inv_c2;
+  H[3] = c[3] * un.inv_c2;
+}
+__device__ __forceinline__ void enthalpy_poly(const double (&c)[4], float Rm, const Units& un,
+                                              float (&H)[4]) {
+  H[0] = float(c[0] * un.inv_c2);
+  H[1] = float((c[1] + double(Rm) * R_U) * un.inv_c2);
+  H[2] = float(c[2] * un.inv_c2);
+  H[3] = float(c[3] * un.inv_c2);
+}
+__device__ __forceinline__ void enthalpy_poly(const ff (&c)[4], float Rm, const Units& un,
+                                              float (&H)[4]) {
+  H[0] = (c[0] * un.inv_c2_f).hi;
+  H[1] = ((c[1] + ff(Rm * float(R_U))) * un.inv_c2_f).hi;
+  H[2] = (c[2] * un.inv_c2_f).hi;
+  H[3] = (c[3] * un.inv_c2_f).hi;
+}
+// ln(T / T0)
+__device__ __forceinline__ float ln_T0(float T) { return log(T * float(1.0 / T_REF)); }
+__device__ __forceinline__ double ln_T0(double T) { return log(T * (1.0 / T_REF)); }
+// q - u . P
+template <int D, typename R, typename QT, typename PT>
+__device__ __forceinline__ R flux_less_work(int d, const R (&u)[D], const QT& q, const PT& P) {
+  R v = q[d];
+#pragma unroll
+  for (int b = 0; b < D; ++b)
+    v = fma(-u[b], P[b == d ? b : (D == 3 ? (b + d == 1 ? 3 : (b + d == 2 ? 4 : 5)) : 2)], v);
+  return v;
 }
 
 // ------------------------------------------------------------------------

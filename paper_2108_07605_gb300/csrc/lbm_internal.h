@@ -16,6 +16,7 @@ namespace lbm {
 
 constexpr double R_U = 8.314462618;       // J/(mol K)
 constexpr double T_REF = 298.15;          // K, T0 of Sec. 3.6
+constexpr double LN_T_REF = 5.697596715569115;   // ln(T_REF)
 constexpr double P_REF = 101325.0;        // Pa, P0 of Sec. 3.6
 constexpr double RHO_TINY = 1e-300;       // u_a := u below this species density
 
@@ -80,8 +81,7 @@ struct Units {
   double dt_sub;         // dt / substeps
   double dtmm[LBM_MAX_SPECIES];   // dt_sub times the molar mass
   ff dtmm_f[LBM_MAX_SPECIES];
-  // species enthalpies H_a/c^2 = sum_k hl[k][a] T^k (with formation)
-  double hl[4][LBM_MAX_SPECIES];
+  // species enthalpies H_a/c^2 = sum_k hl_f[k][a] T^k (with formation)
   ff hl_f[4][LBM_MAX_SPECIES];
   // mixed path: float-float and FP32 copies
   ff c2_f, inv_c2_f, dt_sub_f;   // c^2, 1/c^2, dt / substeps

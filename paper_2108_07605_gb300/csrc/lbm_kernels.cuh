@@ -184,7 +184,8 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
 #pragma unroll
         for (int a = 0; a < M; ++a) Ys[a] = r[a] / rho_f;
         bool oks;
-        Ts = newton_T_ff<M>(mech, Ys, Uphys, Ts, un.newton_max_iter, un.newton_rtol_f, oks);
+        ff c[4];
+        Ts = newton_T_ff<M>(mech, Ys, Uphys, Ts, un.newton_max_iter, un.newton_rtol_f, oks, c);
         if (!oks) atomicOr(status, ST_NEWTON);
       }
 #pragma unroll
@@ -256,10 +257,10 @@ __device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __r
   const RT ER = rhoE * inv_rho;
   bool ok;
   double T;
-  RT thR;
+  RT thR, H[4];
   if constexpr (kFF<RT>) {
     // mixed path: the temperature solve in float-float
-    ff Yf[M];
+    ff Yf[M], c[4];
     float Rm = 0.f;
 #pragma unroll
     for (int a = 0; a < M; ++a) {
@@ -268,20 +269,21 @@ __device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __r
     }
     const ff U = (ff(ER) + ff(-0.5f * usqR)) * un.c2_f;
     const ff Tx = newton_T_ff<M>(mech, Yf, U, ff_from_double(__ldcg(Tf + n)), un.newton_max_iter,
-                                 un.newton_rtol_f, ok);
+                                 un.newton_rtol_f, ok, c);
     T = ff_to_double(Tx);
     thR = Rm * float(R_U) * Tx.hi * un.inv_c2_s;
+    enthalpy_poly(c, Rm, un, H);
   } else {
-    double Y[M];
+    double Y[M], c[4];
 #pragma unroll
     for (int a = 0; a < M; ++a) Y[a] = double(YR[a]);
     const double U = (double(ER) - 0.5 * double(usqR)) * un.c * un.c;
-    T = newton_T<M>(mech, Y, U, __ldcg(Tf + n), un.newton_max_iter, un.newton_rtol, ok);
-    double Rmix = 0.0;
+    T = newton_T<M>(mech, Y, U, __ldcg(Tf + n), un.newton_max_iter, un.newton_rtol, ok, c);
+    float Rm = 0.f;
 #pragma unroll
-    for (int a = 0; a < M; ++a) Rmix += Y[a] * mech.inv_mm[a];
-    Rmix *= R_U;
-    thR = RT(Rmix * T * un.inv_c2);
+    for (int a = 0; a < M; ++a) Rm += float(YR[a]) * mech.inv_mm_s[a];
+    thR = RT(Rm * float(R_U) * float(T) * un.inv_c2_s);
+    enthalpy_poly(c, RT(Rm), un, H);
   }
   if (!ok) atomicOr(status, ST_NEWTON);
   if (!(rho > RT(0)) || !isfinite(double(rho)) || !isfinite(T)) atomicOr(status, ST_NONFINITE);
@@ -299,12 +301,14 @@ __device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __r
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     rec[(RC::U + d) * N + n] = uR[d];
-    rec[(RC::QF + d) * N + n] = q[d];
+    rec[(RC::Z + d) * N + n] = flux_less_work<D, RT>(d, uR, q, P);
     rec[(RC::PHI + d) * N + n] = rho * uR[d] * (RT(1) - RT(3) * thR) - rho * uR[d] * uR[d] * uR[d];
   }
-#pragma unroll
-  for (int k = 0; k < NP; ++k) rec[(RC::P + k) * N + n] = P[k];
   rec[RC::E * N + n] = ER;
+  rec[RC::TH * N + n] = thR;
+  rec[RC::LNT * N + n] = ln_T0(RT(T));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) rec[(RC::H + k) * N + n] = H[k];
 #pragma unroll
   for (int a = 0; a < M; ++a) {
     rec[(RC::Y + a) * N + n] = YR[a];
@@ -370,7 +374,7 @@ __device__ __forceinline__ void moments_body64(const S* __restrict__ src,
              (wrap1(y - (r % 3 - 1), g.ny) +
               (long long)g.ny * (D == 3 ? wrap1(z - (r / 3 - 1), g.nz) : 0));
 
-  double rho = 0.0, inv_rho = 0.0, u[D], usq = 0.0, ER = 0.0;
+  double rho = 0.0, inv_rho = 0.0, u[D], usq = 0.0, ER = 0.0, Z[D];
   double Rm = 0.0, cU[4] = {0.0, 0.0, 0.0, 0.0};   // sum Y/m, energy polynomial
   // the slaved species' sums: the f lattice's minus the others', in fixed
   // point at exponent eR (momenta: eR - 6); ex: sums that do not fit there
@@ -381,7 +385,7 @@ __device__ __forceinline__ void moments_body64(const S* __restrict__ src,
 #pragma unroll
   for (int d = 0; d <= D; ++d) { rem[d] = 0; ex[d] = 0.0; }
 #pragma unroll
-  for (int d = 0; d < D; ++d) u[d] = 0.0;
+  for (int d = 0; d < D; ++d) u[d] = Z[d] = 0.0;
 
   // species a's state from its sums: record, concentration, energy polynomial
   auto species = [&](int a, double rs, const double (&js)[D]) {
@@ -479,14 +483,16 @@ __device__ __forceinline__ void moments_body64(const S* __restrict__ src,
         usq = fma(u[d], u[d], usq);
         rec[(RC::U + d) * N + n] = u[d];
       }
+      double P[NP];
 #pragma unroll
-      for (int k = 0; k < NP; ++k)
-        rec[(RC::P + k) * N + n] = double_of_fix(fix_sum(sP[k], e));
+      for (int k = 0; k < NP; ++k) P[k] = double_of_fix(fix_sum(sP[k], e));
+#pragma unroll
+      for (int d = 0; d < D; ++d) Z[d] = flux_less_work<D, double>(d, u, Z, P);
     } else if (it == 1) {
       ER = s0 * inv_rho;
       rec[RC::E * N + n] = ER;
 #pragma unroll
-      for (int d = 0; d < D; ++d) rec[(RC::QF + d) * N + n] = s1[d];
+      for (int d = 0; d < D; ++d) rec[(RC::Z + d) * N + n] = s1[d] + Z[d];
     }
     if (it != 1) {
       const long long sg = it == 0 ? 1 : -1;
@@ -518,7 +524,12 @@ __device__ __forceinline__ void moments_body64(const S* __restrict__ src,
   if (!ok) atomicOr(status, ST_NEWTON);
   if (!(rho > 0.0) || !isfinite(rho) || !isfinite(T)) atomicOr(status, ST_NONFINITE);
   Tf[n] = T;
-  const double b3 = fma(-3.0, R_U * Rm * T * un.inv_c2, 1.0);    // 1 - 3 theta
+  const double th = R_U * Rm * T * un.inv_c2, b3 = fma(-3.0, th, 1.0);    // 1 - 3 theta
+  double H[4];
+  enthalpy_poly(cU, Rm, un, H);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) rec[(RC::H + k) * N + n] = H[k];
+  rec[RC::TH * N + n] = th;
 #pragma unroll
   for (int d = 0; d < D; ++d)
     rec[(RC::PHI + d) * N + n] = rho * u[d] * fma(-u[d], u[d], b3);
@@ -541,7 +552,9 @@ __device__ __forceinline__ void moments_body64(const S* __restrict__ src,
     }
 #pragma unroll
     for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
-    add_reactions<M>(mech, tbasis(Ts), Cs, Ws, 0, 1);
+    const TBasis<double> tb = tbasis(Ts);
+    if (s == 0) rec[RC::LNT * N + n] = tb.lnT - LN_T_REF;
+    add_reactions<M>(mech, tb, Cs, Ws, 0, 1);
     const bool last = s + 1 == un.substeps;
 #pragma unroll 1
     for (int a = 0; a < M; ++a) {
@@ -725,9 +738,10 @@ __device__ __forceinline__ CT pick(const CT (&r)[M], int a) {
 template <int M, int L, typename CT>
 __device__ __forceinline__ CT group_newton(const DevMech& m, const CT (&r)[M], CT irho, CT U,
                                            CT T, const Units& un, int sub, unsigned gmask,
-                                           bool& ok) {
+                                           bool& ok, CT (&c)[4]) {
   using X = Chem<CT>;
-  CT c[4] = {CT(), CT(), CT(), CT()};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c[k] = CT();
 #pragma unroll
   for (int j = 0; j < (M + L - 1) / L; ++j) {
     const int a = sub + j * L;
@@ -758,7 +772,8 @@ __device__ __forceinline__ void chem_group_substeps(CT (&r)[M], const CT irho, c
   for (int s = 0; s < un.substeps; ++s) {
     if (s > 0) {
       bool ok;
-      Ts = group_newton<M, L, CT>(m, r, irho, U, Ts, un, sub, gmask, ok);
+      CT c[4];
+      Ts = group_newton<M, L, CT>(m, r, irho, U, Ts, un, sub, gmask, ok, c);
       if (!ok && sub == 0) atomicOr(status, ST_NEWTON);
     }
 #pragma unroll
@@ -933,21 +948,25 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
   for (int a = 0; a < M; ++a) r[a] = X::of(rs[a]);
   const CT irho = X::inv(X::of(rho));
   bool ok;
-  const CT Tx = group_newton<M, L, CT>(mg, r, irho, U, X::of_T(Tf[n]), un, sub, gmask, ok);
+  CT c[4];
+  const CT Tx = group_newton<M, L, CT>(mg, r, irho, U, X::of_T(Tf[n]), un, sub, gmask, ok, c);
   double T;
-  RT thR;
-  if constexpr (kFF<RT>) {
+  RT thR, H[4];
+  if constexpr (sizeof(RT) == 4) {
     float Rm = 0.f;
 #pragma unroll
     for (int a = 0; a < M; ++a) Rm += YR[a] * m.inv_mm_s[a];
-    T = ff_to_double(Tx);
-    thR = Rm * float(R_U) * Tx.hi * un.inv_c2_s;
+    if constexpr (kFF<RT>) T = ff_to_double(Tx);
+    else T = Tx;
+    thR = Rm * float(R_U) * float(T) * un.inv_c2_s;
+    enthalpy_poly(c, Rm, un, H);
   } else {
-    double Rmix = 0.0;
+    double Rm = 0.0;
 #pragma unroll
-    for (int a = 0; a < M; ++a) Rmix += double(YR[a]) * m.inv_mm[a];
+    for (int a = 0; a < M; ++a) Rm += YR[a] * m.inv_mm[a];
     T = Tx;
-    thR = RT(Rmix * R_U * T * un.inv_c2);
+    thR = RT(Rm * R_U * T * un.inv_c2);
+    enthalpy_poly(c, Rm, un, H);
   }
   if (sub == 0) {
     if (!ok) atomicOr(status, ST_NEWTON);
@@ -962,12 +981,14 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     put(RC::U + d, uR[d]);
-    put(RC::QF + d, q[d]);
+    put(RC::Z + d, flux_less_work<D, RT>(d, uR, q, P));
     put(RC::PHI + d, rho * uR[d] * (RT(1) - RT(3) * thR) - rho * uR[d] * uR[d] * uR[d]);
   }
-#pragma unroll
-  for (int k = 0; k < NP; ++k) put(RC::P + k, P[k]);
   put(RC::E, ER);
+  put(RC::TH, thR);
+  put(RC::LNT, ln_T0(RT(T)));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) put(RC::H + k, H[k]);
 #pragma unroll
   for (int a = 0; a < M; ++a) {
     put(RC::Y + a, YR[a]);
@@ -1085,46 +1106,29 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
   const double T_d = __ldcg(Tf + n);
   const RT T = RT(T_d);
   const RT E = rec[RC::E * N + n];
-  RT u[D], Y[M], q[D], P[NP], usq = RT(0);
+  const RT theta = rec[RC::TH * N + n];
+  RT u[D], Y[M], Z[D], usq = RT(0);
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     u[d] = rec[(RC::U + d) * N + n];
-    q[d] = rec[(RC::QF + d) * N + n];
+    Z[d] = rec[(RC::Z + d) * N + n];
     usq += u[d] * u[d];
   }
 #pragma unroll
-  for (int k = 0; k < NP; ++k) P[k] = rec[(RC::P + k) * N + n];
-#pragma unroll
   for (int a = 0; a < M; ++a) Y[a] = rec[(RC::Y + a) * N + n];
 
-  // species enthalpies H_a/c^2 (Horner in FP64; in the mixed path summed in
-  // float-float, rounded)
-  RT Ha[M];
-  if constexpr (sizeof(RT) == 8) {
-#pragma unroll
-    for (int a = 0; a < M; ++a)
-      Ha[a] = fma(T, fma(T, fma(T, un.hl[3][a], un.hl[2][a]), un.hl[1][a]), un.hl[0][a]);
-  } else {
-    const ff T1 = ff_of_double(T_d), T2 = T1 * T1, T3 = T2 * T1;
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-      ff h = un.hl_f[0][a];
-      ff_fma_acc(h, un.hl_f[1][a], T1);
-      ff_fma_acc(h, un.hl_f[2][a], T2);
-      ff_fma_acc(h, un.hl_f[3][a], T3);
-      Ha[a] = ff_norm(h).hi;
-    }
-  }
-
-  // isotropic gradients: d_a Phi_a, and sum_a H_a grad Y_a with this node's
-  // H_a, whose sum over the species is taken at each neighbour first (M + 3
-  // multiply-adds per neighbour instead of 3 M, and three sums in registers
-  // instead of 3 M): 3 sum_i w_i c_i phi(x + c_i)
-  RT dPhi[D], corr[D], HYself = RT(0);
+  // isotropic gradients 3 sum_i w_i c_i phi(x + c_i): d_a Phi_a, and
+  // sum_a H_a grad Y_a with this node's H_a, from the neighbours' enthalpy
+  // polynomials at this node's T (three multiply-adds per neighbour instead of
+  // M, and M - 4 fewer loads)
+  RT dPhi[D], corr[D];
 #pragma unroll
   for (int d = 0; d < D; ++d) dPhi[d] = corr[d] = RT(0);
-#pragma unroll
-  for (int a = 0; a < M; ++a) HYself += Ha[a] * Y[a];
+  auto enthalpy = [&](long long nb) {
+    const RT* h = rec + (long long)RC::H * N + nb;
+    return fma(T, fma(T, fma(T, __ldg(h + 3 * N), __ldg(h + 2 * N)), __ldg(h + N)), __ldg(h));
+  };
+  const RT HYself = enthalpy(n);
   // ghost values beyond non-periodic faces and on solid nodes: walls Phi = 0,
   // inlet the inlet state's Phi, outlet the node's own Phi; Y the node's own
   RT phi_self[D], phi_in[D];
@@ -1176,12 +1180,7 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
       const RT wy = cyi == 0 ? RT(2.0 / 3.0) : RT(1.0 / 6.0);
       const RT wz = D == 3 ? (czi == 0 ? RT(2.0 / 3.0) : RT(1.0 / 6.0)) : RT(1);
       const RT w3 = RT(3) * ((ix == 1 ? RT(2.0 / 3.0) : RT(1.0 / 6.0)) * wy * wz);
-      RT hy = HYself;
-      if (gk == BK_NONE) {
-        hy = RT(0);
-#pragma unroll
-        for (int a = 0; a < M; ++a) hy += Ha[a] * __ldg(rec + (RC::Y + a) * N + nb);
-      }
+      const RT hy = gk == BK_NONE ? enthalpy(nb) : HYself;
 #pragma unroll
       for (int d = 0; d < D; ++d) {
         if (cvi[d] == 0) continue;
@@ -1197,12 +1196,7 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
   // relaxation parameters (Sec. 2.3 Eqs. betaa, taua; Sec. 3.5 Eqs. mu,
   // lambda): 1/tau_ab = s K_ab; with xr = nu/theta, omega = 1/(xr + 1/2),
   // omega1 = 1/(xr/Pr + 1/2) and (2 - omega)/(2 omega) = xr
-  RT Rmix = RT(0);
-#pragma unroll
-  for (int a = 0; a < M; ++a) Rmix += Y[a] * MP::inv_mm(mech, a);
-  Rmix *= RT(R_U);
-  const RT theta = Rmix * T * MP::inv_c2(un);
-  const RT lnTr = log(T * RT(1.0 / T_REF));
+  const RT lnTr = rec[RC::LNT * N + n];
   const RT s_tau = MP::s_pref(un) * rho * T * T * exp_of(-MP::D_T_exp(mech) * lnTr);
   RT mu = MP::mu0(mech);
   if (mech.wilke) {
@@ -1304,36 +1298,36 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
   const RT U_lat = E - RT(0.5) * usq;
   RT W[D];
   {
+    // diffusion flux sum_a H_a Y_a V_a, H_a/c^2 in float-float
     VT diff[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) diff[d] = VT();
+    const ff T1 = ff_of_double(T_d), T2 = T1 * T1, T3 = T2 * T1;
 #pragma unroll
     for (int a = 0; a < M; ++a) {
+      ff h = un.hl_f[0][a];
+      ff_fma_acc(h, un.hl_f[1][a], T1);
+      ff_fma_acc(h, un.hl_f[2][a], T2);
+      ff_fma_acc(h, un.hl_f[3][a], T3);
       if constexpr (sizeof(RT) == 8) {
-        const ff HY = ff_of_double(Ha[a] * Y[a]);
+        const ff HY = ff_norm(h) * ff_of_double(Y[a]);
 #pragma unroll
         for (int d = 0; d < D; ++d) ff_fma_acc(diff[d], HY, V[a][d]);
       } else {
-        const RT HY = Ha[a] * Y[a];
+        const RT HY = ff_norm(h).hi * Y[a];
 #pragma unroll
         for (int d = 0; d < D; ++d) diff[d] += HY * V[a][d];
       }
     }
+    // q - q^eq - u . (P - P^eq) = (q - u . P) - rho u (E - u^2)
+    const RT b = rho * (E - usq);
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      const RT ud = u[d];
-      const RT q_eq = rho * ud * (E + theta);
-      RT uP = RT(0);
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        const RT Peq = rho * u[b] * ud + (b == d ? Pres : RT(0));
-        uP += u[b] * (P[pidx<D>(b, d)] - Peq);
-      }
-      const RT q_ex = RT(-0.5) * ud * dPhi[d];
       RT df;
       if constexpr (sizeof(RT) == 8) df = double_of_ff(diff[d]);
       else df = diff[d];
-      W[d] = (omega - omega1) * (q[d] - q_eq - uP + q_ex) + omega1 * rho * df +
+      const RT qd = fma(-b, u[d], Z[d]) - RT(0.5) * u[d] * dPhi[d];     // with q^ex
+      W[d] = (omega - omega1) * qd + omega1 * rho * df +
              (RT(0.5) * (RT(2) - omega1)) * Pres * corr[d];
     }
   }
