@@ -294,22 +294,10 @@ __device__ __forceinline__ ExpArg exp_arg(ff x) {
   a.rl = r.lo;
   return a;
 }
-// x in FP64: integer part and rest from its fixed-point form with 46 fraction
-// bits, in integer arithmetic (the FP64 pipe would take three additions)
-__device__ __forceinline__ ExpArg exp_arg(double x) {
-  const int h = __double2hiint(x), l = __double2loint(x);
-  const int mag = h & 0x7fffffff;
-  if (mag >= 0x40cf4000) {                 // 16000 and above
-    ExpArg b{h < 0 ? -16000 : 16000, 0.f, 0.f};
-    if (x != x) b.rh = __int_as_float(0x7fffffff);
-    return b;
-  }
-  const unsigned long long m =
-      ((unsigned long long)(unsigned)((mag & 0xfffff) | 0x100000) << 42) |
-      ((unsigned long long)(unsigned)l << 10);            // mantissa, 62 fraction bits
-  const int sh = min(1039 - (mag >> 20), 63);             // 16 - exponent
-  long long v = (long long)(m >> sh);
-  if (h < 0) v = -v;
+// x in fixed point with 46 fraction bits, |x| < 2^17
+__device__ __forceinline__ ExpArg exp_arg(long long v) {
+  const long long top = 16000LL << 46;
+  v = v > top ? top : (v < -top ? -top : v);
   const int vh = (int)(v >> 32);
   ExpArg a;
   a.n = (vh + (1 << 13)) >> 14;
@@ -319,6 +307,26 @@ __device__ __forceinline__ ExpArg exp_arg(double x) {
   a.rh = __fmul_rn(__int2float_rn(f1 & ~0xff), 0x1p-32f);
   a.rl = __fmul_rn(__int2float_rn(((f1 & 0xff) << 14) | (int)(fl & 0x3fffu)), 0x1p-46f);
   return a;
+}
+// 0 <= d < 2^(63 - bits) as an integer with `bits` fraction bits
+__device__ __forceinline__ long long fixed_of(double d, int bits) {
+  const int h = __double2hiint(d);
+  const unsigned long long m =
+      ((unsigned long long)(unsigned)((h & 0xfffff) | 0x100000) << 42) |
+      ((unsigned long long)(unsigned)__double2loint(d) << 10);    // 62 fraction bits
+  const int sh = 62 + 1023 - bits - (h >> 20);
+  return (long long)(m >> min(max(sh, 0), 63));
+}
+// x in FP64, through its fixed-point form
+__device__ __forceinline__ ExpArg exp_arg(double x) {
+  const int h = __double2hiint(x);
+  if ((h & 0x7fffffff) >= 0x40cf4000) {                 // 16000 and above
+    ExpArg b{h < 0 ? -16000 : 16000, 0.f, 0.f};
+    if (x != x) b.rh = __int_as_float(0x7fffffff);
+    return b;
+  }
+  const long long v = fixed_of(__hiloint2double(h & 0x7fffffff, __double2loint(x)), 46);
+  return exp_arg(h < 0 ? -v : v);
 }
 
 __device__ __forceinline__ ff exp_frac(const ExpArg& a) {

@@ -280,6 +280,15 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
   }
   const long double ln_p0 = std::log(P_REF / R_U), S = 64.0L / std::log(2.0L);
   int n = 0;
+  d.fixed_args = 1;
+  // coefficient of basis function j in fixed point; the sum of a reaction's
+  // terms has to stay below 2^62
+  auto fixed = [&](long double c, int j) {
+    const int bits[5] = {64, kBitsLnT, kBitsInvT, kBitsT, kBitsT2};
+    const long double v = std::ldexp(c, kArgBits + 64 - bits[j]);
+    if (!(std::fabs(v) < std::ldexp(1.0L, j ? 63 : 61))) { d.fixed_args = 0; return 0LL; }
+    return (long long)std::llround(v);
+  };
   for (int k = -1; k < rows; ++k)
     for (int r = 0; r < m.n_reactions; ++r) {
       if (set[r] != k) continue;
@@ -303,8 +312,23 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
         for (int j = 0; j < m.nu_r[r][a]; ++j) { x.prod[x.np++] = a; molecule(a, 1.0L); }
       }
       const long double f[3] = {lnA, b, -EaR};
-      for (int j = 0; j < 3; ++j) x.f_f[j] = ff_host(x.f[j] = (double)(S * f[j]));
-      for (int j = 0; j < 5; ++j) x.r_f[j] = ff_host(x.r[j] = (double)(S * c[j]));
+      for (int j = 0; j < 3; ++j) {
+        x.f_f[j] = ff_host(x.f[j] = (double)(S * f[j]));
+        x.fq[j] = fixed(S * f[j], j);
+      }
+      for (int j = 0; j < 5; ++j) {
+        x.r_f[j] = ff_host(x.r[j] = (double)(S * c[j]));
+        x.rq[j] = fixed(S * c[j], j);
+      }
+      // |sum| over the temperature range, in units of ln2/64
+      auto reach = [&](const long double* q, int nq) {
+        const long double top[5] = {1.0L, 9.8L, 1.0L / 128, 16384.0L, 268435456.0L};
+        long double t = 0.0L;
+        for (int j = 0; j < nq; ++j) t += std::fabs(S * q[j]) * top[j];
+        if (!(t < 65536.0L)) d.fixed_args = 0;
+      };
+      reach(f, 3);
+      reach(c, 5);
     }
   d.D_T_exp = m.D_T_exponent;
   d.mu0 = m.mu0;

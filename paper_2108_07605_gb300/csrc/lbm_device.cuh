@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "exp64.cuh"
+#include "log64.cuh"
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -274,7 +275,7 @@ __device__ __forceinline__ void enthalpy_poly(const ff (&c)[4], float Rm, const 
 }
 // ln(T / T0)
 __device__ __forceinline__ float ln_T0(float T) { return log(T * float(1.0 / T_REF)); }
-__device__ __forceinline__ double ln_T0(double T) { return log(T * (1.0 / T_REF)); }
+__device__ __forceinline__ double ln_T0(double T) { return log_tang(T) - LN_T_REF; }
 // q - u . P
 template <int D, typename R, typename QT, typename PT>
 __device__ __forceinline__ R flux_less_work(int d, const R (&u)[D], const QT& q, const PT& P) {
@@ -295,24 +296,49 @@ __device__ __forceinline__ R flux_less_work(int d, const R (&u)[D], const QT& q,
 // per SM quarter, in float-float ~410 FP32 instructions.  So (1) the
 // logarithm of each rate constant is one sum over the basis (1, ln T, 1/T, T,
 // T^2) with coefficients folded on the host, which replaces the species' Gibbs
-// functions; (2) only these sums run in FP64 (six instructions per
-// reaction), where the argument's size (up to ~100) would cost a
-// float-float its accuracy; the exponentials, products and sums that follow
-// keep ~48 bits in pairs of FP32, below the ~1e-14 that the rounding of T
-// leaves in a rate constant; (3) sums stay unnormalised (ff_acc); (4) the
+// functions; (2) of FP64 temperatures these sums are taken in 64-bit fixed
+// point (the argument's size, up to ~100, would cost a float-float its
+// accuracy); the exponentials, products and sums that follow keep ~48 bits in
+// pairs of FP32, below the ~1e-14 that the rounding of T leaves in a rate
+// constant; (3) sums stay unnormalised (ff_acc); (4) the
 // third-body sums are formed once per distinct row of efficiencies.
 template <typename CT> struct TBasis { CT lnT, invT, T, T2; };
+// FP64: also in fixed point, in which a sum takes no FP64 instruction (and is
+// exact to 2^-46; FP64's own rounding of it is up to 2^-40); usable for
+// mechanisms and temperatures inside its range
+template <> struct TBasis<double> {
+  double lnT, invT, T, T2;
+  long long q[5];
+  bool fixed;
+};
 
-__device__ __forceinline__ TBasis<double> tbasis(double T) {
-  return TBasis<double>{log(T), 1.0 / T, T, T * T};
+__device__ __forceinline__ TBasis<double> tbasis(const DevMech& m, double T) {
+  TBasis<double> b;
+  b.lnT = log_tang(T);
+  b.invT = 1.0 / T;
+  b.T = T;
+  b.T2 = T * T;
+  const int h = __double2hiint(T);              // 128 <= T < 16384
+  b.fixed = m.fixed_args && h >= 0x40600000 && h < 0x40d00000;
+  b.q[0] = 0;
+  b.q[1] = fixed_of(b.lnT, kBitsLnT);
+  b.q[2] = fixed_of(b.invT, kBitsInvT);
+  b.q[3] = fixed_of(T, kBitsT);
+  b.q[4] = fixed_of(b.T2, kBitsT2);
+  return b;
 }
-__device__ __forceinline__ TBasis<ff> tbasis(ff T) {
+__device__ __forceinline__ TBasis<ff> tbasis(const DevMech&, ff T) {
   return TBasis<ff>{ff_log(T), ff(1.f) / T, T, T * T};
 }
 __device__ __forceinline__ ExpArg forward_arg(const DevReaction& x, const TBasis<double>& b) {
+  if (b.fixed)
+    return exp_arg(x.fq[0] + __mul64hi(x.fq[1], b.q[1]) + __mul64hi(x.fq[2], b.q[2]));
   return exp_arg(fma(x.f[2], b.invT, fma(x.f[1], b.lnT, x.f[0])));
 }
 __device__ __forceinline__ ExpArg reverse_arg(const DevReaction& x, const TBasis<double>& b) {
+  if (b.fixed)
+    return exp_arg(x.rq[0] + __mul64hi(x.rq[1], b.q[1]) + __mul64hi(x.rq[2], b.q[2]) +
+                   __mul64hi(x.rq[3], b.q[3]) + __mul64hi(x.rq[4], b.q[4]));
   return exp_arg(fma(x.r[2], b.invT,
                      fma(x.r[1], b.lnT, fma(x.r[4], b.T2, fma(x.r[3], b.T, x.r[0])))));
 }
@@ -393,7 +419,7 @@ __device__ __forceinline__ void molar_rates(const DevMech& m, CT T, ff (&w)[M], 
   ff* const Ws = Cs + M * kChemThreads;
 #pragma unroll
   for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
-  add_reactions<M>(m, tbasis(T), Cs, Ws, 0, 1);
+  add_reactions<M>(m, tbasis(m, T), Cs, Ws, 0, 1);
 #pragma unroll
   for (int a = 0; a < M; ++a) w[a] = ff_norm(Ws[a * kChemThreads]);
 }

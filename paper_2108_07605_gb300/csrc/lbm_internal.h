@@ -38,11 +38,19 @@ struct DevReaction {
   int third_body;        // row of DevMech::eff_f, -1: none
   double f[3], r[5];
   ff f_f[3], r_f[5];     // the same as float-float (mixed path)
+  // and in fixed point, each against its basis function's units (kArgBits)
+  long long fq[3], rq[5];
 };
+// Fixed-point rate-constant logarithms: 46 fraction bits in the sum; the basis
+// functions ln T, 1/T, T, T^2 with these many (below 2^63 for 128 K <= T <
+// 16384 K), so the coefficients with 46 + 64 less those.
+constexpr int kArgBits = 46;
+constexpr int kBitsLnT = 59, kBitsInvT = 70, kBitsT = 49, kBitsT2 = 35;
 
 // Mechanism in the forms the kernels evaluate (built on the host).
 struct DevMech {
   int M, R;
+  int fixed_args;        // every reaction's fq and rq fit
   double mm[LBM_MAX_SPECIES], inv_mm[LBM_MAX_SPECIES], Ra[LBM_MAX_SPECIES];
   // U_a(T) = u0 + u1 T + u2 T^2 + u3 T^3  (J/kg, incl. formation)
   double u0[LBM_MAX_SPECIES], u1[LBM_MAX_SPECIES], u2[LBM_MAX_SPECIES],

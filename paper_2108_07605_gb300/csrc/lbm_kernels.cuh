@@ -552,7 +552,7 @@ __device__ __forceinline__ void moments_body64(const S* __restrict__ src,
     }
 #pragma unroll
     for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
-    const TBasis<double> tb = tbasis(Ts);
+    const TBasis<double> tb = tbasis(mech, Ts);
     if (s == 0) rec[RC::LNT * N + n] = tb.lnT - LN_T_REF;
     add_reactions<M>(mech, tb, Cs, Ws, 0, 1);
     const bool last = s + 1 == un.substeps;
@@ -781,7 +781,7 @@ __device__ __forceinline__ void chem_group_substeps(CT (&r)[M], const CT irho, c
       Cs[a * kChemThreads] = X::concentration(m, a, r[a]);
       Ws[a * kChemThreads] = ff();
     }
-    add_reactions<M>(m, tbasis(Ts), Cs, Ws, sub, L);
+    add_reactions<M>(m, tbasis(m, Ts), Cs, Ws, sub, L);
     ff w[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) w[a] = Ws[a * kChemThreads];
@@ -1733,6 +1733,22 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   const int tag = n < N ? (bc.tag ? bc.tag[n] : TAG_BULK) : TAG_SOLID;
   const bool valid = tag != TAG_SOLID;
   double* const s = sm + lane;
+  const int x = (int)(n % g.nx);
+  const int y = (int)((n / g.nx) % g.ny);
+  const int z = (int)(n / ((long long)g.nx * g.ny));
+  constexpr int NZ = D == 3 ? 3 : 1;
+  constexpr int CH = (Q + TPN - 1) / TPN;
+  const int k0 = w * CH, k1 = min(k0 + CH, Q);
+  // the first direction's populations are in flight while the block's tables
+  // are built
+  double fin[M + 1];
+#pragma unroll
+  for (int l = 0; l <= M; ++l) fin[l] = 0.0;
+  if (valid && k0 < k1) {
+    const int i = k0 / NZ + 9 * (k0 % NZ);
+    load_direction<D, M, S, double>(src, bc, tag, N, node_shift<D>(x, y, z, i, -1, g), i,
+                                    g.codec, fin);
+  }
   for (int f = w; f < CP::NF; f += TPN)
     s[f * kCollNodes] = valid ? __ldcg(cp + f * N + n) : 0.0;
   __syncthreads();
@@ -1777,12 +1793,6 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   if (!valid) return;
   auto P = [&](int f) { return s[f * kCollNodes]; };
   auto PF = [&](int f) { return ff_unpack(s[f * kCollNodes]); };
-  const int x = (int)(n % g.nx);
-  const int y = (int)((n / g.nx) % g.ny);
-  const int z = (int)(n / ((long long)g.nx * g.ny));
-  constexpr int NZ = D == 3 ? 3 : 1;
-  constexpr int CH = (Q + TPN - 1) / TPN;
-  const int k0 = w * CH, k1 = min(k0 + CH, Q);
   if (k0 >= k1) return;
   ff A[M], SS[M];              // t_x e_y + s_x t_y and s_x s_y, times -rho_b
   double eh[M - 1];            // hh_a e_x e_y
@@ -1793,9 +1803,13 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   for (int k = k0; k < k1; ++k) {
     const int j = k / NZ, i = j + 9 * (k % NZ);
     const int cx = cvel(j, 0), cy = cvel(j, 1), cz = D == 3 ? k % NZ - 1 : 0;
-    double fin[M + 1];
-    load_direction<D, M, S, double>(src, bc, tag, N, node_shift<D>(x, y, z, i, -1, g), i,
-                                    g.codec, fin);
+    // the next direction, whose populations take the places of this one's as
+    // these are used up (the last direction loads its own again)
+    const int kn = min(k + 1, k1 - 1), in = kn / NZ + 9 * (kn % NZ);
+    const long long sn = node_shift<D>(x, y, z, in, -1, g);
+    auto next = [&](int l) {
+      return pop_in<double>(src, bc, tag, N, sn, l * Q + in, g.codec);
+    };
     if (j != jcur) {
       jcur = j;
 #pragma unroll
@@ -1838,6 +1852,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
       F = PF(CP::CF + a) * ff_norm(F);
       const double ez = D == 3 ? P(T::e(a, D - 1, cz)) : 1.0;
       const double base = fma(fin[a], P(CP::OM1 + a), double_join(F));
+      fin[a] = next(a);
       dst[(long long)(a * Q + i) * N + n] = D == 3 ? fma(eh[a], ez, base) : eh[a] + base;
     }
     double fex = fxy, geq = gQ;
@@ -1846,7 +1861,9 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
       geq = fma(P(T::AF + 6 + cz + 1), gQ, gP * P(T::BF + 6 + cz + 1));
     }
     dst[(long long)((M - 1) * Q + i) * N + n] = fma(om, fex - fin[M - 1], fin[M - 1]);
+    fin[M - 1] = next(M - 1);
     double gn = fma(om, fma(rho, geq, -fin[M]), fin[M]);
+    fin[M] = next(M);
     if (csq(i, D) == 1) {
 #pragma unroll
       for (int d = 0; d < D; ++d)
