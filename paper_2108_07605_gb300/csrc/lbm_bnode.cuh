@@ -379,13 +379,13 @@ template <int D, int M, typename S, typename R> struct BPull {
 template <int D, int M, typename S, typename R> struct BStorePull {
   static constexpr int Q = Lat<D>::Q;
   BPull<D, M, S, R> p;
-  double* P;
+  R* P;
   long long st;
   template <int l> __device__ __forceinline__ void setup() {}
   template <int l> __device__ __forceinline__ void row(int, int) {}
   template <int l> __device__ __forceinline__ R get(int i, const int (&)[3]) const {
     const R v = p.template pull<l>(i);
-    P[(long long)(l * Q + i) * st] = double(v);
+    P[(long long)(l * Q + i) * st] = v;
     return v;
   }
 };
@@ -422,44 +422,115 @@ template <int D, int M, typename S, typename R> struct BLocal {
   }
 };
 
-// Step 4: the target Bt + the local populations - the local equilibria L;
-// the simplified inlet takes the local equilibria.  Stored as the node's
-// reconstructed populations.
+// Step 4: the target + the local populations - the local equilibria L, stored
+// as the node's reconstructed populations (the simplified inlet: the local
+// equilibria).  same: the target is the state A of the incoming links, else Bt.
 template <int D, int M, typename S, typename R> struct BFinal {
   static constexpr int Q = Lat<D>::Q;
   BLocal<D, M, S, R> lo;
   const BState<D, M, R>* Bt;
   const BState<D, M, R>* L;
-  bool simple, same;        // same: Bt is the state A of the incoming links
-  double* P;
+  bool simple, same;
+  R* P;
   long long st;
   ETab<D, M, R> tb, tl;
-  template <int l> __device__ __forceinline__ void setup() {
-    lo.template setup<l>();
-    if (!same) tb.template build<l>(*Bt, *lo.m, *lo.un);
-    tl.template build<l>(*L, *lo.m, *lo.un);
-  }
-  template <int l> __device__ __forceinline__ void row(int cy, int cz) {
-    lo.template row<l>(cy, cz);
-    if (!same) tb.template row<l>(cy, cz);
-    tl.template row<l>(cy, cz);
-  }
-  template <int l> __device__ __forceinline__ R get(int i, const int (&c)[3]) const {
-    const R loc = tl.template evalx<l>(c[0]);
-    R v;
-    if (simple) {
-      v = loc;
-    } else if (lo.p.incoming(i)) {
-      const R a = lo.ta.template evalx<l>(c[0]);
-      v = (same ? a : tb.template evalx<l>(c[0])) + a - loc;
-    } else {
-      v = (same ? lo.ta.template evalx<l>(c[0]) : tb.template evalx<l>(c[0])) +
-          lo.p.template pull<l>(i) - loc;
-    }
-    P[(long long)(l * Q + i) * st] = double(v);
-    return v;
+  __device__ __forceinline__ void store() {
+    ForL<0, M + 1>::run([&](auto lc) {
+      constexpr int l = decltype(lc)::value;
+      lo.template setup<l>();
+      if (!same) tb.template build<l>(*Bt, *lo.m, *lo.un);
+      tl.template build<l>(*L, *lo.m, *lo.un);
+#pragma unroll 1
+      for (int yz = 0; yz < Q / 3; ++yz) {
+        const int cy = yz % 3 - 1, cz = D == 3 ? yz / 3 - 1 : 0;
+        lo.template row<l>(cy, cz);
+        if (!same) tb.template row<l>(cy, cz);
+        tl.template row<l>(cy, cz);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const int i = 3 * yz + k;
+          const R loc = tl.template evalx<l>(k - 1), a = lo.ta.template evalx<l>(k - 1);
+          const R t = same ? a : tb.template evalx<l>(k - 1);
+          const R v = t + (lo.p.incoming(i) ? a : lo.p.template pull<l>(i)) - loc;
+          P[(long long)(l * Q + i) * st] = simple ? loc : v;
+        }
+      }
+    });
   }
 };
+
+// The sums of the reconstructed populations, target t + local populations
+// (whose sums these are) - local equilibria l: the two equilibria's moments are
+// known, so no pass over the populations is needed.  Explicitly fused (see
+// mul1).
+template <typename R>
+__device__ __forceinline__ R final_momentum(R rt, R ut, R j, R rl, R ul) {
+  return fma(rt, ut, fma(-rl, ul, j));
+}
+template <int D, int M, typename R, typename ST>
+__device__ __forceinline__ R final_flux(int a, int b, const ST& t, R P, const ST& l) {
+  const R pt = a == b ? fma(t.u[a], t.u[a], t.th) : mul1(t.u[a], t.u[b]);
+  const R pl = a == b ? fma(l.u[a], l.u[a], l.th) : mul1(l.u[a], l.u[b]);
+  return fma(t.rho, pt, fma(-l.rho, pl, P));
+}
+template <int D, typename R, typename ST>
+__device__ __forceinline__ R state_energy(const ST& s) {       // U + u^2/2
+  R q = mul1(s.u[0], s.u[0]);
+#pragma unroll
+  for (int d = 1; d < D; ++d) q = fma(s.u[d], s.u[d], q);
+  return fma(R(0.5), q, s.U);
+}
+template <int D, int M, typename R>
+__device__ __forceinline__ void final_sums(BSums<D, M, R>& z, const BState<D, M, R>& t,
+                                           const BState<D, M, R>& l) {
+  const R Et = state_energy<D, R>(t), El = state_energy<D, R>(l);
+#pragma unroll
+  for (int a = 0; a < M - 1; ++a) {
+    const R rt = mul1(t.rho, t.Y[a * kBnd]), rl = mul1(l.rho, l.Y[a * kBnd]);
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+      z.js[a][d] = final_momentum(rt, t.us ? t.us[(a * D + d) * kBnd] : t.u[d], z.js[a][d], rl,
+                                  l.us ? l.us[(a * D + d) * kBnd] : l.u[d]);
+    z.rs[a] = rt;
+  }
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    z.j[d] = mul1(t.rho, t.u[d]);
+    z.q[d] = final_momentum(mul1(t.rho, Et + t.th), t.u[d], z.q[d], mul1(l.rho, El + l.th),
+                            l.u[d]);
+  }
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll
+    for (int b = a; b < D; ++b)
+      z.P[pidx<D>(a, b)] = final_flux<D, M, R>(a, b, t, z.P[pidx<D>(a, b)], l);
+  z.rhoE = final_momentum(t.rho, Et, z.rhoE, l.rho, El);
+  z.rho = t.rho;
+}
+// ... and of the local equilibria alone (simplified inlet)
+template <int D, int M, typename R>
+__device__ __forceinline__ void equilibrium_sums(BSums<D, M, R>& z, const BState<D, M, R>& l) {
+#pragma unroll
+  for (int a = 0; a < M - 1; ++a) {
+    z.rs[a] = mul1(l.rho, l.Y[a * kBnd]);
+#pragma unroll
+    for (int d = 0; d < D; ++d) z.js[a][d] = mul1(z.rs[a], l.u[d]);
+  }
+  const R E = state_energy<D, R>(l);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    z.j[d] = mul1(l.rho, l.u[d]);
+    z.q[d] = mul1(mul1(l.rho, E + l.th), l.u[d]);
+  }
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll
+    for (int b = a; b < D; ++b)
+      z.P[pidx<D>(a, b)] =
+          mul1(l.rho, a == b ? fma(l.u[a], l.u[a], l.th) : mul1(l.u[a], l.u[b]));
+  z.rhoE = mul1(l.rho, E);
+  z.rho = l.rho;
+}
 
 // The boundary procedure of interface node k and its moment record.
 // col: this thread's shared-memory column of R entries, sncol: its column of
@@ -498,7 +569,8 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
   if (kind == BK_BB) {
     // Eq. bb: incoming links take the node's own opposite post-collision
     // populations
-    BStorePull<D, M, S, R> out{Pull{src, codec, N, n, sncol, inc, true}, bc.pops + k, st};
+    BStorePull<D, M, S, R> out{Pull{src, codec, N, n, sncol, inc, true},
+                               static_cast<R*>(bc.pops) + k, st};
     bsums<D, M, R>(out, z);
   } else {
     if (kind == BK_TMS) {
@@ -620,14 +692,16 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
       bstate_prepare<D, M, R>(B, m, un);
     }
     // step 4 (Eqs. ftms-fatms, f_inlet-fa_inlet, f_outlet-fa_outlet)
-    BFinal<D, M, S, R> fin{local, &B, &L, kind == BK_INLET && bc.inlet_simplified != 0,
-                           kind != BK_INLET, bc.pops + k, st, {}, {}};
-    bsums<D, M, R>(fin, z);
+    const bool simple = kind == BK_INLET && bc.inlet_simplified != 0, same = kind != BK_INLET;
+    BFinal<D, M, S, R> fin{local, &B, &L, simple, same, static_cast<R*>(bc.pops) + k, st, {}, {}};
+    fin.store();
+    if (simple) equilibrium_sums<D, M, R>(z, L);
+    else final_sums<D, M, R>(z, same ? A : B, L);
   }
 
-  // the record from the reconstructed populations (the fields the moments
-  // kernel records: state with Newton from the node's previous T, energy
-  // flux, momentum flux tensor); the reaction sub-steps follow in their own kernel
+  // the record from the sums of the reconstructed populations (the fields the
+  // moments kernel records, T by Newton from the node's previous T); the
+  // reaction sub-steps follow in their own kernel
   BState<D, M, R> s;
   s.Y = A.Y;                                    // the target columns are free now
   s.us = col + 3 * M * kBnd;
@@ -663,7 +737,7 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
 
 // ---------------------------------------------------------------------------
 // The same procedure with one warp per interface node, for grids with few of
-// them (bnode_warp_limit): a thread per node is then a single chain of some
+// them (kBnodeWarpNodes): a thread per node is then a single chain of some
 // thousand dependent loads and sums, whatever the node count (444 us in FP64,
 // 355 us in FP32 for the 32 interface nodes of the 1024x4x4 flame, the
 // critical path of its step; with a warp each, sub-steps included, 70 and 56).  Lane 3 l + p holds lattice l's directions of
@@ -1108,14 +1182,52 @@ __device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDe
 #pragma unroll
       for (int j = 0; j < W::NR; ++j) v[j] = ea[j] + (incoming(j) ? ea[j] : pull[j]) - el[j];
     }
+    // their sums (final_sums, equilibrium_sums), a lattice per lane
+    const bool simple = kind == BK_INLET && bc.inlet_simplified != 0;
+    const WState<D, M, R>& t = simple ? L : (kind == BK_INLET ? B : A);
+    const R Et = state_energy<D, R>(t), El = state_energy<D, R>(L);
+    if (lane <= M) {
+      R* zl = sm + W::Z + lane * W::ZS;
+      if (lane < M - 1) {
+        const R rt = mul1(t.rho, t.Y[lane]), rl = mul1(L.rho, L.Y[lane]);
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          const R ut = t.own_us ? t.us[lane * D + d] : t.u[d];
+          zl[1 + d] = simple ? mul1(rt, ut)
+                             : final_momentum(rt, ut, zl[1 + d], rl,
+                                              L.own_us ? L.us[lane * D + d] : L.u[d]);
+        }
+        zl[0] = rt;
+      } else if (lane == M - 1) {
+        zl[0] = t.rho;
+#pragma unroll
+        for (int d = 0; d < D; ++d) zl[1 + d] = mul1(t.rho, t.u[d]);
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+#pragma unroll
+          for (int b = a; b < D; ++b) {
+            R& P = sm[W::P + pidx<D>(a, b)];
+            P = simple ? mul1(t.rho, a == b ? fma(t.u[a], t.u[a], t.th) : mul1(t.u[a], t.u[b]))
+                       : final_flux<D, M, R>(a, b, t, P, L);
+          }
+      } else {
+        zl[0] = simple ? mul1(t.rho, Et) : final_momentum(t.rho, Et, zl[0], L.rho, El);
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+          zl[1 + d] = simple ? mul1(mul1(t.rho, Et + t.th), t.u[d])
+                             : final_momentum(mul1(t.rho, Et + t.th), t.u[d], zl[1 + d],
+                                              mul1(L.rho, El + L.th), L.u[d]);
+      }
+    }
+    __syncwarp();
   }
+  if (kind == BK_BB) wsums<D, M, R>(v, sm, lane);
   if (on)
 #pragma unroll
     for (int j = 0; j < W::NR; ++j)
-      bc.pops[(long long)(l * Q + i0 + j) * bc.n_if + k] = double(v[j]);
+      static_cast<R*>(bc.pops)[(long long)(l * Q + i0 + j) * bc.n_if + k] = v[j];
 
   // the record
-  wsums<D, M, R>(v, sm, lane);
   WState<D, M, R> s;
   s.Y = Fs;
   s.us = Fs + M;

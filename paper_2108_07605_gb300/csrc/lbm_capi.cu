@@ -89,8 +89,7 @@ void fill_domains(lbm_ctx* const* hs, int n, const Launch& lc, std::vector<Domai
   doms.assign(n, DomainDev());
   gr = BatchGrids();
   for (int k = 0; k < n; ++k) gr.n_if_total += hs[k]->bc.n_if;
-  gr.bnd_warp = n > 0 && gr.n_if_total <= bnode_warp_limit(
-                                        hs[0]->D, hs[0]->cfg.precision == LBM_FP64);
+  gr.bnd_warp = gr.n_if_total <= kBnodeWarpNodes;
   const int per_bnd = gr.bnd_warp ? kBnodeWarps : kBndNodesPerBlock;
   for (int k = 0; k < n; ++k) {
     lbm_ctx* h = hs[k];
@@ -886,7 +885,7 @@ lbm_status lbm_create(const lbm_config* cfg, lbm_t* out) {
     unsigned* if_inc = reinterpret_cast<unsigned*>(take(nif * sizeof(unsigned)));
     double* wallT = reinterpret_cast<double*>(take(nif * sizeof(double)));
     double* uin = reinterpret_cast<double*>(take(3 * nif * sizeof(double)));
-    b.pops = reinterpret_cast<double*>(take((size_t)h->L * h->Q * nif * sizeof(double)));
+    b.pops = static_cast<void*>(take((size_t)h->L * h->Q * nif * sizeof(double)));
     cudaError_t e = cudaMemcpy(tag, hb.tag.data(), N * sizeof(int), cudaMemcpyHostToDevice);
     if (hb.offgrid) {
       int* nbr = reinterpret_cast<int*>(take(nif * sizeof(int)));

@@ -119,7 +119,7 @@ struct BCDev {
   const unsigned* if_inc = nullptr;  // incoming-link mask (bit i = link i)
   const double* if_wallT = nullptr;  // [n_if] TMS target temperature (K)
   const double* if_uin = nullptr;    // [3][n_if] inlet velocity, lattice units
-  double* pops = nullptr;            // [L][Q][n_if] reconstructed populations
+  void* pops = nullptr;              // [L][Q][n_if] reconstructed populations (lattice type)
   // off-grid TMS targets (nullptr: targets at the node): the fluid node x_f
   // of each interface node (-1: none), its normal projection h and the
   // node's normal wall distance delta (lattice units)
@@ -244,10 +244,9 @@ struct BatchGrids {
 // the boundary kernel with a warp per node, which does more work in all but
 // not in one chain.  Steps of the 1024x4x4 flame (32 nodes): 0.29 ms against
 // 0.60 in FP64, 0.15 against 0.34 in FP32; of a mixed FP32 batch (2816 nodes)
-// 2.2 against 2.7; of the 2000x40 channel (4078 nodes, D2Q9) 0.69 against 0.75
-// in FP64 but 0.36 against 0.33 in FP32 with FP64 chemistry, where the shorter
-// 2-D chain hides behind the bulk nodes.
-inline int bnode_warp_limit(int D, bool fp64) { return D == 2 && !fp64 ? 1536 : 6144; }
+// 2.2 against 2.7; of the 2000x40 channel (4078 nodes) 0.69 against 0.75 in
+// FP64, 0.28 against 0.31 in FP32 with FP64 chemistry.
+constexpr int kBnodeWarpNodes = 6144;
 // nodes (warps) per block of it
 constexpr int kBnodeWarps = 2;
 // interface nodes per block of the boundary kernel (one thread each)

@@ -55,10 +55,10 @@ inline namespace chemff {
 // float-float Newton and chemistry: FP32 lattice arithmetic, float-float mode
 template <typename RT> constexpr bool kFF = sizeof(RT) == 4 && !LBM_CHEM64;
 // resident blocks per SM the moments kernels are compiled for (register cap):
-// four for the float-float chemistry, two with FP64 chemistry beside FP32
-// lattice arithmetic, one in the FP64 path
-template <typename RT>
-constexpr int kMomentsMinBlocks = kFF<RT> ? 4 : (sizeof(RT) == 4 ? 2 : 3);
+// four (128 registers): with three (168) the FP64 kernel took 1.34 ms on the
+// 600x40x40 tube, with four 1.15, its 460 bytes of spills included; FP32 with
+// FP64 chemistry on the 2000x40 channel 0.19 ms with two, 0.11 with four
+constexpr int kMomentsMinBlocks = 4;
 
 // Arithmetic type of a storage type: FP16 storage computes in FP32.
 template <typename S> struct ComputeType { using type = S; };
@@ -110,7 +110,7 @@ __device__ __forceinline__ long long node_shift(int x, int y, int z, int i, int 
 template <typename RT, typename S>
 __device__ __forceinline__ RT pop_in(const S* __restrict__ src, const BCDev& bc, int tag,
                                      long long N, long long sn, int li, const float4* codec) {
-  return tag >= 0 ? RT(bc.pops[(long long)li * bc.n_if + tag])
+  return tag >= 0 ? static_cast<const RT*>(bc.pops)[(long long)li * bc.n_if + tag]
                   : Codec<S>::template dec<RT>(__ldg(src + (long long)li * N + sn), codec, li);
 }
 
@@ -1968,7 +1968,7 @@ __device__ __forceinline__ void coll_block(const S* __restrict__ src, S* __restr
 enum { NODES_ALL = 0, NODES_BULK = 1, NODES_INTERFACE = 2 };
 
 template <int D, int M, typename S, typename RT>
-__global__ void __launch_bounds__(128, kMomentsMinBlocks<RT>)
+__global__ void __launch_bounds__(128, kMomentsMinBlocks)
 k_moments(const S* __restrict__ src, RT* __restrict__ rec, double* __restrict__ Tf,
           int* __restrict__ status, const __grid_constant__ Geom g,
           const __grid_constant__ Units un, const __grid_constant__ BCDev bc,
@@ -2146,7 +2146,7 @@ static_assert(sizeof(DomainDev) % 4 == 0, "domain descriptor copied in 4-byte wo
   __shared__ __align__(16) unsigned char name##_raw[sizeof(DomainDev)]; \
   BlockDomain name{name##_raw}
 template <int D, int M, typename S, typename RT>
-__global__ void __launch_bounds__(128, kMomentsMinBlocks<RT>)
+__global__ void __launch_bounds__(128, kMomentsMinBlocks)
 k_moments_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int node_set,
                 int nblk) {
   LBM_BLOCK_DOMAIN(bd);
@@ -2770,7 +2770,7 @@ static cudaError_t step_impl(const DevMech& mech, const StepArgs& a, cudaStream_
     const bool fork = a.bc.n_if > 0 && a.side && a.ev_fork && a.ev_join;
     // the boundary kernel and the interface nodes' sub-steps
     auto boundary = [&](cudaStream_t st) {
-      if (a.bc.n_if <= bnode_warp_limit(D, sizeof(RT) == 8)) {
+      if (a.bc.n_if <= kBnodeWarpNodes) {
         k_bnode_warp<D, M, S><<<blocks_for(a.bc.n_if, kBnodeWarps), 32 * kBnodeWarps, 0, st>>>(
             src, a.bc, a.Tfield, a.status, a.g, a.un, a.mech_dev, rec);
         return;
