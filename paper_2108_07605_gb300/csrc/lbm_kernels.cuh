@@ -1656,34 +1656,11 @@ __device__ __forceinline__ void prep_body(const RT* __restrict__ rec,
 
 constexpr int kCollNodes = kCollNodesPerBlock;   // nodes per block of k_coll (the lanes)
 constexpr int kCollTPN = 9;      // threads per node (warps per block)
+constexpr int kColl32Blocks = 3; // FP32 blocks per SM the registers are held to
 
 // shared-memory entries per node of k_coll: parameters, energy factors,
 // species axis-factor tables
 template <int D, int M, typename RT> constexpr int coll_smem_entries();
-
-// Parameters of node j of the block, field f at s[f * kCollNodes + j].
-template <int D, int M, typename RT> struct SmemPar {
-  using CP = CPar<D, M>;
-  static constexpr int AF = CP::NF, BF = CP::NF + 3 * D, TAB = CP::NF + 6 * D;
-  const RT* s;
-  int j;
-  __device__ RT get(int f) const { return s[f * kCollNodes + j]; }
-  __device__ RT rho() const { return get(CP::RHO); }
-  __device__ RT om() const { return get(CP::OM); }
-  __device__ RT U() const { return get(CP::UL); }
-  __device__ RT u(int d) const { return get(CP::U + d); }
-  __device__ RT Pex(int d) const { return get(CP::PEX + d); }
-  __device__ RT W(int d) const { return get(CP::W + d); }
-  __device__ RT rs(int a) const { return get(CP::RS + a); }
-  __device__ RT cF(int a) const { return get(CP::CF + a); }
-  __device__ RT om1(int a) const { return get(CP::OM1 + a); }
-  __device__ RT hh(int a) const { return get(CP::HH + a); }
-  __device__ RT Af(int d, int c) const { return get(AF + d * 3 + c + 1); }
-  __device__ RT Bf(int d, int c) const { return get(BF + d * 3 + c + 1); }
-  __device__ RT sp(int set, int b, int d, int c) const {
-    return get(TAB + ((set * M + b) * D + d) * 3 + c + 1);
-  }
-};
 
 // Layout of k_coll's shared memory in FP64 (8-byte entries per node): the
 // parameters, the energy factors, the FP64 axis factors E of every species'
@@ -1701,8 +1678,20 @@ template <int D, int M> struct Coll64 {
   // first of a pair: x: -rho s(c), then -rho t(c); y, z: e(c), then t(c)
   static constexpr int f(int b, int d, int c) { return F + (b * D + d) * 6 + c + 1; }
 };
+// ... and in FP32 (4-byte entries per node): per axis d and c the species' axis
+// factors e of psi(u, theta_b) and s of psi(u + V_b, theta_b) (x: times rho_b, and
+// e times hh_b), the factors of the extended equilibrium and the energy
+// factors, then the species coefficients cF and 1 - 2 beta and the scalars.
+template <int D, int M> struct Coll32 {
+  static constexpr int E = 0, S = E + D * 3 * M, H = S + D * 3 * M;
+  static constexpr int EX = H + 3 * M, AF = EX + 3 * D, BF = AF + 3 * D;
+  static constexpr int CF = BF + 3 * D, OM1 = CF + M - 1;
+  static constexpr int RHO = OM1 + M - 1, OM = RHO + 1, U = OM + 1, W = U + 1;
+  static constexpr int N = W + D;
+  static constexpr int f(int b, int d, int c) { return (d * 3 + c + 1) * M + b; }
+};
 template <int D, int M, typename RT> constexpr int coll_smem_entries() {
-  return sizeof(RT) == 8 ? Coll64<D, M>::N : CPar<D, M>::NF + 6 * D + 2 * M * D * 3;
+  return sizeof(RT) == 8 ? Coll64<D, M>::N : Coll32<D, M>::N;
 }
 
 // The FP64 collision of one block of TPN warps, 32 nodes (lane = node), the
@@ -1877,6 +1866,13 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
 // kCollNodes.  The Q directions, taken in the order k = 0 .. Q - 1 with
 // direction (k / NZ) + 9 (k % NZ) (NZ = 3 in 3D: the directions of one
 // (c_x, c_y) pair in a row), are dealt to the warps in contiguous chunks.
+//
+// FP32 lattice arithmetic: bound by instruction issue (of 744 instructions per
+// direction and warp, most formed addresses and shared (c_x, c_y) products
+// again; now ~250), then by HBM.  The products with rho_b, hh_b and of x and y
+// are taken once per (c_x, c_y) pair, a species update is two multiply-adds
+// beside its Stefan-Maxwell sum, and every lattice's address is the
+// direction's plus a constant stride.
 template <int D, int M, typename S, typename RT, int TPN = kCollTPN>
 __device__ __forceinline__ void coll_block(const S* __restrict__ src, S* __restrict__ dst,
                                            const RT* __restrict__ cp, const Geom& g,
@@ -1885,77 +1881,161 @@ __device__ __forceinline__ void coll_block(const S* __restrict__ src, S* __restr
   if constexpr (sizeof(RT) == 8) {
     coll_block64<D, M, S, TPN>(src, dst, cp, g, bc, mech, n0, sm);
   } else {
-  using CP = CPar<D, M>;
-  using SP = SmemPar<D, M, RT>;
-  constexpr int Q = Lat<D>::Q;
-  constexpr int NT = 2 * M * D * 3;
-  const long long N = g.N;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const long long n = n0 + lane;
-  const int tag = n < N ? (bc.tag ? bc.tag[n] : TAG_BULK) : TAG_SOLID;
-  const bool valid = tag != TAG_SOLID;
-  for (int f = w; f < CP::NF; f += TPN)
-    sm[f * kCollNodes + lane] = valid ? __ldcg(cp + f * N + n) : RT(0);
-  __syncthreads();
-  if (valid) {
-    if (w == 0) {
-      RT u[D], Af[D][3], Bf[D][3];
+    using CP = CPar<D, M>;
+    using T = Coll32<D, M>;
+    constexpr int Q = Lat<D>::Q, CN = kCollNodes;
+    const long long N = g.N;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long n = n0 + lane;
+    const int tag = n < N ? (bc.tag ? bc.tag[n] : TAG_BULK) : TAG_SOLID;
+    const bool valid = tag != TAG_SOLID;
+    RT* const s = sm + lane;
+    const int x = (int)(n % g.nx);
+    const int y = (int)((n / g.nx) % g.ny);
+    const int z = (int)(n / ((long long)g.nx * g.ny));
+    constexpr int NZ = D == 3 ? 3 : 1;
+    constexpr int CH = (Q + TPN - 1) / TPN;
+    const int k0 = w * CH, k1 = min(k0 + CH, Q);
+    // populations entering direction i of lattice l (pop_in)
+    const long long ls = (long long)Q * N;              // stride of a lattice
+    auto load = [&](long long sn, int i, RT (&fin)[M + 1]) {
+      if (tag >= 0) {
+        const RT* p = static_cast<const RT*>(bc.pops) + (long long)i * bc.n_if + tag;
+        const long long st = (long long)Q * bc.n_if;
 #pragma unroll
-      for (int d = 0; d < D; ++d) u[d] = sm[(CP::U + d) * kCollNodes + lane];
-      energy_factors<D, RT>(u, sm[CP::THETA * kCollNodes + lane], Af, Bf);
+        for (int l = 0; l <= M; ++l, p += st) fin[l] = *p;
+      } else {
+        const S* p = src + (long long)i * N + sn;
 #pragma unroll
-      for (int d = 0; d < D; ++d)
+        for (int l = 0; l <= M; ++l, p += ls)
+          fin[l] = Codec<S>::template dec<RT>(__ldg(p), g.codec, l * Q + i);
+      }
+    };
+    RT fin[M + 1];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          sm[(SP::AF + d * 3 + k) * kCollNodes + lane] = Af[d][k];
-          sm[(SP::BF + d * 3 + k) * kCollNodes + lane] = Bf[d][k];
+    for (int l = 0; l <= M; ++l) fin[l] = RT(0);
+    if (valid) {
+      // the first direction's populations are in flight while the block's
+      // tables are built
+      if (k0 < k1) {
+        const int i = k0 / NZ + 9 * (k0 % NZ);
+        load(node_shift<D>(x, y, z, i, -1, g), i, fin);
+      }
+      auto P = [&](int f) { return __ldcg(cp + (long long)f * N + n); };
+      for (int e = w; e < M * D; e += TPN) {
+        const int b = e / D, d = e % D;
+        const RT u = P(CP::U + d), th = P(CP::TH + b), us = u + P(CP::V + b * D + d);
+        const RT pe = th + u * u, ps = th + us * us;
+        const RT r = d == 0 ? P(CP::RS + b) : RT(1);
+        const RT ee[3] = {RT(0.5) * (pe - u), RT(1) - pe, RT(0.5) * (pe + u)};
+        const RT ss[3] = {RT(0.5) * (ps - us), RT(1) - ps, RT(0.5) * (ps + us)};
+        const RT hh = d == 0 && b < M - 1 ? P(CP::HH + b) : RT(0);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          s[(T::E + T::f(b, d, c - 1)) * CN] = r * ee[c];
+          s[(T::S + T::f(b, d, c - 1)) * CN] = r * ss[c];
+          if (d == 0) s[(T::H + c * M + b) * CN] = hh * ee[c];
         }
-    }
-    for (int e = w; e < NT; e += TPN) {
-      const int c = e % 3 - 1;
-      const int d = (e / 3) % D;
-      const int b = (e / (3 * D)) % M;
-      const int set = e / (3 * D * M);
-      const RT ud = sm[(CP::U + d) * kCollNodes + lane];
-      const RT xs = set ? ud + sm[(CP::V + b * D + d) * kCollNodes + lane] : ud;
-      const RT Ps = sm[(CP::TH + b) * kCollNodes + lane] + xs * xs;
-      sm[(SP::TAB + e) * kCollNodes + lane] =
-          c == 0 ? RT(1) - Ps : (c > 0 ? RT(0.5) * (Ps + xs) : RT(0.5) * (Ps - xs));
-    }
-  }
-  __syncthreads();
-  if (!valid) return;
-  const SP ps{sm, lane};
-  const int x = (int)(n % g.nx);
-  const int y = (int)((n / g.nx) % g.ny);
-  const int z = (int)(n / ((long long)g.nx * g.ny));
-  // software pipeline: the next direction's populations are in flight while
-  // this one collides.  The (c_x, c_y) part is formed per direction, which
-  // keeps k_coll within its 56-register budget.
-  constexpr int NZ = D == 3 ? 3 : 1;
-  constexpr int CH = (Q + TPN - 1) / TPN;
-  const int k0 = w * CH, k1 = min(k0 + CH, Q);
-  if (k0 >= k1) return;
-  RT fa[M + 1], fb[M + 1];
-  int i = k0 / NZ + 9 * (k0 % NZ);
-  load_direction<D, M, S, RT>(src, bc, tag, N, node_shift<D>(x, y, z, i, -1, g), i, g.codec, fa);
-#pragma unroll 1
-  for (int k = k0; k < k1; ++k) {
-    const int inext = k + 1 < k1 ? (k + 1) / NZ + 9 * ((k + 1) % NZ) : -1;
-    if (inext >= 0)
-      load_direction<D, M, S, RT>(src, bc, tag, N, node_shift<D>(x, y, z, inext, -1, g), inext,
-                                  g.codec, fb);
-    const int j = k / NZ;
-    XYPart<D, M, RT> h;
-    xy_part<D, M, RT>(ps, cvel(j, 0), cvel(j, 1), h);
-    collide_direction<D, M, S, RT>(ps, h, i, fa, dst, N, n, mech, g.codec);
+      }
+      if (w == TPN - 1) {
+        RT u[D], Af[D][3], Bf[D][3];
 #pragma unroll
-    for (int l = 0; l <= M; ++l) fa[l] = fb[l];
-    i = inext;
-  }
+        for (int d = 0; d < D; ++d) u[d] = P(CP::U + d);
+        energy_factors<D, RT>(u, P(CP::THETA), Af, Bf);
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          const RT px = P(CP::PEX + d);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            s[(T::AF + d * 3 + k) * CN] = Af[d][k];
+            s[(T::BF + d * 3 + k) * CN] = Bf[d][k];
+            s[(T::EX + d * 3 + k) * CN] = psi1<RT>(k - 1, u[d], px);
+          }
+          s[(T::W + d) * CN] = P(CP::W + d);
+        }
+        s[T::RHO * CN] = P(CP::RHO);
+        s[T::OM * CN] = P(CP::OM);
+        s[T::U * CN] = P(CP::UL);
+      }
+      for (int a = w; a < M - 1; a += TPN) {
+        s[(T::CF + a) * CN] = P(CP::CF + a);
+        s[(T::OM1 + a) * CN] = P(CP::OM1 + a);
+      }
+    }
+    __syncthreads();
+    if (!valid || k0 >= k1) return;
+    RT re[M], rss[M], eh[M - 1];     // rho_b e_x e_y, rho_b s_x s_y, hh_a e_x e_y
+    RT fxy = RT(0), gP = RT(0), gQ = RT(0);
+    const RT rho = s[T::RHO * CN], om = s[T::OM * CN];
+    int jcur = -1;
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+      const int j = k / NZ, i = j + 9 * (k % NZ);
+      const int cx = cvel(j, 0), cy = cvel(j, 1), cz = D == 3 ? k % NZ - 1 : 0;
+      if (j != jcur) {
+        jcur = j;
+        const RT *ex = s + (T::E + T::f(0, 0, cx)) * CN, *ey = s + (T::E + T::f(0, 1, cy)) * CN;
+        const RT *sx = s + (T::S + T::f(0, 0, cx)) * CN, *sy = s + (T::S + T::f(0, 1, cy)) * CN;
+        const RT* hx = s + (T::H + (cx + 1) * M) * CN;
+#pragma unroll
+        for (int b = 0; b < M; ++b) {
+          const RT e = ey[b * CN];
+          re[b] = ex[b * CN] * e;
+          rss[b] = sx[b * CN] * sy[b * CN];
+          if (b < M - 1) eh[b] = hx[b * CN] * e;
+        }
+        fxy = rho * s[(T::EX + cx + 1) * CN] * s[(T::EX + 3 + cy + 1) * CN];
+        const RT ax = s[(T::AF + cx + 1) * CN], ay = s[(T::AF + 3 + cy + 1) * CN];
+        gP = ax * ay;
+        gQ = s[T::U * CN] * gP + s[(T::BF + cx + 1) * CN] * ay + ax * s[(T::BF + 3 + cy + 1) * CN];
+      }
+      RT dd[M], pe[M - 1];
+      if constexpr (D == 3) {
+        const RT *ez = s + (T::E + T::f(0, 2, cz)) * CN, *sz = s + (T::S + T::f(0, 2, cz)) * CN;
+#pragma unroll
+        for (int b = 0; b < M; ++b) {
+          const RT e = ez[b * CN];
+          dd[b] = re[b] * e - rss[b] * sz[b * CN];
+          if (b < M - 1) pe[b] = eh[b] * e;
+        }
+      } else {
+#pragma unroll
+        for (int b = 0; b < M; ++b) {
+          dd[b] = re[b] - rss[b];
+          if (b < M - 1) pe[b] = eh[b];
+        }
+      }
+      S* out = dst + (long long)i * N + n;
+      const RT f = fin[M - 1], gv = fin[M];
+#pragma unroll
+      for (int a = 0; a < M - 1; ++a) {
+        RT F = RT(0);
+#pragma unroll
+        for (int b = 0; b < M; ++b)
+          if (b != a) F += kcoef<RT>(mech, a, b) * dd[b];
+        const RT fn = fin[a] * s[(T::OM1 + a) * CN] + (pe[a] + s[(T::CF + a) * CN] * F);
+        *out = Codec<S>::enc(fn, g.codec, a * Q + i);
+        out += ls;
+      }
+      // the next direction's populations (the last direction's again)
+      const int kn = min(k + 1, k1 - 1), in = kn / NZ + 9 * (kn % NZ);
+      load(node_shift<D>(x, y, z, in, -1, g), in, fin);
+      RT fex = fxy, geq = gQ;
+      if constexpr (D == 3) {
+        fex *= s[(T::EX + 6 + cz + 1) * CN];
+        geq = s[(T::AF + 6 + cz + 1) * CN] * gQ + gP * s[(T::BF + 6 + cz + 1) * CN];
+      }
+      *out = Codec<S>::enc(f + om * (fex - f), g.codec, (M - 1) * Q + i);
+      RT gn = gv + om * (rho * geq - gv);
+      if (csq(i, D) == 1) {
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+          if (cvel(i, d) != 0) gn += (cvel(i, d) > 0 ? RT(0.5) : RT(-0.5)) * s[(T::W + d) * CN];
+      }
+      out[ls] = Codec<S>::enc(gn, g.codec, M * Q + i);
+    }
   }
 }
-
 
 #include "lbm_bnode.cuh"
 
@@ -2053,7 +2133,7 @@ k_prep(const RT* __restrict__ rec, const double* __restrict__ Tf, RT* __restrict
 // FP32: four 288-thread blocks per SM (at most 56 registers), so a grid of
 // the 16k-node flame fits the GPU in one wave
 template <int D, int M, typename S, typename RT>
-__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? 4 : 2)
+__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? kColl32Blocks : 2)
 k_coll(const S* __restrict__ src, S* __restrict__ dst, const RT* __restrict__ cp,
        const __grid_constant__ Geom g, const __grid_constant__ BCDev bc,
        const __grid_constant__ DevMech mech) {
@@ -2231,7 +2311,7 @@ k_prep_batch(const DomainDev* __restrict__ doms, int ndom, int nblk) {
 }
 
 template <int D, int M, typename S, typename RT>
-__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? 4 : 2)
+__global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? kColl32Blocks : 2)
 k_coll_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   extern __shared__ __align__(16) unsigned char coll_raw[];
