@@ -153,23 +153,20 @@ __device__ __forceinline__ constexpr int pidx(int a, int b) {
 // included), rho, ER = E / rho and usqR = |u|^2 of the moments, T_0 = T
 // their temperature; dr receives the increments drho_a (a < M - 1).  The
 // temperature solve in float-float (mixed path) or FP64; the rate arrays live
-// in the thread's shared-memory slice (kDynChem: chem_slice, the block's
-// slices of chem_slice_bytes in dynamic shared memory; else a static array of
-// the calling kernel).  Blocks of kChemThreads threads.
+// in the thread's slice of shared memory (chem_slice: the block's slices,
+// chem_slice_bytes).  Blocks of at most kChemThreads threads.
 template <int M>
 __device__ __forceinline__ ff* chem_static_slice() {
   __shared__ __align__(8) unsigned char chem_raw[chem_slice_bytes<M>()];
   return reinterpret_cast<ff*>(chem_raw);
 }
 
-template <int M, typename RT, bool kDynChem>
+template <int M, typename RT>
 __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, RT usqR,
                                               double T, const Units& un, const DevMech& mech,
                                               int* __restrict__ status, void* chem_slice,
                                               RT (&dr)[M - 1]) {
-  ff* Cs;
-  if constexpr (kDynChem) Cs = static_cast<ff*>(chem_slice) + threadIdx.x;
-  else Cs = chem_static_slice<M>() + threadIdx.x;
+  ff* const Cs = static_cast<ff*>(chem_slice) + threadIdx.x;
   ff w[M];
   if constexpr (kFF<RT>) {
     const ff Uphys = (ff(ER) + ff(-0.5f * usqR)) * un.c2_f;
@@ -224,454 +221,6 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
 }
 
 // ---------------------------------------------------------------------------
-// The node's record from its population sums (Sec. 2.1, Sec. 3.1-3.2, Sec.
-// 3.7 slaving): fields, temperature by Newton from the node's previous T, and
-// the reaction sub-steps.  FP32 lattice arithmetic.
-template <int D, int M, typename RT, bool kDynChem = false>
-__device__ __forceinline__ void moments_finish(RT* __restrict__ rec, double* __restrict__ Tf,
-                                               int* __restrict__ status, long long N,
-                                               const Units& un, const DevMech& mech,
-                                               long long n, RT rho, RT rhoE,
-                                               const RT (&j)[D], const RT (&q)[D],
-                                               const RT (&P)[Lat<D>::NP], RT (&rs)[M],
-                                               RT (&js)[M][D], void* chem_slice) {
-  constexpr int NP = Lat<D>::NP;
-  using RC = Rec<D, M>;
-  // slaved species M (Eq. strongest)
-  rs[M - 1] = rho;
-#pragma unroll
-  for (int d = 0; d < D; ++d) js[M - 1][d] = j[d];
-#pragma unroll
-  for (int a = 0; a < M - 1; ++a) {
-    rs[M - 1] -= rs[a];
-#pragma unroll
-    for (int d = 0; d < D; ++d) js[M - 1][d] -= js[a][d];
-  }
-  // node fields in the lattice type; FP64 only for the temperature solve
-  const RT inv_rho = RT(1) / rho;
-  RT uR[D], YR[M], usqR = RT(0);
-#pragma unroll
-  for (int d = 0; d < D; ++d) { uR[d] = j[d] * inv_rho; usqR += uR[d] * uR[d]; }
-#pragma unroll
-  for (int a = 0; a < M; ++a) YR[a] = rs[a] * inv_rho;
-  const RT ER = rhoE * inv_rho;
-  bool ok;
-  double T;
-  RT thR, H[4];
-  if constexpr (kFF<RT>) {
-    // mixed path: the temperature solve in float-float
-    ff Yf[M], c[4];
-    float Rm = 0.f;
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-      Yf[a] = ff(YR[a]);
-      Rm += YR[a] * mech.inv_mm_s[a];
-    }
-    const ff U = (ff(ER) + ff(-0.5f * usqR)) * un.c2_f;
-    const ff Tx = newton_T_ff<M>(mech, Yf, U, ff_from_double(__ldcg(Tf + n)), un.newton_max_iter,
-                                 un.newton_rtol_f, ok, c);
-    T = ff_to_double(Tx);
-    thR = Rm * float(R_U) * Tx.hi * un.inv_c2_s;
-    enthalpy_poly(c, Rm, un, H);
-  } else {
-    double Y[M], c[4];
-#pragma unroll
-    for (int a = 0; a < M; ++a) Y[a] = double(YR[a]);
-    const double U = (double(ER) - 0.5 * double(usqR)) * un.c * un.c;
-    T = newton_T<M>(mech, Y, U, __ldcg(Tf + n), un.newton_max_iter, un.newton_rtol, ok, c);
-    float Rm = 0.f;
-#pragma unroll
-    for (int a = 0; a < M; ++a) Rm += float(YR[a]) * mech.inv_mm_s[a];
-    thR = RT(Rm * float(R_U) * float(T) * un.inv_c2_s);
-    enthalpy_poly(c, RT(Rm), un, H);
-  }
-  if (!ok) atomicOr(status, ST_NEWTON);
-  if (!(rho > RT(0)) || !isfinite(double(rho)) || !isfinite(T)) atomicOr(status, ST_NONFINITE);
-  Tf[n] = T;
-
-  // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3): a zero-dimensional
-  // reactor per node from its post-stream species densities; T_0 is the T
-  // just solved.  The increments drho_a (a < M) go to the record.
-  RT dr[M - 1];
-  node_substeps<M, RT, kDynChem>(rs, rho, ER, usqR, T, un, mech, status, chem_slice, dr);
-#pragma unroll
-  for (int a = 0; a < M - 1; ++a) rec[(RC::DRHO + a) * N + n] = dr[a];
-
-  rec[RC::RHO * N + n] = rho;
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    rec[(RC::U + d) * N + n] = uR[d];
-    rec[(RC::Z + d) * N + n] = flux_less_work<D, RT>(d, uR, q, P);
-    rec[(RC::PHI + d) * N + n] = rho * uR[d] * (RT(1) - RT(3) * thR) - rho * uR[d] * uR[d] * uR[d];
-  }
-  rec[RC::E * N + n] = ER;
-  rec[RC::TH * N + n] = thR;
-  rec[RC::LNT * N + n] = ln_T0(RT(T));
-#pragma unroll
-  for (int k = 0; k < 4; ++k) rec[(RC::H + k) * N + n] = H[k];
-#pragma unroll
-  for (int a = 0; a < M; ++a) {
-    rec[(RC::Y + a) * N + n] = YR[a];
-    // where defined, |j_a| < rho_a, so the quotient lies in (-1, 1) even when
-    // rho_a is denormal (its reciprocal would overflow)
-    const bool tiny = species_velocity_undefined<D, RT>(rs[a], js[a]);
-#pragma unroll
-    for (int d = 0; d < D; ++d)
-      rec[(RC::US + a * D + d) * N + n] = tiny ? RT(0) : js[a][d] / rs[a] - uR[d];
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Shared memory of the FP64 moments: per thread the chemistry's slice (C, W),
-// then the concentrations and the summed rates in FP64 (M each).
-template <int M> constexpr size_t moments64_bytes() {
-  return chem_slice_bytes<M>() + (size_t)2 * M * kChemThreads * sizeof(double);
-}
-template <int M>
-__device__ __forceinline__ void* moments64_static() {
-  __shared__ __align__(16) unsigned char mom_raw[moments64_bytes<M>()];
-  return mom_raw;
-}
-
-// The moments, record and reaction sub-steps of bulk node n in FP64, one
-// thread per node, lattice by lattice.
-//
-// What bounds it is the count of FP64 instructions (75 cycles of an SM
-// quarter each), then their latency.  So: a lattice's 27 populations are
-// loaded together (27 loads in flight; three before) and summed in fixed point
-// (fix_of), as are the remainders of the slaved species; u_a - u, which only
-// becomes a diffusion velocity, is a float-float quotient of the FP64 j_a -
-// rho_a u; comparisons are made on the bit patterns; a sub-step's energy
-// coefficients are those of the moments plus float-float increments.  ~500
-// FP64 instructions per node remain of ~1500.  The loop over the lattices is
-// rolled: its sums need no register arrays (so more warps fit) and the code
-// stays in the instruction cache.
-template <int D, int M, typename S>
-__device__ __forceinline__ void moments_body64(const S* __restrict__ src,
-                                               double* __restrict__ rec,
-                                               double* __restrict__ Tf,
-                                               int* __restrict__ status, const Geom& g,
-                                               const Units& un, const BCDev& bc,
-                                               const DevMech& mech, long long n, void* smem) {
-  constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP, NZ = Q / 9;
-  using RC = Rec<D, M>;
-  const long long N = g.N;
-  if (n >= N) return;
-  if (bc.tag && bc.tag[n] == TAG_SOLID) return;
-  ff* const Cs = static_cast<ff*>(smem) + threadIdx.x;
-  ff* const Ws = Cs + M * kChemThreads;
-  double* const Cd = static_cast<double*>(smem) + 2 * M * kChemThreads + threadIdx.x;
-  double* const Wd = Cd + M * kChemThreads;
-  const int x = (int)(n % g.nx);
-  const int y = (int)((n / g.nx) % g.ny);
-  const int z = (int)(n / ((long long)g.nx * g.ny));
-  // pull sources: x of c_x = -1, 0, 1 and the offsets of (c_y, c_z)
-  const int xs[3] = {wrap1(x + 1, g.nx), x, wrap1(x - 1, g.nx)};
-  long long row[Q / 3];
-#pragma unroll
-  for (int r = 0; r < Q / 3; ++r)
-    row[r] = (long long)g.nx *
-             (wrap1(y - (r % 3 - 1), g.ny) +
-              (long long)g.ny * (D == 3 ? wrap1(z - (r / 3 - 1), g.nz) : 0));
-
-  double rho = 0.0, inv_rho = 0.0, u[D], usq = 0.0, ER = 0.0, Z[D];
-  double Rm = 0.0, cU[4] = {0.0, 0.0, 0.0, 0.0};   // sum Y/m, energy polynomial
-  // the slaved species' sums: the f lattice's minus the others', in fixed
-  // point at exponent eR (momenta: eR - 6); ex: sums that do not fit there
-  // (beyond any physical state)
-  long long rem[1 + D];
-  double ex[1 + D];
-  int eR = 0;
-#pragma unroll
-  for (int d = 0; d <= D; ++d) { rem[d] = 0; ex[d] = 0.0; }
-#pragma unroll
-  for (int d = 0; d < D; ++d) u[d] = Z[d] = 0.0;
-
-  // species a's state from its sums: record, concentration, energy polynomial
-  auto species = [&](int a, double rs, const double (&js)[D]) {
-    const double Y = rs * inv_rho;
-    rec[(RC::Y + a) * N + n] = Y;
-    Rm = fma(Y, mech.inv_mm[a], Rm);
-    cU[0] = fma(Y, mech.u0[a], cU[0]);
-    cU[1] = fma(Y, mech.u1[a], cU[1]);
-    cU[2] = fma(Y, mech.u2[a], cU[2]);
-    cU[3] = fma(Y, mech.u3[a], cU[3]);
-    const double c = rs * mech.inv_mm[a];
-    Cd[a * kChemThreads] = c;
-    Wd[a * kChemThreads] = 0.0;
-    Cs[a * kChemThreads] = ff_of_double(c);
-    // reading R5 on the bit patterns (positive doubles order as integers; a
-    // negative rho_a is below every |j_a|)
-    const long long rb = __double_as_longlong(rs);
-    bool undef = rb <= __double_as_longlong(RHO_TINY);
-#pragma unroll
-    for (int d = 0; d < D; ++d)
-      undef |= (__double_as_longlong(js[d]) & 0x7fffffffffffffffLL) >= rb;
-    // (j_a - rho_a u) / rho_a, both scaled by rho_a's power of two
-    const int de = 1023 - ((__double2hiint(rs) >> 20) & 0x7ff);
-    const ff ir = ff_rcp(ff_of_double(
-        __hiloint2double((__double2hiint(rs) & 0x800fffff) | 0x3ff00000, __double2loint(rs))));
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const double w = fma(-rs, u[d], js[d]);
-      const int h = __double2hiint(w), ew = ((h >> 20) & 0x7ff) + de;
-      const double ws = ew <= 0 || undef
-                            ? 0.0
-                            : __hiloint2double((h & 0x800fffff) | (ew << 20), __double2loint(w));
-      rec[(RC::US + a * D + d) * N + n] = ff_pack(ff_of_double(ws) * ir);
-    }
-  };
-
-#pragma unroll 1
-  for (int it = 0; it <= M; ++it) {
-    const int l = it == 0 ? M - 1 : (it == 1 ? M : it - 2);   // f, g, the species
-    double v[Q];
-    int e = 0;
-    const S* pl = src + (long long)l * Q * N;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) v[i] = __ldg(pl + (long long)i * N + row[i / 3] + xs[i % 3]);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) e = max(e, fix_exponent(v[i]));
-    Fix sum, sj[D], sP[NP];
-#pragma unroll
-    for (int pz = 0; pz < NZ; ++pz) {
-      Fix ps, pd, py, pxy;
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const int i = 9 * pz + 3 * r;
-        const Fix f0 = fix_of(v[i], e), f1 = fix_of(v[i + 1], e), f2 = fix_of(v[i + 2], e);
-        const Fix sx = f0 + f2, sr = sx + f1, dx = f2 - f0;
-        ps = ps + sr;
-        pd = pd + dx;
-        sP[pidx<D>(0, 0)] = sP[pidx<D>(0, 0)] + sx;
-        if (r != 1) {
-          py = r == 2 ? py + sr : py - sr;
-          pxy = r == 2 ? pxy + dx : pxy - dx;
-          sP[pidx<D>(1, 1)] = sP[pidx<D>(1, 1)] + sr;
-        }
-      }
-      sum = sum + ps;
-      sj[0] = sj[0] + pd;
-      sj[1] = sj[1] + py;
-      sP[pidx<D>(0, 1)] = sP[pidx<D>(0, 1)] + pxy;
-      if constexpr (D == 3) {
-        if (pz != 1) {
-          sj[2] = pz == 2 ? sj[2] + ps : sj[2] - ps;
-          sP[pidx<D>(2, 2)] = sP[pidx<D>(2, 2)] + ps;
-          sP[pidx<D>(0, 2)] = pz == 2 ? sP[pidx<D>(0, 2)] + pd : sP[pidx<D>(0, 2)] - pd;
-          sP[pidx<D>(1, 2)] = pz == 2 ? sP[pidx<D>(1, 2)] + py : sP[pidx<D>(1, 2)] - py;
-        }
-      }
-    }
-    const FixSum t0 = fix_sum(sum, e);
-    const double s0 = double_of_fix(t0);
-    FixSum t1[D];
-    double s1[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      t1[d] = fix_sum(sj[d], e);
-      s1[d] = double_of_fix(t1[d]);
-    }
-    if (it == 0) {
-      eR = e + 2;
-      rho = s0;
-      inv_rho = 1.0 / rho;
-      rec[RC::RHO * N + n] = rho;
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        u[d] = s1[d] * inv_rho;
-        usq = fma(u[d], u[d], usq);
-        rec[(RC::U + d) * N + n] = u[d];
-      }
-      double P[NP];
-#pragma unroll
-      for (int k = 0; k < NP; ++k) P[k] = double_of_fix(fix_sum(sP[k], e));
-#pragma unroll
-      for (int d = 0; d < D; ++d) Z[d] = flux_less_work<D, double>(d, u, Z, P);
-    } else if (it == 1) {
-      ER = s0 * inv_rho;
-      rec[RC::E * N + n] = ER;
-#pragma unroll
-      for (int d = 0; d < D; ++d) rec[(RC::Z + d) * N + n] = s1[d] + Z[d];
-    }
-    if (it != 1) {
-      const long long sg = it == 0 ? 1 : -1;
-      if (t0.e <= eR) rem[0] += sg * fix_down(t0.s, eR - t0.e);
-      else ex[0] += sg * s0;
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        if (t1[d].e <= eR - 6) rem[1 + d] += sg * fix_down(t1[d].s, eR - 6 - t1[d].e);
-        else ex[1 + d] += sg * s1[d];
-      }
-      if (it > 1) species(l, s0, s1);
-    }
-  }
-  {   // slaved species M (Eq. strongest)
-    double rs = double_of_fix(rem[0], eR), js[D];
-    if (ex[0] != 0.0) rs += ex[0];
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      js[d] = double_of_fix(rem[1 + d], eR - 6);
-      if (ex[1 + d] != 0.0) js[d] += ex[1 + d];
-    }
-    species(M - 1, rs, js);
-  }
-
-  // temperature (Eq. temperature) from the node's previous T
-  const double U = (ER - 0.5 * usq) * un.c * un.c;
-  bool ok;
-  const double T = newton_poly(cU, U, __ldcg(Tf + n), un.newton_max_iter, un.newton_rtol, ok);
-  if (!ok) atomicOr(status, ST_NEWTON);
-  if (!(rho > 0.0) || !isfinite(rho) || !isfinite(T)) atomicOr(status, ST_NONFINITE);
-  Tf[n] = T;
-  const double th = R_U * Rm * T * un.inv_c2, b3 = fma(-3.0, th, 1.0);    // 1 - 3 theta
-  double H[4];
-  enthalpy_poly(cU, Rm, un, H);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) rec[(RC::H + k) * N + n] = H[k];
-  rec[RC::TH * N + n] = th;
-#pragma unroll
-  for (int d = 0; d < D; ++d)
-    rec[(RC::PHI + d) * N + n] = rho * u[d] * fma(-u[d], u[d], b3);
-
-  // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3): a zero-dimensional
-  // reactor per node from its post-stream species densities; T_0 is the T just
-  // solved
-  double Ts = T;
-  ff dU[4];                              // increments of rho cU
-  const ff irho = ff_of_double(inv_rho);
-#pragma unroll 1
-  for (int s = 0; s < un.substeps; ++s) {
-    if (s > 0) {
-      double c[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) c[k] = cU[k] + double_of_ff(ff_norm(dU[k]) * irho);
-      bool oks;
-      Ts = newton_poly(c, U, Ts, un.newton_max_iter, un.newton_rtol, oks);
-      if (!oks) atomicOr(status, ST_NEWTON);
-    }
-#pragma unroll
-    for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
-    const TBasis<double> tb = tbasis(mech, Ts);
-    if (s == 0) rec[RC::LNT * N + n] = tb.lnT - LN_T_REF;
-    add_reactions<M>(mech, tb, Cs, Ws, 0, 1);
-    const bool last = s + 1 == un.substeps;
-#pragma unroll 1
-    for (int a = 0; a < M; ++a) {
-      const ff w = ff_norm(Ws[a * kChemThreads]);
-      const double wd = double_join(w);
-      Wd[a * kChemThreads] += wd;
-      if (last) continue;
-      const double c = fma(wd, un.dt_sub, Cd[a * kChemThreads]);
-      Cd[a * kChemThreads] = c;
-      Cs[a * kChemThreads] = ff_of_double(c);
-      const ff inc = w * un.dtmm_f[a];
-      ff_fma_acc(dU[0], inc, mech.u0_f[a]);
-      ff_fma_acc(dU[1], inc, mech.u1_f[a]);
-      ff_fma_acc(dU[2], inc, mech.u2_f[a]);
-      ff_fma_acc(dU[3], inc, mech.u3_f[a]);
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < M - 1; ++a)
-    rec[(RC::DRHO + a) * N + n] = Wd[a * kChemThreads] * un.dtmm[a];
-}
-
-// ---------------------------------------------------------------------------
-// Moments of the post-stream state + temperature (Sec. 2.1, Sec. 3.1-3.2,
-// Sec. 3.7 slaving, Sec. 4.1 pull streaming), and the reaction sub-steps.
-template <int D, int M, typename S, typename RT, bool kDynChem = false>
-__device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __restrict__ rec,
-                                             double* __restrict__ Tf, int* __restrict__ status,
-                                             const Geom& g, const Units& un, const BCDev& bc,
-                                             const DevMech& mech, long long n,
-                                             void* chem_slice = nullptr) {
-  if constexpr (sizeof(RT) == 8) {
-    if constexpr (!kDynChem) chem_slice = moments64_static<M>();
-    moments_body64<D, M>(src, rec, Tf, status, g, un, bc, mech, n, chem_slice);
-  } else {
-  constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP;
-  const long long N = g.N;
-  if (n >= N) return;
-  const int tag = bc.tag ? bc.tag[n] : TAG_BULK;
-  if (tag == TAG_SOLID) return;
-  const int x = (int)(n % g.nx);
-  const int y = (int)((n / g.nx) % g.ny);
-  const int z = (int)(n / ((long long)g.nx * g.ny));
-  const float4* codec = g.codec;
-
-  // sums in the lattice compute type RT
-  RT rho = RT(0), rhoE = RT(0), j[D], q[D], P[NP], rs[M], js[M][D];
-#pragma unroll
-  for (int d = 0; d < D; ++d) { j[d] = RT(0); q[d] = RT(0); }
-#pragma unroll
-  for (int k = 0; k < NP; ++k) P[k] = RT(0);
-#pragma unroll
-  for (int a = 0; a < M; ++a) {
-    rs[a] = RT(0);
-#pragma unroll
-    for (int d = 0; d < D; ++d) js[a][d] = RT(0);
-  }
-  // rows of three velocities (c_x = -1, 0, 1 at fixed c_y, c_z), rows
-  // rolled: the fully unrolled loop is ~27 copies of the body, whose
-  // instruction fetch dominates grids too small to keep many warps per SM.
-  // A row's populations enter through their sum s and difference d = f_+ -
-  // f_- (and f_+ + f_- for P_xx): sum_i c_ix f_i = sum_rows d,
-  // sum_i c_iy f_i = sum_rows c_y s, and so on.
-#pragma unroll 1
-  for (int r = 0; r < Q / 3; ++r) {
-    const RT cy = RT(r % 3 - 1), cz = RT(D == 3 ? r / 3 - 1 : 0);
-    const long long sn0 = node_shift<D>(x, y, z, 3 * r, -1, g);
-    const long long sn1 = node_shift<D>(x, y, z, 3 * r + 1, -1, g);
-    const long long sn2 = node_shift<D>(x, y, z, 3 * r + 2, -1, g);
-#pragma unroll
-    for (int a = 0; a < M - 1; ++a) {
-      const RT v0 = pop_in<RT>(src, bc, tag, N, sn0, a * Q + 3 * r, codec);
-      const RT v1 = pop_in<RT>(src, bc, tag, N, sn1, a * Q + 3 * r + 1, codec);
-      const RT v2 = pop_in<RT>(src, bc, tag, N, sn2, a * Q + 3 * r + 2, codec);
-      const RT sr = v0 + v1 + v2;
-      rs[a] += sr;
-      js[a][0] += v2 - v0;
-      js[a][1] += cy * sr;
-      if (D == 3) js[a][D - 1] += cz * sr;
-    }
-    {
-      const int l = M - 1;
-      const RT f0 = pop_in<RT>(src, bc, tag, N, sn0, l * Q + 3 * r, codec);
-      const RT f1 = pop_in<RT>(src, bc, tag, N, sn1, l * Q + 3 * r + 1, codec);
-      const RT f2 = pop_in<RT>(src, bc, tag, N, sn2, l * Q + 3 * r + 2, codec);
-      const RT sx = f0 + f2, sr = sx + f1, dx = f2 - f0;
-      rho += sr;
-      j[0] += dx;
-      j[1] += cy * sr;
-      P[pidx<D>(0, 0)] += sx;
-      P[pidx<D>(1, 1)] += (cy * cy) * sr;
-      P[pidx<D>(0, 1)] += cy * dx;
-      if constexpr (D == 3) {
-        j[2] += cz * sr;
-        P[pidx<D>(2, 2)] += (cz * cz) * sr;
-        P[pidx<D>(0, 2)] += cz * dx;
-        P[pidx<D>(1, 2)] += (cy * cz) * sr;
-      }
-    }
-    {
-      const int l = M;
-      const RT g0 = pop_in<RT>(src, bc, tag, N, sn0, l * Q + 3 * r, codec);
-      const RT g1 = pop_in<RT>(src, bc, tag, N, sn1, l * Q + 3 * r + 1, codec);
-      const RT g2 = pop_in<RT>(src, bc, tag, N, sn2, l * Q + 3 * r + 2, codec);
-      const RT sr = g0 + g1 + g2;
-      rhoE += sr;
-      q[0] += g2 - g0;
-      q[1] += cy * sr;
-      if (D == 3) q[D - 1] += cz * sr;
-    }
-  }
-  moments_finish<D, M, RT, kDynChem>(rec, Tf, status, N, un, mech, n, rho, rhoE, j, q, P, rs, js,
-                                     chem_slice);
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Reaction sub-steps with several lanes per node (Sec. 2.4 Eq. R3), for
 // grids too small to fill the GPU at one thread per node: the node's
 // reactions are dealt out over the lanes, which cuts the latency of a node's
@@ -691,6 +240,7 @@ template <> struct Chem<double> {
   __device__ static double inv(double x) { return 1.0 / x; }
   __device__ static double of(double v) { return v; }
   __device__ static double of_T(double T) { return T; }
+  __device__ static double of_ff(ff v) { return double_of_ff(v); }
   __device__ static ff concentration(const DevMech& m, int a, double r) {
     return ff_of_double(r * m.inv_mm[a]);
   }
@@ -706,6 +256,7 @@ template <> struct Chem<ff> {
   __device__ static ff inv(ff x) { return ff(1.f) / x; }
   __device__ static ff of(float v) { return ff(v); }
   __device__ static ff of_T(double T) { return ff_from_double(T); }
+  __device__ static ff of_ff(ff v) { return v; }
   __device__ static ff concentration(const DevMech& m, int a, ff r) { return r * m.inv_mm_f[a]; }
   __device__ static ff increment(const DevMech& m, const Units& u, int a, ff w) {
     return u.dt_sub_f * (w * m.mm_f[a]);
@@ -1007,6 +558,382 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
   for (int a = 0; a < M - 1; ++a) {
     if constexpr (kFF<RT>) put(RC::DRHO + a, (r[a] - r0[a]).hi);
     else put(RC::DRHO + a, RT(r[a] - r0[a]));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Shared memory of the moments kernels: per thread the chemistry's slice (C,
+// W), the sums of W over the sub-steps and, with FP64 chemistry, the
+// concentrations in FP64 (M entries of 8 bytes each).
+template <int M> constexpr size_t moments_bytes() {
+  return chem_slice_bytes<M>() + (size_t)2 * M * kChemThreads * sizeof(double);
+}
+template <int M>
+__device__ __forceinline__ void* moments_static() {
+  __shared__ __align__(16) unsigned char mom_raw[moments_bytes<M>()];
+  return mom_raw;
+}
+
+// Sums over a lattice's 27 (9) populations: density, momentum, momentum flux.
+// FP32: plain sums, row by row and plane by plane; FP64: fixed point.
+template <typename RT> struct SumType { using type = RT; };
+template <> struct SumType<double> { using type = Fix; };
+__device__ __forceinline__ float sum_of(float v, int) { return v; }
+__device__ __forceinline__ Fix sum_of(double v, int e) { return fix_of(v, e); }
+
+template <int D, typename RT>
+__device__ __forceinline__ void lattice_sums(const RT (&v)[Lat<D>::Q], int e,
+                                             typename SumType<RT>::type& sum,
+                                             typename SumType<RT>::type (&sj)[D],
+                                             typename SumType<RT>::type (&sP)[Lat<D>::NP]) {
+  using ST = typename SumType<RT>::type;
+  constexpr int NZ = Lat<D>::Q / 9;
+  sum = ST();
+#pragma unroll
+  for (int d = 0; d < D; ++d) sj[d] = ST();
+#pragma unroll
+  for (int k = 0; k < Lat<D>::NP; ++k) sP[k] = ST();
+#pragma unroll
+  for (int pz = 0; pz < NZ; ++pz) {
+    ST ps = ST(), pd = ST(), py = ST(), pxy = ST();
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int i = 9 * pz + 3 * r;
+      const ST f0 = sum_of(v[i], e), f1 = sum_of(v[i + 1], e), f2 = sum_of(v[i + 2], e);
+      const ST sx = f0 + f2, sr = sx + f1, dx = f2 - f0;
+      ps = ps + sr;
+      pd = pd + dx;
+      sP[pidx<D>(0, 0)] = sP[pidx<D>(0, 0)] + sx;
+      if (r != 1) {
+        py = r == 2 ? py + sr : py - sr;
+        pxy = r == 2 ? pxy + dx : pxy - dx;
+        sP[pidx<D>(1, 1)] = sP[pidx<D>(1, 1)] + sr;
+      }
+    }
+    sum = sum + ps;
+    sj[0] = sj[0] + pd;
+    sj[1] = sj[1] + py;
+    sP[pidx<D>(0, 1)] = sP[pidx<D>(0, 1)] + pxy;
+    if constexpr (D == 3) {
+      if (pz != 1) {
+        sj[2] = pz == 2 ? sj[2] + ps : sj[2] - ps;
+        sP[pidx<D>(2, 2)] = sP[pidx<D>(2, 2)] + ps;
+        sP[pidx<D>(0, 2)] = pz == 2 ? sP[pidx<D>(0, 2)] + pd : sP[pidx<D>(0, 2)] - pd;
+        sP[pidx<D>(1, 2)] = pz == 2 ? sP[pidx<D>(1, 2)] + py : sP[pidx<D>(1, 2)] - py;
+      }
+    }
+  }
+}
+
+// The slaved species' sums: the f lattice's less the other species' (Eq.
+// strongest).  FP64: in fixed point at exponent eR (momenta: eR - 6); ex: sums
+// that do not fit there (beyond any physical state).
+template <int D, typename RT> struct Remainder {
+  RT v[1 + D];
+  __device__ Remainder() {
+#pragma unroll
+    for (int d = 0; d <= D; ++d) v[d] = RT(0);
+  }
+  __device__ __forceinline__ void start(int) {}
+  __device__ __forceinline__ void add(int d, RT, RT value, bool first) {
+    v[d] = first ? value : v[d] - value;
+  }
+  __device__ __forceinline__ RT get(int d) const { return v[d]; }
+};
+template <int D> struct Remainder<D, double> {
+  long long rem[1 + D];
+  double ex[1 + D];
+  int eR;
+  __device__ Remainder() : eR(0) {
+#pragma unroll
+    for (int d = 0; d <= D; ++d) { rem[d] = 0; ex[d] = 0.0; }
+  }
+  __device__ __forceinline__ void start(int e) { eR = e + 2; }
+  __device__ __forceinline__ void add(int d, FixSum t, double value, bool first) {
+    const int to = d == 0 ? eR : eR - 6;
+    if (t.e <= to) {
+      const long long r = fix_down(t.s, to - t.e);
+      rem[d] += first ? r : -r;
+    } else {
+      ex[d] += first ? value : -value;
+    }
+  }
+  __device__ __forceinline__ double get(int d) const {
+    const double r = double_of_fix(rem[d], d == 0 ? eR : eR - 6);
+    return ex[d] != 0.0 ? r + ex[d] : r;
+  }
+};
+__device__ __forceinline__ float sum_value(float s) { return s; }
+__device__ __forceinline__ double sum_value(FixSum s) { return double_of_fix(s); }
+__device__ __forceinline__ float close_sum(float s, int) { return s; }
+__device__ __forceinline__ FixSum close_sum(Fix s, int e) { return fix_sum(s, e); }
+
+// (j_a - rho_a u) / rho_a where u_a is defined (reading R5), else 0, as the
+// record holds it.  FP64: the quotient in float-float, numerator and rho_a
+// scaled by rho_a's power of two, comparisons on the bit patterns (positive
+// doubles order as integers; a negative rho_a is below every |j_a|).
+template <int D>
+__device__ __forceinline__ void record_velocities(double rs, const double (&js)[D],
+                                                  const double (&u)[D], double (&out)[D]) {
+  const long long rb = __double_as_longlong(rs);
+  bool undef = rb <= __double_as_longlong(RHO_TINY);
+#pragma unroll
+  for (int d = 0; d < D; ++d)
+    undef |= (__double_as_longlong(js[d]) & 0x7fffffffffffffffLL) >= rb;
+  const int de = 1023 - ((__double2hiint(rs) >> 20) & 0x7ff);
+  const ff ir = ff_rcp(ff_of_double(
+      __hiloint2double((__double2hiint(rs) & 0x800fffff) | 0x3ff00000, __double2loint(rs))));
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const double w = fma(-rs, u[d], js[d]);
+    const int h = __double2hiint(w), ew = ((h >> 20) & 0x7ff) + de;
+    const double ws = ew <= 0 || undef
+                          ? 0.0
+                          : __hiloint2double((h & 0x800fffff) | (ew << 20), __double2loint(w));
+    out[d] = ff_pack(ff_of_double(ws) * ir);
+  }
+}
+template <int D>
+__device__ __forceinline__ void record_velocities(float rs, const float (&js)[D],
+                                                  const float (&u)[D], float (&out)[D]) {
+  // where defined, |j_a| < rho_a, so the quotient lies in (-1, 1) even when
+  // rho_a is denormal (its reciprocal would overflow)
+  const bool undef = species_velocity_undefined<D, float>(rs, js);
+#pragma unroll
+  for (int d = 0; d < D; ++d) out[d] = undef ? 0.f : js[d] / rs - u[d];
+}
+
+// The moments (Sec. 2.1, Sec. 3.1-3.2, Sec. 3.7 slaving, Sec. 4.1 pull
+// streaming), record and reaction sub-steps (Sec. 2.4 Eq. R3) of bulk node n by
+// one thread, lattice by lattice.
+//
+// What bounds it: in FP64 the count of FP64 instructions (75 cycles of an SM
+// quarter each), in FP32 instruction issue, and in both the latency of the
+// loads at the few warps that the registers leave.  So a lattice's 27
+// populations are loaded together (27 loads in flight), and the loop over the
+// lattices is rolled: its sums need no register arrays and the code stays in
+// the instruction cache.  FP64: the sums run in fixed point (fix_of), u_a - u,
+// which only becomes a diffusion velocity, is a float-float quotient, and a
+// sub-step's energy coefficients are those of the moments plus float-float
+// increments (~300 FP64 instructions per node remain of ~1500).
+// smem: the block's shared memory (moments_bytes).
+template <int D, int M, typename S, typename RT>
+__device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __restrict__ rec,
+                                             double* __restrict__ Tf, int* __restrict__ status,
+                                             const Geom& g, const Units& un, const BCDev& bc,
+                                             const DevMech& mech, long long n, void* smem) {
+  constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP;
+  using RC = Rec<D, M>;
+  using ST = typename SumType<RT>::type;
+  using CT = typename ChemType<RT>::type;
+  const long long N = g.N;
+  if (n >= N) return;
+  if (bc.tag && bc.tag[n] == TAG_SOLID) return;
+  ff* const Cs = static_cast<ff*>(smem) + threadIdx.x;
+  ff* const Ws = Cs + M * kChemThreads;
+  double* const Wd = static_cast<double*>(smem) + 2 * M * kChemThreads + threadIdx.x;
+  double* const Cd = Wd + M * kChemThreads;
+  const int x = (int)(n % g.nx);
+  const int y = (int)((n / g.nx) % g.ny);
+  const int z = (int)(n / ((long long)g.nx * g.ny));
+  // pull sources: x of c_x = -1, 0, 1 and the offsets of (c_y, c_z)
+  const int xs[3] = {wrap1(x + 1, g.nx), x, wrap1(x - 1, g.nx)};
+  int row[Q / 3];      // (a grid of 2^31 nodes would not fit any memory)
+#pragma unroll
+  for (int r = 0; r < Q / 3; ++r)
+    row[r] = g.nx * (wrap1(y - (r % 3 - 1), g.ny) +
+                     g.ny * (D == 3 ? wrap1(z - (r / 3 - 1), g.nz) : 0));
+
+  RT rho = RT(0), inv_rho = RT(0), u[D], usq = RT(0), ER = RT(0), Z[D];
+  RT Rm = RT(0);                                   // sum Y_a / m_a
+  CT cU[4] = {CT(), CT(), CT(), CT()};             // energy polynomial
+  Remainder<D, RT> rest;
+#pragma unroll
+  for (int d = 0; d < D; ++d) u[d] = Z[d] = RT(0);
+
+  // species a's state from its sums: record, concentration, energy polynomial
+  auto species = [&](int a, RT rs, const RT (&js)[D]) {
+    const RT Y = rs * inv_rho;
+    rec[(RC::Y + a) * N + n] = Y;
+    if constexpr (kFF<RT>) {
+      Rm += Y * mech.inv_mm_s[a];
+      ff_fma_acc(cU[0], ff(Y), mech.u0_f[a]);
+      ff_fma_acc(cU[1], ff(Y), mech.u1_f[a]);
+      ff_fma_acc(cU[2], ff(Y), mech.u2_f[a]);
+      ff_fma_acc(cU[3], ff(Y), mech.u3_f[a]);
+      Cs[a * kChemThreads] = ff(rs) * mech.inv_mm_f[a];
+      Wd[a * kChemThreads] = ff_pack(ff());
+    } else {
+      double Yd, rd;
+      if constexpr (sizeof(RT) == 8) {
+        Yd = Y;
+        rd = rs;
+        Rm = fma(Y, mech.inv_mm[a], Rm);
+      } else {
+        Yd = double_of_float(Y);
+        rd = double_of_float(rs);
+        Rm += Y * mech.inv_mm_s[a];
+      }
+      cU[0] = fma(Yd, mech.u0[a], cU[0]);
+      cU[1] = fma(Yd, mech.u1[a], cU[1]);
+      cU[2] = fma(Yd, mech.u2[a], cU[2]);
+      cU[3] = fma(Yd, mech.u3[a], cU[3]);
+      const double c = rd * mech.inv_mm[a];
+      Cd[a * kChemThreads] = c;
+      Wd[a * kChemThreads] = 0.0;
+      Cs[a * kChemThreads] = ff_of_double(c);
+    }
+    RT us[D];
+    record_velocities<D>(rs, js, u, us);
+#pragma unroll
+    for (int d = 0; d < D; ++d) rec[(RC::US + a * D + d) * N + n] = us[d];
+  };
+
+#pragma unroll 1
+  for (int it = 0; it <= M; ++it) {
+    const int l = it == 0 ? M - 1 : (it == 1 ? M : it - 2);   // f, g, the species
+    RT v[Q];
+    int e = 0;
+    const S* pl = src + (long long)l * Q * N;
+#pragma unroll
+    for (int i = 0; i < Q; ++i, pl += N)
+      v[i] = Codec<S>::template dec<RT>(__ldg(pl + (row[i / 3] + xs[i % 3])), g.codec, l * Q + i);
+    if constexpr (sizeof(RT) == 8) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) e = max(e, fix_exponent(v[i]));
+    }
+    ST sum, sj[D], sP[NP];
+    lattice_sums<D, RT>(v, e, sum, sj, sP);
+    const auto t0 = close_sum(sum, e);
+    const RT s0 = sum_value(t0);
+    RT s1[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) s1[d] = sum_value(close_sum(sj[d], e));
+    if (it == 0) {
+      rho = s0;
+      inv_rho = RT(1) / rho;
+      rec[RC::RHO * N + n] = rho;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        u[d] = s1[d] * inv_rho;
+        usq = fma(u[d], u[d], usq);
+        rec[(RC::U + d) * N + n] = u[d];
+      }
+      RT P[NP];
+#pragma unroll
+      for (int k = 0; k < NP; ++k) P[k] = sum_value(close_sum(sP[k], e));
+#pragma unroll
+      for (int d = 0; d < D; ++d) Z[d] = flux_less_work<D, RT>(d, u, Z, P);
+      rest.start(e);
+    } else if (it == 1) {
+      ER = s0 * inv_rho;
+      rec[RC::E * N + n] = ER;
+#pragma unroll
+      for (int d = 0; d < D; ++d) rec[(RC::Z + d) * N + n] = s1[d] + Z[d];
+    }
+    if (it != 1) {
+      rest.add(0, t0, s0, it == 0);
+#pragma unroll
+      for (int d = 0; d < D; ++d) rest.add(1 + d, close_sum(sj[d], e), s1[d], it == 0);
+      if (it > 1) species(l, s0, s1);
+    }
+  }
+  {   // slaved species M (Eq. strongest)
+    RT js[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) js[d] = rest.get(1 + d);
+    species(M - 1, rest.get(0), js);
+  }
+
+  // temperature (Eq. temperature) from the node's previous T
+  using X = Chem<CT>;
+  CT U;
+  if constexpr (kFF<RT>) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) cU[k] = ff_norm(cU[k]);
+    U = (ff(ER) + ff(-0.5f * usq)) * un.c2_f;
+  } else {
+    U = (double(ER) - 0.5 * double(usq)) * un.c * un.c;
+  }
+  bool ok;
+  CT Ts = newton_poly(cU, U, X::of_T(__ldcg(Tf + n)), un.newton_max_iter, X::rtol(un), ok);
+  double T;
+  RT th, H[4];
+  if constexpr (kFF<RT>) {
+    T = ff_to_double(Ts);
+    th = Rm * float(R_U) * Ts.hi * un.inv_c2_s;
+  } else if constexpr (sizeof(RT) == 4) {
+    T = Ts;
+    th = Rm * float(R_U) * float(T) * un.inv_c2_s;
+  } else {
+    T = Ts;
+    th = R_U * Rm * T * un.inv_c2;
+  }
+  if (!ok) atomicOr(status, ST_NEWTON);
+  if (!(rho > RT(0)) || !isfinite(rho) || !isfinite(T)) atomicOr(status, ST_NONFINITE);
+  Tf[n] = T;
+  enthalpy_poly(cU, Rm, un, H);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) rec[(RC::H + k) * N + n] = H[k];
+  rec[RC::TH * N + n] = th;
+  const RT b3 = fma(RT(-3), th, RT(1));                            // 1 - 3 theta
+#pragma unroll
+  for (int d = 0; d < D; ++d)
+    rec[(RC::PHI + d) * N + n] = rho * u[d] * fma(-u[d], u[d], b3);
+  if constexpr (sizeof(RT) == 4) rec[RC::LNT * N + n] = ln_T0(RT(T));
+
+  // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3): a zero-dimensional
+  // reactor per node from its post-stream species densities; T_0 is the T just
+  // solved
+  ff dU[4];                              // increments of rho cU
+  ff irho;
+  if constexpr (sizeof(RT) == 8) irho = ff_of_double(inv_rho);
+  else irho = ff_rcp(ff(rho));
+#pragma unroll 1
+  for (int s = 0; s < un.substeps; ++s) {
+    if (s > 0) {
+      CT c[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) c[k] = cU[k] + X::of_ff(ff_norm(dU[k]) * irho);
+      bool oks;
+      Ts = newton_poly(c, U, Ts, un.newton_max_iter, X::rtol(un), oks);
+      if (!oks) atomicOr(status, ST_NEWTON);
+    }
+#pragma unroll
+    for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
+    const TBasis<CT> tb = tbasis(mech, Ts);
+    if constexpr (sizeof(RT) == 8)
+      if (s == 0) rec[RC::LNT * N + n] = tb.lnT - LN_T_REF;
+    add_reactions<M>(mech, tb, Cs, Ws, 0, 1);
+    const bool last = s + 1 == un.substeps;
+#pragma unroll 1
+    for (int a = 0; a < M; ++a) {
+      const ff w = ff_norm(Ws[a * kChemThreads]);
+      if constexpr (kFF<RT>) {
+        Wd[a * kChemThreads] = ff_pack(ff_unpack(Wd[a * kChemThreads]) + w);
+        if (last) continue;
+        Cs[a * kChemThreads] += un.dt_sub_f * w;
+      } else {
+        const double wd = double_join(w);
+        Wd[a * kChemThreads] += wd;
+        if (last) continue;
+        const double c = fma(wd, un.dt_sub, Cd[a * kChemThreads]);
+        Cd[a * kChemThreads] = c;
+        Cs[a * kChemThreads] = ff_of_double(c);
+      }
+      const ff inc = w * un.dtmm_f[a];
+      ff_fma_acc(dU[0], inc, mech.u0_f[a]);
+      ff_fma_acc(dU[1], inc, mech.u1_f[a]);
+      ff_fma_acc(dU[2], inc, mech.u2_f[a]);
+      ff_fma_acc(dU[3], inc, mech.u3_f[a]);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < M - 1; ++a) {
+    if constexpr (kFF<RT>)
+      rec[(RC::DRHO + a) * N + n] = (ff_unpack(Wd[a * kChemThreads]) * un.dtmm_f[a]).hi;
+    else
+      rec[(RC::DRHO + a) * N + n] = RT(Wd[a * kChemThreads] * un.dtmm[a]);
   }
 }
 
@@ -2056,7 +1983,7 @@ k_moments(const S* __restrict__ src, RT* __restrict__ rec, double* __restrict__ 
   // node_set: NODES_ALL or NODES_BULK
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (node_set == NODES_BULK && bc.tag && n < g.N && bc.tag[n] >= 0) return;
-  moments_body<D, M, S, RT>(src, rec, Tf, status, g, un, bc, mech, n);
+  moments_body<D, M, S, RT>(src, rec, Tf, status, g, un, bc, mech, n, moments_static<M>());
 }
 
 // reaction sub-steps, L lanes per node, 128 threads per block.  Node sets:
@@ -2238,7 +2165,7 @@ k_moments_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int no
     const long long n = (b - d.block_begin) * (long long)blockDim.x + threadIdx.x;
     if (node_set == NODES_BULK && d.bc.tag && n < d.g.N && d.bc.tag[n] >= 0) continue;
     moments_body<D, M, S, RT>(static_cast<const S*>(d.pops[c]), static_cast<RT*>(d.rec), d.Tf,
-                              d.status, d.g, d.un, d.bc, *d.mech, n);
+                              d.status, d.g, d.un, d.bc, *d.mech, n, moments_static<M>());
   }
 }
 
@@ -2402,7 +2329,7 @@ __device__ __forceinline__ void iface_substeps(RT* __restrict__ rec, const doubl
   }
   rs[M - 1] = last;
   RT dr[M - 1];
-  node_substeps<M, RT, true>(rs, rho, ER, usq, __ldcg(Tf + n), un, mech, status, chem_slice, dr);
+  node_substeps<M, RT>(rs, rho, ER, usq, __ldcg(Tf + n), un, mech, status, chem_slice, dr);
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) rec[(RC::DRHO + a) * N + n] = dr[a];
 }
@@ -2513,8 +2440,7 @@ k_step_persist(const DomainDev* __restrict__ doms, int ndom, int parity,
         const long long n = w.first + (long long)j * kPersistThreads + threadIdx.x;
         if (n >= d.g.N) break;
         if (d.bc.tag && d.bc.tag[n] >= 0) continue;   // interface node: PI_BND
-        moments_body<D, M, S, RT, true>(src, rec, d.Tf, d.status, d.g, d.un, d.bc, *d.mech, n,
-                                        ps_raw);
+        moments_body<D, M, S, RT>(src, rec, d.Tf, d.status, d.g, d.un, d.bc, *d.mech, n, ps_raw);
       }
     } else if (w.kind == PI_PREP) {
       for (int j = 0; j < npt; ++j)
@@ -2552,7 +2478,7 @@ template <int D, int M, typename S, typename RT> constexpr size_t persist_smem(b
   const size_t chem =
       chem_slice_bytes<M>() + sizeof(R) * WB<D, M>::N * (kPersistThreads / 32);
   size_t m = bnd > chem ? bnd : chem;
-  if (sizeof(RT) == 8) m = m > moments64_bytes<M>() ? m : moments64_bytes<M>();
+  m = m > moments_bytes<M>() ? m : moments_bytes<M>();
   if (split) {
     m = m > prep ? m : prep;
     m = m > coll ? m : coll;
