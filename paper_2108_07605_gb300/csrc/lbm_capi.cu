@@ -566,29 +566,11 @@ lbm_status init_fp16(lbm_ctx* h, const double* drho, int is_pressure, const doub
                      const double* dT, const double* dY) {
   const long long N = h->g.N;
   const int M = h->M, L = h->L, Q = h->Q, LQ = L * Q;
-  // mean fields (host)
-  std::vector<double> rp(N), T(N), Y((size_t)M * N);
-  cudaError_t e = cudaMemcpyAsync(rp.data(), drho, N * sizeof(double), cudaMemcpyDeviceToHost,
-                                  h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(T.data(), dT, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(Y.data(), dY, (size_t)M * N * sizeof(double), cudaMemcpyDeviceToHost,
-                        h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e, "FP16 codec: field download");
-  std::vector<double> mean(1 + 3 + 1 + M, 0.0);   // rho or P, u (0), T, Y
-  for (long long n = 0; n < N; ++n) {
-    mean[0] += rp[n];
-    mean[4] += T[n];
-    for (int a = 0; a < M; ++a) mean[5 + a] += Y[(size_t)a * N + n];
-  }
-  mean[0] /= N;
-  mean[4] /= N;
-  for (int a = 0; a < M; ++a) mean[5 + a] /= N;
-  // scratch: mean state (1 node), offsets, FP32 equilibria, extents
-  const size_t b_mean = mean.size() * sizeof(double), b_off = LQ * sizeof(float),
-               b_eq = (size_t)LQ * N * sizeof(float), b_ext = 2 * L * sizeof(unsigned);
+  // scratch: mean state (1 node) with its partial sums, offsets, FP32
+  // equilibria, extents
+  const size_t b_mean = (5 + M + (size_t)kCodecMeanBlocks * (2 + M)) * sizeof(double),
+               b_off = LQ * sizeof(float), b_eq = (size_t)LQ * N * sizeof(float),
+               b_ext = 2 * L * sizeof(unsigned);
   char* tmp = static_cast<char*>(dalloc(h->cfg, b_mean + b_off + b_eq + b_ext + 256 * 4));
   if (!tmp) return fail(h, LBM_ERR_OOM, "FP16 codec: scratch allocation failed");
   double* dmean = reinterpret_cast<double*>(tmp);
@@ -602,44 +584,20 @@ lbm_status init_fp16(lbm_ctx* h, const double* drho, int is_pressure, const doub
   g1.N = 1;
   Geom gq = h->g;
   gq.codec = nullptr;
-  e = cudaMemcpyAsync(dmean, mean.data(), b_mean, cudaMemcpyHostToDevice, h->stream);
+  cudaError_t e = launch_codec_mean(drho, dT, dY, M, N, dmean + 5 + M, dmean, h->stream);
   if (e == cudaSuccess)
     e = launch_init(h->D, M, LBM_FP32_STORE, h->mech, g1, h->un, dmean, is_pressure, dmean + 1,
-                    dmean + 4, dmean + 5, off, Tdummy, h->status, h->stream);
+                    dmean + 4, dmean + 5, off, nullptr, Tdummy, h->status, h->stream);
   if (e == cudaSuccess)
     e = launch_init(h->D, M, LBM_FP32_STORE, h->mech, gq, h->un, drho, is_pressure, du, dT, dY,
-                    eq, h->Tf, h->status, h->stream);
+                    eq, nullptr, h->Tf, h->status, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ext, 0, b_ext, h->stream);
   if (e == cudaSuccess) e = launch_codec_extent(eq, off, L, Q, N, ext, ext + L, h->stream);
-  std::vector<float> hoff(LQ);
-  std::vector<unsigned> hext(2 * L);
+  if (e == cudaSuccess) e = launch_codec_table(off, ext, ext + L, M, Q, h->codec, h->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(hoff.data(), off, b_off, cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(hext.data(), ext, b_ext, cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) {
-    dfree(h->cfg, tmp);
-    return cuda_fail(h, e, "FP16 codec");
-  }
-  double rho_ref = 0.0;
-  for (int i = 0; i < Q; ++i) rho_ref += hoff[(M - 1) * Q + i];
-  std::vector<float4> table(LQ);
-  for (int l = 0; l < L; ++l) {
-    float dev, amax;
-    std::memcpy(&dev, &hext[l], sizeof(float));
-    std::memcpy(&amax, &hext[L + l], sizeof(float));
-    const double floor_s = l < M ? rho_ref / 27.0 * 0x1p-12 : amax * 0x1p-12;
-    double sc = std::max(16.0 * dev / 65504.0, floor_s);
-    if (!(sc > 0.0) || !std::isfinite(sc)) sc = 1.0;
-    for (int i = 0; i < Q; ++i)
-      table[l * Q + i] = make_float4(hoff[l * Q + i], (float)sc, (float)(1.0 / sc), 0.f);
-  }
-  e = cudaMemcpyAsync(h->codec, table.data(), LQ * sizeof(float4), cudaMemcpyHostToDevice,
-                      h->stream);
-  if (e == cudaSuccess)
-    e = launch_codec_encode(eq, h->pops[h->cur], (long long)LQ * N, N, h->codec, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);   // table and scratch in use
+    e = launch_codec_encode(eq, h->pops[h->cur], h->pops[1 - h->cur], (long long)LQ * N, N,
+                            h->codec, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);   // the scratch is in use
   dfree(h->cfg, tmp);
   if (e != cudaSuccess) return cuda_fail(h, e, "FP16 encode");
   return LBM_OK;
@@ -673,14 +631,11 @@ lbm_status init_common(lbm_ctx* h, const double* rho_or_P, int is_pressure, cons
     if (st != LBM_OK) return st;
   } else {
     e = launch_init(h->D, M, kernel_precision(h->cfg), h->mech, h->g, h->un, drho, is_pressure, du, dT,
-                    dY, h->pops[h->cur], h->Tf, h->status, h->stream);
+                    dY, h->pops[h->cur], h->pops[1 - h->cur], h->Tf, h->status, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "init kernel");
   }
-  // Both buffers start equal: the kernels never write solid nodes, which
-  // keep their initial (equilibrium) populations in either buffer.
-  e = cudaMemcpyAsync(h->pops[1 - h->cur], h->pops[h->cur],
-                      (size_t)h->L * h->Q * N * h->elem, cudaMemcpyDeviceToDevice, h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e, "buffer copy");
+  // (both buffers start equal: the kernels never write solid nodes, which
+  // keep their initial equilibrium populations in either buffer)
   h->initialized = true;
   h->steps = 0;
   if (!on_device) return check_status(h);

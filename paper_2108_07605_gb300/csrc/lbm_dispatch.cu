@@ -44,10 +44,10 @@ cudaError_t launch_step(int D, int M, lbm_precision prec, const DevMech& mech,
 cudaError_t launch_init(int D, int M, lbm_precision prec, const DevMech& mech,
                         const Geom& g, const Units& un, const double* rho_or_P,
                         int is_pressure, const double* u, const double* T,
-                        const double* Y, void* pops, double* Tfield, int* status,
+                        const double* Y, void* pops, void* pops2, double* Tfield, int* status,
                         cudaStream_t s) {
   const KernelSet* k = kernel_set(D, M, prec);
-  return k ? k->init(mech, g, un, rho_or_P, is_pressure, u, T, Y, pops, Tfield, status, s)
+  return k ? k->init(mech, g, un, rho_or_P, is_pressure, u, T, Y, pops, pops2, Tfield, status, s)
            : cudaErrorInvalidValue;
 }
 
@@ -192,15 +192,80 @@ __global__ void k_codec_extent(const float* __restrict__ eq, const float* __rest
   }
 }
 
-// FP32 populations to FP16 offsets with the codec
+// FP32 populations to FP16 offsets with the codec, in both buffers
 __global__ void k_codec_encode(const float* __restrict__ eq, __half* __restrict__ out,
-                               long long count, long long N,
+                               __half* __restrict__ out2, long long N,
                                const float4* __restrict__ codec) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
-       k += (long long)gridDim.x * blockDim.x) {
-    const float4 c = __ldg(codec + k / N);
-    out[k] = __float2half_rn((eq[k] - c.x) * c.z);
+  const float4 c = __ldg(codec + blockIdx.y);          // one population index per grid row
+  const long long base = (long long)blockIdx.y * N;
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
+       n += (long long)gridDim.x * blockDim.x) {
+    const __half h = __float2half_rn((eq[base + n] - c.x) * c.z);
+    out[base + n] = h;
+    out2[base + n] = h;
   }
+}
+
+// Per field (0: rho or P, 1: T, 2 + a: Y_a) and block a partial sum, then the
+// means: on the device, where the fields are (read back and summed on the host
+// they took most of an FP16 initialisation)
+__global__ void k_codec_sum(const double* __restrict__ rho_or_P, const double* __restrict__ T,
+                            const double* __restrict__ Y, long long N,
+                            double* __restrict__ part) {
+  __shared__ double s[256];
+  const int f = blockIdx.y;
+  const double* v = f == 0 ? rho_or_P : (f == 1 ? T : Y + (long long)(f - 2) * N);
+  double a = 0.0;
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
+       n += (long long)gridDim.x * blockDim.x)
+    a += v[n];
+  s[threadIdx.x] = a;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[f * gridDim.x + blockIdx.x] = s[0];
+}
+__global__ void k_codec_mean(const double* __restrict__ part, int nf, int nb, long long N,
+                             double* __restrict__ mean) {
+  const int f = threadIdx.x;
+  if (f >= 1 && f <= 3) mean[f] = 0.0;
+  if (f >= nf) return;
+  double a = 0.0;
+  for (int b = 0; b < nb; ++b) a += part[f * nb + b];
+  mean[f == 0 ? 0 : 3 + f] = a / (double)N;
+}
+
+// The codec table (reading R19): offsets off, per lattice the scale that maps
+// 16x the largest initial deviation to the FP16 maximum, with its floor.
+__global__ void k_codec_table(const float* __restrict__ off, const unsigned* __restrict__ dev_max,
+                              const unsigned* __restrict__ abs_max, int M, int Q,
+                              float4* __restrict__ table) {
+  double rho_ref = 0.0;
+  for (int i = 0; i < Q; ++i) rho_ref += off[(M - 1) * Q + i];
+  for (int k = threadIdx.x; k < (M + 1) * Q; k += blockDim.x) {
+    const int l = k / Q;
+    const double floor_s = l < M ? rho_ref / 27.0 * 0x1p-12 : __uint_as_float(abs_max[l]) * 0x1p-12;
+    double sc = fmax(16.0 * __uint_as_float(dev_max[l]) / 65504.0, floor_s);
+    if (!(sc > 0.0) || !isfinite(sc)) sc = 1.0;
+    table[k] = make_float4(off[k], (float)sc, (float)(1.0 / sc), 0.f);
+  }
+}
+
+cudaError_t launch_codec_mean(const double* rho_or_P, const double* T, const double* Y, int M,
+                              long long N, double* part, double* mean, cudaStream_t s) {
+  const int nb = (int)std::min<long long>((N + 255) / 256, kCodecMeanBlocks);
+  k_codec_sum<<<dim3(nb, 2 + M), 256, 0, s>>>(rho_or_P, T, Y, N, part);
+  k_codec_mean<<<1, 32, 0, s>>>(part, 2 + M, nb, N, mean);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_codec_table(const float* off, const unsigned* dev_max,
+                               const unsigned* abs_max, int M, int Q, float4* table,
+                               cudaStream_t s) {
+  k_codec_table<<<1, 128, 0, s>>>(off, dev_max, abs_max, M, Q, table);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_codec_extent(const float* eq, const float* off, int L, int Q, long long N,
@@ -211,11 +276,12 @@ cudaError_t launch_codec_extent(const float* eq, const float* off, int L, int Q,
   return cudaGetLastError();
 }
 
-cudaError_t launch_codec_encode(const float* eq, void* out, long long count, long long N,
-                                const float4* codec, cudaStream_t s) {
-  const long long nb = std::min<long long>((count + 255) / 256, 152LL * 16);
-  if (nb <= 0) return cudaSuccess;
-  k_codec_encode<<<(unsigned)nb, 256, 0, s>>>(eq, static_cast<__half*>(out), count, N, codec);
+cudaError_t launch_codec_encode(const float* eq, void* out, void* out2, long long count,
+                                long long N, const float4* codec, cudaStream_t s) {
+  if (count <= 0) return cudaSuccess;
+  const long long bx = std::min<long long>((N + 255) / 256, 152LL * 4);
+  k_codec_encode<<<dim3((unsigned)bx, (unsigned)(count / N)), 256, 0, s>>>(
+      eq, static_cast<__half*>(out), static_cast<__half*>(out2), N, codec);
   return cudaGetLastError();
 }
 

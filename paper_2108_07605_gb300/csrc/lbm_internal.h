@@ -284,8 +284,8 @@ struct KernelSet {
   cudaError_t (*prepare)();
   cudaError_t (*init)(const DevMech& mech, const Geom& g, const Units& un,
                       const double* rho_or_P, int is_pressure, const double* u,
-                      const double* T, const double* Y, void* pops, double* Tfield,
-                      int* status, cudaStream_t s);
+                      const double* T, const double* Y, void* pops, void* pops2,
+                      double* Tfield, int* status, cudaStream_t s);
   cudaError_t (*out)(const DevMech& mech, const Geom& g, const Units& un, const void* pops,
                      const double* Tfield, double* rho, double* u, double* T, double* Y,
                      double* E, int* status, cudaStream_t s);
@@ -312,8 +312,8 @@ cudaError_t launch_step(int D, int M, lbm_precision prec, const DevMech& mech,
 cudaError_t launch_init(int D, int M, lbm_precision prec, const DevMech& mech,
                         const Geom& g, const Units& un, const double* rho_or_P,
                         int is_pressure, const double* u, const double* T,
-                        const double* Y, void* pops, double* Tfield, int* status,
-                        cudaStream_t s);
+                        const double* Y, void* pops, void* pops2, double* Tfield, int* status,
+                        cudaStream_t s);   // pops2: a second copy (nullptr: none)
 cudaError_t launch_moments_out(int D, int M, lbm_precision prec, const DevMech& mech,
                                const Geom& g, const Units& un, const void* pops,
                                const double* Tfield, double* rho, double* u,
@@ -331,8 +331,17 @@ cudaError_t launch_diagnostics(int D, int M, lbm_precision prec, const DevMech& 
 // FP16 storage codec (lbm_dispatch.cu)
 cudaError_t launch_codec_extent(const float* eq, const float* off, int L, int Q, long long N,
                                 unsigned* dev_max, unsigned* abs_max, cudaStream_t s);
-cudaError_t launch_codec_encode(const float* eq, void* out, long long count, long long N,
-                                const float4* codec, cudaStream_t s);
+cudaError_t launch_codec_encode(const float* eq, void* out, void* out2, long long count,
+                                long long N, const float4* codec, cudaStream_t s);
+// means over the N nodes of rho or P, T and Y (fixed order), as a one-node state
+// at rest: mean[0], 0 (u), mean[4], mean[5 ..]; part: kCodecMeanBlocks (2 + M)
+// doubles of scratch
+constexpr int kCodecMeanBlocks = 128;
+cudaError_t launch_codec_mean(const double* rho_or_P, const double* T, const double* Y, int M,
+                              long long N, double* part, double* mean, cudaStream_t s);
+cudaError_t launch_codec_table(const float* off, const unsigned* dev_max,
+                               const unsigned* abs_max, int M, int Q, float4* table,
+                               cudaStream_t s);
 int record_fields(int D, int M);
 
 // Host helpers defined in lbm_capi.cu.
