@@ -1582,19 +1582,22 @@ constexpr int kColl32Blocks = 3; // FP32 blocks per SM the registers are held to
 // species axis-factor tables
 template <int D, int M, typename RT> constexpr int coll_smem_entries();
 
-// Layout of k_coll's shared memory in FP64 (8-byte entries per node): the
-// parameters, the energy factors, the FP64 axis factors E of every species'
-// equilibrium, and float-float tables (packed pairs) of the Stefan-Maxwell
-// term's factors:
+// Layout of k_coll's shared memory in FP64 (8-byte entries per node): the FP64
+// axis factors E of the stored species' equilibria (x: times hh_a), float-float
+// tables (packed pairs) of the Stefan-Maxwell term's factors, the extended
+// equilibrium's and the energy factors, the species coefficients cF (a pair)
+// and 1 - 2 beta, and the scalars.  The pairs:
 //   e_d(c), the axis factor of psi(u, theta_b), and t_d(c) = s_d(c) - e_d(c),
 //   s_d(c) that of psi(u + V_b, theta_b), formed without cancellation from
 //   V_b (t(0) = -V (2u + V), t(+-1) = (V (2u + V) +- V)/2); for x, s and t
 //   times -rho_b.
 template <int D, int M> struct Coll64 {
-  static constexpr int AF = CPar<D, M>::NF, BF = AF + 3 * D, E = BF + 3 * D;
-  static constexpr int F = E + M * D * 3;       // ff pairs of (b, d): 6 entries
-  static constexpr int N = F + M * D * 6;
-  static constexpr int e(int b, int d, int c) { return E + (b * D + d) * 3 + c + 1; }
+  static constexpr int E = 0, F = E + (M - 1) * D * 3;
+  static constexpr int EX = F + M * D * 6, AF = EX + 3 * D, BF = AF + 3 * D;
+  static constexpr int CF = BF + 3 * D, OM1 = CF + M - 1;
+  static constexpr int RHO = OM1 + M - 1, OM = RHO + 1, U = OM + 1, W = U + 1;
+  static constexpr int N = W + D;
+  static constexpr int e(int a, int d, int c) { return E + (a * D + d) * 3 + c + 1; }
   // first of a pair: x: -rho s(c), then -rho t(c); y, z: e(c), then t(c)
   static constexpr int f(int b, int d, int c) { return F + (b * D + d) * 6 + c + 1; }
 };
@@ -1658,44 +1661,54 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
     load_direction<D, M, S, double>(src, bc, tag, N, node_shift<D>(x, y, z, i, -1, g), i,
                                     g.codec, fin);
   }
-  for (int f = w; f < CP::NF; f += TPN)
-    s[f * kCollNodes] = valid ? __ldcg(cp + f * N + n) : 0.0;
-  __syncthreads();
   if (valid) {
-    if (w == TPN - 1) {
-      double u[D], Af[D][3], Bf[D][3];
-#pragma unroll
-      for (int d = 0; d < D; ++d) u[d] = s[(CP::U + d) * kCollNodes];
-      energy_factors<D, double>(u, s[CP::THETA * kCollNodes], Af, Bf);
-#pragma unroll
-      for (int d = 0; d < D; ++d)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          s[(T::AF + d * 3 + k) * kCollNodes] = Af[d][k];
-          s[(T::BF + d * 3 + k) * kCollNodes] = Bf[d][k];
-        }
-    }
+    auto G = [&](int f) { return __ldcg(cp + (long long)f * N + n); };
     for (int e = w; e < M * D; e += TPN) {
       const int b = e / D, d = e % D;
-      const double u = s[(CP::U + d) * kCollNodes];
-      const double P = fma(u, u, s[(CP::TH + b) * kCollNodes]), hu = 0.5 * u;
+      const double u = G(CP::U + d), th = G(CP::TH + b);
+      const ff V = ff_unpack(G(CP::V + b * D + d));
+      const ff mr = d == 0 ? -ff_of_double(G(CP::RS + b)) : ff(1.f);
+      const double hh = d == 0 && b < M - 1 ? G(CP::HH + b) : 1.0;
+      const double P = fma(u, u, th), hu = 0.5 * u;
       const double E[3] = {fma(0.5, P, -hu), 1.0 - P, fma(0.5, P, hu)};
-      const ff V = ff_unpack(s[(CP::V + b * D + d) * kCollNodes]);
       ff uf = ff_of_double(u);
       uf = ff(2.f * uf.hi, 2.f * uf.lo) + V;
       const ff dP = V * uf;                     // V (2u + V)
       const ff t0 = -dP, tp = dP + V, tm = dP - V;
       const ff t[3] = {ff(0.5f * tm.hi, 0.5f * tm.lo), t0, ff(0.5f * tp.hi, 0.5f * tp.lo)};
-      const ff mr = -ff_of_double(s[(CP::RS + b) * kCollNodes]);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        s[(T::E + e * 3 + c) * kCollNodes] = E[c];
+        if (b < M - 1) s[(T::E + e * 3 + c) * kCollNodes] = d == 0 ? hh * E[c] : E[c];
         const ff ef = ff_of_double(E[c]);
         const ff first = d == 0 ? mr * (ef + t[c]) : ef;
         const ff second = d == 0 ? mr * t[c] : t[c];
         s[(T::F + e * 6 + c) * kCollNodes] = ff_pack(first);
         s[(T::F + e * 6 + 3 + c) * kCollNodes] = ff_pack(second);
       }
+    }
+    if (w == TPN - 1) {
+      double u[D], Af[D][3], Bf[D][3];
+#pragma unroll
+      for (int d = 0; d < D; ++d) u[d] = G(CP::U + d);
+      energy_factors<D, double>(u, G(CP::THETA), Af, Bf);
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const double px = G(CP::PEX + d);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          s[(T::AF + d * 3 + k) * kCollNodes] = Af[d][k];
+          s[(T::BF + d * 3 + k) * kCollNodes] = Bf[d][k];
+          s[(T::EX + d * 3 + k) * kCollNodes] = psi1<double>(k - 1, u[d], px);
+        }
+        s[(T::W + d) * kCollNodes] = G(CP::W + d);
+      }
+      s[T::RHO * kCollNodes] = G(CP::RHO);
+      s[T::OM * kCollNodes] = G(CP::OM);
+      s[T::U * kCollNodes] = G(CP::UL);
+    }
+    for (int a = w; a < M - 1; a += TPN) {
+      s[(T::CF + a) * kCollNodes] = G(CP::CF + a);
+      s[(T::OM1 + a) * kCollNodes] = G(CP::OM1 + a);
     }
   }
   __syncthreads();
@@ -1706,7 +1719,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   ff A[M], SS[M];              // t_x e_y + s_x t_y and s_x s_y, times -rho_b
   double eh[M - 1];            // hh_a e_x e_y
   double fxy = 0.0, gP = 0.0, gQ = 0.0;
-  const double rho = P(CP::RHO), om = P(CP::OM);
+  const double rho = P(T::RHO), om = P(T::OM);
   int jcur = -1;
 #pragma unroll 1
   for (int k = k0; k < k1; ++k) {
@@ -1733,13 +1746,12 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
           ff_acc(sy, ty);
           SS[b] = sx * ff_norm(sy);
         }
-        if (b < M - 1) eh[b] = P(T::e(b, 0, cx)) * P(T::e(b, 1, cy)) * P(CP::HH + b);
+        if (b < M - 1) eh[b] = P(T::e(b, 0, cx)) * P(T::e(b, 1, cy));
       }
-      fxy = rho * psi1<double>(cx, P(CP::U), P(CP::PEX)) *
-            psi1<double>(cy, P(CP::U + 1), P(CP::PEX + 1));
+      fxy = rho * P(T::EX + cx + 1) * P(T::EX + 3 + cy + 1);
       const double ax = P(T::AF + cx + 1), ay = P(T::AF + 3 + cy + 1);
       gP = ax * ay;
-      gQ = fma(P(CP::UL), gP, fma(P(T::BF + cx + 1), ay, ax * P(T::BF + 3 + cy + 1)));
+      gQ = fma(P(T::U), gP, fma(P(T::BF + cx + 1), ay, ax * P(T::BF + 3 + cy + 1)));
     }
     ff dd[M];
 #pragma unroll
@@ -1758,15 +1770,15 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
 #pragma unroll
       for (int b = 0; b < M; ++b)
         if (b != a) ff_fma_acc(F, mech.K_f[a][b], dd[b]);
-      F = PF(CP::CF + a) * ff_norm(F);
+      F = PF(T::CF + a) * ff_norm(F);
       const double ez = D == 3 ? P(T::e(a, D - 1, cz)) : 1.0;
-      const double base = fma(fin[a], P(CP::OM1 + a), double_join(F));
+      const double base = fma(fin[a], P(T::OM1 + a), double_join(F));
       fin[a] = next(a);
       dst[(long long)(a * Q + i) * N + n] = D == 3 ? fma(eh[a], ez, base) : eh[a] + base;
     }
     double fex = fxy, geq = gQ;
     if constexpr (D == 3) {
-      fex *= psi1<double>(cz, P(CP::U + 2), P(CP::PEX + 2));
+      fex *= P(T::EX + 6 + cz + 1);
       geq = fma(P(T::AF + 6 + cz + 1), gQ, gP * P(T::BF + 6 + cz + 1));
     }
     dst[(long long)((M - 1) * Q + i) * N + n] = fma(om, fex - fin[M - 1], fin[M - 1]);
@@ -1776,7 +1788,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
     if (csq(i, D) == 1) {
 #pragma unroll
       for (int d = 0; d < D; ++d)
-        if (cvel(i, d) != 0) gn += (cvel(i, d) > 0 ? 0.5 : -0.5) * P(CP::W + d);
+        if (cvel(i, d) != 0) gn = fma(cvel(i, d) > 0 ? 0.5 : -0.5, P(T::W + d), gn);
     }
     dst[(long long)(M * Q + i) * N + n] = gn;
   }
