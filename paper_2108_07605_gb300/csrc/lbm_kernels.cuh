@@ -1614,7 +1614,19 @@ template <int D, int M> struct Coll32 {
   static constexpr int f(int b, int d, int c) { return (d * 3 + c + 1) * M + b; }
 };
 template <int D, int M, typename RT> constexpr int coll_smem_entries() {
-  return sizeof(RT) == 8 ? Coll64<D, M>::N : Coll32<D, M>::N;
+  return sizeof(RT) == 8 ? Coll64<D, M>::N + kCollTPN * (M + 1) : Coll32<D, M>::N;
+}
+
+// Asynchronous 8-byte copy from global to this thread's shared memory (8-byte
+// aligned), and the wait for this thread's copies.
+__device__ __forceinline__ void copy_async8(double* to, const double* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(to)),
+               "l"(from)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // The FP64 collision of one block of TPN warps, 32 nodes (lane = node), the
@@ -1651,15 +1663,19 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   constexpr int NZ = D == 3 ? 3 : 1;
   constexpr int CH = (Q + TPN - 1) / TPN;
   const int k0 = w * CH, k1 = min(k0 + CH, Q);
-  // the first direction's populations are in flight while the block's tables
-  // are built
-  double fin[M + 1];
-#pragma unroll
-  for (int l = 0; l <= M; ++l) fin[l] = 0.0;
+  // This lane's slots of the warp's buffer hold the populations of one
+  // direction; the next direction's are copied into them as they are used up,
+  // past the registers (the first direction's while the tables are built).
+  double* const fin = sm + T::N * kCollNodes + w * (M + 1) * kCollNodes + lane;
+  const long long stride = Q * (tag >= 0 ? (long long)bc.n_if : N);
+  auto first_of = [&](int i) {
+    return tag >= 0 ? static_cast<const double*>(bc.pops) + (long long)i * bc.n_if + tag
+                    : src + i * N + node_shift<D>(x, y, z, i, -1, g);
+  };
   if (valid && k0 < k1) {
-    const int i = k0 / NZ + 9 * (k0 % NZ);
-    load_direction<D, M, S, double>(src, bc, tag, N, node_shift<D>(x, y, z, i, -1, g), i,
-                                    g.codec, fin);
+    const double* p = first_of(k0 / NZ + 9 * (k0 % NZ));
+#pragma unroll
+    for (int l = 0; l <= M; ++l, p += stride) copy_async8(fin + l * kCollNodes, p);
   }
   if (valid) {
     auto G = [&](int f) { return __ldcg(cp + (long long)f * N + n); };
@@ -1725,12 +1741,13 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   for (int k = k0; k < k1; ++k) {
     const int j = k / NZ, i = j + 9 * (k % NZ);
     const int cx = cvel(j, 0), cy = cvel(j, 1), cz = D == 3 ? k % NZ - 1 : 0;
-    // the next direction, whose populations take the places of this one's as
-    // these are used up (the last direction loads its own again)
-    const int kn = min(k + 1, k1 - 1), in = kn / NZ + 9 * (kn % NZ);
-    const long long sn = node_shift<D>(x, y, z, in, -1, g);
+    // the next direction
+    const bool more = k + 1 < k1;
+    const double* pn = more ? first_of((k + 1) / NZ + 9 * ((k + 1) % NZ)) : src;
+    auto take = [&](int l) { return fin[l * kCollNodes]; };
     auto next = [&](int l) {
-      return pop_in<double>(src, bc, tag, N, sn, l * Q + in, g.codec);
+      if (more) copy_async8(fin + l * kCollNodes, pn);
+      pn += stride;
     };
     if (j != jcur) {
       jcur = j;
@@ -1764,6 +1781,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
         dd[b] = A[b];
       }
     }
+    copy_async_wait();
 #pragma unroll
     for (int a = 0; a < M - 1; ++a) {
       ff F;
@@ -1772,8 +1790,8 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
         if (b != a) ff_fma_acc(F, mech.K_f[a][b], dd[b]);
       F = PF(T::CF + a) * ff_norm(F);
       const double ez = D == 3 ? P(T::e(a, D - 1, cz)) : 1.0;
-      const double base = fma(fin[a], P(T::OM1 + a), double_join(F));
-      fin[a] = next(a);
+      const double base = fma(take(a), P(T::OM1 + a), double_join(F));
+      next(a);
       dst[(long long)(a * Q + i) * N + n] = D == 3 ? fma(eh[a], ez, base) : eh[a] + base;
     }
     double fex = fxy, geq = gQ;
@@ -1781,10 +1799,12 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
       fex *= P(T::EX + 6 + cz + 1);
       geq = fma(P(T::AF + 6 + cz + 1), gQ, gP * P(T::BF + 6 + cz + 1));
     }
-    dst[(long long)((M - 1) * Q + i) * N + n] = fma(om, fex - fin[M - 1], fin[M - 1]);
-    fin[M - 1] = next(M - 1);
-    double gn = fma(om, fma(rho, geq, -fin[M]), fin[M]);
-    fin[M] = next(M);
+    const double fm = take(M - 1);
+    dst[(long long)((M - 1) * Q + i) * N + n] = fma(om, fex - fm, fm);
+    next(M - 1);
+    const double gm = take(M);
+    double gn = fma(om, fma(rho, geq, -gm), gm);
+    next(M);
     if (csq(i, D) == 1) {
 #pragma unroll
       for (int d = 0; d < D; ++d)
