@@ -2606,6 +2606,32 @@ __device__ __forceinline__ double wide(float v) { return double_of_float(v); }
 template <typename S> struct StoredType { using type = float; };
 template <> struct StoredType<double> { using type = double; };
 
+// Q populations of a lattice from pl, N apart, and their largest biased
+// exponent.  FP32: from the largest bit pattern, so that all loads are in flight
+// before the first is widened.
+template <typename S, int Q>
+__device__ __forceinline__ int load_lattice(const S* __restrict__ pl, long long N,
+                                            const float4* codec, int li, double (&v)[Q]) {
+  int e = 0;
+  if constexpr (sizeof(S) == 8) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i, pl += N) v[i] = __ldg(pl);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) e = max(e, fix_exponent(v[i]));
+  } else {
+    float f[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i, pl += N)
+      f[i] = Codec<S>::template dec<float>(__ldg(pl), codec, li + i);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) e = max(e, __float_as_int(f[i]) & 0x7fffffff);
+    e = fix_exponent(wide(__int_as_float(e)));
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = wide(f[i]);
+  }
+  return e;
+}
+
 template <int D, int M, typename S, typename F>
 __device__ __forceinline__ void stored_sums(const S* __restrict__ pops, long long N, long long n,
                                             const float4* codec, double& rho, double (&j)[D],
@@ -2616,14 +2642,8 @@ __device__ __forceinline__ void stored_sums(const S* __restrict__ pops, long lon
   for (int it = 0; it <= M; ++it) {
     const int l = it == 0 ? M - 1 : (it == 1 ? M : it - 2);   // f, g, the species
     double v[Q];
-    int e = 0;
     const S* pl = pops + (long long)l * Q * N + n;
-#pragma unroll
-    for (int i = 0; i < Q; ++i, pl += N)
-      v[i] = wide(Codec<S>::template dec<typename StoredType<S>::type>(__ldg(pl), codec,
-                                                                       l * Q + i));
-#pragma unroll
-    for (int i = 0; i < Q; ++i) e = max(e, fix_exponent(v[i]));
+    const int e = load_lattice<S>(pl, N, codec, l * Q, v);
     Fix sum, sj[D], sP[NP];
     lattice_sums<D, double>(v, e, sum, sj, sP);
     const FixSum t = fix_sum(sum, e);
@@ -2713,8 +2733,9 @@ k_diag(const S* __restrict__ pops, const double* __restrict__ Tf, const int* __r
 }
 
 // Fields of the stored state: rho, u (m/s), T (Newton, not stored), Y, E (J/kg).
-// Bound by its one pass over the populations (600x40x40 tube, FP64: 0.98 ms
-// with the sums in FP64 instructions).
+// Bound by its one pass over the populations (600x40x40 tube: 0.40 ms in FP64,
+// 0.98 with the sums in FP64 instructions; 0.47 in FP32, 1.5 with a lattice's
+// loads one after the other).
 template <int D, int M, typename S>
 __global__ void __launch_bounds__(128)
 k_out(const S* __restrict__ pops, const double* __restrict__ Tf, double* __restrict__ orho,
