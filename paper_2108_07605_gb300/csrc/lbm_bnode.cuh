@@ -26,13 +26,20 @@
 // thread's shared-memory column, stride kBnd.
 
 constexpr int kBnd = kBndNodesPerBlock;   // threads per block of the boundary kernel
+// Blocks per SM its registers are held to.  Bound by latency, not by a pipe
+// (FP64: pipe 45 % busy; FP32: 3.8 warps per SM quarter in all): what counts is
+// loads in flight, by the directions unrolled three rows deep, and warps.
+// 600x40x40 tube, 74k interface nodes: FP64 1.22 -> 1.11 ms (255 registers);
+// FP32 0.44 -> 0.32 ms at 168 registers and six blocks, 0.41 at eight (128
+// registers, spills) and at four (240); FP16 0.52 -> 0.37.
+template <typename S> constexpr int kBnodeMinBlocks = sizeof(S) == 8 ? 4 : 6;
 
 // shared memory per thread: target Y, local Y, a spare Y, the local u_a and
-// the target u_a (off-grid TMS targets) (R entries), then the Q pull sources
-// (long long)
+// the target u_a (off-grid TMS targets) (R entries), then the pull sources of
+// the Q / 3 rows of directions (long long)
 template <int D, int M> constexpr int bnode_col_entries() { return 3 * M + 2 * M * D; }
 template <int D, int M, typename R> constexpr size_t bnode_smem() {
-  return (sizeof(R) * bnode_col_entries<D, M>() + sizeof(long long) * Lat<D>::Q) * kBnd;
+  return (sizeof(R) * bnode_col_entries<D, M>() + sizeof(long long) * (Lat<D>::Q / 3)) * kBnd;
 }
 
 // An equilibrium state of the boundary procedures (Eqs. faEqGeneral,
@@ -282,8 +289,8 @@ template <int E> struct ForL<E, E> {
 // Population sums of a pass, lattice by lattice: fn.template setup<l>()
 // once per lattice, then, row by row, fn.template row<l>(c_y, c_z) and
 // fn.template get<l>(i, c) for the row's three directions.
-// Directions in rows of three (c_x = -1, 0, 1 at compile time, a row's loads
-// in flight together); a row enters through its sum s and difference
+// Directions in rows of three (c_x = -1, 0, 1 at compile time), three rows'
+// loads in flight together; a row enters through its sum s and difference
 // d = f_+ - f_- (and f_+ + f_- for P_xx).  kDensOnly: the densities rho_a,
 // rho and rho E only (the bounce-back pass of a wall).
 template <int D, int M, typename R, bool kDensOnly = false, typename F>
@@ -297,7 +304,7 @@ __device__ __forceinline__ void bsums(F& fn, BSums<D, M, R>& z) {
     for (int d = 0; d < D; ++d) sj[d] = R(0);
 #pragma unroll
     for (int p = 0; p < NP; ++p) sP[p] = R(0);
-#pragma unroll 1
+#pragma unroll 3
     for (int yz = 0; yz < Q / 3; ++yz) {
       const int cy = yz % 3 - 1, cz = D == 3 ? yz / 3 - 1 : 0;
       fn.template row<l>(cy, cz);
@@ -357,21 +364,22 @@ template <int D, int M, typename S, typename R> struct BPull {
   const S* src;
   const float4* codec;
   long long N, n;
-  const long long* sn;      // pull source of direction i at sn[i kBnd]
+  const long long* sn;      // row r's pull source is node sn[r kBnd] + dx[k], c_x = k - 1
+  int dx[3];
   unsigned inc;
   bool bbk;
   __device__ __forceinline__ bool incoming(int i) const { return inc >> i & 1u; }
   template <int l> __device__ __forceinline__ void setup() {}
   template <int l> __device__ __forceinline__ void row(int, int) {}
-  template <int l> __device__ __forceinline__ R pull(int i) const {
+  template <int l> __device__ __forceinline__ R pull(int i, int k) const {
     const bool bb = bbk && incoming(i);
-    const long long mm = bb ? n : sn[i * kBnd];
+    const long long mm = bb ? n : sn[i / 3 * kBnd] + dx[k];
     const int ii = bb ? Q - 1 - i : i;
     return Codec<S>::template dec<R>(__ldg(src + (long long)(l * Q + ii) * N + mm), codec,
                                      l * Q + ii);
   }
-  template <int l> __device__ __forceinline__ R get(int i, const int (&)[3]) const {
-    return pull<l>(i);
+  template <int l> __device__ __forceinline__ R get(int i, const int (&c)[3]) const {
+    return pull<l>(i, c[0] + 1);
   }
 };
 
@@ -383,8 +391,8 @@ template <int D, int M, typename S, typename R> struct BStorePull {
   long long st;
   template <int l> __device__ __forceinline__ void setup() {}
   template <int l> __device__ __forceinline__ void row(int, int) {}
-  template <int l> __device__ __forceinline__ R get(int i, const int (&)[3]) const {
-    const R v = p.template pull<l>(i);
+  template <int l> __device__ __forceinline__ R get(int i, const int (&c)[3]) const {
+    const R v = p.template pull<l>(i, c[0] + 1);
     P[(long long)(l * Q + i) * st] = v;
     return v;
   }
@@ -418,7 +426,7 @@ template <int D, int M, typename S, typename R> struct BLocal {
     ta.template row<l>(cy, cz);
   }
   template <int l> __device__ __forceinline__ R get(int i, const int (&c)[3]) const {
-    return p.incoming(i) ? ta.template evalx<l>(c[0]) : p.template pull<l>(i);
+    return p.incoming(i) ? ta.template evalx<l>(c[0]) : p.template pull<l>(i, c[0] + 1);
   }
 };
 
@@ -451,7 +459,7 @@ template <int D, int M, typename S, typename R> struct BFinal {
           const int i = 3 * yz + k;
           const R loc = tl.template evalx<l>(k - 1), a = lo.ta.template evalx<l>(k - 1);
           const R t = same ? a : tb.template evalx<l>(k - 1);
-          const R v = t + (lo.p.incoming(i) ? a : lo.p.template pull<l>(i)) - loc;
+          const R v = t + (lo.p.incoming(i) ? a : lo.p.template pull<l>(i, k)) - loc;
           P[(long long)(l * Q + i) * st] = simple ? loc : v;
         }
       }
@@ -541,7 +549,7 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
                                            int* __restrict__ status, const Geom& g,
                                            const Units& un, const DevMech& m, int k,
                                            R* col, long long* sncol) {
-  constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP;
+  constexpr int Q = Lat<D>::Q;
   using RC = Rec<D, M>;
   using Pull = BPull<D, M, S, R>;
   const long long N = g.N;
@@ -549,12 +557,15 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
   const int info = bc.if_info[k];
   const int kind = info & 15;
   const unsigned inc = bc.if_inc[k];
+  // the pull sources: a row's directions share y and z
+  const int x = (int)(n % g.nx);
+  const int dx[3] = {wrap1(x + 1, g.nx), x, wrap1(x - 1, g.nx)};
   {
-    const int x = (int)(n % g.nx);
     const int y = (int)((n / g.nx) % g.ny);
     const int z = (int)(n / ((long long)g.nx * g.ny));
 #pragma unroll 1
-    for (int i = 0; i < Q; ++i) sncol[i * kBnd] = node_shift<D>(x, y, z, i, -1, g);
+    for (int r = 0; r < Q / 3; ++r)
+      sncol[r * kBnd] = node_shift<D>(x, y, z, 3 * r + 1, -1, g) - x;
   }
   const long long st = bc.n_if;
   const float4* codec = g.codec;
@@ -569,13 +580,13 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
   if (kind == BK_BB) {
     // Eq. bb: incoming links take the node's own opposite post-collision
     // populations
-    BStorePull<D, M, S, R> out{Pull{src, codec, N, n, sncol, inc, true},
+    BStorePull<D, M, S, R> out{Pull{src, codec, N, n, sncol, {dx[0], dx[1], dx[2]}, inc, true},
                                static_cast<R*>(bc.pops) + k, st};
     bsums<D, M, R>(out, z);
   } else {
     if (kind == BK_TMS) {
       // step 1, Eqs. BBrho and BBY: bounce-back density and mass fractions
-      Pull pull{src, codec, N, n, sncol, inc, true};
+      Pull pull{src, codec, N, n, sncol, {dx[0], dx[1], dx[2]}, inc, true};
       bsums<D, M, R, true>(pull, z);
       A.rho = z.rho;
       const R irho = R(1) / z.rho;
@@ -679,7 +690,8 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
     }
     // the local state: incoming links at A, the others pulled (Eqs.
     // locRho-locT and their inlet / outlet analogues)
-    BLocal<D, M, S, R> local{Pull{src, codec, N, n, sncol, inc, false}, &A, &m, &un, {}};
+    BLocal<D, M, S, R> local{Pull{src, codec, N, n, sncol, {dx[0], dx[1], dx[2]}, inc, false},
+                             &A, &m, &un, {}};
     bsums<D, M, R>(local, z);
     if (kind != BK_TMS) L.us = nullptr;               // TMS local species use u_a^loc
     bstate_of<D, M, R>(L, z, __ldcg(Tf + n), m, un, status);

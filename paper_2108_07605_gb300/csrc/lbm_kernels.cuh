@@ -2097,7 +2097,7 @@ k_coll(const S* __restrict__ src, S* __restrict__ dst, const RT* __restrict__ cp
 // One thread per interface node: reconstruction and record (lbm_bnode.cuh);
 // the interface nodes' reaction sub-steps follow in k_chem.
 template <int D, int M, typename S>
-__global__ void __launch_bounds__(kBnd)
+__global__ void __launch_bounds__(kBnd, kBnodeMinBlocks<S>)
 k_bnode(const S* __restrict__ src, const __grid_constant__ BCDev bc, double* __restrict__ Tf,
         int* __restrict__ status, const __grid_constant__ Geom g,
         const __grid_constant__ Units un, const __grid_constant__ DevMech mech,
@@ -2282,7 +2282,7 @@ k_coll_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nblk)
 
 // One thread per interface node over every domain (the batched k_bnode).
 template <int D, int M, typename S>
-__global__ void __launch_bounds__(kBnd)
+__global__ void __launch_bounds__(kBnd, kBnodeMinBlocks<S>)
 k_bnode_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   using R = typename ComputeType<S>::type;
@@ -2451,7 +2451,7 @@ k_step_persist(const DomainDev* __restrict__ doms, int ndom, int parity,
       R* col = reinterpret_cast<R*>(ps_raw) + grp * E * kBnd + t;
       long long* sncol =
           reinterpret_cast<long long*>(ps_raw + sizeof(R) * E * kBnd * (kPersistThreads / kBnd)) +
-          grp * Q * kBnd + t;
+          grp * (Q / 3) * kBnd + t;
       const long long k = w.first + threadIdx.x;
       if (k < d.bc.n_if)
         bnode_body<D, M, S, R>(src, d.bc, static_cast<R*>(d.rec), d.Tf, d.status, d.g, d.un,
