@@ -59,6 +59,11 @@ template <typename RT> constexpr bool kFF = sizeof(RT) == 4 && !LBM_CHEM64;
 // 600x40x40 tube, with four 1.15, its 460 bytes of spills included; FP32 with
 // FP64 chemistry on the 2000x40 channel 0.19 ms with two, 0.11 with four
 constexpr int kMomentsMinBlocks = 4;
+// Blocks per SM that k_prep's registers are held to.  FP32 (latency of the
+// gradients' loads and of the elimination): four, 128 registers; with three, as
+// the compiler chose, 600x40x40 tube 47.5 against 45.4 ms per 24 steps, uneven
+// FP32 batch 43.0 against 39.7.  FP64: two, by its shared memory (110 KB).
+template <typename RT> constexpr int kPrepMinBlocks = sizeof(RT) == 4 ? 4 : 2;
 
 // Arithmetic type of a storage type: FP16 storage computes in FP32.
 template <typename S> struct ComputeType { using type = S; };
@@ -2074,7 +2079,7 @@ k_collide(const S* __restrict__ src, S* __restrict__ dst, const RT* __restrict__
 }
 
 template <int D, int M, typename RT>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, kPrepMinBlocks<RT>)
 k_prep(const RT* __restrict__ rec, const double* __restrict__ Tf, RT* __restrict__ cp,
        const __grid_constant__ Geom g, const __grid_constant__ Units un,
        const __grid_constant__ BCDev bc, const __grid_constant__ DevMech mech) {
@@ -2251,7 +2256,7 @@ k_collide_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nb
 }
 
 template <int D, int M, typename RT>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, kPrepMinBlocks<RT>)
 k_prep_batch(const DomainDev* __restrict__ doms, int ndom, int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
