@@ -29,7 +29,7 @@ constexpr int kBnd = kBndNodesPerBlock;   // threads per block of the boundary k
 // Blocks per SM its registers are held to.  Bound by latency, not by a pipe
 // (FP64: pipe 45 % busy; FP32: 3.8 warps per SM quarter in all): what counts is
 // loads in flight, by the directions unrolled three rows deep, and warps.
-// 600x40x40 tube, 74k interface nodes: FP64 1.22 -> 1.11 ms (255 registers);
+// 600x40x40 tube, 91k interface nodes: FP64 1.22 -> 1.11 ms (255 registers);
 // FP32 0.44 -> 0.32 ms at 168 registers and six blocks, 0.41 at eight (128
 // registers, spills) and at four (240); FP16 0.52 -> 0.37.
 template <typename S> constexpr int kBnodeMinBlocks = sizeof(S) == 8 ? 4 : 6;

@@ -139,7 +139,7 @@ struct BCDev {
 
 // Kernel placement of a step (lbm_launch, resolved).
 struct Launch {
-  int chem_lanes = 1;    // 1: chemistry inside the moments kernel; 4 or 8: k_chem lanes per node
+  int chem_lanes = 1;    // 1: a thread per bulk node (k_moments); 4 or 8: lanes per node (k_mchem)
   int coll_split = 0;    // 0: fused collision; 1: k_prep + k_coll
   int persistent = 0;    // batched kernels: 1 = grids of the resident blocks, looping over
                          // tiles; 2 = the whole step as one launch over a work-list
@@ -181,7 +181,7 @@ struct DomainDev {
   int block_begin = 0;         // first block of this domain in the node grids
   int bblock_begin = 0;        // first block in the interface-chemistry grid
   int tblock_begin = 0;        // first block in the thread-per-interface-node grid (k_bnode)
-  int cblock_begin = 0;        // first block in the chemistry grid (k_chem)
+  int cblock_begin = 0;        // first block in the lane-group grid (k_mchem)
   int kblock_begin = 0;        // first block in the split-collision grid (k_coll)
 };
 
@@ -226,7 +226,7 @@ struct BatchGrids {
   int nblocks = 0;    // node kernels, 128 nodes per block
   int nbblocks = 0;   // interface-chemistry grid, kIfChemNodesPerBlock nodes per block
   int ntblocks = 0;   // k_bnode, kBndNodesPerBlock interface nodes per block
-  int ncblocks = 0;   // k_chem, 128 / chem_lanes nodes per block (0 without it)
+  int ncblocks = 0;   // k_mchem, 128 / chem_lanes nodes per block (0 without it)
   int nkblocks = 0;   // k_coll, 32 nodes per block (0 without it)
   long long n_if_total = 0;   // interface nodes of every domain
   int bnd_warp = 0;           // the boundary grid holds kBnodeWarps nodes per block
@@ -244,7 +244,7 @@ struct BatchGrids {
 // the boundary kernel with a warp per node, which does more work in all but
 // not in one chain.  Steps of the 1024x4x4 flame (32 nodes): 0.29 ms against
 // 0.60 in FP64, 0.15 against 0.34 in FP32; of a mixed FP32 batch (2816 nodes)
-// 2.2 against 2.7; of the 2000x40 channel (4078 nodes) 0.69 against 0.75 in
+// 2.2 against 2.7; of the 2000x40 channel (4076 nodes) 0.69 against 0.75 in
 // FP64, 0.28 against 0.31 in FP32 with FP64 chemistry.
 constexpr int kBnodeWarpNodes = 6144;
 // nodes (warps) per block of it

@@ -4,8 +4,10 @@
 //   k_bnode     one thread per interface node: gather, bounce-back / TMS /
 //               inlet / LODI outlet reconstruction, the node's moment record
 //               (lbm_bnode.cuh).
-//   k_iface_chem, k_chem  the interface nodes' reaction sub-steps (a thread
-//               or a lane group per node).
+//   k_bnode_warp  the same and the node's reaction sub-steps with one warp per
+//               interface node (few of them).
+//   k_iface_chem, k_chem  the interface nodes' reaction sub-steps after k_bnode
+//               (a thread or eight lanes per node).
 //   k_moments   one thread per bulk node: pull-stream all lattices, moments,
 //               temperature Newton, the reaction sub-steps, the moment
 //               record (scratch) and the T guess.
@@ -23,7 +25,9 @@
 //
 // Template parameters: D (2 or 3), M (species), S (storage type), RT (type
 // of the lattice arithmetic: moments, equilibria, collision).  FP64 storage
-// computes everything in FP64.  FP32 and FP16 storage compute the lattice
+// computes to FP64 rounding; what can runs beside the FP64 pipe (population sums
+// in fixed point, rates, diffusion velocities and the Stefan-Maxwell term in
+// float-float).  FP32 and FP16 storage compute the lattice
 // arithmetic and transport in FP32 and the temperature Newton solve and the
 // chemistry in float-float (ff.cuh) or, with LBM_CHEM64, in FP64.
 #include <atomic>
@@ -59,6 +63,10 @@ template <typename RT> constexpr bool kFF = sizeof(RT) == 4 && !LBM_CHEM64;
 // 600x40x40 tube, with four 1.15, its 460 bytes of spills included; FP32 with
 // FP64 chemistry on the 2000x40 channel 0.19 ms with two, 0.11 with four
 constexpr int kMomentsMinBlocks = 4;
+// ... of the single-domain kernel with float-float chemistry five: 24 steps of
+// the tube 45.4 against 44.3 ms; the batch kernel, which holds its domain's
+// descriptor as well, four (uneven FP32 batch 39.7 against 41.0 with five)
+template <typename RT> constexpr int kMoments1MinBlocks = kFF<RT> ? 5 : kMomentsMinBlocks;
 // Blocks per SM that k_prep's registers are held to.  FP32 (latency of the
 // gradients' loads and of the elimination): four, 128 registers; with three, as
 // the compiler chose, 600x40x40 tube 47.5 against 45.4 ms per 24 steps, uneven
@@ -353,9 +361,8 @@ template <int D, int M, typename RT, int L>
 __device__ __forceinline__ void chem_lanes_body(RT* __restrict__ rec,
                                                 const double* __restrict__ Tf,
                                                 int* __restrict__ status, long long N,
-                                                const int* __restrict__ tag, const Units& un,
-                                                const DevMech& m, long long n, int sub,
-                                                unsigned gmask) {
+                                                const Units& un, const DevMech& m,
+                                                long long n, int sub, unsigned gmask) {
   using CT = typename ChemType<RT>::type;
   using X = Chem<CT>;
   using RC = Rec<D, M>;
@@ -1017,7 +1024,7 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
                                             const Units& un, const BCDev& bc,
                                             const DevMech& mech, long long n, int tag,
                                             NodePar<D, M, RT>& p) {
-  constexpr int Q = Lat<D>::Q, NP = Lat<D>::NP;
+  constexpr int Q = Lat<D>::Q;
   using RC = Rec<D, M>;
   const long long N = g.N;
   const int x = (int)(n % g.nx);
@@ -1999,13 +2006,12 @@ __device__ __forceinline__ void coll_block(const S* __restrict__ src, S* __restr
 // ---------------------------------------------------------------------------
 // Single-domain kernels: one thread per node (moments, collision), one thread
 // per interface node (k_bnode: boundary reconstruction and record).
-// Node sets: every node, the nodes without boundary reconstruction (the
-// bulk), or the interface nodes (whose sub-steps follow k_bnode, on a side
-// stream concurrent with the bulk).
-enum { NODES_ALL = 0, NODES_BULK = 1, NODES_INTERFACE = 2 };
+// Node sets: every node, or the nodes without boundary reconstruction (the
+// bulk; the interface nodes run on a side stream concurrent with it).
+enum { NODES_ALL = 0, NODES_BULK = 1 };
 
 template <int D, int M, typename S, typename RT>
-__global__ void __launch_bounds__(128, kMomentsMinBlocks)
+__global__ void __launch_bounds__(128, kMoments1MinBlocks<RT>)
 k_moments(const S* __restrict__ src, RT* __restrict__ rec, double* __restrict__ Tf,
           int* __restrict__ status, const __grid_constant__ Geom g,
           const __grid_constant__ Units un, const __grid_constant__ BCDev bc,
@@ -2016,37 +2022,29 @@ k_moments(const S* __restrict__ src, RT* __restrict__ rec, double* __restrict__ 
   moments_body<D, M, S, RT>(src, rec, Tf, status, g, un, bc, mech, n, moments_static<M>());
 }
 
-// reaction sub-steps, L lanes per node, 128 threads per block.  Node sets:
-// every node, the nodes without boundary reconstruction (their chemistry
-// runs beside the boundary kernel on the side stream), or the interface
-// nodes (entry `first` of the interface list, after the boundary kernel)
-template <int D, int M, typename RT, int L>
+// The reaction sub-steps of the interface nodes from entry `first` of their
+// list, after the boundary kernel: kIfLanes lanes per node, 128 threads per block.
+constexpr int kIfLanes = 8;
+static_assert(128 / kIfLanes == kIfChemNodesPerBlock, "the interface-chemistry grid");
+template <int D, int M, typename RT>
 __device__ __forceinline__ void chem_entry(RT* rec, const double* Tf, int* status, long long N,
-                                           const int* tag, const Units& un, const DevMech& m,
-                                           long long first, int node_set, const int* if_node,
-                                           int n_if) {
+                                           const Units& un, const DevMech& m, long long first,
+                                           const int* if_node, int n_if) {
   const int lane = threadIdx.x & 31;
-  const long long idx = first + threadIdx.x / L;
-  long long n = idx;
-  if (node_set == NODES_INTERFACE) {                    // the whole group leaves
-    if (idx >= n_if) return;
-    n = if_node[idx];
-  } else {
-    if (n >= N) return;
-    if (tag && (tag[n] == TAG_SOLID || (node_set == NODES_BULK && tag[n] >= 0))) return;
-  }
-  const unsigned gmask = (L == 32 ? 0xffffffffu : ((1u << L) - 1u) << (lane & ~(L - 1)));
-  chem_lanes_body<D, M, RT, L>(rec, Tf, status, N, tag, un, m, n, lane & (L - 1), gmask);
+  const long long k = first + threadIdx.x / kIfLanes;
+  if (k >= n_if) return;                                // the whole group leaves
+  const unsigned gmask = ((1u << kIfLanes) - 1u) << (lane & ~(kIfLanes - 1));
+  chem_lanes_body<D, M, RT, kIfLanes>(rec, Tf, status, N, un, m, if_node[k],
+                                      lane & (kIfLanes - 1), gmask);
 }
 
-template <int D, int M, typename RT, int L>
+template <int D, int M, typename RT>
 __global__ void __launch_bounds__(128)
 k_chem(RT* __restrict__ rec, const double* __restrict__ Tf, int* __restrict__ status,
-       long long N, const int* __restrict__ tag, const __grid_constant__ Units un,
-       const DevMech* __restrict__ mech, int node_set, const int* __restrict__ if_node,
-       int n_if) {
-  chem_entry<D, M, RT, L>(rec, Tf, status, N, tag, un, *mech, blockIdx.x * (128LL / L), node_set,
-                          if_node, n_if);
+       long long N, const __grid_constant__ Units un, const DevMech* __restrict__ mech,
+       const int* __restrict__ if_node, int n_if) {
+  chem_entry<D, M, RT>(rec, Tf, status, N, un, *mech, blockIdx.x * (128LL / kIfLanes), if_node,
+                       n_if);
 }
 
 // moments and reaction sub-steps, L lanes per node, 128 threads per block,
@@ -2199,24 +2197,15 @@ k_moments_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int no
   }
 }
 
-// NODES_INTERFACE: the interface-chemistry grid (128 / L interface nodes
-// per block, L lanes each, as k_chem)
-template <int D, int M, typename RT, int L>
+// k_chem over the interface nodes of several handles
+template <int D, int M, typename RT>
 __global__ void __launch_bounds__(128)
-k_chem_batch(const DomainDev* __restrict__ doms, int ndom, int node_set, int nblk) {
+k_chem_batch(const DomainDev* __restrict__ doms, int ndom, int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
-    if (node_set == NODES_INTERFACE) {
-      const DomainDev& d = bd.get(doms, domain_of_block(doms, ndom, b, GRID_BOUNDARY));
-      chem_entry<D, M, RT, L>(static_cast<RT*>(d.rec), d.Tf, d.status, d.g.N, d.bc.tag, d.un,
-                              *d.mech, (b - d.bblock_begin) * (128LL / L), NODES_INTERFACE,
-                              d.bc.if_node, d.bc.n_if);
-    } else {
-      const DomainDev& d = bd.get(doms, domain_of_block(doms, ndom, b, GRID_CHEM));
-      chem_entry<D, M, RT, L>(static_cast<RT*>(d.rec), d.Tf, d.status, d.g.N, d.bc.tag, d.un,
-                              *d.mech, (b - d.cblock_begin) * (128LL / L), node_set, nullptr,
-                              0);
-    }
+    const DomainDev& d = bd.get(doms, domain_of_block(doms, ndom, b, GRID_BOUNDARY));
+    chem_entry<D, M, RT>(static_cast<RT*>(d.rec), d.Tf, d.status, d.g.N, d.un, *d.mech,
+                         (b - d.bblock_begin) * (128LL / kIfLanes), d.bc.if_node, d.bc.n_if);
   }
 }
 
@@ -2681,7 +2670,6 @@ __global__ void __launch_bounds__(128)
 k_diag(const S* __restrict__ pops, const double* __restrict__ Tf, const int* __restrict__ tag,
        DiagPart* __restrict__ part, int* __restrict__ status, Geom g, Units un,
        const __grid_constant__ DevMech mech, int x0, int x1) {
-  constexpr int Q = Lat<D>::Q;
   __shared__ double s_sum[128], s_qmax[128], s_T[128], s_u[128];
   __shared__ long long s_n[128];
   const long long N = g.N;
@@ -2814,27 +2802,18 @@ static cudaError_t prepare_impl() {
   return e;
 }
 
+// the interface nodes' reaction sub-steps after k_bnode: a thread each where
+// these fill the GPU, else eight lanes
 template <int D, int M, typename RT>
-static void launch_chem(const Launch& lc, cudaStream_t s, RT* rec, const double* Tf,
-                        int* status, long long N, const BCDev& bc, const Units& un,
-                        const DevMech* mech, int node_set) {
-  if (node_set == NODES_INTERFACE && bc.n_if >= kIfChemThreadNodes) {
-    const size_t sm = chem_slice_bytes<M>();
-    k_iface_chem<D, M, RT><<<blocks_for(bc.n_if, kChemThreads), kChemThreads, sm, s>>>(
-        rec, Tf, status, N, bc.if_node, bc.n_if, un, mech);
-    return;
-  }
-  // fewer interface nodes: on the critical path, 8 lanes each
-  const int lanes = node_set == NODES_INTERFACE ? 8 : lc.chem_lanes;
-  const long long n = node_set == NODES_INTERFACE ? bc.n_if : N;
-  const unsigned nblk = blocks_for(n, 128 / lanes);
-  if (nblk == 0) return;
-  if (lanes == 4)
-    k_chem<D, M, RT, 4><<<nblk, 128, 0, s>>>(rec, Tf, status, N, bc.tag, un, mech, node_set,
-                                             bc.if_node, bc.n_if);
+static void launch_chem(cudaStream_t s, RT* rec, const double* Tf, int* status, long long N,
+                        const BCDev& bc, const Units& un, const DevMech* mech) {
+  if (bc.n_if >= kIfChemThreadNodes)
+    k_iface_chem<D, M, RT>
+        <<<blocks_for(bc.n_if, kChemThreads), kChemThreads, chem_slice_bytes<M>(), s>>>(
+            rec, Tf, status, N, bc.if_node, bc.n_if, un, mech);
   else
-    k_chem<D, M, RT, 8><<<nblk, 128, 0, s>>>(rec, Tf, status, N, bc.tag, un, mech, node_set,
-                                             bc.if_node, bc.n_if);
+    k_chem<D, M, RT><<<blocks_for(bc.n_if, kIfChemNodesPerBlock), 128, 0, s>>>(
+        rec, Tf, status, N, un, mech, bc.if_node, bc.n_if);
 }
 
 // prepare_impl once per device and instantiation
@@ -2865,10 +2844,8 @@ static cudaError_t step_impl(const DevMech& mech, const StepArgs& a, cudaStream_
     const S* src = static_cast<const S*>(a.src);
     RT* rec = reinterpret_cast<RT*>(a.rec);
     // chem_lanes > 1: the bulk nodes' moments and reaction sub-steps in one
-    // kernel with chem_lanes lanes per node (k_mchem); the boundary warps
-    // write their nodes' records and the interface nodes' sub-steps follow
-    // in k_chem.  chem_lanes = 1: k_moments with the sub-steps inline, the
-    // interface nodes' moments after the boundary kernel.
+    // kernel with chem_lanes lanes per node (k_mchem).  chem_lanes = 1:
+    // k_moments with the sub-steps inline.
     auto mchem = [&](cudaStream_t st, int node_set) {
       const unsigned nbm = blocks_for(a.g.N, 128 / lc.chem_lanes);
       if (lc.chem_lanes == 4)
@@ -2893,8 +2870,7 @@ static cudaError_t step_impl(const DevMech& mech, const StepArgs& a, cudaStream_
       }
       k_bnode<D, M, S><<<blocks_for(a.bc.n_if, kBnd), kBnd, bnode_smem<D, M, RT>(), st>>>(
           src, a.bc, a.Tfield, a.status, a.g, a.un, mech, rec);
-      launch_chem<D, M, RT>(lc, st, rec, a.Tfield, a.status, a.g.N, a.bc, a.un, a.mech_dev,
-                            NODES_INTERFACE);
+      launch_chem<D, M, RT>(st, rec, a.Tfield, a.status, a.g.N, a.bc, a.un, a.mech_dev);
     };
     auto bulk = [&](int node_set) {
       if (chem_sep)
@@ -3016,26 +2992,17 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
                                                                     gr.ntblocks);
     }
   };
-  // the reaction sub-steps in k_chem over a node set (the grid of the set)
-  static_assert(128 / 8 == kIfChemNodesPerBlock, "interface chemistry: 8 lanes per node");
-  auto chem = [&](int node_set, cudaStream_t st) {
+  // the interface nodes' reaction sub-steps after the thread-per-node kernel
+  auto chem = [&](cudaStream_t st) {
     if (gr.bnd_warp) return;          // done by the boundary kernel
-    if (node_set == NODES_INTERFACE && gr.n_if_total >= kIfChemThreadNodes) {
+    if (gr.n_if_total >= kIfChemThreadNodes) {
       // enough interface nodes to fill the GPU with one thread each
       auto k = k_iface_chem_batch<D, M, RT>;
       const size_t sm = chem_slice_bytes<M>();
       k<<<batch_grid(k, gr.ntblocks, kBnd, sm, ps), kBnd, sm, st>>>(doms, ndom, gr.ntblocks);
-      return;
-    }
-    const int nb = node_set == NODES_INTERFACE ? gr.nbblocks : gr.ncblocks;
-    if (nb == 0) return;
-    // the interface nodes are few and on the critical path: 8 lanes each
-    if (lc.chem_lanes == 4 && node_set != NODES_INTERFACE) {
-      auto k = k_chem_batch<D, M, RT, 4>;
-      k<<<batch_grid(k, nb, 128, 0, ps), 128, 0, st>>>(doms, ndom, node_set, nb);
     } else {
-      auto k = k_chem_batch<D, M, RT, 8>;
-      k<<<batch_grid(k, nb, 128, 0, ps), 128, 0, st>>>(doms, ndom, node_set, nb);
+      auto k = k_chem_batch<D, M, RT>;
+      k<<<batch_grid(k, gr.nbblocks, 128, 0, ps), 128, 0, st>>>(doms, ndom, gr.nbblocks);
     }
   };
   // chem_lanes > 1: moments and sub-steps of the nodes in one kernel with
@@ -3054,15 +3021,12 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
   };
   if (gr.nbblocks > 0 && side.stream && side.fork && side.join) {
     // on the side stream, concurrent with the bulk moments: the boundary
-    // kernel, then the interface nodes' moments (reaction sub-steps inline)
-    // or, with the boundary warps writing the records, their sub-steps
+    // kernel and the interface nodes' sub-steps
     cudaError_t e = cudaEventRecord(side.fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side.stream, side.fork, 0);
     if (e != cudaSuccess) return e;
-    // (the interface nodes: records by the boundary warps, sub-steps with
-    // eight lanes per node, whatever the bulk placement)
     bnd(side.stream);
-    chem(NODES_INTERFACE, side.stream);
+    chem(side.stream);
     e = cudaEventRecord(side.join, side.stream);
     if (e != cudaSuccess) return e;
     if (chem_inline)
@@ -3081,7 +3045,7 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
           doms, ndom, parity, bnd_rec ? NODES_BULK : NODES_ALL, gr.nblocks);
     else
       mchem(bnd_rec ? NODES_BULK : NODES_ALL);
-    if (bnd_rec) chem(NODES_INTERFACE, s);
+    if (bnd_rec) chem(s);
   }
   if (lc.coll_split) {
     auto kp = k_prep_batch<D, M, RT>;
