@@ -63,8 +63,11 @@ typedef enum {
 
 typedef enum { LBM_D2Q9 = 0, LBM_D3Q27 = 1 } lbm_lattice;
 
-/* Storage precision of the populations.  LBM_FP64: every operation in FP64
- * (the path checked against the oracle to 1e-10).  LBM_FP32_STORE:
+/* Storage precision of the populations.  LBM_FP64: results to
+ * FP64 rounding (the path checked against the oracle to 1e-10); what is summed
+ * exactly or enters as a small correction runs in fixed point or in pairs of
+ * FP32 (~48 significant bits) beside the FP64 pipe, with no larger error than
+ * in FP64 throughout.  LBM_FP32_STORE:
  * populations, moments and collision in FP32; the temperature Newton solve
  * and the chemistry in float-float (pairs of FP32, ~48 significant bits);
  * transport in FP32.  LBM_FP16_OFFSET: the FP32 path's arithmetic, with
@@ -237,15 +240,13 @@ lbm_status lbm_step(lbm_t h, int nsteps);
 
 /* Advance several handles by nsteps steps together, in the placement a
  * batch plan of the same handles starts with (see lbm_batch_set_launch):
- * FP64 storage under 311,296 nodes in all, each step is ONE persistent
- * launch over a work-list of the handles' tiles (persistent = 2); else one
- * launch per kernel over the concatenated tiles (128-node tiles, 64
- * interface nodes per boundary block), so many small domains fill the GPU.
+ * one launch per kernel over the concatenated tiles (128-node tiles; the
+ * interface nodes with a warp each up to 6,144 of them in all, else with a
+ * thread each), so many small domains fill the GPU.
  * The handles must share lattice, species count, precision and device; each
  * keeps its own mechanism, units and boundaries.  The work runs on hs[0]'s
  * stream after the earlier work of every handle's stream, and every
- * handle's stream waits for it; with the single launch the call returns
- * after the work (its work-list is freed).  Results equal n separate
+ * handle's stream waits for it.  Results equal n separate
  * lbm_step calls to rounding (the same per-node arithmetic, summed in
  * another order where the placements differ). */
 lbm_status lbm_batch_step(lbm_t* hs, int n, int nsteps);
@@ -268,19 +269,19 @@ lbm_status lbm_batch_destroy(lbm_batch_t b);
  *                  group of that many lanes per node shares the pull, the
  *                  temperature solve and the node's reactions (for grids too
  *                  small to fill the GPU at one thread per node); -1 = by
- *                  grid size.  Interface nodes (boundary reconstruction) take
- *                  their sub-steps, in every placement, with one thread each
- *                  when a grid has at least 19,456 of them and with eight
- *                  lanes each otherwise (the single launch of a plan: one
- *                  thread each).
+ *                  grid size.  Interface nodes (boundary reconstruction, then
+ *                  their sub-steps) take, in every placement, a warp each up
+ *                  to 6,144 of them; beyond, a thread each, the sub-steps with
+ *                  eight lanes each below 19,456 (the single launch of a plan:
+ *                  one thread each).
  *   collide_split  0 = one thread per node does the whole collision; 1 = a
  *                  per-node kernel stores the collision parameters and a
  *                  second kernel updates the directions with nine threads
  *                  per node; -1 = default.
- * Defaults (below 77,824 nodes, four 128-thread blocks per SM of a 152-SM
- * GPU, a grid is small): collide_split 0 for FP64 storage on grids that are
- * not small (except the single launch of a plan, see persistent), else 1;
- * chem_lanes 4 for small FP32-storage grids, else 1.
+ * Defaults: collide_split 1; chem_lanes 4 for FP32 and FP16 storage on grids
+ * of up to 14,592 nodes (three 128-thread blocks of four lanes per node on
+ * each SM of a 152-SM GPU), with interface nodes up to 4,864 (one block per
+ * SM), else 1.
  * lbm_set_launch rejects other values with LBM_ERR_INVALID. */
 typedef struct {
   int chem_lanes;
@@ -300,8 +301,7 @@ typedef struct {
                          dependency wait that outlasts 4 s
                          ends the launch and the handles report
                          LBM_ERR_TIMEOUT; 0 = one block per tile; -1 = the
-                         default: 2 for plans of FP64 storage below 311,296
-                         nodes in all, else 0 */
+                         default, 0 */
   int nodes_per_thread;  /* persistent = 2: nodes per thread of the node
                          tiles, 1, 2 or 4 (tiles of 128, 256, 512 nodes);
                          -1 = 1 */

@@ -57,20 +57,23 @@ lbm_status cuda_fail(lbm_ctx* h, cudaError_t e, const char* where) {
 }
 
 // Default placement, measured on one GB300.  The split collision is faster
-// than the fused one on every grid tried (FP64 and FP32).  Below kSmallGrid
-// nodes a thread-per-node grid of the FP32 path holds fewer than four
-// 128-thread blocks per SM of a 152-SM GB300, too few warps to hide the latency
-// of the float-float chemistry, which then runs with four lanes per node; in
-// FP64 the extra redundant work of the lanes costs more than it hides.  Batch
-// plans take one launch per kernel (six reactors and flames of 69k nodes in
-// all, FP64: 0.84 ms per step against 1.05 as a single launch over the
-// work-list, whose registers the kernels' largest stage sets).
-constexpr long long kSmallGrid = 152LL * 4 * 128;
-Launch resolve_launch(const lbm_launch& opt, long long nodes, lbm_precision prec) {
+// than the fused one on every grid tried (FP64 and FP32).  In FP32 and FP16
+// storage a grid whose blocks with four lanes per node are all resident at once
+// hides the latency of the float-float chemistry that way: three 128-thread
+// blocks per SM without interface nodes (ms per step with 1 / 4 lanes, FP32:
+// 4096 nodes 0.084 / 0.068, 13824 0.093 / 0.081, 21952 0.103 / 0.125), one per SM
+// beside the boundary kernel (4096 nodes 0.096 / 0.080, 8192 0.097 / 0.124).  In
+// FP64 the lanes' redundant work costs what it hides (4096 nodes 0.16 / 0.14,
+// 5832 0.170 / 0.175; 2-D channel, 4000 nodes, 0.124 / 0.127).  Batch plans take
+// one launch per kernel (six reactors and flames of 69k nodes in all, FP64: 0.67
+// ms per step against 1.15 as a single launch over the work-list, whose
+// registers the kernels' largest stage sets).
+constexpr long long kLaneNodes = 152LL * 128 / 4;   // four lanes each: one block per SM
+Launch resolve_launch(const lbm_launch& opt, long long nodes, long long n_if,
+                      lbm_precision prec) {
   Launch lc;
-  const bool small = nodes < kSmallGrid;
-  lc.chem_lanes = opt.chem_lanes > 0 ? opt.chem_lanes
-                                     : (small && prec == LBM_FP32_STORE ? 4 : 1);
+  const bool lanes = prec != LBM_FP64 && nodes <= (n_if > 0 ? 1 : 3) * kLaneNodes;
+  lc.chem_lanes = opt.chem_lanes > 0 ? opt.chem_lanes : (lanes ? 4 : 1);
   lc.persistent = opt.persistent >= 0 ? opt.persistent : 0;
   lc.coll_split = opt.collide_split >= 0 ? opt.collide_split : 1;
   lc.npt = opt.nodes_per_thread > 0 ? opt.nodes_per_thread : 1;
@@ -80,6 +83,18 @@ Launch resolve_launch(const lbm_launch& opt, long long nodes, lbm_precision prec
 // every placement the autotuners try
 const Launch kCandidates[] = {{1, 0}, {4, 0}, {8, 0}, {1, 1}, {4, 1}, {8, 1}};
 
+// nodes of several handles
+long long total_nodes(lbm_ctx* const* hs, int n) {
+  long long t = 0;
+  for (int k = 0; k < n; ++k) t += hs[k]->g.N;
+  return t;
+}
+long long total_if(lbm_ctx* const* hs, int n) {      // ... and interface nodes
+  long long t = 0;
+  for (int k = 0; k < n; ++k) t += hs[k]->bc.n_if;
+  return t;
+}
+
 // Domains of a batched step: each handle's tiles follow the previous
 // handle's in every grid (128 nodes per node-kernel block, 16 interface nodes
 // per interface-chemistry block, 128 / chem_lanes nodes per chemistry block,
@@ -88,7 +103,7 @@ void fill_domains(lbm_ctx* const* hs, int n, const Launch& lc, std::vector<Domai
                   BatchGrids& gr) {
   doms.assign(n, DomainDev());
   gr = BatchGrids();
-  for (int k = 0; k < n; ++k) gr.n_if_total += hs[k]->bc.n_if;
+  gr.n_if_total = total_if(hs, n);
   gr.bnd_warp = gr.n_if_total <= kBnodeWarpNodes;
   const int per_bnd = gr.bnd_warp ? kBnodeWarps : kBndNodesPerBlock;
   for (int k = 0; k < n; ++k) {
@@ -120,12 +135,6 @@ void fill_domains(lbm_ctx* const* hs, int n, const Launch& lc, std::vector<Domai
     if (lc.coll_split)
       gr.nkblocks += (int)((h->g.N + kCollNodesPerBlock - 1) / kCollNodesPerBlock);
   }
-}
-
-long long total_nodes(lbm_ctx* const* hs, int n) {
-  long long t = 0;
-  for (int k = 0; k < n; ++k) t += hs[k]->g.N;
-  return t;
 }
 
 void* dalloc(const lbm_config& c, size_t bytes) {
@@ -930,7 +939,7 @@ lbm_status lbm_step(lbm_t h, int nsteps) {
   a.g = h->g;
   a.un = h->un;
   a.bc = h->bc;
-  a.lc = resolve_launch(h->opt, h->g.N, h->cfg.precision);
+  a.lc = resolve_launch(h->opt, h->g.N, h->bc.n_if, h->cfg.precision);
   a.mech_dev = h->mech_dev;
   a.cpar = h->cpar;
   a.side = h->side;
@@ -963,7 +972,7 @@ lbm_status lbm_step_timed(lbm_t h, int nsteps, double* kernel_ms, int n_kernels)
   a.g = h->g;
   a.un = h->un;
   a.bc = h->bc;
-  a.lc = resolve_launch(h->opt, h->g.N, h->cfg.precision);
+  a.lc = resolve_launch(h->opt, h->g.N, h->bc.n_if, h->cfg.precision);
   a.mech_dev = h->mech_dev;
   a.cpar = h->cpar;
   a.side = h->side;
@@ -1012,7 +1021,7 @@ lbm_status lbm_set_launch(lbm_t h, const lbm_launch* l) {
 
 lbm_status lbm_get_launch(lbm_t h, lbm_launch* l) {
   if (!h || !l) return fail(h, LBM_ERR_INVALID, "handle or launch is NULL");
-  const Launch lc = resolve_launch(h->opt, h->g.N, h->cfg.precision);
+  const Launch lc = resolve_launch(h->opt, h->g.N, h->bc.n_if, h->cfg.precision);
   l->chem_lanes = lc.chem_lanes;
   l->collide_split = lc.coll_split;
   l->persistent = lc.persistent;
@@ -1081,7 +1090,7 @@ lbm_status lbm_autotune(lbm_t h, int trial_steps, lbm_launch* chosen) {
   h->opt.collide_split = best.coll_split;
   if (chosen) {
     *chosen = h->opt;
-    const Launch r = resolve_launch(h->opt, h->g.N, h->cfg.precision);
+    const Launch r = resolve_launch(h->opt, h->g.N, h->bc.n_if, h->cfg.precision);
     chosen->persistent = r.persistent;
     chosen->nodes_per_thread = r.npt;
   }
@@ -1111,7 +1120,7 @@ lbm_status lbm_batch_step(lbm_t* hs, int n, int nsteps) {
   BatchGrids gr;
   // the placement a new plan of these handles starts with
   const Launch lc = resolve_launch(lbm_launch{-1, -1, -1, -1}, total_nodes(hs, n),
-                                   hs[0]->cfg.precision);
+                                   total_if(hs, n), hs[0]->cfg.precision);
   fill_domains(hs, n, lc, doms, gr);
   // every handle's earlier work precedes the batch; the batch runs on the
   // first handle's stream and each handle's stream waits for it afterwards
@@ -1296,7 +1305,8 @@ lbm_status lbm_batch_create(lbm_t* hs, int n, lbm_batch_t* out) {
     b->ddev = static_cast<DomainDev*>(dalloc(h0->cfg, n * sizeof(DomainDev)));
     if (!b->ddev) e = cudaErrorMemoryAllocation;
   }
-  b->lc = resolve_launch(lbm_launch{-1, -1, -1, -1}, total_nodes(hs, n), hs[0]->cfg.precision);
+  b->lc = resolve_launch(lbm_launch{-1, -1, -1, -1}, total_nodes(hs, n), total_if(hs, n),
+                         hs[0]->cfg.precision);
   if (e == cudaSuccess) e = batch_upload(b);
   if (e == cudaSuccess) e = prepare_batch_step(h0->D, h0->M, kernel_precision(h0->cfg));
   if (e == cudaSuccess) e = batch_capture_all(b);
@@ -1357,7 +1367,9 @@ lbm_status lbm_batch_set_launch(lbm_batch_t b, const lbm_launch* l) {
     return fail(h0, LBM_ERR_INVALID, "placement out of range");
   DeviceGuard dg(h0->cfg.device);
   cudaError_t e = cudaStreamSynchronize(b->stream);
-  b->lc = resolve_launch(*l, total_nodes(b->hs.data(), (int)b->hs.size()), h0->cfg.precision);
+  const int n = (int)b->hs.size();
+  b->lc = resolve_launch(*l, total_nodes(b->hs.data(), n), total_if(b->hs.data(), n),
+                         h0->cfg.precision);
   if (e == cudaSuccess) e = batch_upload(b);
   if (e == cudaSuccess) e = batch_capture_all(b);
   return e == cudaSuccess ? LBM_OK : cuda_fail(h0, e, "batch placement");
