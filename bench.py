@@ -228,20 +228,47 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def launch_groups(launch, has_bnd):
-    """Names of the two timed launch groups of a step (lbm_step_timed): the
-    kernels before the collision, and the collision."""
-    g0 = (["k_boundary", "k_chem"] if has_bnd else []) + \
-        ["k_mchem" if launch["chem_lanes"] > 1 else "k_moments"]
-    return ["+".join(g0), "k_prep+k_coll" if launch["collide_split"] else "k_collide"]
+def interface_nodes(w):
+    """Nodes whose incoming populations the boundary kernel reconstructs: fluid
+    nodes on a face that is not periodic or with a solid neighbour."""
+    import numpy as np
+    if boundary_spec(w) is None:
+        return 0
+    nx, ny, nz = w["shape"]
+    mark = np.zeros((nz, ny, nx), bool)
+    for axis, (lo, hi) in enumerate(zip(w["faces"][0::2], w["faces"][1::2])):
+        plane = np.moveaxis(mark, 2 - axis, 0)
+        plane[0] |= lo != "periodic"
+        plane[-1] |= hi != "periodic"
+    if w.get("solid") is not None:
+        near = np.asarray(w["solid"], bool)
+        fluid = ~near
+        for axis in range(3):
+            near = near | np.roll(near, 1, axis) | np.roll(near, -1, axis)
+        mark = (mark | near) & fluid
+    return int(mark.sum())
 
 
-def launches_per_step(launch, has_bnd):
-    """Kernels one step launches: the moments with the reaction sub-steps
-    (k_moments or k_mchem), the collision (k_collide, or k_prep + k_coll);
-    with interface nodes also the boundary kernel and the interface nodes'
-    sub-steps (k_chem)."""
-    return 1 + (2 if has_bnd else 0) + (2 if launch["collide_split"] else 1)
+WARP_BOUNDARY_NODES = 6144    # up to here a warp per interface node, sub-steps included
+
+
+def step_kernels(launch, n_if):
+    """Kernels one step launches, in two groups (lbm_step_timed): the boundary
+    kernel with, for many interface nodes, their sub-steps in a kernel of
+    their own, and the moments with the reaction sub-steps; the collision."""
+    bnd = [] if n_if == 0 else \
+        ["k_bnode_warp"] if n_if <= WARP_BOUNDARY_NODES else ["k_bnode", "k_iface_chem"]
+    return (bnd + ["k_mchem" if launch["chem_lanes"] > 1 else "k_moments"],
+            ["k_prep", "k_coll"] if launch["collide_split"] else ["k_collide"])
+
+
+def launch_groups(launch, n_if):
+    """Names of the two timed launch groups of a step."""
+    return ["+".join(g) for g in step_kernels(launch, n_if)]
+
+
+def launches_per_step(launch, n_if):
+    return sum(len(g) for g in step_kernels(launch, n_if))
 
 
 def step_counters(workload, mode):
@@ -483,7 +510,7 @@ def main():
     N = int(w["P"].size)
     Nf = fluid_nodes(w)
     M = mech.n_species
-    has_bnd = boundary_spec(w) is not None
+    n_if = interface_nodes(w)
     peaks = measured_peaks()
     fma = {"fp64": lbm.lbm_fma_peak(True), "fp32": lbm.lbm_fma_peak(False)}
     stream = torch.cuda.current_stream()
@@ -530,7 +557,7 @@ def main():
     ms_per_step = total_ms / args.steps
     value = node_updates_per_s(Nf, args.steps, world, M, total_ms * 1e-3)
     roof = roofline(args.workload, args.precision, info, Nf, ms_per_step, peaks, fma)
-    names = launch_groups(launch, has_bnd)
+    names = launch_groups(launch, n_if)
 
     # end to end through the C ABI with host buffers
     e2e = None
@@ -621,7 +648,7 @@ def main():
                    else "state larger than L2", "parallelism": f"replicas x{world}",
                    "launch": launch},
         "roofline": roof, "cpu_baseline": cpu, "e2e": e2e,
-        "gpu_launches": launches_per_step(launch, has_bnd) * args.steps,
+        "gpu_launches": launches_per_step(launch, n_if) * args.steps,
         "kernel_ms_per_step": {names[0]: kms[0] / args.steps, names[1]: kms[1] / args.steps},
         "fma_peak_tflops": fma,
         "variants": variants,
