@@ -1,5 +1,5 @@
-// FP64 exponential of the reaction rates.  No counterpart in the paper (its
-// rates come from Cantera); a published method, restated.
+// FP64 exponential of the FP64 path's transport laws (powers of T/T0).  A
+// published method, restated.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -12,7 +12,7 @@ namespace lbm {
 // e^x = 2^m 2^(j/32) e^r, e^r - 1 by its Taylor polynomial to degree 6
 // (truncation below 4e-18), 2^(j/32) from a table of the nearest doubles
 // (60-digit arithmetic), 2^m added to the exponent field.  Within 2 ulp of
-// e^x; arguments beyond |x| = 700 (never met by the rates) and NaN go to
+// e^x; arguments beyond |x| = 700 (never met there) and NaN go to
 // the library exp.
 static __device__ const double kExp2Tab32[32] = {
     0x1.0000000000000p+0, 0x1.059b0d3158574p+0, 0x1.0b5586cf9890fp+0,
