@@ -186,7 +186,7 @@ typedef struct lbm_config {
   int chem_fp64;              /* with LBM_FP32_STORE: 1 runs the temperature
                                  Newton solves (Sec. 3.1 Eq. temperature) and
                                  the reaction sub-steps (Sec. 2.4 Eq. R3) in
-                                 native FP64 instead of float-float; the
+                                 LBM_FP64's way instead of float-float; the
                                  populations, moments, transport and
                                  collision stay FP32.  Ignored for LBM_FP64;
                                  LBM_ERR_INVALID with LBM_FP16_OFFSET.
