@@ -308,14 +308,15 @@ __device__ __forceinline__ ExpArg exp_arg(long long v) {
   a.rl = __fmul_rn(__int2float_rn(((f1 & 0xff) << 14) | (int)(fl & 0x3fffu)), 0x1p-46f);
   return a;
 }
-// 0 <= d < 2^(63 - bits) as an integer with `bits` fraction bits
+// 0 <= d < 2^(63 - bits) as an integer with `bits` fraction bits; the largest
+// integer above
 __device__ __forceinline__ long long fixed_of(double d, int bits) {
   const int h = __double2hiint(d);
   const unsigned long long m =
       ((unsigned long long)(unsigned)((h & 0xfffff) | 0x100000) << 42) |
       ((unsigned long long)(unsigned)__double2loint(d) << 10);    // 62 fraction bits
   const int sh = 62 + 1023 - bits - (h >> 20);
-  return (long long)(m >> min(max(sh, 0), 63));
+  return sh < 0 ? 0x7fffffffffffffffLL : (long long)(m >> min(sh, 63));
 }
 // x in FP64, through its fixed-point form
 __device__ __forceinline__ ExpArg exp_arg(double x) {

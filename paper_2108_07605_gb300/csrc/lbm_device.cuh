@@ -318,8 +318,11 @@ __device__ __forceinline__ TBasis<double> tbasis(const DevMech& m, double T) {
   b.invT = 1.0 / T;
   b.T = T;
   b.T2 = T * T;
-  const int h = __double2hiint(T);              // 128 <= T < 16384
-  b.fixed = m.fixed_args && h >= 0x40600000 && h < 0x40d00000;
+  // 128 < T < 16384: at 128 K itself 1/T = 2^-7 is one past its kBitsInvT bits
+  // (one bit fewer of it would leave the coefficients no room for activation
+  // energies above 377 kJ/mol)
+  const long long Tb = __double_as_longlong(T);
+  b.fixed = m.fixed_args && Tb > 0x4060000000000000LL && Tb < 0x40d0000000000000LL;
   b.q[0] = 0;
   b.q[1] = fixed_of(b.lnT, kBitsLnT);
   b.q[2] = fixed_of(b.invT, kBitsInvT);

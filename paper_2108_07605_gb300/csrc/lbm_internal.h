@@ -42,7 +42,7 @@ struct DevReaction {
   long long fq[3], rq[5];
 };
 // Fixed-point rate-constant logarithms: 46 fraction bits in the sum; the basis
-// functions ln T, 1/T, T, T^2 with these many (below 2^63 for 128 K <= T <
+// functions ln T, 1/T, T, T^2 with these many (below 2^63 for 128 K < T <
 // 16384 K), so the coefficients with 46 + 64 less those.
 constexpr int kArgBits = 46;
 constexpr int kBitsLnT = 59, kBitsInvT = 70, kBitsT = 49, kBitsT2 = 35;

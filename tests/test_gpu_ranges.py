@@ -1,0 +1,63 @@
+"""The kernels' arithmetic at the edges of its ranges, against the CPU oracle."""
+import numpy as np
+import pytest
+
+from lbm_workloads import fields
+from lbm_workloads.mechanism import h2_air_synthetic
+from oracle.diagnostics import diagnostics
+
+from helpers import make_gpu, make_oracle, max_rel_err_per_lattice, oracle_populations
+
+pytestmark = pytest.mark.gpu
+RTOL_FP64 = 1e-10      # relative per lattice, the bound of the other parity tests
+
+
+@pytest.fixture(scope="module")
+def mech():
+    return h2_air_synthetic()
+
+
+def _errors(mech, w, nsteps, precision="fp64"):
+    o, g = make_oracle(mech, w), make_gpu(mech, w, precision=precision)
+    o.step(nsteps)
+    g.step(nsteps)
+    err = max_rel_err_per_lattice(g.populations(), oracle_populations(o))
+    g.close()
+    return err
+
+
+# The fixed-point rate arguments hold 1/T below 2^-7 (T above 128 K) and T below
+# 2^14 K.
+def _at_temperature(mech, shape, T0):
+    w = fields.perturbed_box(shape, "D2Q9", mech=mech, T0=T0, amp_T=0.0, amp_u=0.0,
+                             dx=1e-6 if T0 < 200.0 else 1e-9)
+    w["Y"][:] = w["Y"][:, :1, :1, :1]      # radicals present
+    if T0 > 3000.0:
+        w["T_max"] = 17000.0
+    return w
+
+
+@pytest.mark.parametrize("T0", [128.0, 16384.0])
+def test_heat_release_at_the_bounds_of_the_rate_arguments(mech, T0):
+    """Nodes on the bound itself and a spacing beside it: the temperature solve's
+    rounding spreads them."""
+    w = _at_temperature(mech, (37, 23, 1), T0)
+    o, g = make_oracle(mech, w), make_gpu(mech, w)
+    T = g.moments()["T"]
+    assert (T == T0).any() and (T < T0).any()
+    d, m = g.diagnostics(), o.moments()
+    g.close()
+    ref = diagnostics(mech, m["rho"], m["u"], m["T"], m["Y"], w["dx"], 2, w["shape"][0])
+    for k in ("hrr_integral", "hrr_max"):
+        assert abs(d[k] / ref[k] - 1.0) < RTOL_FP64, (k, d[k], ref[k])
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", RTOL_FP64), ("fp32c64", 1e-4)])
+def test_step_at_the_lower_bound_of_the_rate_arguments(mech, precision, tol):
+    """Forty uniform states at 128 K, each with its own rounding of T."""
+    worst = np.zeros(mech.n_species + 1)
+    w = _at_temperature(mech, (5, 3, 1), 128.0)
+    for k in range(40):
+        w["P"][:] = 101325.0 * (1.0 + 1e-3 * k)
+        worst = np.maximum(worst, _errors(mech, w, 1, precision))
+    assert np.all(worst < tol), worst
