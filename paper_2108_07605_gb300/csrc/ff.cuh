@@ -269,12 +269,22 @@ __device__ __forceinline__ ff ff_unpack(double d) {
   return ff(__int_as_float(__double2hiint(d)), __int_as_float(__double2loint(d)));
 }
 
-// Exponentials of the reaction rates.  The argument comes in units of ln2/64
-// (the mechanism's coefficients are scaled by 64/ln2 on the host), as the
-// nearest integer n and the rest r = rh + rl, |r| <= 1/2; e^x = y 2^e with
+// 0 <= d < 2^(63 - bits) as an integer with `bits` fraction bits; the largest
+// integer above
+__device__ __forceinline__ long long fixed_of(double d, int bits) {
+  const int h = __double2hiint(d);
+  const unsigned long long m =
+      ((unsigned long long)(unsigned)((h & 0xfffff) | 0x100000) << 42) |
+      ((unsigned long long)(unsigned)__double2loint(d) << 10);    // 62 fraction bits
+  const int sh = 62 + 1023 - bits - (h >> 20);
+  return sh < 0 ? 0x7fffffffffffffffLL : (long long)(m >> min(sh, 63));
+}
+
+// Exponentials of the float-float reaction rates.  The argument comes in units
+// of ln2/64 (the mechanism's coefficients are scaled by 64/ln2 on the host), as
+// the nearest integer n and the rest r = rh + rl, |r| <= 1/2; e^x = y 2^e with
 // e = floor(n / 64) and y = 2^(j/64) e^z, z = r ln2/64 (Tang's reduction,
-// as ff_exp).  e is applied after the concentrations (ff_scale), so that a
-// rate constant beyond FP32's range is no overflow by itself.
+// as ff_exp).
 struct ExpArg {
   int n;
   float rh, rl;
@@ -293,41 +303,6 @@ __device__ __forceinline__ ExpArg exp_arg(ff x) {
   a.rh = r.hi;
   a.rl = r.lo;
   return a;
-}
-// x in fixed point with 46 fraction bits, |x| < 2^17
-__device__ __forceinline__ ExpArg exp_arg(long long v) {
-  const long long top = 16000LL << 46;
-  v = v > top ? top : (v < -top ? -top : v);
-  const int vh = (int)(v >> 32);
-  ExpArg a;
-  a.n = (vh + (1 << 13)) >> 14;
-  const int fh = vh - (a.n << 14);
-  const unsigned fl = (unsigned)v;
-  const int f1 = (int)__funnelshift_l(fl, (unsigned)fh, 18);      // rest, 32 fraction bits
-  a.rh = __fmul_rn(__int2float_rn(f1 & ~0xff), 0x1p-32f);
-  a.rl = __fmul_rn(__int2float_rn(((f1 & 0xff) << 14) | (int)(fl & 0x3fffu)), 0x1p-46f);
-  return a;
-}
-// 0 <= d < 2^(63 - bits) as an integer with `bits` fraction bits; the largest
-// integer above
-__device__ __forceinline__ long long fixed_of(double d, int bits) {
-  const int h = __double2hiint(d);
-  const unsigned long long m =
-      ((unsigned long long)(unsigned)((h & 0xfffff) | 0x100000) << 42) |
-      ((unsigned long long)(unsigned)__double2loint(d) << 10);    // 62 fraction bits
-  const int sh = 62 + 1023 - bits - (h >> 20);
-  return sh < 0 ? 0x7fffffffffffffffLL : (long long)(m >> min(sh, 63));
-}
-// x in FP64, through its fixed-point form
-__device__ __forceinline__ ExpArg exp_arg(double x) {
-  const int h = __double2hiint(x);
-  if ((h & 0x7fffffff) >= 0x40cf4000) {                 // 16000 and above
-    ExpArg b{h < 0 ? -16000 : 16000, 0.f, 0.f};
-    if (x != x) b.rh = __int_as_float(0x7fffffff);
-    return b;
-  }
-  const long long v = fixed_of(__hiloint2double(h & 0x7fffffff, __double2loint(x)), 46);
-  return exp_arg(h < 0 ? -v : v);
 }
 
 __device__ __forceinline__ ff exp_frac(const ExpArg& a) {

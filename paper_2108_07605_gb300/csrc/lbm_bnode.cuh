@@ -1022,14 +1022,14 @@ __device__ __forceinline__ void wequilibrium(const WState<D, M, R>& s, const Dev
 }
 
 // Interface node k by one warp; sm: the warp's WB::N entries; m: the
-// mechanism's global copy (indexed by lane); Cs: this thread's slice for the
+// mechanism's global copy (indexed by lane); cs: this thread's slice for the
 // sub-steps.
-template <int D, int M, typename S, typename R>
+template <int D, int M, typename S, typename R, typename Slice>
 __device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDev& bc,
                                            R* __restrict__ rec, double* __restrict__ Tf,
                                            int* __restrict__ status, const Geom& g,
                                            const Units& un, const DevMech& m, int k, R* sm,
-                                           int lane, ff* const Cs) {
+                                           int lane, Slice& cs) {
   using W = WB<D, M>;
   using RC = Rec<D, M>;
   constexpr int Q = W::Q;
@@ -1292,7 +1292,7 @@ __device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDe
   if constexpr (kFF<R>) U = (ff(ER) + ff(-0.5f * usq)) * un.c2_f;
   else U = (double(ER) - 0.5 * double(usq)) * un.c * un.c;
   chem_group_substeps<M, CT, 32>(r, X::inv(X::of(rr)), U, X::of_T(s.T_full), un, m, lane,
-                                 0xffffffffu, status, Cs);
+                                 0xffffffffu, status, cs);
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
     if (a != lane) continue;

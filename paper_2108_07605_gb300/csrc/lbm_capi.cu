@@ -283,7 +283,8 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
       if (std::equal(m.efficiency[r], m.efficiency[r] + m.n_species, eff[k])) set[r] = k;
     if (set[r] >= 0) continue;
     std::copy(m.efficiency[r], m.efficiency[r] + m.n_species, eff[rows]);
-    for (int a = 0; a < m.n_species; ++a) d.eff_f[rows][a] = ff_host(m.efficiency[r][a]);
+    for (int a = 0; a < m.n_species; ++a)
+      d.eff_f[rows][a] = ff_host(d.eff[rows][a] = m.efficiency[r][a]);
     set[r] = rows++;
   }
   const long double ln_p0 = std::log(P_REF / R_U), S = 64.0L / std::log(2.0L);

@@ -11,6 +11,7 @@
 
 #include "exp64.cuh"
 #include "log64.cuh"
+#include "sig64.cuh"
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -130,16 +131,7 @@ __device__ __forceinline__ long long fix_down(long long s, int sh) {
 }
 // the value, rounded to nearest; NaN when e is near that of infinities
 __device__ __forceinline__ double double_of_fix(long long s, int e) {
-  if (e >= 0x7f0) return __longlong_as_double(0x7ff8000000000000LL);
-  if (s == 0) return 0.0;
-  const unsigned sgn = (unsigned)(s >> 32) & 0x80000000u;
-  unsigned long long a = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
-  const int z = __clzll((long long)a);
-  a <<= z;                                     // leading bit at 63
-  const unsigned long long r = ((a >> 10) + 1) >> 1;          // 53 bits, rounded
-  const int ex = e + 6 - z;                    // biased exponent of the leading bit
-  const unsigned long long d = ex <= 0 ? 0 : ((unsigned long long)(ex - 1) << 52) + r;
-  return __longlong_as_double((long long)(d | (unsigned long long)sgn << 32));
+  return e >= 0x7f0 ? __longlong_as_double(0x7ff8000000000000LL) : double_of_sig(Sig{s, e - 1080});
 }
 __device__ __forceinline__ double double_of_fix(FixSum v) { return double_of_fix(v.s, v.e); }
 
@@ -292,16 +284,17 @@ __device__ __forceinline__ R flux_less_work(int d, const R (&u)[D], const QT& q,
 // chem_fp64) or float-float.
 //
 // What bounds it is the arithmetic of two exponentials per reaction.  In
-// FP64 the whole took ~42 FP64 instructions per reaction of 64 cycles each
-// per SM quarter, in float-float ~410 FP32 instructions.  So (1) the
+// FP64 the whole took ~42 FP64 instructions per reaction of 64 to 75 cycles
+// each per SM quarter, in float-float ~410 FP32 instructions.  So (1) the
 // logarithm of each rate constant is one sum over the basis (1, ln T, 1/T, T,
 // T^2) with coefficients folded on the host, which replaces the species' Gibbs
 // functions; (2) of FP64 temperatures these sums are taken in 64-bit fixed
-// point (the argument's size, up to ~100, would cost a float-float its
-// accuracy); the exponentials, products and sums that follow keep ~48 bits in
-// pairs of FP32, below the ~1e-14 that the rounding of T leaves in a rate
-// constant; (3) sums stay unnormalised (ff_acc); (4) the
-// third-body sums are formed once per distinct row of efficiencies.
+// point, the exponentials and their products with the concentrations in 64-bit
+// significands (Sig), and only a rate of progress becomes a double: FP64 is
+// left with the third body and the sums over the reactions (~6 instructions per
+// reaction), its range and rounding with all of it; (3) float-float sums stay
+// unnormalised (ff_acc); (4) the third-body sums are formed once per distinct
+// row of efficiencies.
 template <typename CT> struct TBasis { CT lnT, invT, T, T2; };
 // FP64: also in fixed point, in which a sum takes no FP64 instruction (and is
 // exact to 2^-46; FP64's own rounding of it is up to 2^-40); usable for
@@ -333,16 +326,17 @@ __device__ __forceinline__ TBasis<double> tbasis(const DevMech& m, double T) {
 __device__ __forceinline__ TBasis<ff> tbasis(const DevMech&, ff T) {
   return TBasis<ff>{ff_log(T), ff(1.f) / T, T, T * T};
 }
-__device__ __forceinline__ ExpArg forward_arg(const DevReaction& x, const TBasis<double>& b) {
+// the rate constants
+__device__ __forceinline__ Sig forward_constant(const DevReaction& x, const TBasis<double>& b) {
   if (b.fixed)
-    return exp_arg(x.fq[0] + __mul64hi(x.fq[1], b.q[1]) + __mul64hi(x.fq[2], b.q[2]));
-  return exp_arg(fma(x.f[2], b.invT, fma(x.f[1], b.lnT, x.f[0])));
+    return exp_sig(x.fq[0] + __mul64hi(x.fq[1], b.q[1]) + __mul64hi(x.fq[2], b.q[2]));
+  return exp_sig(fma(x.f[2], b.invT, fma(x.f[1], b.lnT, x.f[0])));
 }
-__device__ __forceinline__ ExpArg reverse_arg(const DevReaction& x, const TBasis<double>& b) {
+__device__ __forceinline__ Sig reverse_constant(const DevReaction& x, const TBasis<double>& b) {
   if (b.fixed)
-    return exp_arg(x.rq[0] + __mul64hi(x.rq[1], b.q[1]) + __mul64hi(x.rq[2], b.q[2]) +
+    return exp_sig(x.rq[0] + __mul64hi(x.rq[1], b.q[1]) + __mul64hi(x.rq[2], b.q[2]) +
                    __mul64hi(x.rq[3], b.q[3]) + __mul64hi(x.rq[4], b.q[4]));
-  return exp_arg(fma(x.r[2], b.invT,
+  return exp_sig(fma(x.r[2], b.invT,
                      fma(x.r[1], b.lnT, fma(x.r[4], b.T2, fma(x.r[3], b.T, x.r[0])))));
 }
 __device__ __forceinline__ ExpArg forward_arg(const DevReaction& x, const TBasis<ff>& b) {
@@ -360,71 +354,121 @@ __device__ __forceinline__ ExpArg reverse_arg(const DevReaction& x, const TBasis
   return exp_arg(ff_norm(s));
 }
 
-// The arrays the reaction loop indexes by species (concentrations C, molar
-// rates W) live in a per-thread slice of shared memory: a runtime index into
-// a register array would put it in local memory.  Every kernel that runs the
-// rates has kChemThreads threads per block (or fewer).
+// The arrays the reaction loop indexes by species (concentrations, molar
+// rates) live in a per-thread slice of shared memory: a runtime index into a
+// register array would put it in local memory.  ST: threads per block (or more),
+// the stride of a slice's entries; kBytes: the block's slices.
 constexpr int kChemThreads = 128;
+template <int M, typename CT, int ST = kChemThreads> struct ChemSlice;
+template <int M, int ST> struct ChemSlice<M, ff, ST> {
+  static constexpr size_t kBytes = (size_t)2 * M * ST * sizeof(ff);
+  ff* p;
+  __device__ __forceinline__ ChemSlice(void* block, int t) : p(static_cast<ff*>(block) + t) {}
+  __device__ __forceinline__ ff c(int a) const { return p[a * ST]; }
+  __device__ __forceinline__ void set(int a, ff c) { p[a * ST] = c; }
+  __device__ __forceinline__ void clear(int a) { p[(M + a) * ST] = ff(); }
+  __device__ __forceinline__ void add(int a, ff q) { ff_acc(p[(M + a) * ST], q); }
+  __device__ __forceinline__ ff sum(int a) const { return p[(M + a) * ST]; }   // unnormalised
+  __device__ __forceinline__ ff rate(int a) const { return ff_norm(sum(a)); }
+  __device__ __forceinline__ ff third_body(const DevMech& m, int row) const {
+    ff s;
+#pragma unroll
+    for (int a = 0; a < M; ++a) ff_fma_acc(s, m.eff_f[row][a], c(a));
+    return ff_norm(s);
+  }
+};
+// FP64: the concentrations also as significand and exponent
+template <int M, int ST> struct ChemSlice<M, double, ST> {
+  static constexpr size_t kBytes = (size_t)M * ST * (3 * sizeof(double) + sizeof(int));
+  double* p;      // C, W, then the significands
+  int* e;
+  __device__ __forceinline__ ChemSlice(void* block, int t)
+      : p(static_cast<double*>(block) + t), e(static_cast<int*>(block) + 6 * M * ST + t) {}
+  __device__ __forceinline__ double c(int a) const { return p[a * ST]; }
+  __device__ __forceinline__ Sig sig(int a) const {
+    return Sig{__double_as_longlong(p[(2 * M + a) * ST]), e[a * ST]};
+  }
+  __device__ __forceinline__ void set(int a, double c) {
+    const Sig s = sig_of(c);
+    p[a * ST] = c;
+    p[(2 * M + a) * ST] = __longlong_as_double(s.m);
+    e[a * ST] = s.e;
+  }
+  __device__ __forceinline__ void clear(int a) { p[(M + a) * ST] = 0.0; }
+  __device__ __forceinline__ void add(int a, double q) { p[(M + a) * ST] += q; }
+  __device__ __forceinline__ double sum(int a) const { return p[(M + a) * ST]; }
+  __device__ __forceinline__ double rate(int a) const { return sum(a); }
+  __device__ __forceinline__ double third_body(const DevMech& m, int row) const {
+    double s = 0.0;
+#pragma unroll
+    for (int a = 0; a < M; ++a) s = fma(m.eff[row][a], c(a), s);
+    return s;
+  }
+};
 
-// bytes of one block's slices (kChemThreads threads, C and W per species)
-template <int M> constexpr size_t chem_slice_bytes() {
-  return (size_t)2 * M * kChemThreads * sizeof(ff);
-}
-
-// Rate of progress of a reaction without its third body; C: this thread's
-// concentrations (entry a at C[a kChemThreads]).
-template <typename CT>
-__device__ __forceinline__ ff reaction_rate(const DevReaction& x, const TBasis<CT>& b,
-                                            const ff* C) {
-  const ExpArg af = forward_arg(x, b);
-  ff q = exp_frac(af);
-  for (int j = 0; j < x.nr; ++j) q *= C[x.reac[j] * kChemThreads];
-  q = ff_scale(q, af.n >> 6);
+// Rate of progress of a reaction without its third body, from this thread's
+// concentrations.
+template <int M, int ST>
+__device__ __forceinline__ double reaction_rate(const DevReaction& x, const TBasis<double>& b,
+                                                const ChemSlice<M, double, ST>& s) {
+  Sig q = forward_constant(x, b);
+  for (int j = 0; j < x.nr; ++j) q = q * s.sig(x.reac[j]);
   if (x.reversible) {
-    const ExpArg ar = reverse_arg(x, b);
-    ff rev = exp_frac(ar);
-    for (int j = 0; j < x.np; ++j) rev *= C[x.prod[j] * kChemThreads];
-    ff_acc(q, -ff_scale(rev, ar.n >> 6));
+    Sig rev = reverse_constant(x, b);
+    for (int j = 0; j < x.np; ++j) rev = rev * s.sig(x.prod[j]);
+    q = q - rev;
+  }
+  return double_of_sig(q);
+}
+// Float-float: of a rate constant 2^e1 y, what FP32 holds of 2^e1 goes before the
+// concentrations and the rest after them.
+template <int M, int ST>
+__device__ __forceinline__ ff scaled_product(const ExpArg& x, int n, const int* species,
+                                             const ChemSlice<M, ff, ST>& s) {
+  const int e = x.n >> 6, e1 = min(max(e, -100), 126);
+  ff q = ff_scale(exp_frac(x), e1);
+  for (int j = 0; j < n; ++j) q *= s.c(species[j]);
+  return e == e1 ? q : ff_scale(q, e - e1);
+}
+template <int M, int ST>
+__device__ __forceinline__ ff reaction_rate(const DevReaction& x, const TBasis<ff>& b,
+                                            const ChemSlice<M, ff, ST>& s) {
+  ff q = scaled_product(forward_arg(x, b), x.nr, x.reac, s);
+  if (x.reversible) {
+    ff_acc(q, -scaled_product(reverse_arg(x, b), x.np, x.prod, s));
     q = ff_norm(q);
   }
   return q;
 }
 
-// The reactions first, first + step, ... added to this thread's molar rates W
-// (entry a at W[a kChemThreads], unnormalised).
-template <int M, typename CT>
+// The reactions first, first + step, ... added to this thread's molar rates.
+template <int M, typename CT, int ST>
 __device__ __forceinline__ void add_reactions(const DevMech& m, const TBasis<CT>& b,
-                                              const ff* C, ff* W, int first, int step) {
+                                              ChemSlice<M, CT, ST>& s, int first, int step) {
   int row = -1;
-  ff cm;
+  CT cm = CT();
   for (int k = first; k < m.R; k += step) {
     const DevReaction& x = m.rx[k];
-    ff q = reaction_rate(x, b, C);
+    CT q = reaction_rate(x, b, s);
     if (x.third_body >= 0) {
       if (x.third_body != row) {
         row = x.third_body;
-        cm = ff();
-#pragma unroll
-        for (int a = 0; a < M; ++a) ff_fma_acc(cm, m.eff_f[row][a], C[a * kChemThreads]);
-        cm = ff_norm(cm);
+        cm = s.third_body(m, row);
       }
       q *= cm;
     }
-    for (int j = 0; j < x.nr; ++j) ff_acc(W[x.reac[j] * kChemThreads], -q);
-    for (int j = 0; j < x.np; ++j) ff_acc(W[x.prod[j] * kChemThreads], q);
+    for (int j = 0; j < x.nr; ++j) s.add(x.reac[j], -q);
+    for (int j = 0; j < x.np; ++j) s.add(x.prod[j], q);
   }
 }
 
-// Molar rates w_a (mol/(m^3 s)) at T of the concentrations already in this
-// thread's slice Cs; the slice's rates are overwritten.
-template <int M, typename CT>
-__device__ __forceinline__ void molar_rates(const DevMech& m, CT T, ff (&w)[M], ff* const Cs) {
-  ff* const Ws = Cs + M * kChemThreads;
+// Molar rates (mol/(m^3 s)) at T of the concentrations already in this
+// thread's slice; the slice's rates are overwritten.
+template <int M, typename CT, int ST>
+__device__ __forceinline__ void molar_rates(const DevMech& m, CT T, ChemSlice<M, CT, ST>& s) {
 #pragma unroll
-  for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
-  add_reactions<M>(m, tbasis(m, T), Cs, Ws, 0, 1);
-#pragma unroll
-  for (int a = 0; a < M; ++a) w[a] = ff_norm(Ws[a * kChemThreads]);
+  for (int a = 0; a < M; ++a) s.clear(a);
+  add_reactions(m, tbasis(m, T), s, 0, 1);
 }
 
 // ------------------------------------------------------------------------

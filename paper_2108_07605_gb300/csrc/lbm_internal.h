@@ -26,7 +26,7 @@ constexpr int ST_NONFINITE = 2;
 constexpr int ST_RANGE = 4;
 constexpr int ST_TIMEOUT = 8;   // a bounded device wait gave up
 
-// Logarithms of a reaction's rate constants, in units of ln2/64 (ExpArg), as
+// Logarithms of a reaction's rate constants, in units of ln2/64, as
 // sums over T alone:
 //   forward  f[0] + f[1] ln T + f[2] / T
 //   reverse  r[0] + r[1] ln T + r[2] / T + r[3] T + r[4] T^2,
@@ -35,7 +35,7 @@ struct DevReaction {
   int nr, np;            // number of reactant / product molecules (<= 3)
   int reac[3], prod[3];  // species index per molecule (repeated for nu = 2)
   int reversible;
-  int third_body;        // row of DevMech::eff_f, -1: none
+  int third_body;        // row of DevMech::eff, -1: none
   double f[3], r[5];
   ff f_f[3], r_f[5];     // the same as float-float (mixed path)
   // and in fixed point, each against its basis function's units (kArgBits)
@@ -56,8 +56,9 @@ struct DevMech {
   double u0[LBM_MAX_SPECIES], u1[LBM_MAX_SPECIES], u2[LBM_MAX_SPECIES],
       u3[LBM_MAX_SPECIES];
   // reactions, those of equal third-body efficiencies in a row (the sum over
-  // the species is formed once per row)
+  // the species is formed once per distinct row of efficiencies)
   DevReaction rx[LBM_MAX_REACTIONS];
+  double eff[LBM_MAX_REACTIONS][LBM_MAX_SPECIES];
   // 1/tau_ab = s(node) * K[a][b], K = 1/(m_a m_b D0_ab)
   double K[LBM_MAX_SPECIES][LBM_MAX_SPECIES];
   float Kf[LBM_MAX_SPECIES][LBM_MAX_SPECIES];   // K rounded to FP32 (mixed path)
@@ -73,7 +74,7 @@ struct DevMech {
   // float-float copies for the mixed path's temperature solve and chemistry
   ff mm_f[LBM_MAX_SPECIES], inv_mm_f[LBM_MAX_SPECIES];
   ff u0_f[LBM_MAX_SPECIES], u1_f[LBM_MAX_SPECIES], u2_f[LBM_MAX_SPECIES], u3_f[LBM_MAX_SPECIES];
-  ff eff_f[LBM_MAX_REACTIONS][LBM_MAX_SPECIES];   // distinct rows of third-body efficiencies
+  ff eff_f[LBM_MAX_REACTIONS][LBM_MAX_SPECIES];
   // FP32 copies for the mixed path's transport and energy-flux terms
   float inv_mm_s[LBM_MAX_SPECIES], Ra_s[LBM_MAX_SPECIES];
   float D_T_exp_s, mu0_s, mu_T_exp_s, inv_prandtl_s;

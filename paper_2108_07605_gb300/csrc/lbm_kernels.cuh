@@ -58,6 +58,8 @@ inline namespace chemff {
 
 // float-float Newton and chemistry: FP32 lattice arithmetic, float-float mode
 template <typename RT> constexpr bool kFF = sizeof(RT) == 4 && !LBM_CHEM64;
+template <typename RT> struct ChemType { using type = double; };
+template <> struct ChemType<float> { using type = std::conditional_t<LBM_CHEM64 != 0, double, ff>; };
 // resident blocks per SM the moments kernels are compiled for (register cap):
 // four (128 registers): with three (168) the FP64 kernel took 1.34 ms on the
 // 600x40x40 tube, with four 1.15, its 460 bytes of spills included; FP32 with
@@ -159,12 +161,12 @@ __device__ __forceinline__ constexpr int pidx(int a, int b) {
 // included), rho, ER = E / rho and usqR = |u|^2 of the moments, T_0 = T
 // their temperature; dr receives the increments drho_a (a < M - 1).  The
 // temperature solve in float-float (mixed path) or FP64; the rate arrays live
-// in the thread's slice of shared memory (chem_slice: the block's slices,
-// chem_slice_bytes).  Blocks of at most kChemThreads threads.
-template <int M>
-__device__ __forceinline__ ff* chem_static_slice() {
-  __shared__ __align__(8) unsigned char chem_raw[chem_slice_bytes<M>()];
-  return reinterpret_cast<ff*>(chem_raw);
+// in the thread's slice of shared memory (chem_slice: the block's slices).
+// Blocks of at most kChemThreads threads.
+template <int M, typename CT, int ST = kChemThreads>
+__device__ __forceinline__ void* chem_static_slice() {
+  __shared__ __align__(8) unsigned char chem_raw[ChemSlice<M, CT, ST>::kBytes];
+  return chem_raw;
 }
 
 template <int M, typename RT>
@@ -172,8 +174,7 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
                                               double T, const Units& un, const DevMech& mech,
                                               int* __restrict__ status, void* chem_slice,
                                               RT (&dr)[M - 1]) {
-  ff* const Cs = static_cast<ff*>(chem_slice) + threadIdx.x;
-  ff w[M];
+  ChemSlice<M, typename ChemType<RT>::type> cs(chem_slice, threadIdx.x);
   if constexpr (kFF<RT>) {
     const ff Uphys = (ff(ER) + ff(-0.5f * usqR)) * un.c2_f;
     ff r[M];
@@ -192,10 +193,10 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
         if (!oks) atomicOr(status, ST_NEWTON);
       }
 #pragma unroll
-      for (int a = 0; a < M; ++a) Cs[a * kChemThreads] = r[a] * mech.inv_mm_f[a];
-      molar_rates<M>(mech, Ts, w, Cs);
+      for (int a = 0; a < M; ++a) cs.set(a, r[a] * mech.inv_mm_f[a]);
+      molar_rates(mech, Ts, cs);
 #pragma unroll
-      for (int a = 0; a < M; ++a) r[a] += un.dt_sub_f * (w[a] * mech.mm_f[a]);
+      for (int a = 0; a < M; ++a) r[a] += un.dt_sub_f * (cs.rate(a) * mech.mm_f[a]);
     }
 #pragma unroll
     for (int a = 0; a < M - 1; ++a) dr[a] = (r[a] - ff(rs[a])).hi;
@@ -216,10 +217,10 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
         if (!oks) atomicOr(status, ST_NEWTON);
       }
 #pragma unroll
-      for (int a = 0; a < M; ++a) Cs[a * kChemThreads] = ff_of_double(r[a] * mech.inv_mm[a]);
-      molar_rates<M>(mech, Ts, w, Cs);
+      for (int a = 0; a < M; ++a) cs.set(a, r[a] * mech.inv_mm[a]);
+      molar_rates(mech, Ts, cs);
 #pragma unroll
-      for (int a = 0; a < M; ++a) r[a] = fma(double_of_ff(w[a]), dtr * mech.mm[a], r[a]);
+      for (int a = 0; a < M; ++a) r[a] = fma(cs.rate(a), dtr * mech.mm[a], r[a]);
     }
 #pragma unroll
     for (int a = 0; a < M - 1; ++a) dr[a] = RT(r[a] - double(rs[a]));
@@ -247,11 +248,26 @@ template <> struct Chem<double> {
   __device__ static double of(double v) { return v; }
   __device__ static double of_T(double T) { return T; }
   __device__ static double of_ff(ff v) { return double_of_ff(v); }
-  __device__ static ff concentration(const DevMech& m, int a, double r) {
-    return ff_of_double(r * m.inv_mm[a]);
+  __device__ static double concentration(const DevMech& m, int a, double r) {
+    return r * m.inv_mm[a];
   }
-  __device__ static double increment(const DevMech& m, const Units& u, int a, ff w) {
-    return double_of_ff(w) * (u.dt_sub * m.mm[a]);
+  __device__ static double increment(const DevMech& m, const Units& u, int a, double w) {
+    return w * (u.dt_sub * m.mm[a]);
+  }
+  // sum over the group, the same in every lane: significands shifted to the
+  // largest exponent and added in integers (a butterfly of FP64 additions would
+  // occupy the FP64 pipe for 75 cycles per stage)
+  template <int L> __device__ __forceinline__ static double group_sum(double v, unsigned gmask) {
+    constexpr int G = L == 32 ? 6 : (L == 8 ? 4 : 3);       // log2 L and the sign
+    const Sig s = sig_of(v);
+    int e = s.m == 0 ? -(1 << 16) : s.e;
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) e = max(e, __shfl_xor_sync(gmask, e, o));
+    long long m = s.m >> min(e - s.e + G, 63);
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) m += __shfl_xor_sync(gmask, m, o);
+    return e >= kSigNaN / 2 ? __longlong_as_double(0x7ff8000000000000LL)
+                            : double_of_sig(Sig{m, e + G});
   }
   __device__ static double ucoef(const DevMech& m, int k, int a) {
     return k == 0 ? m.u0[a] : (k == 1 ? m.u1[a] : (k == 2 ? m.u2[a] : m.u3[a]));
@@ -265,16 +281,19 @@ template <> struct Chem<ff> {
   __device__ static ff of_ff(ff v) { return v; }
   __device__ static ff concentration(const DevMech& m, int a, ff r) { return r * m.inv_mm_f[a]; }
   __device__ static ff increment(const DevMech& m, const Units& u, int a, ff w) {
-    return u.dt_sub_f * (w * m.mm_f[a]);
+    return u.dt_sub_f * (ff_norm(w) * m.mm_f[a]);
+  }
+  // (unnormalised)
+  template <int L> __device__ __forceinline__ static ff group_sum(ff v, unsigned gmask) {
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) ff_acc(v, shfl_xor_ct(gmask, v, o));
+    return v;
   }
   __device__ static ff ucoef(const DevMech& m, int k, int a) {
     return k == 0 ? m.u0_f[a] : (k == 1 ? m.u1_f[a] : (k == 2 ? m.u2_f[a] : m.u3_f[a]));
   }
   __device__ static float rtol(const Units& u) { return u.newton_rtol_f; }
 };
-
-template <typename RT> struct ChemType { using type = double; };
-template <> struct ChemType<float> { using type = std::conditional_t<LBM_CHEM64 != 0, double, ff>; };
 
 // Register r[a] for a lane-dependent species index a (a select per species:
 // a runtime index into a register array would put it in local memory).
@@ -318,14 +337,14 @@ __device__ __forceinline__ CT group_newton(const DevMech& m, const CT (&r)[M], C
 // The reaction sub-steps of one node by its lane group (Sec. 2.4 Eq. R3),
 // from the post-stream species densities r (replaced by the densities after
 // the sub-steps), 1/rho, the internal energy U and the temperature T_0 of
-// the moments.  Cs: this thread's slice for concentrations and rates.
-template <int M, typename CT, int L>
+// the moments.  cs: this thread's slice for concentrations and rates.
+template <int M, typename CT, int L, int ST>
 __device__ __forceinline__ void chem_group_substeps(CT (&r)[M], const CT irho, const CT U,
                                                     CT Ts, const Units& un, const DevMech& m,
                                                     int sub, unsigned gmask,
-                                                    int* __restrict__ status, ff* const Cs) {
+                                                    int* __restrict__ status,
+                                                    ChemSlice<M, CT, ST>& cs) {
   using X = Chem<CT>;
-  ff* const Ws = Cs + M * kChemThreads;
   for (int s = 0; s < un.substeps; ++s) {
     if (s > 0) {
       bool ok;
@@ -335,20 +354,14 @@ __device__ __forceinline__ void chem_group_substeps(CT (&r)[M], const CT irho, c
     }
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-      Cs[a * kChemThreads] = X::concentration(m, a, r[a]);
-      Ws[a * kChemThreads] = ff();
+      cs.set(a, X::concentration(m, a, r[a]));
+      cs.clear(a);
     }
-    add_reactions<M>(m, tbasis(m, Ts), Cs, Ws, sub, L);
-    ff w[M];
+    add_reactions(m, tbasis(m, Ts), cs, sub, L);
+    // the group's sums: every lane ends with the same total
 #pragma unroll
-    for (int a = 0; a < M; ++a) w[a] = Ws[a * kChemThreads];
-    // butterfly sums over the group: every lane ends with the same total
-#pragma unroll
-    for (int o = 1; o < L; o <<= 1)
-#pragma unroll
-      for (int a = 0; a < M; ++a) ff_acc(w[a], shfl_xor_ct(gmask, w[a], o));
-#pragma unroll
-    for (int a = 0; a < M; ++a) r[a] += X::increment(m, un, a, ff_norm(w[a]));
+    for (int a = 0; a < M; ++a)
+      r[a] += X::increment(m, un, a, X::template group_sum<L>(cs.sum(a), gmask));
   }
 }
 
@@ -389,8 +402,9 @@ __device__ __forceinline__ void chem_lanes_body(RT* __restrict__ rec,
     r[a] = r0[a];
   }
   r[M - 1] = X::of(last);
+  ChemSlice<M, CT> cs(chem_static_slice<M, CT>(), threadIdx.x);
   chem_group_substeps<M, CT, L>(r, X::inv(X::of(rho)), U, X::of_T(Tf[n]), un, m, sub, gmask,
-                                status, chem_static_slice<M>() + threadIdx.x);
+                                status, cs);
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
     if (a % L != sub) continue;
@@ -557,8 +571,8 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
   CT r0[M - 1];
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) r0[a] = r[a];
-  chem_group_substeps<M, CT, L>(r, irho, U, X::of_T(T), un, mg, sub, gmask, status,
-                                chem_static_slice<M>() + threadIdx.x);
+  ChemSlice<M, CT> cs(chem_static_slice<M, CT>(), threadIdx.x);
+  chem_group_substeps<M, CT, L>(r, irho, U, X::of_T(T), un, mg, sub, gmask, status, cs);
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
     if constexpr (kFF<RT>) put(RC::DRHO + a, (r[a] - r0[a]).hi);
@@ -567,15 +581,15 @@ __device__ __forceinline__ void mchem_body(const S* __restrict__ src, RT* __rest
 }
 
 // ---------------------------------------------------------------------------
-// Shared memory of the moments kernels: per thread the chemistry's slice (C,
-// W), the sums of W over the sub-steps and, with FP64 chemistry, the
-// concentrations in FP64 (M entries of 8 bytes each).
-template <int M> constexpr size_t moments_bytes() {
-  return chem_slice_bytes<M>() + (size_t)2 * M * kChemThreads * sizeof(double);
+// Shared memory of the moments kernels: per thread the chemistry's slice and
+// the sums of its rates over the sub-steps.
+template <int M, typename RT> constexpr size_t moments_bytes() {
+  return ChemSlice<M, typename ChemType<RT>::type>::kBytes +
+         (size_t)M * kChemThreads * sizeof(double);
 }
-template <int M>
+template <int M, typename RT>
 __device__ __forceinline__ void* moments_static() {
-  __shared__ __align__(16) unsigned char mom_raw[moments_bytes<M>()];
+  __shared__ __align__(16) unsigned char mom_raw[moments_bytes<M, RT>()];
   return mom_raw;
 }
 
@@ -734,10 +748,8 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   const long long N = g.N;
   if (n >= N) return;
   if (bc.tag && bc.tag[n] == TAG_SOLID) return;
-  ff* const Cs = static_cast<ff*>(smem) + threadIdx.x;
-  ff* const Ws = Cs + M * kChemThreads;
-  double* const Wd = static_cast<double*>(smem) + 2 * M * kChemThreads + threadIdx.x;
-  double* const Cd = Wd + M * kChemThreads;
+  double* const Wd = static_cast<double*>(smem) + threadIdx.x;
+  ChemSlice<M, CT> cs(static_cast<double*>(smem) + M * kChemThreads, threadIdx.x);
   const int x = (int)(n % g.nx);
   const int y = (int)((n / g.nx) % g.ny);
   const int z = (int)(n / ((long long)g.nx * g.ny));
@@ -766,7 +778,7 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
       ff_fma_acc(cU[1], ff(Y), mech.u1_f[a]);
       ff_fma_acc(cU[2], ff(Y), mech.u2_f[a]);
       ff_fma_acc(cU[3], ff(Y), mech.u3_f[a]);
-      Cs[a * kChemThreads] = ff(rs) * mech.inv_mm_f[a];
+      cs.set(a, ff(rs) * mech.inv_mm_f[a]);
       Wd[a * kChemThreads] = ff_pack(ff());
     } else {
       double Yd, rd;
@@ -783,10 +795,8 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
       cU[1] = fma(Yd, mech.u1[a], cU[1]);
       cU[2] = fma(Yd, mech.u2[a], cU[2]);
       cU[3] = fma(Yd, mech.u3[a], cU[3]);
-      const double c = rd * mech.inv_mm[a];
-      Cd[a * kChemThreads] = c;
+      cs.set(a, rd * mech.inv_mm[a]);
       Wd[a * kChemThreads] = 0.0;
-      Cs[a * kChemThreads] = ff_of_double(c);
     }
     RT us[D];
     record_velocities<D>(rs, js, u, us);
@@ -905,28 +915,27 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
       if (!oks) atomicOr(status, ST_NEWTON);
     }
 #pragma unroll
-    for (int a = 0; a < M; ++a) Ws[a * kChemThreads] = ff();
+    for (int a = 0; a < M; ++a) cs.clear(a);
     const TBasis<CT> tb = tbasis(mech, Ts);
     if constexpr (sizeof(RT) == 8)
       if (s == 0) rec[RC::LNT * N + n] = tb.lnT - LN_T_REF;
-    add_reactions<M>(mech, tb, Cs, Ws, 0, 1);
+    add_reactions(mech, tb, cs, 0, 1);
     const bool last = s + 1 == un.substeps;
 #pragma unroll 1
     for (int a = 0; a < M; ++a) {
-      const ff w = ff_norm(Ws[a * kChemThreads]);
+      const CT w = cs.rate(a);
+      ff inc;
       if constexpr (kFF<RT>) {
         Wd[a * kChemThreads] = ff_pack(ff_unpack(Wd[a * kChemThreads]) + w);
         if (last) continue;
-        Cs[a * kChemThreads] += un.dt_sub_f * w;
+        cs.set(a, cs.c(a) + un.dt_sub_f * w);
+        inc = w * un.dtmm_f[a];
       } else {
-        const double wd = double_join(w);
-        Wd[a * kChemThreads] += wd;
+        Wd[a * kChemThreads] += w;
         if (last) continue;
-        const double c = fma(wd, un.dt_sub, Cd[a * kChemThreads]);
-        Cd[a * kChemThreads] = c;
-        Cs[a * kChemThreads] = ff_of_double(c);
+        cs.set(a, fma(w, un.dt_sub, cs.c(a)));
+        inc = ff_of_double(w) * un.dtmm_f[a];
       }
-      const ff inc = w * un.dtmm_f[a];
       ff_fma_acc(dU[0], inc, mech.u0_f[a]);
       ff_fma_acc(dU[1], inc, mech.u1_f[a]);
       ff_fma_acc(dU[2], inc, mech.u2_f[a]);
@@ -2019,7 +2028,7 @@ k_moments(const S* __restrict__ src, RT* __restrict__ rec, double* __restrict__ 
   // node_set: NODES_ALL or NODES_BULK
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (node_set == NODES_BULK && bc.tag && n < g.N && bc.tag[n] >= 0) return;
-  moments_body<D, M, S, RT>(src, rec, Tf, status, g, un, bc, mech, n, moments_static<M>());
+  moments_body<D, M, S, RT>(src, rec, Tf, status, g, un, bc, mech, n, moments_static<M, RT>());
 }
 
 // The reaction sub-steps of the interface nodes from entry `first` of their
@@ -2128,8 +2137,9 @@ k_bnode_warp(const S* __restrict__ src, const __grid_constant__ BCDev bc,
   __shared__ R ws[kBnodeWarps][WB<D, M>::N];
   const int w = threadIdx.x >> 5, k = blockIdx.x * kBnodeWarps + w;
   if (k >= bc.n_if) return;
-  bnode_warp<D, M, S, R>(src, bc, rec, Tf, status, g, un, *mech, k, ws[w], threadIdx.x & 31,
-                         chem_static_slice<M>() + threadIdx.x);
+  using CT = typename ChemType<R>::type;
+  ChemSlice<M, CT, 32 * kBnodeWarps> cs(chem_static_slice<M, CT, 32 * kBnodeWarps>(), threadIdx.x);
+  bnode_warp<D, M, S, R>(src, bc, rec, Tf, status, g, un, *mech, k, ws[w], threadIdx.x & 31, cs);
 }
 
 // ---------------------------------------------------------------------------
@@ -2193,7 +2203,7 @@ k_moments_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int no
     const long long n = (b - d.block_begin) * (long long)blockDim.x + threadIdx.x;
     if (node_set == NODES_BULK && d.bc.tag && n < d.g.N && d.bc.tag[n] >= 0) continue;
     moments_body<D, M, S, RT>(static_cast<const S*>(d.pops[c]), static_cast<RT*>(d.rec), d.Tf,
-                              d.status, d.g, d.un, d.bc, *d.mech, n, moments_static<M>());
+                              d.status, d.g, d.un, d.bc, *d.mech, n, moments_static<M, RT>());
   }
 }
 
@@ -2300,7 +2310,9 @@ __global__ void __launch_bounds__(32 * kBnodeWarps)
 k_bnode_warp_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   using R = typename ComputeType<S>::type;
+  using CT = typename ChemType<R>::type;
   __shared__ R ws[kBnodeWarps][WB<D, M>::N];
+  ChemSlice<M, CT, 32 * kBnodeWarps> cs(chem_static_slice<M, CT, 32 * kBnodeWarps>(), threadIdx.x);
   const int w = threadIdx.x >> 5;
   for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
     const DomainDev& d = bd.get(doms, domain_of_block(doms, ndom, b, GRID_BNODE));
@@ -2308,7 +2320,7 @@ k_bnode_warp_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int
     if (k >= d.bc.n_if) continue;
     bnode_warp<D, M, S, R>(static_cast<const S*>(d.pops[d.cur0 ^ parity]), d.bc,
                            static_cast<R*>(d.rec), d.Tf, d.status, d.g, d.un, *d.mech, k, ws[w],
-                           threadIdx.x & 31, chem_static_slice<M>() + threadIdx.x);
+                           threadIdx.x & 31, cs);
   }
 }
 
@@ -2357,7 +2369,7 @@ __device__ __forceinline__ void iface_substeps(RT* __restrict__ rec, const doubl
 // least kIfChemThreadNodes interface nodes, which fill the GPU this way):
 // the same arithmetic as the lane groups of k_chem without their redundant
 // per-lane temperature and Gibbs evaluations.  Float-float rate arrays in
-// dynamic shared memory (chem_slice_bytes).
+// dynamic shared memory.
 constexpr long long kIfChemThreadNodes = 152LL * 128;
 
 template <int D, int M, typename RT>
@@ -2433,11 +2445,12 @@ k_step_persist(const DomainDev* __restrict__ doms, int ndom, int parity,
     if (w.kind == PI_BND && d.bc.n_if - w.first <= kPersistWarpNodes) {
       // few interface nodes: the block's warps take them in turn
       const int wp = threadIdx.x >> 5;
-      R* ws = reinterpret_cast<R*>(ps_raw + chem_slice_bytes<M>()) + wp * WB<D, M>::N;
+      using CT = typename ChemType<R>::type;
+      R* ws = reinterpret_cast<R*>(ps_raw + ChemSlice<M, CT>::kBytes) + wp * WB<D, M>::N;
+      ChemSlice<M, CT> cs(ps_raw, threadIdx.x);
       for (int k = (int)w.first + wp; k < d.bc.n_if; k += kPersistThreads / 32)
         bnode_warp<D, M, S, R>(src, d.bc, static_cast<R*>(d.rec), d.Tf, d.status, d.g, d.un,
-                               *d.mech, k, ws, threadIdx.x & 31,
-                               reinterpret_cast<ff*>(ps_raw) + threadIdx.x);
+                               *d.mech, k, ws, threadIdx.x & 31, cs);
     } else if (w.kind == PI_BND) {
       // two groups of kBnd threads, each with its boundary columns
       const int grp = threadIdx.x / kBnd, t = threadIdx.x % kBnd;
@@ -2494,10 +2507,10 @@ template <int D, int M, typename S, typename RT> constexpr size_t persist_smem(b
   const size_t prep = (size_t)solve_smem_entries<D, M, RT>() * kBS * sizeof(RT);
   const size_t coll = (size_t)coll_smem_entries<D, M, RT>() * kCollNodes * sizeof(RT);
   const size_t fused = (size_t)collide_smem_entries<D, M, RT>() * kBS * sizeof(RT);
-  const size_t chem =
-      chem_slice_bytes<M>() + sizeof(R) * WB<D, M>::N * (kPersistThreads / 32);
+  const size_t chem = ChemSlice<M, typename ChemType<RT>::type>::kBytes +
+                      sizeof(R) * WB<D, M>::N * (kPersistThreads / 32);
   size_t m = bnd > chem ? bnd : chem;
-  m = m > moments_bytes<M>() ? m : moments_bytes<M>();
+  m = m > moments_bytes<M, RT>() ? m : moments_bytes<M, RT>();
   if (split) {
     m = m > prep ? m : prep;
     m = m > coll ? m : coll;
@@ -2679,7 +2692,7 @@ k_diag(const S* __restrict__ pops, const double* __restrict__ Tf, const int* __r
   const int xn = (int)(n % g.nx);   // the nodes with x in [x0, x1) only
   if (n < N && xn >= x0 && xn < x1 && !(tag && tag[n] == TAG_SOLID)) {
     double rho, rhoE, j[D], c[4] = {0.0, 0.0, 0.0, 0.0}, ir = 0.0, usq = 0.0;
-    ff* const Cs = chem_static_slice<M>() + threadIdx.x;
+    ChemSlice<M, double> cs(chem_static_slice<M, double>(), threadIdx.x);
     stored_sums<D, M, S>(pops, N, n, g.codec, rho, j, rhoE, [&](int a, double rs) {
       if (a == 0) ir = 1.0 / rho;
       const double Y = rs * ir;
@@ -2687,17 +2700,16 @@ k_diag(const S* __restrict__ pops, const double* __restrict__ Tf, const int* __r
       c[1] = fma(Y, mech.u1[a], c[1]);
       c[2] = fma(Y, mech.u2[a], c[2]);
       c[3] = fma(Y, mech.u3[a], c[3]);
-      Cs[a * kChemThreads] = ff_of_double(rs * mech.inv_mm[a]);
+      cs.set(a, rs * mech.inv_mm[a]);
     });
     for (int d = 0; d < D; ++d) usq += (j[d] * ir) * (j[d] * ir);
     bool ok;
     const double T = newton_poly(c, (rhoE * ir - 0.5 * usq) * un.c * un.c, Tf[n],
                                  un.newton_max_iter, un.newton_rtol, ok);
     if (!ok) atomicOr(status, ST_NEWTON);
-    ff w[M];
-    molar_rates<M>(mech, T, w, Cs);
+    molar_rates(mech, T, cs);
     for (int a = 0; a < M; ++a)
-      q -= (species_U(mech, a, T) + mech.Ra[a] * T) * (double_of_ff(w[a]) * mech.mm[a]);
+      q -= (species_U(mech, a, T) + mech.Ra[a] * T) * (cs.rate(a) * mech.mm[a]);
     qmax = q;
     nmax = n;
     Tmax = T;
@@ -2809,7 +2821,8 @@ static void launch_chem(cudaStream_t s, RT* rec, const double* Tf, int* status, 
                         const BCDev& bc, const Units& un, const DevMech* mech) {
   if (bc.n_if >= kIfChemThreadNodes)
     k_iface_chem<D, M, RT>
-        <<<blocks_for(bc.n_if, kChemThreads), kChemThreads, chem_slice_bytes<M>(), s>>>(
+        <<<blocks_for(bc.n_if, kChemThreads), kChemThreads,
+           ChemSlice<M, typename ChemType<RT>::type>::kBytes, s>>>(
             rec, Tf, status, N, bc.if_node, bc.n_if, un, mech);
   else
     k_chem<D, M, RT><<<blocks_for(bc.n_if, kIfChemNodesPerBlock), 128, 0, s>>>(
@@ -2998,7 +3011,7 @@ static cudaError_t batch_impl(const DomainDev* doms, int ndom, const BatchGrids&
     if (gr.n_if_total >= kIfChemThreadNodes) {
       // enough interface nodes to fill the GPU with one thread each
       auto k = k_iface_chem_batch<D, M, RT>;
-      const size_t sm = chem_slice_bytes<M>();
+      const size_t sm = ChemSlice<M, typename ChemType<RT>::type>::kBytes;
       k<<<batch_grid(k, gr.ntblocks, kBnd, sm, ps), kBnd, sm, st>>>(doms, ndom, gr.ntblocks);
     } else {
       auto k = k_chem_batch<D, M, RT>;

@@ -1,4 +1,6 @@
 """The kernels' arithmetic at the edges of its ranges, against the CPU oracle."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -61,3 +63,45 @@ def test_step_at_the_lower_bound_of_the_rate_arguments(mech, precision, tol):
         w["P"][:] = 101325.0 * (1.0 + 1e-3 * k)
         worst = np.maximum(worst, _errors(mech, w, 1, precision))
     assert np.all(worst < tol), worst
+
+
+# Trace species: rates of progress from 1e-36 down to 1e-56 mol/(m^3 s) below those
+# of the main species, and a rate constant beyond e^200.  Relative to the species'
+# own lattice, as everywhere; rounding of T (Ea / (R T) up to 175) leaves 4e-14.
+def _without_radicals(mech, T0):
+    w = fields.perturbed_box((9, 5, 3), "D3Q27", mech=mech, T0=T0, dx=25e-6)
+    for s in ("H2O", "H", "O", "OH", "HO2", "H2O2"):
+        w["Y"][mech.index(s)] = 0.0
+    w["Y"] /= w["Y"].sum(axis=0)
+    return w
+
+
+def _one_step_errors(mech, w, lanes):
+    o, g = make_oracle(mech, w), make_gpu(mech, w)
+    g.set_launch(chem_lanes=lanes)
+    o.step(1)
+    g.step(1)
+    got, ref = g.populations(), oracle_populations(o)
+    g.close()
+    present = np.abs(ref).max(axis=(1, 2)) > 0.0
+    assert np.all(got[~present] == 0.0)
+    return max_rel_err_per_lattice(got[present], ref[present])
+
+
+@pytest.mark.parametrize("lanes", [1, 8])
+@pytest.mark.parametrize("T0", [300.0, 700.0])
+def test_radicals_formed_in_a_fresh_mixture(mech, T0, lanes):
+    err = _one_step_errors(mech, _without_radicals(mech, T0), lanes)
+    assert np.all(err < RTOL_FP64), err
+
+
+@pytest.mark.parametrize("lanes", [1, 8])
+def test_rate_constant_far_beyond_its_products(mech, lanes):
+    arr, rev = mech.arrhenius.copy(), mech.reversible.copy()
+    arr[-1], rev[-1] = (1e88, 0.0, 0.0), 0            # H2O2 + OH, both at 1e-45
+    m = dataclasses.replace(mech, arrhenius=arr, reversible=rev)
+    w = _without_radicals(m, 700.0)
+    for s in ("H2O2", "OH"):
+        w["Y"][m.index(s)] = 1e-45
+    err = _one_step_errors(m, w, lanes)
+    assert np.all(err < RTOL_FP64), err
