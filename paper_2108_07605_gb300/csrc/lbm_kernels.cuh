@@ -1168,7 +1168,8 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
   // in shared memory, entry-major with the block's threads contiguous (no
   // bank conflicts): in registers it would not fit beside the node's other
   // state and spills to local memory.
-  VT V[M][D], inv_tau_a[M], sv;
+  VT V[M][D], sv;
+  RT inv_tau_a[M];               // FP64: 2 + 1/tau_a
   {
     extern __shared__ unsigned char smem_raw[];
     VT* As = reinterpret_cast<VT*>(smem_raw) + threadIdx.x;
@@ -1192,14 +1193,15 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
       }
 #pragma unroll
       for (int a = 0; a < M; ++a) {
-        ff acc;
+        // in FP64: beta_a moves whole populations, not a correction (in
+        // float-float the lightest species lost two bits of FP64's accuracy)
+        double acc = 0.0;
 #pragma unroll
         for (int b = 0; b < M; ++b)
-          if (b != a) ff_fma_acc(acc, mech.K_f[a][b], Yv[b]);
-        inv_tau_a[a] = sv * ff_norm(acc);
-        ff dg(1.f);
-        ff_acc(dg, ff(0.5f * inv_tau_a[a].hi, 0.5f * inv_tau_a[a].lo));
-        As[(a * W + a) * st] = ff_norm(dg);
+          if (b != a) acc = fma(mech.K[a][b], Y[b], acc);
+        inv_tau_a[a] = fma(s_tau, acc, 2.0);
+        const ff dg = ff_of_double(inv_tau_a[a]);
+        As[(a * W + a) * st] = ff(0.5f * dg.hi, 0.5f * dg.lo);
       }
       solve_dd_ff<M, D>(As, st);
 #pragma unroll
@@ -1295,17 +1297,16 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
   //   f_a + 2 beta_a (rho_a psi_a - f_a) + cF_a sum_b K_ab d_b + drho_a psi_a
   //     = f_a om1_a + psi_a hh_a + cF_a sum_b K_ab d_b,
   // cF_a = (beta_a - 1) Y_a s (1/tau_ab = s K_ab), om1_a = 1 - 2 beta_a,
-  // hh_a = 2 beta_a rho_a + drho_a; beta = 1 / (2 tau + 1) to the precision of
-  // the diffusion velocities (om1 and hh share its rounding, so that mass is
-  // conserved)
+  // hh_a = 2 beta_a rho_a + drho_a; beta = 1 / (2 tau + 1) = 1 - 2 r, r =
+  // 1 / (2 + 1/tau) (om1 and hh share its rounding, so that mass is conserved)
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
     RT beta;
     if constexpr (sizeof(RT) == 8) {
-      ff den(2.f);
-      ff_acc(den, inv_tau_a[a]);
-      const ff r = ff_rcp(ff_norm(den));
-      beta = double_of_ff(inv_tau_a[a] * r);
+      // r in float-float and a Newton step in FP64
+      const ff r = ff_rcp(ff_of_double(inv_tau_a[a]));
+      const double r0 = double_of_ff(r);
+      beta = fma(-2.0, fma(r0, fma(-inv_tau_a[a], r0, 1.0), r0), 1.0);
       // beta - 1 = -2 / (2 + 1/tau)
       p.cF[a] = ff(-2.f * r.hi, -2.f * r.lo) * (ff_of_double(Y[a]) * sv);
     } else {

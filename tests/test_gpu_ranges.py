@@ -28,6 +28,15 @@ def _errors(mech, w, nsteps, precision="fp64"):
     return err
 
 
+def _inert(mech, D0):
+    """The mechanism's species without reactions."""
+    M = mech.n_species
+    return dataclasses.replace(
+        mech, nu_f=np.zeros((0, M)), nu_r=np.zeros((0, M)), arrhenius=np.zeros((0, 3)),
+        third_body=np.zeros(0, dtype=np.int32), efficiency=np.ones((0, M)),
+        reversible=np.zeros(0, dtype=np.int32), D0=D0)
+
+
 # The fixed-point rate arguments hold 1/T below 2^-7 (T above 128 K) and T below
 # 2^14 K.
 def _at_temperature(mech, shape, T0):
@@ -105,3 +114,22 @@ def test_rate_constant_far_beyond_its_products(mech, lanes):
         w["Y"][m.index(s)] = 1e-45
     err = _one_step_errors(m, w, lanes)
     assert np.all(err < RTOL_FP64), err
+
+
+# One step without reactions, composition as noise (diffusion velocities of the
+# order of the lattice speed for the lightest species), 1/tau from 3 to 3e5.  A
+# population is some ten roundings of terms of up to twice its size: 18 spacings
+# of FP64.  (Coefficients of 48 bits would leave 2^-48 of the same terms, 6e-15
+# and more.)
+@pytest.mark.parametrize("split", [0, 1])
+@pytest.mark.parametrize("scale", [10.0, 1.0, 0.1, 1e-2, 1e-4])
+def test_species_relaxation_keeps_fp64(mech, scale, split):
+    m = _inert(mech, mech.D0 * scale)
+    w = fields.perturbed_box((9, 5, 3), "D3Q27", mech=m, T0=1300.0, dx=25e-6)
+    o, g = make_oracle(m, w), make_gpu(m, w)
+    g.set_launch(collide_split=split)
+    o.step(1)
+    g.step(1)
+    err = max_rel_err_per_lattice(g.populations(), oracle_populations(o))
+    g.close()
+    assert np.all(err < 18 * 2.0 ** -52), err
