@@ -245,6 +245,22 @@ __device__ __forceinline__ double double_join(ff a) {
       ((unsigned long long)((m >> 3) + (896 << 20)) << 32 | ((unsigned)b << 29)) + (long long)l;
   return __longlong_as_double((long long)(d | (unsigned long long)(b & 0x80000000u) << 32));
 }
+// d = m 2^e, 1 <= |m| < 2 (0 and denormals: m = 0; infinities, NaN: m = NaN)
+__device__ __forceinline__ ff ff_mantissa(double d, int& e) {
+  const int h = __double2hiint(d), ex = (h >> 20) & 0x7ff;
+  e = ex - 1023;
+  if (ex == 0x7ff) return ff(__int_as_float(0x7fffffff), 0.f);
+  return ex == 0 ? ff() : ff_of_double(__hiloint2double((h & 0x800fffff) | 0x3ff00000,
+                                                        __double2loint(d)));
+}
+// a 2^e for a normalised pair, 0 below FP64's normal numbers
+__device__ __forceinline__ double double_join(ff a, int e) {
+  const double d = double_join(a);
+  const int h = __double2hiint(d), ex = (h >> 20) & 0x7ff;
+  if (ex == 0x7ff) return d;
+  if (ex == 0 || ex + e <= 0) return 0.0;
+  return __hiloint2double(h + (e << 20), __double2loint(d));
+}
 // 1 / a
 __device__ __forceinline__ ff ff_rcp(ff a) {
   const float q = __fdiv_rn(1.f, a.hi);

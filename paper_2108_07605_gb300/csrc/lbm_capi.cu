@@ -250,6 +250,7 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
   // Gibbs functions g_a/(R_U T) = gi/T + g0 + g1 T + g2 T^2 - a0 ln T
   double gi[LBM_MAX_SPECIES], g0[LBM_MAX_SPECIES], g1[LBM_MAX_SPECIES], g2[LBM_MAX_SPECIES],
       ga[LBM_MAX_SPECIES];
+  double Kmax = 0.0;
   for (int a = 0; a < m.n_species; ++a) {
     const double mm = m.molar_mass[a];
     const double a0 = m.cp[a][0], a1 = m.cp[a][1], a2 = m.cp[a][2];
@@ -269,9 +270,13 @@ void build_mech(const lbm_mechanism& m, DevMech& d) {
     for (int b = 0; b < m.n_species; ++b) {
       d.K[a][b] = a == b ? 0.0 : 1.0 / (mm * m.molar_mass[b] * m.D0[a][b]);
       d.Kf[a][b] = (float)d.K[a][b];
-      d.K_f[a][b] = ff_host(d.K[a][b]);
+      Kmax = std::max(Kmax, d.K[a][b]);
     }
   }
+  d.K_exp = std::ilogb(Kmax);
+  d.K_unit = std::ldexp(1.0, d.K_exp);
+  for (int a = 0; a < m.n_species; ++a)
+    for (int b = 0; b < m.n_species; ++b) d.K_f[a][b] = ff_host(d.K[a][b] / d.K_unit);
   // the reactions without a third body, then those of each distinct row of
   // efficiencies
   int rows = 0, set[LBM_MAX_REACTIONS];

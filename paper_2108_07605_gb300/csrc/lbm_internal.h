@@ -62,7 +62,11 @@ struct DevMech {
   // 1/tau_ab = s(node) * K[a][b], K = 1/(m_a m_b D0_ab)
   double K[LBM_MAX_SPECIES][LBM_MAX_SPECIES];
   float Kf[LBM_MAX_SPECIES][LBM_MAX_SPECIES];   // K rounded to FP32 (mixed path)
-  ff K_f[LBM_MAX_SPECIES][LBM_MAX_SPECIES];     // and as float-float (FP64 path)
+  // and as float-float (FP64 path), over K_unit = 2^K_exp, the largest one's power
+  // of two (K may lie outside FP32's range; s K_unit goes with it)
+  ff K_f[LBM_MAX_SPECIES][LBM_MAX_SPECIES];
+  double K_unit;
+  int K_exp;
   double D_T_exp, mu0, mu_T_exp, inv_prandtl;
   // Wilke's mixing rule (wilke = 1): species viscosities at T0 and the
   // T-independent Phi_ab (the species share the T exponent)

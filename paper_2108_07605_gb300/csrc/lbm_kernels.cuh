@@ -1000,8 +1000,9 @@ template <int D, int M, typename RT> struct NodePar {
   RT rho, om, U, theta;          // density, omega, internal energy, R T (lattice)
   RT u[D], Pex[D], W[D];         // velocity, extended diagonal pressure, energy-flux term
   RT th[M], rs[M];               // theta_b, rho_b
-  typename DiffType<RT>::type V[M][D], cF[M - 1];  // diffusion velocities, (beta_a - 1) Y_a s
-  RT om1[M - 1], hh[M - 1];      // 1 - 2 beta_a, 2 beta_a rho_a + drho_a
+  typename DiffType<RT>::type V[M][D];             // diffusion velocities
+  // (beta_a - 1) Y_a s, 1 - 2 beta_a, 2 beta_a rho_a + drho_a
+  RT cF[M - 1], om1[M - 1], hh[M - 1];
 };
 
 // Field offsets of NodePar stored field-major [field][N] (split collision);
@@ -1175,7 +1176,7 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
     VT* As = reinterpret_cast<VT*>(smem_raw) + threadIdx.x;
     const int st = kBS;
     if constexpr (sizeof(RT) == 8) {
-      sv = ff_of_double(s_tau);
+      sv = ff_of_double(s_tau * mech.K_unit);
       constexpr int W = M + D;
       ff Yv[M], yh[M];
 #pragma unroll
@@ -1304,11 +1305,13 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
     RT beta;
     if constexpr (sizeof(RT) == 8) {
       // r in float-float and a Newton step in FP64
-      const ff r = ff_rcp(ff_of_double(inv_tau_a[a]));
-      const double r0 = double_of_ff(r);
-      beta = fma(-2.0, fma(r0, fma(-inv_tau_a[a], r0, 1.0), r0), 1.0);
-      // beta - 1 = -2 / (2 + 1/tau)
-      p.cF[a] = ff(-2.f * r.hi, -2.f * r.lo) * (ff_of_double(Y[a]) * sv);
+      int e;
+      const ff x = ff_mantissa(inv_tau_a[a], e);
+      const double r0 = double_join(ff_rcp(x), -e);
+      const double r = fma(r0, fma(-inv_tau_a[a], r0, 1.0), r0);
+      beta = fma(-2.0, r, 1.0);
+      // beta - 1 = -2 r; FP64's range, which trace species need
+      p.cF[a] = r * (Y[a] * (-2.0 * s_tau));
     } else {
       beta = inv_tau_a[a] / (RT(2) + inv_tau_a[a]);
       p.cF[a] = (beta - RT(1)) * Y[a] * s_tau;
@@ -1457,14 +1460,12 @@ __device__ __forceinline__ double stored(ff v) { return ff_pack(v); }
 // kBS, d = 1, 2).
 template <int D, int M, typename RT> struct RegPar {
   const NodePar<D, M, RT>& p;
-  RT Afv[D][3], Bfv[D][3], cFv[M - 1], Vx[M];
+  RT Afv[D][3], Bfv[D][3], Vx[M];
   const RT* tab;
   const RT* yztab;
   __device__ RegPar(const NodePar<D, M, RT>& p_, const RT* tab_, const RT* yztab_ = nullptr)
       : p(p_), tab(tab_), yztab(yztab_) {
     energy_factors<D, RT>(p.u, p.theta, Afv, Bfv);
-#pragma unroll
-    for (int a = 0; a < M - 1; ++a) cFv[a] = value_of(p.cF[a]);
 #pragma unroll
     for (int b = 0; b < M; ++b) Vx[b] = value_of(p.V[b][0]);
   }
@@ -1475,7 +1476,7 @@ template <int D, int M, typename RT> struct RegPar {
   __device__ RT Pex(int d) const { return p.Pex[d]; }
   __device__ RT W(int d) const { return p.W[d]; }
   __device__ RT rs(int a) const { return p.rs[a]; }
-  __device__ RT cF(int a) const { return cFv[a]; }
+  __device__ RT cF(int a) const { return p.cF[a]; }
   __device__ RT om1(int a) const { return p.om1[a]; }
   __device__ RT hh(int a) const { return p.hh[a]; }
   __device__ RT Af(int d, int c) const { return c == 0 ? Afv[d][1] : (c > 0 ? Afv[d][2] : Afv[d][0]); }
@@ -1580,7 +1581,7 @@ __device__ __forceinline__ void prep_body(const RT* __restrict__ rec,
   }
 #pragma unroll
   for (int a = 0; a < M - 1; ++a) {
-    cp[(CP::CF + a) * N + n] = stored(p.cF[a]);
+    cp[(CP::CF + a) * N + n] = p.cF[a];
     cp[(CP::OM1 + a) * N + n] = p.om1[a];
     cp[(CP::HH + a) * N + n] = p.hh[a];
   }
@@ -1607,8 +1608,9 @@ template <int D, int M, typename RT> constexpr int coll_smem_entries();
 // Layout of k_coll's shared memory in FP64 (8-byte entries per node): the FP64
 // axis factors E of the stored species' equilibria (x: times hh_a), float-float
 // tables (packed pairs) of the Stefan-Maxwell term's factors, the extended
-// equilibrium's and the energy factors, the species coefficients cF (a pair)
-// and 1 - 2 beta, and the scalars.  The pairs:
+// equilibrium's and the energy factors, the species coefficients cF (a pair with
+// an exponent of its own, cF being as small as Y_a) and 1 - 2 beta, and the
+// scalars.  The pairs:
 //   e_d(c), the axis factor of psi(u, theta_b), and t_d(c) = s_d(c) - e_d(c),
 //   s_d(c) that of psi(u + V_b, theta_b), formed without cancellation from
 //   V_b (t(0) = -V (2u + V), t(+-1) = (V (2u + V) +- V)/2); for x, s and t
@@ -1618,7 +1620,7 @@ template <int D, int M> struct Coll64 {
   static constexpr int EX = F + M * D * 6, AF = EX + 3 * D, BF = AF + 3 * D;
   static constexpr int CF = BF + 3 * D, OM1 = CF + M - 1;
   static constexpr int RHO = OM1 + M - 1, OM = RHO + 1, U = OM + 1, W = U + 1;
-  static constexpr int N = W + D;
+  static constexpr int CE = W + D, N = CE + M / 2;       // CE: M - 1 ints per node
   static constexpr int e(int a, int d, int c) { return E + (a * D + d) * 3 + c + 1; }
   // first of a pair: x: -rho s(c), then -rho t(c); y, z: e(c), then t(c)
   static constexpr int f(int b, int d, int c) { return F + (b * D + d) * 6 + c + 1; }
@@ -1679,6 +1681,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   const int tag = n < N ? (bc.tag ? bc.tag[n] : TAG_BULK) : TAG_SOLID;
   const bool valid = tag != TAG_SOLID;
   double* const s = sm + lane;
+  int* const ce = reinterpret_cast<int*>(sm + T::CE * kCollNodes) + lane;
   const int x = (int)(n % g.nx);
   const int y = (int)((n / g.nx) % g.ny);
   const int z = (int)(n / ((long long)g.nx * g.ny));
@@ -1745,7 +1748,9 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
       s[T::U * kCollNodes] = G(CP::UL);
     }
     for (int a = w; a < M - 1; a += TPN) {
-      s[(T::CF + a) * kCollNodes] = G(CP::CF + a);
+      int e;
+      s[(T::CF + a) * kCollNodes] = ff_pack(ff_mantissa(G(CP::CF + a), e));
+      ce[a * kCollNodes] = e + mech.K_exp;
       s[(T::OM1 + a) * kCollNodes] = G(CP::OM1 + a);
     }
   }
@@ -1812,7 +1817,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
         if (b != a) ff_fma_acc(F, mech.K_f[a][b], dd[b]);
       F = PF(T::CF + a) * ff_norm(F);
       const double ez = D == 3 ? P(T::e(a, D - 1, cz)) : 1.0;
-      const double base = fma(take(a), P(T::OM1 + a), double_join(F));
+      const double base = fma(take(a), P(T::OM1 + a), double_join(F, ce[a * kCollNodes]));
       next(a);
       dst[(long long)(a * Q + i) * N + n] = D == 3 ? fma(eh[a], ez, base) : eh[a] + base;
     }

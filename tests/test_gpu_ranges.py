@@ -133,3 +133,37 @@ def test_species_relaxation_keeps_fp64(mech, scale, split):
     err = max_rel_err_per_lattice(g.populations(), oracle_populations(o))
     g.close()
     assert np.all(err < 18 * 2.0 ** -52), err
+
+
+# Trace species between main ones: their Stefan-Maxwell term scales with their mass
+# fraction, its coefficient far below FP32's numbers.  And diffusivities so small
+# that m_a m_b D_ab alone leaves FP32's range.
+@pytest.mark.parametrize("split", [0, 1])
+@pytest.mark.parametrize("trace", [1e-25, 1e-36, 1e-60])
+def test_trace_species_diffuse_as_the_others(mech, trace, split):
+    m = _inert(mech, mech.D0)
+    w = fields.perturbed_box((9, 5, 3), "D3Q27", mech=m, T0=1300.0, dx=25e-6, amp_Y=0.2)
+    for s in ("H", "O", "OH", "HO2", "H2O2"):
+        w["Y"][m.index(s)] *= trace
+    w["Y"][8] = 1.0 - w["Y"][:8].sum(axis=0)
+    o, g = make_oracle(m, w), make_gpu(m, w)
+    g.set_launch(collide_split=split)
+    o.step(3)
+    g.step(3)
+    err = max_rel_err_per_lattice(g.populations(), oracle_populations(o))
+    g.close()
+    assert np.all(err < RTOL_FP64), err
+
+
+def test_formed_radicals_diffuse(mech):
+    err = _errors(mech, _without_radicals(mech, 300.0), 3)
+    assert np.all(err < RTOL_FP64), err
+
+
+@pytest.mark.parametrize("shape,lattice", [((9, 5, 3), "D3Q27"), ((13, 11, 1), "D2Q9")])
+def test_tiny_diffusivities(mech, shape, lattice):
+    m = _inert(mech, mech.D0 * 1e-28)
+    m.D0[0, :] *= 1e-4
+    m.D0[:, 0] = m.D0[0, :]
+    err = _errors(m, fields.perturbed_box(shape, lattice, mech=m, T0=1300.0, dx=25e-6), 2)
+    assert np.all(err < RTOL_FP64), err
