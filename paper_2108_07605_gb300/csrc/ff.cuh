@@ -228,6 +228,23 @@ __device__ __forceinline__ double double_of_float(float f) {
   if (m >= 0x7f800000) h = m > 0x7f800000 ? 0x7ff80000 : 0x7ff00000;
   return __hiloint2double(h | (b & 0x80000000), m < 0x00800000 ? 0 : b << 29);
 }
+// exact for denormals too
+__device__ __forceinline__ double double_of_float_exact(float f) {
+  const bool sub = (__float_as_int(f) & 0x7fffffff) < 0x00800000;
+  const double d = double_of_float(sub ? f * 16777216.f : f);
+  const int h = __double2hiint(d), l = __double2loint(d);
+  return __hiloint2double(sub && (h << 1) != 0 ? h - (24 << 20) : h, l);
+}
+// rounded to nearest (the conversion instruction for results that are denormal
+// or infinite)
+__device__ __forceinline__ float float_of_double(double d) {
+  const int h = __double2hiint(d), l = __double2loint(d), mag = h & 0x7fffffff;
+  if ((unsigned)(mag - 0x38100000) >= 0x0fe00000u)
+    return mag < 0x36900000 ? __int_as_float(h & 0x80000000) : __double2float_rn(d);
+  const unsigned up = (unsigned)(l & 0x1fffffff) + ((l >> 29) & 1) > 0x10000000u;
+  return __int_as_float(((int)(__funnelshift_l(l, mag, 3) - (896u << 23)) + (int)up) |
+                        (h & 0x80000000));
+}
 __device__ __forceinline__ double double_of_ff(ff a) {
   return double_of_float(a.hi) + double_of_float(a.lo);
 }

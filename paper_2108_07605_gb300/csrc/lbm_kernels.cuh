@@ -787,8 +787,8 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
         rd = rs;
         Rm = fma(Y, mech.inv_mm[a], Rm);
       } else {
-        Yd = double_of_float(Y);
-        rd = double_of_float(rs);
+        Yd = double_of_float_exact(Y);
+        rd = double_of_float_exact(rs);
         Rm += Y * mech.inv_mm_s[a];
       }
       cU[0] = fma(Yd, mech.u0[a], cU[0]);
@@ -2531,7 +2531,7 @@ template <int D, int M, typename S, typename RT> constexpr size_t persist_smem(b
 // pattern, the conversion instruction runs at the FP64 pipe's rate).
 __device__ __forceinline__ void store_pop(double* p, double v, const float4*, int) { *p = v; }
 __device__ __forceinline__ void store_pop(float* p, double v, const float4*, int) {
-  *p = ff_of_double(v).hi;
+  *p = float_of_double(v);
 }
 __device__ __forceinline__ void store_pop(__half* p, double v, const float4* codec, int li) {
   *p = Codec<__half>::enc(v, codec, li);
@@ -2614,18 +2614,18 @@ k_init(const double* __restrict__ rho_or_P, int is_pressure, const double* __res
 
 // Sums of node n's stored populations in FP64 (fixed point): rho, j, rho E, and
 // species(a, rho_a) for every species, the slaved one last.
-__device__ __forceinline__ double wide(double v) { return v; }
-__device__ __forceinline__ double wide(float v) { return double_of_float(v); }
 template <typename S> struct StoredType { using type = float; };
 template <> struct StoredType<double> { using type = double; };
 
-// Q populations of a lattice from pl, N apart, and their largest biased
-// exponent.  FP32: from the largest bit pattern, so that all loads are in flight
-// before the first is widened.
+// Q populations of a lattice from pl, N apart, times 2^shift, and their largest
+// biased exponent.  FP32: from the largest bit pattern, so that all loads are in
+// flight before the first is widened; shift: 64 where FP32's denormals count.
 template <typename S, int Q>
 __device__ __forceinline__ int load_lattice(const S* __restrict__ pl, long long N,
-                                            const float4* codec, int li, double (&v)[Q]) {
+                                            const float4* codec, int li, double (&v)[Q],
+                                            int& shift) {
   int e = 0;
+  shift = 0;
   if constexpr (sizeof(S) == 8) {
 #pragma unroll
     for (int i = 0; i < Q; ++i, pl += N) v[i] = __ldg(pl);
@@ -2638,9 +2638,11 @@ __device__ __forceinline__ int load_lattice(const S* __restrict__ pl, long long 
       f[i] = Codec<S>::template dec<float>(__ldg(pl), codec, li + i);
 #pragma unroll
     for (int i = 0; i < Q; ++i) e = max(e, __float_as_int(f[i]) & 0x7fffffff);
-    e = fix_exponent(wide(__int_as_float(e)));
+    if (e < (67 << 23)) shift = 64;                // all below 2^-60
+    const float sc = shift ? 0x1p64f : 1.f;
+    e = fix_exponent(double_of_float(sc * __int_as_float(e)));
 #pragma unroll
-    for (int i = 0; i < Q; ++i) v[i] = wide(f[i]);
+    for (int i = 0; i < Q; ++i) v[i] = double_of_float(sc * f[i]);
   }
   return e;
 }
@@ -2656,9 +2658,10 @@ __device__ __forceinline__ void stored_sums(const S* __restrict__ pops, long lon
     const int l = it == 0 ? M - 1 : (it == 1 ? M : it - 2);   // f, g, the species
     double v[Q];
     const S* pl = pops + (long long)l * Q * N + n;
-    const int e = load_lattice<S>(pl, N, codec, l * Q, v);
+    int shift, e = load_lattice<S>(pl, N, codec, l * Q, v, shift);
     Fix sum, sj[D], sP[NP];
     lattice_sums<D, double>(v, e, sum, sj, sP);
+    e -= shift;
     const FixSum t = fix_sum(sum, e);
     const double s0 = double_of_fix(t);
     if (it == 0) {

@@ -167,3 +167,16 @@ def test_tiny_diffusivities(mech, shape, lattice):
     m.D0[:, 0] = m.D0[0, :]
     err = _errors(m, fields.perturbed_box(shape, lattice, mech=m, T0=1300.0, dx=25e-6), 2)
     assert np.all(err < RTOL_FP64), err
+
+
+def test_fp32_storage_holds_denormal_populations(mech):
+    """A species at mass fractions of 1e-40 to 1e-38 in FP32 storage: populations
+    rounded to FP32 (its denormals among them), read out as they are stored."""
+    w = fields.perturbed_box((9, 5, 3), "D3Q27", mech=mech, T0=1300.0, dx=25e-6)
+    Y = w["Y"][3]
+    Y[:] = 1e-40 * (1.0 + 100.0 * np.arange(Y.size).reshape(Y.shape) / Y.size)
+    o, g = make_oracle(mech, w), make_gpu(mech, w, precision="fp32")
+    ref, got, m = oracle_populations(o), g.populations(), g.moments()
+    g.close()
+    assert np.all(np.abs(got[3] - ref[3]) <= 2.0 ** -24 * np.abs(ref[3]) + 2.0 ** -150)
+    assert np.allclose(m["Y"][3], got[3].sum(axis=0) / got[8].sum(axis=0), rtol=1e-12, atol=0.0)
