@@ -769,15 +769,16 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   for (int d = 0; d < D; ++d) u[d] = Z[d] = RT(0);
 
   // species a's state from its sums: record, concentration, energy polynomial
+  // (FP32: rho times it, Y rounded to FP32 would cost the sub-steps' energies bits)
   auto species = [&](int a, RT rs, const RT (&js)[D]) {
     const RT Y = rs * inv_rho;
     rec[(RC::Y + a) * N + n] = Y;
     if constexpr (kFF<RT>) {
       Rm += Y * mech.inv_mm_s[a];
-      ff_fma_acc(cU[0], ff(Y), mech.u0_f[a]);
-      ff_fma_acc(cU[1], ff(Y), mech.u1_f[a]);
-      ff_fma_acc(cU[2], ff(Y), mech.u2_f[a]);
-      ff_fma_acc(cU[3], ff(Y), mech.u3_f[a]);
+      ff_fma_acc(cU[0], ff(rs), mech.u0_f[a]);
+      ff_fma_acc(cU[1], ff(rs), mech.u1_f[a]);
+      ff_fma_acc(cU[2], ff(rs), mech.u2_f[a]);
+      ff_fma_acc(cU[3], ff(rs), mech.u3_f[a]);
       cs.set(a, ff(rs) * mech.inv_mm_f[a]);
       Wd[a * kChemThreads] = ff_pack(ff());
     } else {
@@ -787,8 +788,7 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
         rd = rs;
         Rm = fma(Y, mech.inv_mm[a], Rm);
       } else {
-        Yd = double_of_float_exact(Y);
-        rd = double_of_float_exact(rs);
+        rd = Yd = double_of_float_exact(rs);
         Rm += Y * mech.inv_mm_s[a];
       }
       cU[0] = fma(Yd, mech.u0[a], cU[0]);
@@ -863,11 +863,21 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   // temperature (Eq. temperature) from the node's previous T
   using X = Chem<CT>;
   CT U;
+  ff irho;
   if constexpr (kFF<RT>) {
+    irho = ff_rcp(ff(rho));
 #pragma unroll
-    for (int k = 0; k < 4; ++k) cU[k] = ff_norm(cU[k]);
+    for (int k = 0; k < 4; ++k) cU[k] = ff_norm(cU[k]) * irho;
     U = (ff(ER) + ff(-0.5f * usq)) * un.c2_f;
   } else {
+    if constexpr (sizeof(RT) == 8) {
+      irho = ff_of_double(inv_rho);
+    } else {
+      const double ir = 1.0 / double(rho);
+      irho = ff_of_double(ir);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) cU[k] *= ir;
+    }
     U = (double(ER) - 0.5 * double(usq)) * un.c * un.c;
   }
   bool ok;
@@ -901,9 +911,6 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   // reactor per node from its post-stream species densities; T_0 is the T just
   // solved
   ff dU[4];                              // increments of rho cU
-  ff irho;
-  if constexpr (sizeof(RT) == 8) irho = ff_of_double(inv_rho);
-  else irho = ff_rcp(ff(rho));
 #pragma unroll 1
   for (int s = 0; s < un.substeps; ++s) {
     if (s > 0) {

@@ -5,8 +5,9 @@ import numpy as np
 import pytest
 
 from lbm_workloads import fields
-from lbm_workloads.mechanism import h2_air_synthetic
+from lbm_workloads.mechanism import R_UNIVERSAL, binary_inert, h2_air_synthetic
 from oracle.diagnostics import diagnostics
+from paper_2108_07605_gb300 import lbm
 
 from helpers import make_gpu, make_oracle, max_rel_err_per_lattice, oracle_populations
 
@@ -180,3 +181,28 @@ def test_fp32_storage_holds_denormal_populations(mech):
     g.close()
     assert np.all(np.abs(got[3] - ref[3]) <= 2.0 ** -24 * np.abs(ref[3]) + 2.0 ** -150)
     assert np.allclose(m["Y"][3], got[3].sum(axis=0) / got[8].sum(axis=0), rtol=1e-12, atol=0.0)
+
+
+@pytest.mark.parametrize("lattice,shape", [("D3Q27", (5, 4, 3)), ("D2Q9", (7, 5, 1))])
+@pytest.mark.parametrize("lanes", [1, 4])
+@pytest.mark.parametrize("precision", ["fp32", "fp32c64"])
+def test_energies_of_unrounded_mass_fractions(precision, lanes, lattice, shape):
+    """A uniform state at rest is a fixed point.  rho = 13, Y = (10/13, 3/13)
+    and theta = 1/4 make its populations and their sums exact in FP32, the mass
+    fractions not; formation enthalpies that cancel in the mixture turn FP32
+    rounding of Y into 0.02 K (6e-5).  One step (its own rounding of the species
+    populations is as large in the next); what FP32 rounds of the rest (energy,
+    theta, relaxation) stays below 16 of its spacings."""
+    m = binary_inert(h_formation=(1e7, -1e7 / 0.3))
+    T, N = 300.0, int(np.prod(shape))
+    c_ref = float(np.sqrt(4.0 * R_UNIVERSAL / m.molar_mass[0] * T))
+    s = lbm.Solver(m, lattice=lattice, shape=shape, dx=1e-6, precision="fp32",
+                   chem_fp64=int(precision == "fp32c64"), substeps=2, c_ref=c_ref)
+    s.set_launch(chem_lanes=lanes)
+    Y = np.repeat([[10.0 / 13.0], [3.0 / 13.0]], N, axis=1)
+    s.init_fields(np.full(N, 13.0), np.zeros((3, N)), np.full(N, T), Y)
+    before = s.populations()
+    s.step(1)
+    err = max_rel_err_per_lattice(s.populations(), before)
+    s.close()
+    assert np.all(err < 16 * 2.0 ** -23), err
