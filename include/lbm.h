@@ -441,6 +441,25 @@ lbm_status lbm_ff_check(const double* x, long long n, double* exp_out, double* l
  * device error. */
 lbm_status lbm_exp64_check(const double* x, long long n, double* exp_out);
 
+/* The arithmetic that the kernels use beside the FP64 pipe, at the n points x
+ * (host arrays; out receives n values).  A test hook; synchronous.
+ * LBM_ERR_INVALID for NULL buffers, n < 0 or an unknown operation,
+ * LBM_ERR_RANGE for n > 2^24, LBM_ERR_CUDA on a device error. */
+typedef enum {
+  LBM_ARITH_LOG = 0,       /* ln x of temperatures                                */
+  LBM_ARITH_EXP2 = 1,      /* 2^(x/64) as 64-bit significand (FP64 rate constants) */
+  LBM_ARITH_EXP2_PAIR = 2, /* the same as a pair of FP32 (float-float rates)      */
+  LBM_ARITH_SUM = 3,       /* n a multiple of 27; of each group of 27: its sum,
+                              then the sum of its terms k = 2 mod 3 less that of
+                              those k = 0 mod 3 (a momentum), then zeros, by
+                              fixed-point addition                             */
+  LBM_ARITH_PAIR = 4,      /* x to a pair of FP32 and back                        */
+  LBM_ARITH_SIG = 5,       /* x to a 64-bit significand and back                  */
+  LBM_ARITH_FLOAT = 6,     /* x to FP32 and back                                  */
+  LBM_ARITH_MANTISSA = 7   /* x to a pair with an exponent and back               */
+} lbm_arith;
+lbm_status lbm_arith_check(lbm_arith op, const double* x, long long n, double* out);
+
 /* Measured fused-multiply-add throughput of the current device in TFLOP/s
  * (2 FLOP per FMA), FP64 when fp64 != 0, else FP32.  No counterpart in the
  * paper: the ALU roof against which the step's executed operation counts

@@ -8,8 +8,7 @@
 #include <string>
 #include <vector>
 
-#include "exp64.cuh"
-#include "ff.cuh"
+#include "lbm_device.cuh"
 #include "lbm_internal.h"
 
 using namespace lbm;
@@ -1777,6 +1776,66 @@ lbm_status lbm_exp64_check(const double* x, long long n, double* exp_out) {
   if (e == cudaSuccess) e = cudaMemcpy(exp_out, d + n, b, cudaMemcpyDeviceToHost);
   cudaFree(d);
   return e == cudaSuccess ? LBM_OK : cuda_fail(nullptr, e, "lbm_exp64_check");
+}
+
+// ---------------------------------------------------------------------------
+// The kernels' own arithmetic at given points (a test hook).
+__global__ void k_arith_check(int op, const double* __restrict__ x, long long n,
+                              double* __restrict__ out) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double v = x[i];
+  switch (op) {
+    case LBM_ARITH_LOG: out[i] = log_tang(v); break;
+    case LBM_ARITH_EXP2: out[i] = double_of_sig(exp_sig(v)); break;
+    case LBM_ARITH_EXP2_PAIR: {
+      const ExpArg a = exp_arg(ff_of_double(v));
+      out[i] = ff_to_double(ff_scale(exp_frac(a), a.n >> 6));
+      break;
+    }
+    case LBM_ARITH_SUM: {
+      const double* g = x + i / 27 * 27;
+      const int p = (int)(i % 27);
+      int e = 0;
+      for (int k = 0; k < 27; ++k) e = max(e, fix_exponent(g[k]));
+      Fix s;
+      for (int k = 0; k < 27; ++k) {
+        const Fix f = fix_of(g[k], e);
+        if (p == 0 || k % 3 == 2) s = s + f;
+        else if (k % 3 == 0) s = s - f;
+      }
+      out[i] = p < 2 ? double_of_fix(fix_sum(s, e)) : 0.0;
+      break;
+    }
+    case LBM_ARITH_PAIR: out[i] = double_join(ff_of_double(v)); break;
+    case LBM_ARITH_SIG: out[i] = double_of_sig(sig_of(v)); break;
+    case LBM_ARITH_FLOAT: out[i] = double_of_float_exact(float_of_double(v)); break;
+    default: {
+      int e;
+      const ff m = ff_mantissa(v, e);
+      out[i] = double_join(m, e);
+    }
+  }
+}
+
+lbm_status lbm_arith_check(lbm_arith op, const double* x, long long n, double* out) {
+  if (!x || !out || n < 0 || op < LBM_ARITH_LOG || op > LBM_ARITH_MANTISSA ||
+      (op == LBM_ARITH_SUM && n % 27 != 0))
+    return fail(nullptr, LBM_ERR_INVALID, "lbm_arith_check: bad operation, buffer or count");
+  if (n > (1LL << 24)) return fail(nullptr, LBM_ERR_RANGE, "lbm_arith_check: n above 2^24");
+  if (n == 0) return LBM_OK;
+  double* d = nullptr;
+  const size_t b = (size_t)n * sizeof(double);
+  cudaError_t e = cudaMalloc(&d, 2 * b);
+  if (e != cudaSuccess) return cuda_fail(nullptr, e, "lbm_arith_check allocation");
+  e = cudaMemcpy(d, x, b, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    k_arith_check<<<(unsigned)((n + 255) / 256), 256>>>((int)op, d, n, d + n);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(out, d + n, b, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e == cudaSuccess ? LBM_OK : cuda_fail(nullptr, e, "lbm_arith_check");
 }
 
 // ---------------------------------------------------------------------------

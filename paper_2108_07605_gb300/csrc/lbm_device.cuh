@@ -82,7 +82,7 @@ __device__ __forceinline__ double record_us(double v) { return ff_pack(ff_of_dou
 // lattice's populations at a node) is shifted to a common exponent, that of
 // the largest, and added in integers.  A value is cut at 2^-63 of the largest
 // one's power of two (a double's own last bit lies at 2^-52 of it), and the
-// sums of up to 32 terms are exact; with the small differences that a momentum
+// sums of a lattice's 27 terms are exact (31 fit a); with the small differences that a momentum
 // is made of, this is what FP64 differences keep, and more.
 //
 // Fix: the value modulo 2^64 in units of 2^(e - 63), and a, the same in units
@@ -108,7 +108,7 @@ __device__ __forceinline__ Fix fix_of(double v, int e) {
   unsigned long long m = ((unsigned long long)(hm << 11 | (unsigned)l >> 21) << 32) |
                          (unsigned)(l << 11);
   m >>= min(e - ev, 63);
-  if (ev == 0) m = 0;                          // zeros, denormals
+  if (ev == 0 || e - ev > 63) m = 0;           // zeros, denormals, values far below
   const int a = (int)(m >> 38);
   return h < 0 ? Fix(0ull - m, -a) : Fix(m, a);
 }

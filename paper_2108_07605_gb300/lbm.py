@@ -112,6 +112,7 @@ EXPORTS = {
     "lbm_batch_autotune": (C.c_int, [C.c_void_p, C.c_int, C.POINTER(lbm_launch)]),
     "lbm_ff_check": (C.c_int, [C.c_void_p, C.c_longlong, C.c_void_p, C.c_void_p]),
     "lbm_exp64_check": (C.c_int, [C.c_void_p, C.c_longlong, C.c_void_p]),
+    "lbm_arith_check": (C.c_int, [C.c_int, C.c_void_p, C.c_longlong, C.c_void_p]),
     "lbm_batch_set_launch": (C.c_int, [C.c_void_p, C.POINTER(lbm_launch)]),
     "lbm_batch_get_launch": (C.c_int, [C.c_void_p, C.POINTER(lbm_launch)]),
     "lbm_set_launch": (C.c_int, [C.c_void_p, C.POINTER(lbm_launch)]),
@@ -314,8 +315,21 @@ def lbm_batch_autotune(plan, trial_steps=3):
     return _launch_dict(out)
 
 
+ARITH = {"log": 0, "exp2": 1, "exp2_pair": 2, "sum": 3, "pair": 4, "sig": 5, "float": 6,
+         "mantissa": 7}
+
+
+def lbm_arith_check(op, x):
+    """The kernels' own arithmetic (ARITH) at the points x (1-D float64)."""
+    import numpy as np
+    x = np.ascontiguousarray(x, dtype=np.float64)
+    out = np.empty_like(x)
+    _check(load_library().lbm_arith_check(ARITH[op], x.ctypes.data, x.size, out.ctypes.data))
+    return out
+
+
 def lbm_exp64_check(x):
-    """The library's FP64 exp (reaction rates) at the points x (1-D float64)."""
+    """The library's FP64 exp (transport laws) at the points x (1-D float64)."""
     import numpy as np
     x = np.ascontiguousarray(x, dtype=np.float64)
     e = np.empty_like(x)
