@@ -1198,6 +1198,7 @@ __device__ __forceinline__ void bnode_warp(const S* __restrict__ src, const BCDe
     const bool simple = kind == BK_INLET && bc.inlet_simplified != 0;
     const WState<D, M, R>& t = simple ? L : (kind == BK_INLET ? B : A);
     const R Et = state_energy<D, R>(t), El = state_energy<D, R>(L);
+    __syncwarp();                        // the sums' readers (wstate_of) are done
     if (lane <= M) {
       R* zl = sm + W::Z + lane * W::ZS;
       if (lane < M - 1) {
