@@ -1035,7 +1035,14 @@ template <int D, int M> struct CPar {
 // moments from the record, isotropic gradients, relaxation parameters,
 // diffusion velocities, energy-flux correction.  The diffusion-velocity
 // solve uses this thread's shared-memory column (M*M entries, stride kBS).
-template <int D, int M, typename RT>
+// kLive: the records were written earlier in the same launch (k_step_persist),
+// so the neighbours' fields may not come through the read-only path.
+template <bool kLive, typename RT>
+__device__ __forceinline__ RT record_load(const RT* p) {
+  if constexpr (kLive) return __ldcg(p);
+  else return __ldg(p);
+}
+template <int D, int M, bool kLive, typename RT>
 __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
                                             const double* __restrict__ Tf, const Geom& g,
                                             const Units& un, const BCDev& bc,
@@ -1075,7 +1082,8 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
   for (int d = 0; d < D; ++d) dPhi[d] = corr[d] = RT(0);
   auto enthalpy = [&](long long nb) {
     const RT* h = rec + (long long)RC::H * N + nb;
-    return fma(T, fma(T, fma(T, __ldg(h + 3 * N), __ldg(h + 2 * N)), __ldg(h + N)), __ldg(h));
+    auto H = [&](int k) { return record_load<kLive>(h + k * N); };
+    return fma(T, fma(T, fma(T, H(3), H(2)), H(1)), H(0));
   };
   const RT HYself = enthalpy(n);
   // ghost values beyond non-periodic faces and on solid nodes: walls Phi = 0,
@@ -1134,7 +1142,7 @@ __device__ __forceinline__ void node_params(const RT* __restrict__ rec,
       for (int d = 0; d < D; ++d) {
         if (cvi[d] == 0) continue;
         const RT wc = w3 * RT(cvi[d]);
-        const RT pv = gk == BK_NONE ? __ldg(rec + (RC::PHI + d) * N + nb)
+        const RT pv = gk == BK_NONE ? record_load<kLive>(rec + (RC::PHI + d) * N + nb)
                       : (gk == BK_INLET ? phi_in[d] : (gk == BK_OUTLET ? phi_self[d] : RT(0)));
         dPhi[d] += wc * pv;
         corr[d] += wc * hy;
@@ -1499,7 +1507,7 @@ template <int D, int M, typename RT> struct RegPar {
 
 // Fused placement: one thread per node does the per-node part and then every
 // direction (Sec. 2.3, 3.2-3.4).
-template <int D, int M, typename S, typename RT>
+template <int D, int M, bool kLive, typename S, typename RT>
 __device__ __forceinline__ void collide_body(const S* __restrict__ src, S* __restrict__ dst,
                                              const RT* __restrict__ rec,
                                              const double* __restrict__ Tf,
@@ -1512,7 +1520,7 @@ __device__ __forceinline__ void collide_body(const S* __restrict__ src, S* __res
   const int tag = bc.tag ? bc.tag[n] : TAG_BULK;
   if (tag == TAG_SOLID) return;
   NodePar<D, M, RT> p;
-  node_params<D, M, RT>(rec, Tf, g, un, bc, mech, n, tag, p);
+  node_params<D, M, kLive, RT>(rec, Tf, g, un, bc, mech, n, tag, p);
   const int x = (int)(n % g.nx);
   const int y = (int)((n / g.nx) % g.ny);
   const int z = (int)(n / ((long long)g.nx * g.ny));
@@ -1567,7 +1575,7 @@ __device__ __forceinline__ void collide_body(const S* __restrict__ src, S* __res
 // per direction group, lanes over 32 consecutive nodes), stages the block's
 // parameters and axis-factor tables in shared memory, and updates each
 // direction as the fused kernel does.
-template <int D, int M, typename RT>
+template <int D, int M, bool kLive, typename RT>
 __device__ __forceinline__ void prep_body(const RT* __restrict__ rec,
                                           const double* __restrict__ Tf, RT* __restrict__ cp,
                                           const Geom& g, const Units& un, const BCDev& bc,
@@ -1578,7 +1586,7 @@ __device__ __forceinline__ void prep_body(const RT* __restrict__ rec,
   const int tag = bc.tag ? bc.tag[n] : TAG_BULK;
   if (tag == TAG_SOLID) return;
   NodePar<D, M, RT> p;
-  node_params<D, M, RT>(rec, Tf, g, un, bc, mech, n, tag, p);
+  node_params<D, M, kLive, RT>(rec, Tf, g, un, bc, mech, n, tag, p);
 #pragma unroll
   for (int b = 0; b < M; ++b) {
     cp[(CP::TH + b) * N + n] = p.th[b];
@@ -2094,7 +2102,7 @@ k_collide(const S* __restrict__ src, S* __restrict__ dst, const RT* __restrict__
           const double* __restrict__ Tf, int* __restrict__ status,
           const __grid_constant__ Geom g, const __grid_constant__ Units un,
           const __grid_constant__ BCDev bc, const __grid_constant__ DevMech mech) {
-  collide_body<D, M, S, RT>(src, dst, rec, Tf, status, g, un, bc, mech,
+  collide_body<D, M, false, S, RT>(src, dst, rec, Tf, status, g, un, bc, mech,
                             blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
 
@@ -2103,7 +2111,7 @@ __global__ void __launch_bounds__(128, kPrepMinBlocks<RT>)
 k_prep(const RT* __restrict__ rec, const double* __restrict__ Tf, RT* __restrict__ cp,
        const __grid_constant__ Geom g, const __grid_constant__ Units un,
        const __grid_constant__ BCDev bc, const __grid_constant__ DevMech mech) {
-  prep_body<D, M, RT>(rec, Tf, cp, g, un, bc, mech,
+  prep_body<D, M, false, RT>(rec, Tf, cp, g, un, bc, mech,
                       blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
 
@@ -2260,7 +2268,7 @@ k_collide_batch(const DomainDev* __restrict__ doms, int ndom, int parity, int nb
   for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
     const DomainDev& d = bd.get(doms, domain_of_block(doms, ndom, b, GRID_NODE));
     const int c = d.cur0 ^ parity;
-    collide_body<D, M, S, RT>(static_cast<const S*>(d.pops[c]),
+    collide_body<D, M, false, S, RT>(static_cast<const S*>(d.pops[c]),
                               static_cast<S*>(const_cast<void*>(d.pops[1 - c])),
                               static_cast<const RT*>(d.rec), d.Tf, d.status, d.g, d.un, d.bc,
                               *d.mech, (b - d.block_begin) * (long long)blockDim.x + threadIdx.x);
@@ -2273,7 +2281,7 @@ k_prep_batch(const DomainDev* __restrict__ doms, int ndom, int nblk) {
   LBM_BLOCK_DOMAIN(bd);
   for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
     const DomainDev& d = bd.get(doms, domain_of_block(doms, ndom, b, GRID_NODE));
-    prep_body<D, M, RT>(static_cast<const RT*>(d.rec), d.Tf, static_cast<RT*>(d.cpar), d.g,
+    prep_body<D, M, false, RT>(static_cast<const RT*>(d.rec), d.Tf, static_cast<RT*>(d.cpar), d.g,
                         d.un, d.bc, *d.mech,
                         (b - d.block_begin) * (long long)blockDim.x + threadIdx.x);
   }
@@ -2489,11 +2497,11 @@ k_step_persist(const DomainDev* __restrict__ doms, int ndom, int parity,
       }
     } else if (w.kind == PI_PREP) {
       for (int j = 0; j < npt; ++j)
-        prep_body<D, M, RT>(rec, d.Tf, static_cast<RT*>(d.cpar), d.g, d.un, d.bc, *d.mech,
+        prep_body<D, M, true, RT>(rec, d.Tf, static_cast<RT*>(d.cpar), d.g, d.un, d.bc, *d.mech,
                             w.first + (long long)j * kPersistThreads + threadIdx.x);
     } else if (w.kind == PI_COLLIDE) {
       for (int j = 0; j < npt; ++j)
-        collide_body<D, M, S, RT>(src, static_cast<S*>(const_cast<void*>(d.pops[1 - c])), rec,
+        collide_body<D, M, true, S, RT>(src, static_cast<S*>(const_cast<void*>(d.pops[1 - c])), rec,
                                   d.Tf, d.status, d.g, d.un, d.bc, *d.mech,
                                   w.first + (long long)j * kPersistThreads + threadIdx.x);
     } else {
