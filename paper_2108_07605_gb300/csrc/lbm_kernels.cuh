@@ -1704,8 +1704,9 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
   constexpr int CH = (Q + TPN - 1) / TPN;
   const int k0 = w * CH, k1 = min(k0 + CH, Q);
   // This lane's slots of the warp's buffer hold the populations of one
-  // direction; the next direction's are copied into them as they are used up,
-  // past the registers (the first direction's while the tables are built).
+  // direction; the next direction's are copied into them once all are read (a
+  // barrier of the warp between: nothing else orders a copy after its own
+  // thread's loads), the first direction's while the tables are built.
   double* const fin = sm + T::N * kCollNodes + w * (M + 1) * kCollNodes + lane;
   const long long stride = Q * (tag >= 0 ? (long long)bc.n_if : N);
   auto first_of = [&](int i) {
@@ -1770,6 +1771,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
     }
   }
   __syncthreads();
+  const unsigned lanes = __ballot_sync(0xffffffffu, valid);
   if (!valid) return;
   auto P = [&](int f) { return s[f * kCollNodes]; };
   auto PF = [&](int f) { return ff_unpack(s[f * kCollNodes]); };
@@ -1786,11 +1788,6 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
     // the next direction
     const bool more = k + 1 < k1;
     const double* pn = more ? first_of((k + 1) / NZ + 9 * ((k + 1) % NZ)) : src;
-    auto take = [&](int l) { return fin[l * kCollNodes]; };
-    auto next = [&](int l) {
-      if (more) copy_async8(fin + l * kCollNodes, pn);
-      pn += stride;
-    };
     if (j != jcur) {
       jcur = j;
 #pragma unroll
@@ -1824,6 +1821,14 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
       }
     }
     copy_async_wait();
+    double in[M + 1];
+#pragma unroll
+    for (int l = 0; l <= M; ++l) in[l] = fin[l * kCollNodes];
+    __syncwarp(lanes);
+    if (more) {
+#pragma unroll
+      for (int l = 0; l <= M; ++l, pn += stride) copy_async8(fin + l * kCollNodes, pn);
+    }
 #pragma unroll
     for (int a = 0; a < M - 1; ++a) {
       ff F;
@@ -1832,8 +1837,7 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
         if (b != a) ff_fma_acc(F, mech.K_f[a][b], dd[b]);
       F = PF(T::CF + a) * ff_norm(F);
       const double ez = D == 3 ? P(T::e(a, D - 1, cz)) : 1.0;
-      const double base = fma(take(a), P(T::OM1 + a), double_join(F, ce[a * kCollNodes]));
-      next(a);
+      const double base = fma(in[a], P(T::OM1 + a), double_join(F, ce[a * kCollNodes]));
       dst[(long long)(a * Q + i) * N + n] = D == 3 ? fma(eh[a], ez, base) : eh[a] + base;
     }
     double fex = fxy, geq = gQ;
@@ -1841,12 +1845,10 @@ __device__ __forceinline__ void coll_block64(const S* __restrict__ src, S* __res
       fex *= P(T::EX + 6 + cz + 1);
       geq = fma(P(T::AF + 6 + cz + 1), gQ, gP * P(T::BF + 6 + cz + 1));
     }
-    const double fm = take(M - 1);
+    const double fm = in[M - 1];
     dst[(long long)((M - 1) * Q + i) * N + n] = fma(om, fex - fm, fm);
-    next(M - 1);
-    const double gm = take(M);
+    const double gm = in[M];
     double gn = fma(om, fma(rho, geq, -gm), gm);
-    next(M);
     if (csq(i, D) == 1) {
 #pragma unroll
       for (int d = 0; d < D; ++d)
