@@ -249,26 +249,30 @@ def interface_nodes(w):
     return int(mark.sum())
 
 
-WARP_BOUNDARY_NODES = 6144    # up to here a warp per interface node, sub-steps included
+# up to here a warp per interface node, sub-steps included; beyond, the sub-steps
+# have a kernel of their own, from IFACE_CHEM_THREADS nodes on with a thread each
+WARP_BOUNDARY_NODES = {"fp64": 4096, "fp32": 6144, "fp16": 6144, "fp32c64": 2048}
+IFACE_CHEM_THREADS = 19456
 
 
-def step_kernels(launch, n_if):
+def step_kernels(launch, n_if, precision):
     """Kernels one step launches, in two groups (lbm_step_timed): the boundary
     kernel with, for many interface nodes, their sub-steps in a kernel of
     their own, and the moments with the reaction sub-steps; the collision."""
     bnd = [] if n_if == 0 else \
-        ["k_bnode_warp"] if n_if <= WARP_BOUNDARY_NODES else ["k_bnode", "k_iface_chem"]
+        ["k_bnode_warp"] if n_if <= WARP_BOUNDARY_NODES[precision] else \
+        ["k_bnode", "k_iface_chem" if n_if >= IFACE_CHEM_THREADS else "k_chem"]
     return (bnd + ["k_mchem" if launch["chem_lanes"] > 1 else "k_moments"],
             ["k_prep", "k_coll"] if launch["collide_split"] else ["k_collide"])
 
 
-def launch_groups(launch, n_if):
+def launch_groups(launch, n_if, precision):
     """Names of the two timed launch groups of a step."""
-    return ["+".join(g) for g in step_kernels(launch, n_if)]
+    return ["+".join(g) for g in step_kernels(launch, n_if, precision)]
 
 
-def launches_per_step(launch, n_if):
-    return sum(len(g) for g in step_kernels(launch, n_if))
+def launches_per_step(launch, n_if, precision):
+    return sum(len(g) for g in step_kernels(launch, n_if, precision))
 
 
 def step_counters(workload, mode):
@@ -557,7 +561,7 @@ def main():
     ms_per_step = total_ms / args.steps
     value = node_updates_per_s(Nf, args.steps, world, M, total_ms * 1e-3)
     roof = roofline(args.workload, args.precision, info, Nf, ms_per_step, peaks, fma)
-    names = launch_groups(launch, n_if)
+    names = launch_groups(launch, n_if, args.precision)
 
     # end to end through the C ABI with host buffers
     e2e = None
@@ -648,7 +652,7 @@ def main():
                    else "state larger than L2", "parallelism": f"replicas x{world}",
                    "launch": launch},
         "roofline": roof, "cpu_baseline": cpu, "e2e": e2e,
-        "gpu_launches": launches_per_step(launch, n_if) * args.steps,
+        "gpu_launches": launches_per_step(launch, n_if, args.precision) * args.steps,
         "kernel_ms_per_step": {names[0]: kms[0] / args.steps, names[1]: kms[1] / args.steps},
         "fma_peak_tflops": fma,
         "variants": variants,

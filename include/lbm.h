@@ -241,8 +241,8 @@ lbm_status lbm_step(lbm_t h, int nsteps);
 /* Advance several handles by nsteps steps together, in the placement a
  * batch plan of the same handles starts with (see lbm_batch_set_launch):
  * one launch per kernel over the concatenated tiles (128-node tiles; the
- * interface nodes with a warp each up to 6,144 of them in all, else with a
- * thread each), so many small domains fill the GPU.
+ * interface nodes of all handles together counted for lbm_launch's lines), so
+ * many small domains fill the GPU.
  * The handles must share lattice, species count, precision and device; each
  * keeps its own mechanism, units and boundaries.  The work runs on hs[0]'s
  * stream after the earlier work of every handle's stream, and every
@@ -271,8 +271,10 @@ lbm_status lbm_batch_destroy(lbm_batch_t b);
  *                  small to fill the GPU at one thread per node); -1 = by
  *                  grid size.  Interface nodes (boundary reconstruction, then
  *                  their sub-steps) take, in every placement, a warp each up
- *                  to 6,144 of them; beyond, a thread each, the sub-steps with
- *                  eight lanes each below 19,456 (the single launch of a plan:
+ *                  to 4,096 of them in FP64, 6,144 in FP32 and FP16 and 2,048
+ *                  in FP32 with FP64 chemistry; beyond, a thread each, the
+ *                  sub-steps with eight lanes each below 19,456 (the single
+ *                  launch of a plan: a warp each for an item of up to 32, else
  *                  one thread each).
  *   collide_split  0 = one thread per node does the whole collision; 1 = a
  *                  per-node kernel stores the collision parameters and a

@@ -749,7 +749,7 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
 
 // ---------------------------------------------------------------------------
 // The same procedure with one warp per interface node, for grids with few of
-// them (kBnodeWarpNodes): a thread per node is then a single chain of some
+// them (boundary_warp_nodes): a thread per node is then a single chain of some
 // thousand dependent loads and sums, whatever the node count (444 us in FP64,
 // 355 us in FP32 for the 32 interface nodes of the 1024x4x4 flame, the
 // critical path of its step; with a warp each, sub-steps included, 70 and 56).  Lane 3 l + p holds lattice l's directions of

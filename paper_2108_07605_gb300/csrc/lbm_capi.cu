@@ -103,7 +103,8 @@ void fill_domains(lbm_ctx* const* hs, int n, const Launch& lc, std::vector<Domai
   doms.assign(n, DomainDev());
   gr = BatchGrids();
   gr.n_if_total = total_if(hs, n);
-  gr.bnd_warp = gr.n_if_total <= kBnodeWarpNodes;
+  gr.bnd_warp = gr.n_if_total <=
+                boundary_warp_nodes(hs[0]->cfg.precision == LBM_FP64, hs[0]->cfg.chem_fp64 != 0);
   const int per_bnd = gr.bnd_warp ? kBnodeWarps : kBndNodesPerBlock;
   for (int k = 0; k < n; ++k) {
     lbm_ctx* h = hs[k];

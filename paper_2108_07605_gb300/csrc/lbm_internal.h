@@ -247,11 +247,17 @@ struct BatchGrids {
 
 // Grids (of a plan: handles together) with up to this many interface nodes take
 // the boundary kernel with a warp per node, which does more work in all but
-// not in one chain.  Steps of the 1024x4x4 flame (32 nodes): 0.29 ms against
-// 0.60 in FP64, 0.15 against 0.34 in FP32; of a mixed FP32 batch (2816 nodes)
-// 2.2 against 2.7; of the 2000x40 channel (4076 nodes) 0.69 against 0.75 in
-// FP64, 0.28 against 0.31 in FP32 with FP64 chemistry.
-constexpr int kBnodeWarpNodes = 6144;
+// not in one chain.  Steps in us, warp / thread, of 40-row channels (C) and
+// 40x40 tubes (T) by interface nodes:
+//   FP64            C 2036 294 / 320, C 4076 541 / 567, C 6076 783 / 681;
+//                   T 3136 415 / 436, T 4320 532 / 481
+//   FP32            C 4076 166 / 185, C 6076 236 / 267, C 8076 302 / 309, C 12076
+//                   482 / 426; T 4320 186 / 202, T 6688 256 / 227 (FP16 likewise)
+//   FP32, FP64 chemistry  C 1016 119 / 132, C 2036 154 / 144; T 3136 194 / 185; inlet
+//                   and outlet faces alone, 2048: 302 / 453
+constexpr int boundary_warp_nodes(bool fp64, bool chem64) {
+  return fp64 ? 4096 : (chem64 ? 2048 : 6144);
+}
 // nodes (warps) per block of it
 constexpr int kBnodeWarps = 2;
 // interface nodes per block of the boundary kernel (one thread each)

@@ -2902,7 +2902,7 @@ static cudaError_t step_impl(const DevMech& mech, const StepArgs& a, cudaStream_
     const bool fork = a.bc.n_if > 0 && a.side && a.ev_fork && a.ev_join;
     // the boundary kernel and the interface nodes' sub-steps
     auto boundary = [&](cudaStream_t st) {
-      if (a.bc.n_if <= kBnodeWarpNodes) {
+      if (a.bc.n_if <= boundary_warp_nodes(sizeof(S) == 8, LBM_CHEM64 != 0)) {
         k_bnode_warp<D, M, S><<<blocks_for(a.bc.n_if, kBnodeWarps), 32 * kBnodeWarps, 0, st>>>(
             src, a.bc, a.Tfield, a.status, a.g, a.un, a.mech_dev, rec);
         return;

@@ -206,3 +206,25 @@ def test_energies_of_unrounded_mass_fractions(precision, lanes, lattice, shape):
     err = max_rel_err_per_lattice(s.populations(), before)
     s.close()
     assert np.all(err < 16 * 2.0 ** -23), err
+
+
+# 2 nx + 12 interface nodes either side of the precisions' lines between a warp and
+# a thread per interface node
+@pytest.mark.parametrize("nx,precision", [(2042, "fp64"), (2043, "fp64"), (1018, "fp32c64"),
+                                          (1019, "fp32c64")])
+def test_boundary_kernels_either_side_of_their_line(mech, nx, precision):
+    w = fields.channel_2d(nx=nx, ny=8, dx=25e-6)
+    w["u"][:2] += 0.05 * fields.philox(3).uniform(-1.0, 1.0, size=w["u"][:2].shape)
+    o, g = make_oracle(mech, w), make_gpu(mech, w, precision=precision)
+    o.step(3)
+    g.step(3)
+    if precision == "fp64":
+        err = max_rel_err_per_lattice(g.populations(), oracle_populations(o))
+        g.close()
+        assert np.all(err < RTOL_FP64), err
+        return
+    mo, mg = o.moments(), g.moments()             # FP32 storage's field tolerances
+    g.close()
+    assert np.abs(mg["Y"] - mo["Y"].reshape(mech.n_species, -1)).max() <= 2e-5
+    assert np.abs(mg["T"] - mo["T"].ravel()).max() <= 0.05
+    assert (np.abs(mg["rho"] - mo["rho"].ravel()) / mo["rho"].ravel()).max() <= 1e-4
