@@ -56,17 +56,22 @@ lbm_status cuda_fail(lbm_ctx* h, cudaError_t e, const char* where) {
 }
 
 // Default placement, measured on one GB300.  The split collision is faster
-// than the fused one on every grid tried (FP64 and FP32).  In FP32 and FP16
-// storage a grid whose blocks with four lanes per node are all resident at once
-// hides the latency of the float-float chemistry that way: three 128-thread
-// blocks per SM without interface nodes (ms per step with 1 / 4 lanes, FP32:
-// 4096 nodes 0.084 / 0.068, 13824 0.093 / 0.081, 21952 0.103 / 0.125), one per SM
-// beside the boundary kernel (4096 nodes 0.096 / 0.080, 8192 0.097 / 0.124).  In
-// FP64 the lanes' redundant work costs what it hides (4096 nodes 0.16 / 0.14,
-// 5832 0.170 / 0.175; 2-D channel, 4000 nodes, 0.124 / 0.127).  Batch plans take
-// one launch per kernel (six reactors and flames of 69k nodes in all, FP64: 0.67
-// ms per step against 1.15 as a single launch over the work-list, whose
-// registers the kernels' largest stage sets).
+// than the fused one on every grid tried (FP64 and FP32).  Four lanes per node
+// (chem_lanes) hide the latency of a node's chain where their blocks (32 nodes)
+// are resident at once; us per step with 1 / 4 lanes:
+//   no interface nodes, FP32: 4096 nodes 86 / 68, 12167 92 / 80, 24389 110 / 135;
+//   FP32, FP64 chemistry: 12167 124 / 104, 24389 151 / 182: three blocks per SM;
+//   beside the boundary kernel: 4096 FP32 97 / 79, FP64 chemistry 130 / 92, 8192 FP64
+//   chemistry 131 / 192: one (FP32 alone would gain to 16384 nodes, 104 / 95; one
+//   line serves FP32 storage).
+// FP64 keeps a thread per node at every size, although four lanes are faster on
+// the smallest grids (4096 nodes 184 / 148; 8000 196 / 189, 12167 220 / 240; 4096
+// beside the boundary kernel 196 / 165, 8192 205 / 346): a lane group sums in
+// another order, and a line at some grid size would let a domain and its slabs
+// differ in the last bits.  chem_lanes or the autotuner select them.
+// Batch plans take one launch per kernel (six reactors and flames of 69k nodes in
+// all, FP64: 0.67 ms per step against 1.15 as a single launch over the work-list,
+// whose registers the kernels' largest stage sets).
 constexpr long long kLaneNodes = 152LL * 128 / 4;   // four lanes each: one block per SM
 Launch resolve_launch(const lbm_launch& opt, long long nodes, long long n_if,
                       lbm_precision prec) {
