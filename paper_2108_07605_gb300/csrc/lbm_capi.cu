@@ -1147,35 +1147,15 @@ lbm_status lbm_batch_step(lbm_t* hs, int n, int nsteps) {
   if (!ddev) e = cudaErrorMemoryAllocation;
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ddev, doms.data(), n * sizeof(DomainDev), cudaMemcpyHostToDevice, s0);
-  std::vector<PItem> items;
-  PItem* items_dev = nullptr;
-  int* sync_dev = nullptr;
-  if (e == cudaSuccess && lc.persistent == 2) {
-    int nsync = 0;
-    build_worklist(hs, n, lc.npt, lc.coll_split != 0, items, nsync);
-    items_dev = static_cast<PItem*>(dalloc(h0->cfg, items.size() * sizeof(PItem)));
-    sync_dev = static_cast<int*>(dalloc(h0->cfg, (size_t)nsync * sizeof(int)));
-    if (!items_dev || !sync_dev) e = cudaErrorMemoryAllocation;
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(items_dev, items.data(), items.size() * sizeof(PItem),
-                          cudaMemcpyHostToDevice, s0);
-    gr.items = items_dev;
-    gr.nitems = (int)items.size();
-    gr.sync = sync_dev;
-    gr.nsync = nsync;
-  }
   for (int step = 0; step < nsteps && e == cudaSuccess; ++step)
     e = launch_batch_step(h0->D, h0->M, kernel_precision(h0->cfg), ddev, n, gr, lc, step & 1, s0);
   if (e == cudaSuccess) e = cudaEventRecord(ev, s0);
   for (int k = 1; k < n && e == cudaSuccess; ++k)
     if (hs[k]->stream != s0) e = cudaStreamWaitEvent(hs[k]->stream, ev, 0);
-  if (ddev || items_dev || sync_dev) {
-    // plain cudaFree is not stream-ordered; the host copy of the items must
-    // outlive its asynchronous upload
-    if (!h0->cfg.dev_free || items_dev) cudaStreamSynchronize(s0);
+  if (ddev) {
+    // plain cudaFree is not stream-ordered
+    if (!h0->cfg.dev_free) cudaStreamSynchronize(s0);
     dfree(h0->cfg, ddev);
-    dfree(h0->cfg, items_dev);
-    dfree(h0->cfg, sync_dev);
   }
   if (ev) cudaEventDestroy(ev);
   if (e != cudaSuccess) return cuda_fail(h0, e, "batched step");
