@@ -39,6 +39,8 @@ struct lbm_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   void* cpar = nullptr;     // per-node collision parameters (split collision)
   float4* codec = nullptr;  // FP16 storage: per-population offset and scale
+  DomainDev* batch_dom = nullptr;  // descriptors of lbm_batch_step calls led by this handle
+  int batch_cap = 0;
   std::string err;
 };
 
@@ -1143,7 +1145,15 @@ lbm_status lbm_batch_step(lbm_t* hs, int n, int nsteps) {
       e = cudaEventRecord(ev, hs[k]->stream);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s0, ev, 0);
     }
-  DomainDev* ddev = static_cast<DomainDev*>(dalloc(h0->cfg, n * sizeof(DomainDev)));
+  // the descriptors stay with the first handle: freed here they would need a wait
+  // for the work, or a dev_free that follows the stream
+  if (h0->batch_cap < n) {
+    if (h0->batch_dom) cudaStreamSynchronize(s0);
+    dfree(h0->cfg, h0->batch_dom);
+    h0->batch_dom = static_cast<DomainDev*>(dalloc(h0->cfg, n * sizeof(DomainDev)));
+    h0->batch_cap = h0->batch_dom ? n : 0;
+  }
+  DomainDev* const ddev = h0->batch_dom;
   if (!ddev) e = cudaErrorMemoryAllocation;
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ddev, doms.data(), n * sizeof(DomainDev), cudaMemcpyHostToDevice, s0);
@@ -1152,11 +1162,6 @@ lbm_status lbm_batch_step(lbm_t* hs, int n, int nsteps) {
   if (e == cudaSuccess) e = cudaEventRecord(ev, s0);
   for (int k = 1; k < n && e == cudaSuccess; ++k)
     if (hs[k]->stream != s0) e = cudaStreamWaitEvent(hs[k]->stream, ev, 0);
-  if (ddev) {
-    // plain cudaFree is not stream-ordered
-    if (!h0->cfg.dev_free) cudaStreamSynchronize(s0);
-    dfree(h0->cfg, ddev);
-  }
   if (ev) cudaEventDestroy(ev);
   if (e != cudaSuccess) return cuda_fail(h0, e, "batched step");
   for (int k = 0; k < n; ++k) {
@@ -1724,6 +1729,7 @@ lbm_status lbm_destroy(lbm_t h) {
   dfree(h->cfg, h->io);
   dfree(h->cfg, h->bc_mem);
   dfree(h->cfg, h->mech_dev);
+  dfree(h->cfg, h->batch_dom);
   if (h->ev_fork) cudaEventDestroy(h->ev_fork);
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   if (h->side) cudaStreamDestroy(h->side);
