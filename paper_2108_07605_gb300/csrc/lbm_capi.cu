@@ -530,7 +530,8 @@ Sizes sizes_for(const lbm_config& c, const HostBC& hb) {
   if (hb.needed) {
     const size_t nif = (size_t)hb.n_if;
     s.bc = align256(N * sizeof(int)) + 3 * align256(nif * sizeof(int)) +
-           4 * align256(nif * sizeof(double)) + align256((size_t)(M + 1) * Q * nif * sizeof(double));
+           4 * align256(nif * sizeof(double)) +
+           align256((size_t)(M + 1) * Q * nif * compute_size(c.precision));
     if (hb.offgrid) s.bc += align256(nif * sizeof(int)) + 2 * align256(nif * sizeof(double));
   }
   s.total = 2 * s.pops + s.rec + s.cpar + s.codec + s.tf + s.status + s.bc;
@@ -862,7 +863,7 @@ lbm_status lbm_create(const lbm_config* cfg, lbm_t* out) {
     unsigned* if_inc = reinterpret_cast<unsigned*>(take(nif * sizeof(unsigned)));
     double* wallT = reinterpret_cast<double*>(take(nif * sizeof(double)));
     double* uin = reinterpret_cast<double*>(take(3 * nif * sizeof(double)));
-    b.pops = static_cast<void*>(take((size_t)h->L * h->Q * nif * sizeof(double)));
+    b.pops = take((size_t)h->L * h->Q * nif * compute_size(cfg->precision));
     cudaError_t e = cudaMemcpy(tag, hb.tag.data(), N * sizeof(int), cudaMemcpyHostToDevice);
     if (hb.offgrid) {
       int* nbr = reinterpret_cast<int*>(take(nif * sizeof(int)));
