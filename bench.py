@@ -70,13 +70,13 @@ WORKLOADS = {"reactor": "homogeneous reactor 16^3 periodic D3Q27, M=9, 21 reacti
              "box": "perturbed periodic box 128x64x64 D3Q27, M=9, 21 reactions, "
                     "1400 K +-2%, |u| <= 1 m/s (profiling case larger than L2)"}
 
-# storage / arithmetic modes: (library precision, chemistry in native FP64, dtype text)
+# storage / arithmetic modes: (library precision, chem_fp64, dtype text)
 MODES = {
     "fp64": ("fp64", 0, "f64"),
     "fp32": ("fp32", 0, "f32 storage and lattice arithmetic; temperature Newton and "
                         "chemistry in float-float (two FP32 words, ~48-bit significand)"),
     "fp32c64": ("fp32", 1, "f32 storage and lattice arithmetic; temperature Newton and "
-                           "chemistry in native FP64"),
+                           "chemistry as in the FP64 path"),
     "fp16": ("fp16", 0, "f16 offset storage, f32 lattice arithmetic; temperature Newton "
                         "and chemistry in float-float"),
 }

@@ -64,10 +64,14 @@ typedef enum {
 typedef enum { LBM_D2Q9 = 0, LBM_D3Q27 = 1 } lbm_lattice;
 
 /* Storage precision of the populations.  LBM_FP64: results to
- * FP64 rounding (the path checked against the oracle to 1e-10); what is summed
- * exactly or enters as a small correction runs in fixed point or in pairs of
- * FP32 (~48 significant bits) beside the FP64 pipe, with no larger error than
- * in FP64 throughout.  LBM_FP32_STORE:
+ * FP64 rounding in FP64's range (checked against the oracle to 1e-10 of each
+ * lattice: fresh mixtures from 300 K, mass fractions down to 1e-60, 1/tau_a
+ * from 3 to 3e6 and, with diffusivities of 1e-33 m^2/s, beyond 1e28).  Beside FP64
+ * instructions it uses 64-bit integers (population sums; rate constants and
+ * their products with concentrations) and, for what enters as a correction, pairs
+ * of FP32, ~48 significant bits of the correction within FP32's exponents: the
+ * derivative in the temperature solve, the energy that a reaction sub-step
+ * moves, diffusion velocities and the Stefan-Maxwell term.  LBM_FP32_STORE:
  * populations, moments and collision in FP32; the temperature Newton solve
  * and the chemistry in float-float (pairs of FP32, ~48 significant bits);
  * transport in FP32.  LBM_FP16_OFFSET: the FP32 path's arithmetic, with

@@ -308,7 +308,7 @@ struct KernelSet {
 };
 // nullptr for an unsupported combination.  Besides the lbm_precision values,
 // prec may be LBM_KPREC_FP32_CHEM64: FP32 storage and lattice arithmetic with
-// the temperature solve and the chemistry in native FP64 (cfg->chem_fp64).
+// the temperature solve and the chemistry as in the FP64 path (cfg->chem_fp64).
 constexpr int LBM_KPREC_FP32_CHEM64 = 16;
 const KernelSet* kernel_set(int D, int M, lbm_precision prec);
 // the kernel-set precision of a configuration

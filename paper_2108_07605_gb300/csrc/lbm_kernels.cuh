@@ -42,7 +42,7 @@
 
 // Chemistry mode of the mixed path in this translation unit: with FP32
 // lattice arithmetic, the temperature Newton solve and the reaction
-// chemistry run in float-float (LBM_CHEM64 = 0) or in native FP64
+// chemistry run in float-float (LBM_CHEM64 = 0) or as in the FP64 path
 // (LBM_CHEM64 = 1).  The two modes' templates live in distinct inline
 // namespaces, so both can be instantiated in one library.
 #ifndef LBM_CHEM64
@@ -231,10 +231,10 @@ __device__ __forceinline__ void node_substeps(const RT (&rs)[M], RT rho, RT ER, 
 // Reaction sub-steps with several lanes per node (Sec. 2.4 Eq. R3), for
 // grids too small to fill the GPU at one thread per node: the node's
 // reactions are dealt out over the lanes, which cuts the latency of a node's
-// chemistry by about the lane count.  The formulas are those of
-// production_rates / production_rates_ff; only the production rates are
-// summed in another order (partial sums per lane), so the placements agree
-// to rounding.  CT: double (FP64 path) or float-float (mixed path).
+// chemistry by about the lane count.  The formulas are those of node_substeps;
+// only the production rates are summed in another order (partial sums per
+// lane), so the placements agree to rounding.  CT: double (FP64 path) or
+// float-float (mixed path).
 __device__ __forceinline__ double shfl_xor_ct(unsigned mask, double v, int o) {
   return __shfl_xor_sync(mask, v, o);
 }
@@ -366,8 +366,8 @@ __device__ __forceinline__ void chem_group_substeps(CT (&r)[M], const CT irho, c
 }
 
 // Reaction sub-steps of node n by a group of L lanes (L = 4 or 8, aligned
-// within the warp): every lane forms the node's state, temperature,
-// concentrations and Gibbs functions; lane `sub` takes the reactions
+// within the warp): every lane forms the node's state, temperature and
+// concentrations; lane `sub` takes the reactions
 // k = sub, sub + L, ...; the species production rates are summed across the
 // group with shuffles, after which every lane holds the same densities.
 template <int D, int M, typename RT, int L>
@@ -417,7 +417,7 @@ __device__ __forceinline__ void chem_lanes_body(RT* __restrict__ rec,
 // small to fill the GPU at one thread per node; chem_lanes = L).  Lane `sub`
 // pulls the directions sub, sub + L, ... of every lattice, the group adds the
 // partial sums with a butterfly, every lane forms the node's fields (the
-// formulas of moments_finish), the temperature solve is shared as in
+// formulas of moments_body), the temperature solve is shared as in
 // group_newton, the lanes split the record's stores, and the group runs the
 // sub-steps from the post-stream densities (chem_group_substeps).  m: the
 // mechanism for compile-time indices; mg: its global copy, indexed by lane.
@@ -1000,7 +1000,7 @@ __device__ __forceinline__ double exp_of(double x) { return exp_tang(x); }
 // (Sec. 2.3 Eqs. betaa, taua, transform1; Sec. 3.3 Eq. Pex; Sec. 3.4 Eqs.
 // gstar, qdiff, corrFourier; Sec. 2.4 Eq. R3).
 // The diffusion velocities and what only they need: float-float in the FP64
-// path (solve_dd_strided), FP32 in the mixed path.
+// path (solve_dd_ff), FP32 in the mixed path (solve_dd_strided).
 template <typename RT> struct DiffType { using type = RT; };
 template <> struct DiffType<double> { using type = ff; };
 template <int D, int M, typename RT> struct NodePar {
@@ -1569,12 +1569,11 @@ __device__ __forceinline__ void collide_body(const S* __restrict__ src, S* __res
 }
 
 // ---------------------------------------------------------------------------
-// Split placement of the collision, for grids too small to fill the GPU at
-// one thread per node: k_prep (one thread per node) stores each node's
-// parameters field-major; k_coll gives every node kCollTPN threads (one warp
-// per direction group, lanes over 32 consecutive nodes), stages the block's
-// parameters and axis-factor tables in shared memory, and updates each
-// direction as the fused kernel does.
+// Split placement of the collision (the default): k_prep (one thread per node)
+// stores each node's parameters field-major; k_coll gives every node kCollTPN
+// threads (one warp per direction group, lanes over 32 consecutive nodes),
+// stages the block's parameters and axis-factor tables in shared memory, and
+// updates each direction as the fused kernel does.
 template <int D, int M, bool kLive, typename RT>
 __device__ __forceinline__ void prep_body(const RT* __restrict__ rec,
                                           const double* __restrict__ Tf, RT* __restrict__ cp,
@@ -2117,8 +2116,9 @@ k_prep(const RT* __restrict__ rec, const double* __restrict__ Tf, RT* __restrict
                       blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
 
-// FP32: four 288-thread blocks per SM (at most 56 registers), so a grid of
-// the 16k-node flame fits the GPU in one wave
+// 288-thread blocks: FP64 two per SM (96 registers, 97 KB of shared memory each),
+// FP32 three (72 registers; two or four: 46.4 and 45.7 ms per 24 steps of the
+// 600x40x40 tube against 45.4)
 template <int D, int M, typename S, typename RT>
 __global__ void __launch_bounds__(32 * kCollTPN, sizeof(RT) == 4 ? kColl32Blocks : 2)
 k_coll(const S* __restrict__ src, S* __restrict__ dst, const RT* __restrict__ cp,
@@ -2391,8 +2391,10 @@ __device__ __forceinline__ void iface_substeps(RT* __restrict__ rec, const doubl
 // The interface nodes' sub-steps with one thread per node (grids with at
 // least kIfChemThreadNodes interface nodes, which fill the GPU this way):
 // the same arithmetic as the lane groups of k_chem without their redundant
-// per-lane temperature and Gibbs evaluations.  Float-float rate arrays in
-// dynamic shared memory.
+// per-lane temperature solves.  Rate arrays in dynamic shared memory.  Measured
+// with the tube's steps, eight lanes / a thread per node, us: FP64 20896 interface
+// nodes 1596 / 1598, 31552 2217 / 2177, 90752 6004 / 5828; FP32 20896 529 / 553,
+// 31552 739 / 742, 90752 1850 / 1767; FP32 with FP64 chemistry 20896 682 / 676.
 constexpr long long kIfChemThreadNodes = 152LL * 128;
 
 template <int D, int M, typename RT>
@@ -2631,8 +2633,6 @@ k_init(const double* __restrict__ rho_or_P, int is_pressure, const double* __res
 
 // Sums of node n's stored populations in FP64 (fixed point): rho, j, rho E, and
 // species(a, rho_a) for every species, the slaved one last.
-template <typename S> struct StoredType { using type = float; };
-template <> struct StoredType<double> { using type = double; };
 
 // Q populations of a lattice from pl, N apart, times 2^shift, and their largest
 // biased exponent.  FP32: from the largest bit pattern, so that all loads are in

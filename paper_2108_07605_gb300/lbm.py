@@ -566,7 +566,7 @@ def make_config(mech, lattice="D3Q27", shape=(16, 16, 16), dx=1e-3, precision="f
     solid: optional grid array of solid nodes; inlet: dict(u, T, Y, P) with u
     a 3-vector or a [3, nz, ny, nx] array (m/s); outlet: dict(P, sigma);
     chem_fp64: with precision "fp32", the temperature solve and chemistry in
-    native FP64 instead of float-float; wall_dist [nz, ny, nx] and
+    LBM_FP64's way instead of float-float; wall_dist [nz, ny, nx] and
     wall_normal [3, nz, ny, nx] (together): off-grid TMS targets."""
     cfg = lbm_config_defaults()
     cfg.lattice = LBM_D3Q27 if lattice == "D3Q27" else LBM_D2Q9
