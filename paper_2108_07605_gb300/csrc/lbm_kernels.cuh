@@ -764,21 +764,30 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   RT rho = RT(0), inv_rho = RT(0), u[D], usq = RT(0), ER = RT(0), Z[D];
   RT Rm = RT(0);                                   // sum Y_a / m_a
   CT cU[4] = {CT(), CT(), CT(), CT()};             // energy polynomial
+  // FP32: sum_a (rho_a - rho Y_a) u_k, Y_a as rounded: the sub-steps' energies
+  // are those of rho_a / rho in the chemistry's precision
+  float eU[4] = {0.f, 0.f, 0.f, 0.f};
   Remainder<D, RT> rest;
 #pragma unroll
   for (int d = 0; d < D; ++d) u[d] = Z[d] = RT(0);
 
   // species a's state from its sums: record, concentration, energy polynomial
-  // (FP32: rho times it, Y rounded to FP32 would cost the sub-steps' energies bits)
   auto species = [&](int a, RT rs, const RT (&js)[D]) {
     const RT Y = rs * inv_rho;
     rec[(RC::Y + a) * N + n] = Y;
+    if constexpr (sizeof(RT) == 4) {
+      const float e = __fmaf_rn(-Y, rho, rs);
+      eU[0] = __fmaf_rn(e, mech.u0_f[a].hi, eU[0]);
+      eU[1] = __fmaf_rn(e, mech.u1_f[a].hi, eU[1]);
+      eU[2] = __fmaf_rn(e, mech.u2_f[a].hi, eU[2]);
+      eU[3] = __fmaf_rn(e, mech.u3_f[a].hi, eU[3]);
+    }
     if constexpr (kFF<RT>) {
       Rm += Y * mech.inv_mm_s[a];
-      ff_fma_acc(cU[0], ff(rs), mech.u0_f[a]);
-      ff_fma_acc(cU[1], ff(rs), mech.u1_f[a]);
-      ff_fma_acc(cU[2], ff(rs), mech.u2_f[a]);
-      ff_fma_acc(cU[3], ff(rs), mech.u3_f[a]);
+      ff_fma_acc(cU[0], ff(Y), mech.u0_f[a]);
+      ff_fma_acc(cU[1], ff(Y), mech.u1_f[a]);
+      ff_fma_acc(cU[2], ff(Y), mech.u2_f[a]);
+      ff_fma_acc(cU[3], ff(Y), mech.u3_f[a]);
       cs.set(a, ff(rs) * mech.inv_mm_f[a]);
       Wd[a * kChemThreads] = ff_pack(ff());
     } else {
@@ -788,7 +797,8 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
         rd = rs;
         Rm = fma(Y, mech.inv_mm[a], Rm);
       } else {
-        rd = Yd = double_of_float_exact(rs);
+        Yd = double_of_float_exact(Y);
+        rd = double_of_float_exact(rs);
         Rm += Y * mech.inv_mm_s[a];
       }
       cU[0] = fma(Yd, mech.u0[a], cU[0]);
@@ -867,17 +877,11 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   if constexpr (kFF<RT>) {
     irho = ff_rcp(ff(rho));
 #pragma unroll
-    for (int k = 0; k < 4; ++k) cU[k] = ff_norm(cU[k]) * irho;
+    for (int k = 0; k < 4; ++k) cU[k] = ff_norm(cU[k]);
     U = (ff(ER) + ff(-0.5f * usq)) * un.c2_f;
   } else {
-    if constexpr (sizeof(RT) == 8) {
-      irho = ff_of_double(inv_rho);
-    } else {
-      const double ir = 1.0 / double(rho);
-      irho = ff_of_double(ir);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) cU[k] *= ir;
-    }
+    if constexpr (sizeof(RT) == 8) irho = ff_of_double(inv_rho);
+    else irho = ff_rcp(ff(rho));
     U = (double(ER) - 0.5 * double(usq)) * un.c * un.c;
   }
   bool ok;
@@ -910,7 +914,10 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3): a zero-dimensional
   // reactor per node from its post-stream species densities; T_0 is the T just
   // solved
-  ff dU[4];                              // increments of rho cU
+  // increments of rho cU; FP32: from what its rounding took off Y
+  ff dU[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) dU[k] = ff(eU[k]);
 #pragma unroll 1
   for (int s = 0; s < un.substeps; ++s) {
     if (s > 0) {

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from lbm_workloads import fields
-from lbm_workloads.mechanism import R_UNIVERSAL, binary_inert, h2_air_synthetic
+from lbm_workloads.mechanism import R_UNIVERSAL, h2_air_synthetic
 from oracle.diagnostics import diagnostics
 from paper_2108_07605_gb300 import lbm
 
@@ -184,28 +184,37 @@ def test_fp32_storage_holds_denormal_populations(mech):
 
 
 @pytest.mark.parametrize("lattice,shape", [("D3Q27", (5, 4, 3)), ("D2Q9", (7, 5, 1))])
-@pytest.mark.parametrize("lanes", [1, 4])
 @pytest.mark.parametrize("precision", ["fp32", "fp32c64"])
-def test_energies_of_unrounded_mass_fractions(precision, lanes, lattice, shape):
-    """A uniform state at rest is a fixed point.  rho = 13, Y = (10/13, 3/13)
-    and theta = 1/4 make its populations and their sums exact in FP32, the mass
-    fractions not; formation enthalpies that cancel in the mixture turn FP32
-    rounding of Y into 0.02 K (6e-5).  One step (its own rounding of the species
-    populations is as large in the next); what FP32 rounds of the rest (energy,
-    theta, relaxation) stays below 16 of its spacings."""
-    m = binary_inert(h_formation=(1e7, -1e7 / 0.3))
+def test_substep_energies_of_unrounded_mass_fractions(mech, precision, lattice, shape):
+    """A uniform state at rest: rho = 13, Y = (10/13, 3/13) and theta = 1/4 make
+    its populations and their sums exact in FP32, the mass fractions not, and
+    formation enthalpies that cancel in the mixture turn FP32 rounding of Y into
+    0.02 K (6e-5), Ea / (R T) = 100 times that in a rate.  The first of eight
+    sub-steps takes that temperature, the others that of rho_a / rho: a trace
+    product, constant rate k C_a, is off by 6e-3 / 8, and what FP32 rounds of the
+    energy (1e-7) times 100."""
+    M, a, c, b = mech.n_species, 0, 1, mech.n_species - 1
+    h, nu_f, nu_r = np.zeros(M), np.zeros((1, M)), np.zeros((1, M))
+    h[a], h[b] = 1e7, -1e7 / 0.3
+    nu_f[0, a] = nu_r[0, c] = 1
     T, N = 300.0, int(np.prod(shape))
-    c_ref = float(np.sqrt(4.0 * R_UNIVERSAL / m.molar_mass[0] * T))
+    m = dataclasses.replace(
+        mech, molar_mass=np.full(M, 28e-3), cp_coeffs=np.tile([3.5, 0.0, 0.0], (M, 1)),
+        h_formation=h, s_standard=np.full(M, 150.0), nu_f=nu_f, nu_r=nu_r,
+        arrhenius=np.array([[1e-3 * np.exp(100.0), 0.0, 100.0 * R_UNIVERSAL * T]]),
+        third_body=np.zeros(1, dtype=np.int32), efficiency=np.ones((1, M)),
+        reversible=np.zeros(1, dtype=np.int32), D0=np.full((M, M), 2e-5))
+    c_ref = float(np.sqrt(4.0 * R_UNIVERSAL / 28e-3 * T))
+    Y = np.zeros((M, N))
+    Y[a], Y[b] = 10.0 / 13.0, 3.0 / 13.0
     s = lbm.Solver(m, lattice=lattice, shape=shape, dx=1e-6, precision="fp32",
-                   chem_fp64=int(precision == "fp32c64"), substeps=2, c_ref=c_ref)
-    s.set_launch(chem_lanes=lanes)
-    Y = np.repeat([[10.0 / 13.0], [3.0 / 13.0]], N, axis=1)
+                   chem_fp64=int(precision == "fp32c64"), substeps=8, c_ref=c_ref)
+    s.set_launch(chem_lanes=1)
     s.init_fields(np.full(N, 13.0), np.zeros((3, N)), np.full(N, T), Y)
-    before = s.populations()
     s.step(1)
-    err = max_rel_err_per_lattice(s.populations(), before)
+    made = s.populations()[c].sum(axis=0)
     s.close()
-    assert np.all(err < 16 * 2.0 ** -23), err
+    assert np.abs(made / (1e-3 * 10.0 * 1e-6 / c_ref) - 1.0).max() < 1.5 * 6.4e-3 / 8
 
 
 # 2 nx + 12 interface nodes either side of the precisions' lines between a warp and
