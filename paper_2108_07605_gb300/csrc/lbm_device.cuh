@@ -411,14 +411,15 @@ template <int M, int ST> struct ChemSlice<M, double, ST> {
 template <int M, int ST>
 __device__ __forceinline__ double reaction_rate(const DevReaction& x, const TBasis<double>& b,
                                                 const ChemSlice<M, double, ST>& s) {
-  Sig q = forward_constant(x, b);
-  for (int j = 0; j < x.nr; ++j) q = q * s.sig(x.reac[j]);
-  if (x.reversible) {
-    Sig rev = reverse_constant(x, b);
-    for (int j = 0; j < x.np; ++j) rev = rev * s.sig(x.prod[j]);
-    q = q - rev;
+  // both constants together: two chains in flight (an irreversible reaction's
+  // reverse one goes unused)
+  Sig q = forward_constant(x, b), rev = reverse_constant(x, b);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if (j < x.nr) q = q * s.sig(x.reac[j]);
+    if (j < x.np) rev = rev * s.sig(x.prod[j]);
   }
-  return double_of_sig(q);
+  return double_of_sig(x.reversible ? q - rev : q);
 }
 // Float-float: of a rate constant 2^e1 y, what FP32 holds of 2^e1 goes before the
 // concentrations and the rest after them.
