@@ -764,9 +764,6 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   RT rho = RT(0), inv_rho = RT(0), u[D], usq = RT(0), ER = RT(0), Z[D];
   RT Rm = RT(0);                                   // sum Y_a / m_a
   CT cU[4] = {CT(), CT(), CT(), CT()};             // energy polynomial
-  // FP32: sum_a (rho_a - rho Y_a) u_k, Y_a as rounded: the sub-steps' energies
-  // are those of rho_a / rho in the chemistry's precision
-  float eU[4] = {0.f, 0.f, 0.f, 0.f};
   Remainder<D, RT> rest;
 #pragma unroll
   for (int d = 0; d < D; ++d) u[d] = Z[d] = RT(0);
@@ -775,13 +772,6 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   auto species = [&](int a, RT rs, const RT (&js)[D]) {
     const RT Y = rs * inv_rho;
     rec[(RC::Y + a) * N + n] = Y;
-    if constexpr (sizeof(RT) == 4) {
-      const float e = __fmaf_rn(-Y, rho, rs);
-      eU[0] = __fmaf_rn(e, mech.u0_f[a].hi, eU[0]);
-      eU[1] = __fmaf_rn(e, mech.u1_f[a].hi, eU[1]);
-      eU[2] = __fmaf_rn(e, mech.u2_f[a].hi, eU[2]);
-      eU[3] = __fmaf_rn(e, mech.u3_f[a].hi, eU[3]);
-    }
     if constexpr (kFF<RT>) {
       Rm += Y * mech.inv_mm_s[a];
       ff_fma_acc(cU[0], ff(Y), mech.u0_f[a]);
@@ -914,10 +904,7 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
   // reaction sub-steps at frozen U (Sec. 2.4 Eq. R3): a zero-dimensional
   // reactor per node from its post-stream species densities; T_0 is the T just
   // solved
-  // increments of rho cU; FP32: from what its rounding took off Y
-  ff dU[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) dU[k] = ff(eU[k]);
+  ff dU[4];                              // increments of rho cU
 #pragma unroll 1
   for (int s = 0; s < un.substeps; ++s) {
     if (s > 0) {
@@ -938,6 +925,18 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
 #pragma unroll 1
     for (int a = 0; a < M; ++a) {
       const CT w = cs.rate(a);
+      // FP32: with what its rounding took off rho Y_a, so that the sub-steps'
+      // energies are those of rho_a / rho in the chemistry's precision
+      float e = 0.f;
+      if constexpr (sizeof(RT) == 4) {
+        if (s == 0 && !last) {
+          ff c;
+          if constexpr (kFF<RT>) c = cs.c(a);
+          else c = ff_of_double(cs.c(a));
+          const float rs = (c * mech.mm_f[a]).hi;       // rho_a again
+          e = __fmaf_rn(-(rs * inv_rho), rho, rs);
+        }
+      }
       ff inc;
       if constexpr (kFF<RT>) {
         Wd[a * kChemThreads] = ff_pack(ff_unpack(Wd[a * kChemThreads]) + w);
@@ -950,6 +949,7 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ src, RT* __re
         cs.set(a, fma(w, un.dt_sub, cs.c(a)));
         inc = ff_of_double(w) * un.dtmm_f[a];
       }
+      if constexpr (sizeof(RT) == 4) ff_acc(inc, ff(e));
       ff_fma_acc(dU[0], inc, mech.u0_f[a]);
       ff_fma_acc(dU[1], inc, mech.u1_f[a]);
       ff_fma_acc(dU[2], inc, mech.u2_f[a]);
@@ -2662,11 +2662,15 @@ __device__ __forceinline__ int load_lattice(const S* __restrict__ pl, long long 
       f[i] = Codec<S>::template dec<float>(__ldg(pl), codec, li + i);
 #pragma unroll
     for (int i = 0; i < Q; ++i) e = max(e, __float_as_int(f[i]) & 0x7fffffff);
-    if (e < (67 << 23)) shift = 64;                // all below 2^-60
-    const float sc = shift ? 0x1p64f : 1.f;
-    e = fix_exponent(double_of_float(sc * __int_as_float(e)));
+    if (e < (67 << 23)) {                          // all below 2^-60
+      shift = 64;
+      e = __float_as_int(0x1p64f * __int_as_float(e));
 #pragma unroll
-    for (int i = 0; i < Q; ++i) v[i] = double_of_float(sc * f[i]);
+      for (int i = 0; i < Q; ++i) f[i] *= 0x1p64f;
+    }
+    e = fix_exponent(double_of_float(__int_as_float(e)));
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = double_of_float(f[i]);
   }
   return e;
 }
