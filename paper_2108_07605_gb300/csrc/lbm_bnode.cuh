@@ -26,9 +26,10 @@
 // thread's shared-memory column, stride kBnd.
 
 constexpr int kBnd = kBndNodesPerBlock;   // threads per block of the boundary kernel
-// Blocks per SM its registers are held to.  Bound by latency, not by a pipe
-// (FP64: pipe 45 % busy; FP32: 3.8 warps per SM quarter in all): what counts is
-// loads in flight, by the directions unrolled three rows deep, and warps.
+// Blocks per SM its registers are held to.  FP64 is bound by its FP64 instructions
+// (pipe 72 % of the active cycles) and the tail of its one wave and a half, FP32 by
+// instruction fetch and latency (19 % of the issue slots): what counts is loads in
+// flight, by the directions unrolled three rows deep, and warps.
 // 600x40x40 tube, 91k interface nodes: FP64 1.22 -> 1.11 ms (255 registers);
 // FP32 0.44 -> 0.32 ms at 168 registers and six blocks, 0.41 at eight (128
 // registers, spills) and at four (240); FP16 0.52 -> 0.37.
@@ -752,7 +753,8 @@ __device__ __forceinline__ void bnode_body(const S* __restrict__ src, const BCDe
 // them (boundary_warp_nodes): a thread per node is then a single chain of some
 // thousand dependent loads and sums, whatever the node count (444 us in FP64,
 // 355 us in FP32 for the 32 interface nodes of the 1024x4x4 flame, the
-// critical path of its step; with a warp each, sub-steps included, 70 and 56).  Lane 3 l + p holds lattice l's directions of
+// critical path of its step; with a warp each, sub-steps included, 75 and 59).
+// Lane 3 l + p holds lattice l's directions of
 // c_z = p - 1 (D3Q27: 9 populations; D2Q9: 3, of c_y = p - 1); its loads are
 // in flight together, its sums go through shared memory to every lane, and
 // the sums over the species are butterflies over 16 lanes (lane & 15 = the

@@ -71,8 +71,8 @@ lbm_status cuda_fail(lbm_ctx* h, cudaError_t e, const char* where) {
 // beside the boundary kernel 196 / 165, 8192 205 / 346): a lane group sums in
 // another order, and a line at some grid size would let a domain and its slabs
 // differ in the last bits.  chem_lanes or the autotuner select them.
-// Batch plans take one launch per kernel (six reactors and flames of 69k nodes in
-// all, FP64: 0.67 ms per step against 1.15 as a single launch over the work-list,
+// Batch plans take one launch per kernel (eight reactors and flames of 93k nodes in
+// all, FP64: 0.89 ms per step against 1.24 as a single launch over the work-list,
 // whose registers the kernels' largest stage sets).
 constexpr long long kLaneNodes = 152LL * 128 / 4;   // four lanes each: one block per SM
 Launch resolve_launch(const lbm_launch& opt, long long nodes, long long n_if,

@@ -61,9 +61,9 @@ template <typename RT> constexpr bool kFF = sizeof(RT) == 4 && !LBM_CHEM64;
 template <typename RT> struct ChemType { using type = double; };
 template <> struct ChemType<float> { using type = std::conditional_t<LBM_CHEM64 != 0, double, ff>; };
 // resident blocks per SM the moments kernels are compiled for (register cap):
-// four (128 registers): with three (168) the FP64 kernel took 1.34 ms on the
-// 600x40x40 tube, with four 1.15, its 460 bytes of spills included; FP32 with
-// FP64 chemistry on the 2000x40 channel 0.19 ms with two, 0.11 with four
+// four (128 registers, FP64 spills 340 bytes): with three (168) ten FP64 steps of
+// the 600x40x40 tube took 63.7 ms against 60.9, a 61x37x29 box 13.5 against 10.7, an
+// uneven FP32 batch 43.6 against 40.2
 constexpr int kMomentsMinBlocks = 4;
 // ... of the single-domain kernel with float-float chemistry five: 24 steps of
 // the tube 45.4 against 44.3 ms; the batch kernel, which holds its domain's
